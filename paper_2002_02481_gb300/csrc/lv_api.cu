@@ -131,15 +131,18 @@ lv_status check_sigma(const double* sigma, int64_t n)
 
 // sigma (spot-major, binary64) -> time-major binary32 pairs per cell of a
 // time row: (sigma_{i,j}, sigma_{i+1,j} - sigma_{i,j}), the difference taken
-// in binary64; row 0 is repeated when the grid has a single time node.
-void pack_sigma(const lv_surface_s* h, const double* sigma, float2* dst)
+// in binary64; row 0 is repeated when the grid has a single time node. Keeps
+// the largest sigma on the handle.
+void pack_sigma(lv_surface_s* h, const double* sigma, float2* dst)
 {
+    h->sig_max = 0.0;
     for (int j = 0; j < h->Je; ++j) {
         const int jj = j < h->J ? j : h->J - 1;
         for (int i = 0; i + 1 < h->I; ++i) {
             const double a = sigma[(size_t)i * h->J + jj];
             const double b = sigma[(size_t)(i + 1) * h->J + jj];
             dst[(size_t)j * (h->I - 1) + i] = make_float2((float)a, (float)(b - a));
+            h->sig_max = std::fmax(h->sig_max, std::fmax(a, b));
         }
     }
 }
@@ -386,13 +389,15 @@ lv::McParams base_params(const lv_surface_s* h, const McCall& c)
     P.phi = (float)h->phi;
     P.dt_d = dt;
     P.N = c.n_steps;
-    P.k0 = (uint32_t)(c.seed & 0xffffffffu);
-    P.k1 = (uint32_t)(c.seed >> 32);
+    P.rk = lv::philox_keys((uint32_t)(c.seed & 0xffffffffu), (uint32_t)(c.seed >> 32));
     P.stream_id = c.stream_id;
     P.path_begin = c.path_begin;
     P.n_paths = c.n_paths;
     P.acc_mode = h->acc_mode;
     P.method = LV_ADJ_REVERSE;
+    if (P.log_uniform && lv::index_bounded(on_s, c.n_steps, P.x0, P.rdt, P.hdt, P.sqdt2, h->sig_max, P.cell_scale,
+                                           P.cell_shift))
+        P.log_uniform = 2;
     return P;
 }
 

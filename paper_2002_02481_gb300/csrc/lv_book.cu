@@ -90,19 +90,27 @@ __device__ void build_params(const BookParams& B, int inst, McParams* out)
     P.phi = (float)o.phi;
     P.dt_d = dt;
     P.N = o.N;
-    P.k0 = (uint32_t)(run.seed & 0xffffffffu);
-    P.k1 = (uint32_t)(run.seed >> 32);
+    P.rk = philox_keys((uint32_t)(run.seed & 0xffffffffu), (uint32_t)(run.seed >> 32));
+    if (P.log_uniform && index_bounded(false, o.N, P.x0, P.rdt, P.hdt, P.sqdt2, s.sig_max, P.cell_scale,
+                                       P.cell_shift))
+        P.log_uniform = 2;
     P.stream_id = (uint32_t)o.stream_id;
     P.path_begin = 0;
     P.n_paths = o.n_paths;
     *out = P;
 }
 
+// Launch bound: four blocks of at most 128 registers, as the single-option
+// kernel (8 x 64 options, two paths per lane: 29.7 ms, five blocks 32.7, three
+// 30.9). The option's parameters live in registers here (the single-option
+// kernel reads them from the parameter bank), so the forward pairs stay scalar:
+// packed, with their constants doubled, it took 30.0 ms.
+//
 // PPL: paths per lane of a forward tile, as in the single-option kernel: a
 // warp claims PPL consecutive 32-path tiles of its item and runs them
 // interleaved; the ring groups and the FIFO grow with it.
 template <int KCK, int PPL>
-__global__ void __launch_bounds__(128, 5) book_kernel(const __grid_constant__ BookParams B)
+__global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ BookParams B)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int kSlots = 32 * PPL;
@@ -148,7 +156,8 @@ __global__ void __launch_bounds__(128, 5) book_kernel(const __grid_constant__ Bo
         }
         if (tid == 0) s_ctl[1] = it.first_tile;
         __syncthreads();
-        const McParams P = *s_par;
+        McParams P = *s_par;
+        P.rk = philox_keys(P.rk.k[0], P.rk.k[1]);        // two registers, the other round keys by adds
         const int tile_end = it.first_tile + it.n_tiles;
 
         // per-thread binary64 sums in shared memory (keeps them out of the sweep's registers)
@@ -189,8 +198,7 @@ __global__ void __launch_bounds__(128, 5) book_kernel(const __grid_constant__ Bo
                     path_counter(P, rel_a, c1a, c2a);
                     path_counter(P, rel_b, c1b, c2b);
                     float ya, yb;
-                    forward_path2<KCK, true, false>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a, ckw + slot_b, cks, rel_a,
-                                                    rel_b, false, ya, yb);
+                    forward_path2<KCK, true>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a, ckw + slot_b, cks, ya, yb);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         if (h == 1 && !act_b) break;

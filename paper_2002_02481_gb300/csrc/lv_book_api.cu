@@ -378,6 +378,7 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
         bs.cell_shift = h->cell_shift;
         bs.s_lo = h->s_lo;
         bs.s_hi = h->s_hi;
+        bs.sig_max = h->sig_max;
         bs.off_sig2 = n_sig;
         bs.off_node = n_node;
         bs.off_ab = n_ab;

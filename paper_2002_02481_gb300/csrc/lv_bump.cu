@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(256) bump_kernel(const __grid_constant__ BumpP
             const uint32_t c2 = ((uint32_t)(p >> 32) & 0xffffu) | (P.stream_id << 16);
             float z[4];
             for (int n0 = 0; n0 < P.N; n0 += 4) {
-                normals4((uint32_t)(n0 >> 2), c1, c2, P.k0, P.k1, z);
+                normals4((uint32_t)(n0 >> 2), c1, c2, P.rk, z);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int n = n0 + q;
@@ -118,8 +118,8 @@ __global__ void __launch_bounds__(256) bump_kernel(const __grid_constant__ BumpP
                         if (!used[k]) continue;
                         StepEval e = eval_sigma<false>(P, g, x[k], tb);
                         // time weight of the bumped node: column j (1 - v) or j + 1 (v)
-                        if (b_row[k] == tb.z || b_row[k] == tb.z + P.I) {
-                            const float wt = b_row[k] == tb.z ? 1.0f - v : v;
+                        if (b_row[k] == tb.y || b_row[k] == tb.y + P.I) {
+                            const float wt = b_row[k] == tb.y ? 1.0f - v : v;
                             const float ws = b_i[k] == e.i ? 1.0f - e.u : (b_i[k] == e.i + 1 ? e.u : 0.0f);
                             e.sigma = fmaf(b_h[k], ws * wt, e.sigma);
                         }

@@ -17,13 +17,14 @@ __global__ void normals_kernel(uint32_t k0, uint32_t k1, uint32_t stream_id, con
     const uint32_t c1 = (uint32_t)p;
     const uint32_t c2 = ((uint32_t)(p >> 32) & 0xffffu) | (stream_id << 16);
     uint32_t w0 = blocks[e], w1 = c1, w2 = c2, w3 = 0u;
-    philox4x32_10(w0, w1, w2, w3, k0, k1);
+    const PhiloxKeys K = philox_keys(k0, k1);
+    philox4x32_10(w0, w1, w2, w3, K);
     words[4 * e + 0] = w0;
     words[4 * e + 1] = w1;
     words[4 * e + 2] = w2;
     words[4 * e + 3] = w3;
     float zz[4];
-    normals4(blocks[e], c1, c2, k0, k1, zz);
+    normals4(blocks[e], c1, c2, K, zz);
     for (int q = 0; q < 4; ++q) z[4 * e + q] = zz[q];
 }
 
@@ -32,7 +33,7 @@ __global__ void time_table_kernel(const McParams P, int* __restrict__ out_j, flo
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= P.N) return;
     const int4 tb = step_time(P, n);
-    out_j[n] = tb.z / P.I;                    // tb.z is the bucket row j I
+    out_j[n] = tb.y / P.I;                    // tb.y is the bucket row j I
     out_v[n] = __int_as_float(tb.w);
 }
 

@@ -13,20 +13,18 @@ namespace lv {
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two
 // 32x32->64-bit products and xors with a Weyl-sequence key schedule.
 __device__ __forceinline__ void philox4x32_10(uint32_t& c0, uint32_t& c1, uint32_t& c2,
-                                              uint32_t& c3, uint32_t k0, uint32_t k1)
+                                              uint32_t& c3, const PhiloxKeys& K)
 {
 #pragma unroll
     for (int round = 0; round < 10; ++round) {
         const unsigned long long p0 = (unsigned long long)0xD2511F53u * c0;
         const unsigned long long p1 = (unsigned long long)0xCD9E8D57u * c2;
-        const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k0;
-        const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k1;
+        const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ K.k[2 * round];
+        const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ K.k[2 * round + 1];
         c1 = (uint32_t)p1;
         c3 = (uint32_t)p0;
         c0 = n0;
         c2 = n2;
-        k0 += 0x9E3779B9u;
-        k1 += 0xBB67AE85u;
     }
 }
 
@@ -63,11 +61,11 @@ __device__ __forceinline__ float lg2_approx(float a)
 // rho = sqrt(-2 ln u_a). The angle is evaluated as 2 pi (u_b - 1/2) (exact
 // shift, keeps the hardware sine/cosine inside [-pi, pi)), which flips the
 // sign of both: cos(a + pi) = -cos a, sin(a + pi) = -sin a.
-__device__ __forceinline__ void normals4(uint32_t blk, uint32_t c1, uint32_t c2, uint32_t k0,
-                                         uint32_t k1, float z[4])
+__device__ __forceinline__ void normals4(uint32_t blk, uint32_t c1, uint32_t c2, const PhiloxKeys& K,
+                                         float z[4])
 {
     uint32_t w0 = blk, w1 = c1, w2 = c2, w3 = 0u;
-    philox4x32_10(w0, w1, w2, w3, k0, k1);
+    philox4x32_10(w0, w1, w2, w3, K);
     const float m2ln2 = -1.3862943611198906f;   // -2 ln 2
     const float two_pi = 6.2831853071795865f;
     {
@@ -143,17 +141,24 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
     return r;
 }
 
+__device__ __forceinline__ f32x2 add2_rd(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // The normals of normals4 for two paths at once, as pairs (path a, path b),
 // NEGATED: nz[q] = (-Z_q of a, -Z_q of b), i.e. rho cos / rho sin of the
 // shifted angle without normals4's sign flip. Every element is rounded as in
 // normals4 (a negation is exact), so -nz[q] is normals4's z[q] bit for bit.
 __device__ __forceinline__ void normals4x2_neg(uint32_t blk, uint32_t c1a, uint32_t c2a, uint32_t c1b, uint32_t c2b,
-                                               uint32_t k0, uint32_t k1, f32x2 nz[4])
+                                               const PhiloxKeys& K, f32x2 nz[4])
 {
     uint32_t a0 = blk, a1 = c1a, a2 = c2a, a3 = 0u;
     uint32_t b0 = blk, b1 = c1b, b2 = c2b, b3 = 0u;
-    philox4x32_10(a0, a1, a2, a3, k0, k1);
-    philox4x32_10(b0, b1, b2, b3, k0, k1);
+    philox4x32_10(a0, a1, a2, a3, K);
+    philox4x32_10(b0, b1, b2, b3, K);
     const f32x2 one_m = pk2(__uint_as_float(0x3f7fffffu), __uint_as_float(0x3f7fffffu));
     const f32x2 half = pk2(0.5f, 0.5f);
     const f32x2 m2ln2 = pk2(-1.3862943611198906f, -1.3862943611198906f);
@@ -187,11 +192,11 @@ __device__ __forceinline__ void normals4x2_neg(uint32_t blk, uint32_t c1a, uint3
 // (0, 2) and (1, 3) of its binary32 arithmetic in packed pairs: the uniforms'
 // shift, the -2 ln 2 scale, the angle's shift and scale, and the rho cos / rho
 // sin products, each element rounded as in normals4.
-__device__ __forceinline__ void normals4_neg(uint32_t blk, uint32_t c1, uint32_t c2, uint32_t k0, uint32_t k1,
+__device__ __forceinline__ void normals4_neg(uint32_t blk, uint32_t c1, uint32_t c2, const PhiloxKeys& K,
                                              float nz[4])
 {
     uint32_t w0 = blk, w1 = c1, w2 = c2, w3 = 0u;
-    philox4x32_10(w0, w1, w2, w3, k0, k1);
+    philox4x32_10(w0, w1, w2, w3, K);
     const f32x2 one_m = pk2(__uint_as_float(0x3f7fffffu), __uint_as_float(0x3f7fffffu));
     const f32x2 u02 = sub2(pk2(__uint_as_float((w0 >> 9) | 0x3f800000u), __uint_as_float((w2 >> 9) | 0x3f800000u)),
                            one_m);
@@ -214,8 +219,9 @@ __device__ __forceinline__ void normals4_neg(uint32_t blk, uint32_t c1, uint32_t
 
 // Time data of step n: t_n = n dt, j_n = the largest j <= J-2 with
 // tau_j <= t_n, v_n = (t_n - tau_j) / (tau_{j+1} - tau_j) clamped to
-// [0, 1], decided in binary64. Returned as (j (I-1), (j+1) (I-1), j I, bits
-// of v): the rows of the sigma pairs for j and j + 1 and the bucket row.
+// [0, 1], decided in binary64. Returned as (j (I-1), j I, bits of v twice):
+// the row of the sigma pairs for j (row j + 1 is I - 1 pairs further on), the
+// bucket row, and v as the pair the packed arithmetic takes.
 __device__ __forceinline__ int4 step_time(const McParams& P, int n)
 {
     const double t = (double)n * P.dt_d;
@@ -232,7 +238,8 @@ __device__ __forceinline__ int4 step_time(const McParams& P, int n)
         v = (t - P.tau[j]) / (P.tau[j + 1] - P.tau[j]);
         v = fmin(fmax(v, 0.0), 1.0);
     }
-    return make_int4(j * (P.I - 1), (j + 1) * (P.I - 1), j * P.I, __float_as_int((float)v));
+    const int vb = __float_as_int((float)v);
+    return make_int4(j * (P.I - 1), j * P.I, vb, vb);
 }
 
 // Time slope factor of step n for d price / d T: (n / N) / (tau_{j+1} - tau_j)
@@ -253,19 +260,35 @@ __device__ __forceinline__ float step_tdt(const McParams& P, int n)
 
 // Shared-memory view of the grid for one block.
 struct SmemGrid {
-    const int4* tab;       // [N] per step: (j (I-1), (j+1) (I-1), j I, bits of v)
+    const int4* tab;       // [N] per step: (j (I-1), j I, bits of v, bits of v)
     const float2* sig2;    // [Je][I-1]: (sigma_{i,j}, sigma_{i+1,j} - sigma_{i,j})
     const float* node;     // [I]
     const float2* ab;      // [I - 1]
     const float* tdt;      // [N] step_tdt (kernels that compute d price / d T)
 };
 
+// floor(c) clamped to [0, I-2] for |c| < 2^22 (the launcher's bound on every
+// path of the call, McParams::log_uniform == 2): adding 1.5 * 2^23 rounded
+// down leaves floor(c) in the low bits, and one integer instruction takes the
+// offset off and clamps both sides. A float-to-integer conversion would hold
+// the transcendental unit for 8 cycles a warp, as long as a sine.
+constexpr float kFloorShift = 12582912.0f;          // 1.5 * 2^23 = 0x4B400000
+constexpr int kFloorBits = 0x4B400000;
+
+__device__ __forceinline__ int clamp_floor(const McParams& P, float shifted)
+{
+    return __viaddmin_s32_relu(__float_as_int(shifted), -kFloorBits, P.I - 2);
+}
+
 // Spot cell: the largest i <= I-2 with s_i <= S. On log-uniform grids the
 // index comes from y = log2 S directly (off by one only when S is within
 // binary32 rounding of a node, where the clamped weight gives the same
-// value); on other grids a binary search over the nodes.
+// value); on other grids a binary search over the nodes. FAST: the call has
+// log_uniform == 2 (same index, no branch inside the step).
+template <bool FAST = false>
 __device__ __forceinline__ int spot_cell(const McParams& P, const SmemGrid& g, float y, float S)
 {
+    if (FAST) return clamp_floor(P, __fadd_rd(fmaf(y, P.cell_scale, P.cell_shift), kFloorShift));
     if (P.log_uniform) {
         const int i = __float2int_rd(fmaf(y, P.cell_scale, P.cell_shift));
         return min(max(i, 0), P.I - 2);
@@ -301,7 +324,7 @@ struct StepEval {
 // slope only when WANT_SLOPE. With the ln-S weight the cell coefficients ab
 // are (1 / (y_{i+1} - y_i), -y_i / (y_{i+1} - y_i)) in y = log2 s, so that
 // d u / d ln S = ab.x log2(e); otherwise they are in S.
-template <bool WANT_SLOPE, int MODEL = 0>
+template <bool WANT_SLOPE, int MODEL = 0, bool FAST = false>
 __device__ __forceinline__ StepEval eval_sigma(const McParams& P, const SmemGrid& g, float x,
                                                const int4& tb)
 {
@@ -314,11 +337,11 @@ __device__ __forceinline__ StepEval eval_sigma(const McParams& P, const SmemGrid
         e.S = ex2_approx(x);
         y = x;
     }
-    e.i = spot_cell(P, g, y, e.S);
+    e.i = spot_cell<FAST>(P, g, y, e.S);
     const float2 ab = g.ab[e.i];
     e.u = __saturatef(fmaf((MODEL & kModelLogWeight) ? y : e.S, ab.x, ab.y));
     const float2 lo = g.sig2[tb.x + e.i];      // time row j:     sigma_{i,j},   its spot step
-    const float2 hi = g.sig2[tb.y + e.i];      // time row j + 1
+    const float2 hi = g.sig2[tb.x + e.i + (P.I - 1)];   // time row j + 1
     const float v = __int_as_float(tb.w);
     const float top = fmaf(e.u, lo.y, lo.x);
     const float bot = fmaf(e.u, hi.y, hi.x);
@@ -432,142 +455,186 @@ __device__ __forceinline__ void log_cell_decision(const McParams& P, const SmemG
     }
 }
 
+// The time loop of a forward pass: blocks of four steps on four normals,
+// every block but the last without a bound check. The next block's normals
+// are computed in the same straight-line code as the current block's steps:
+// the Philox products (FMA pipe) and the Box-Muller functions (transcendental
+// unit) then fill the latencies of the steps' loads instead of forming phases
+// of their own in which every warp waits for the same pipe (forward only, 2^20
+// paths: 0.265 -> 0.238 ms; with the body unrolled over two blocks 0.226 ms; the
+// slope-carrying loops spill when unrolled and take one block). PIPE false: the
+// plain loop, for grids whose cell search branches inside the step anyway.
+// `first(blk)` runs before a block's steps, `gen(blk, z)` makes its normals,
+// `step(n, z)` is one step.
+template <typename Z, bool PIPE, int UNROLL, typename First, typename Gen, typename Step>
+__device__ __forceinline__ void time_blocks(int N, First&& first, Gen&& gen, Step&& step)
+{
+    const int nb = (N + 3) >> 2;
+    Z z[4];
+    if constexpr (!PIPE) {
+        for (int blk = 0; blk < nb; ++blk) {
+            first(blk);
+            gen((uint32_t)blk, z);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (4 * blk + q < N) step(4 * blk + q, z[q]);
+        }
+        return;
+    }
+    gen(0u, z);
+#pragma unroll UNROLL
+    for (int blk = 0; blk < nb - 1; ++blk) {
+        first(blk);
+        Z zn[4];
+        gen((uint32_t)(blk + 1), zn);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) step(4 * blk + q, z[q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z[q] = zn[q];
+    }
+    first(nb - 1);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (4 * (nb - 1) + q < N) step(4 * (nb - 1) + q, z[q]);
+}
+
 // Forward pass of one path from x0; checkpoints every KCK steps when STORE.
+template <int KCK, bool STORE, bool DBG, int MODEL, bool FAST>
+__device__ __forceinline__ float forward_path_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
+                                                float* ck, size_t cks, long long rel)
+{
+    float x = P.x0;
+    time_blocks<float, FAST, 2>(
+        P.N, [&](int blk) { if (STORE && (blk * 4) % KCK == 0) ck[(size_t)(blk * 4 / KCK) * cks] = x; },
+        [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
+        [&](int n, float z) {
+            const StepEval e = eval_sigma<false, MODEL, FAST>(P, g, x, g.tab[n]);
+            if (DBG) log_cell_decision(P, g, e, rel, n);
+            x = step_state<MODEL>(P, x, e.sigma, z);
+        });
+    return x;
+}
+
 template <int KCK, bool STORE, bool DBG, int MODEL = 0>
 __device__ __forceinline__ float forward_path(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                               float* ck, size_t cks, long long rel)
 {
-    float x = P.x0;
-    float z[4];
-    const int nseg = (P.N + KCK - 1) / KCK;
-    for (int m = 0; m < nseg; ++m) {
-        if (STORE) ck[(size_t)m * cks] = x;
-#pragma unroll
-        for (int q = 0; q < KCK; ++q) {
-            const int n = m * KCK + q;
-            if (n < P.N) {
-                if ((q & 3) == 0) normals4((uint32_t)(n >> 2), c1, c2, P.k0, P.k1, z);
-                const int4 tb = g.tab[n];
-                const StepEval e = eval_sigma<false, MODEL>(P, g, x, tb);
-                if (DBG) log_cell_decision(P, g, e, rel, n);
-                x = step_state<MODEL>(P, x, e.sigma, z[q & 3]);
-            }
-        }
-    }
-    return x;
+    if (!DBG && P.log_uniform == 2) return forward_path_f<KCK, STORE, DBG, MODEL, true>(P, g, c1, c2, ck, cks, rel);
+    return forward_path_f<KCK, STORE, DBG, MODEL, false>(P, g, c1, c2, ck, cks, rel);
 }
 
 // Forward passes of two paths, interleaved so the scheduler has two
 // independent dependency chains; each path's arithmetic is exactly that of
 // forward_path (its checkpoints and terminal state are bit-identical), and
-// the per-step time data is loaded once for both. Path b is logged only
-// when log_b (it may lie past the end of the call's range). With PACK (every
-// reading, no logging) the two paths' binary32 arithmetic runs in packed
-// pairs: the Box-Muller products and shifts, the spot-cell index, the time
-// blend of sigma and the whole Euler step (on y = log2 S or on S); the loads
-// and the transcendental unit stay per path. The step uses sqdt2 Z =
-// (-sqdt2)(-Z) (sqdt Z on S), exact, so the negated normals need no sign flip.
-template <int KCK, bool STORE, bool DBG, int MODEL = 0, bool PACK = false>
-__device__ __forceinline__ void forward_path2(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
-                                              uint32_t c1b, uint32_t c2b, float* cka, float* ckb, size_t cks,
-                                              long long rel_a, long long rel_b, bool log_b, float& ya_out,
-                                              float& yb_out)
+// the per-step time data is loaded once for both. With PACK the two paths'
+// binary32 arithmetic runs in packed pairs: the Box-Muller products and
+// shifts, the spot-cell index, the time blend of sigma and the whole Euler
+// step (on y = log2 S or on S); the loads and the transcendental unit stay per
+// path. The step uses sqdt2 Z = (-sqdt2)(-Z) (sqdt Z on S), exact, so the
+// negated normals need no sign flip.
+template <int KCK, bool STORE, int MODEL, bool PACK, bool FAST>
+__device__ __forceinline__ void forward_path2_f(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
+                                                uint32_t c1b, uint32_t c2b, float* cka, float* ckb, size_t cks,
+                                                float& ya_out, float& yb_out)
 {
-    const int nseg = (P.N + KCK - 1) / KCK;
-    if constexpr (PACK && !DBG) {
+    if constexpr (PACK) {
         // the path state x is y = log2 S (log-Euler) or S (Euler on S)
         constexpr bool kOnS = (MODEL & kModelEulerS) != 0, kLnW = (MODEL & kModelLogWeight) != 0;
         const f32x2 csc = pk2(P.cell_scale, P.cell_scale), csh = pk2(P.cell_shift, P.cell_shift);
         const f32x2 nsq = pk2(-P.sqdt2, -P.sqdt2), nhdt = pk2(-P.hdt, -P.hdt), rdt = pk2(P.rdt, P.rdt);
-        const f32x2 nsqdt = pk2(-P.sqdt, -P.sqdt);
+        const f32x2 nsqdt = pk2(-P.sqdt, -P.sqdt), fsh = pk2(kFloorShift, kFloorShift);
         f32x2 x = pk2(P.x0, P.x0);
-        f32x2 nz[4];
-        for (int m = 0; m < nseg; ++m) {
-            if (STORE) {
-                cka[(size_t)m * cks] = lo2(x);
-                ckb[(size_t)m * cks] = hi2(x);
-            }
-#pragma unroll
-            for (int q = 0; q < KCK; ++q) {
-                const int n = m * KCK + q;
-                if (n < P.N) {
-                    if ((q & 3) == 0) normals4x2_neg((uint32_t)(n >> 2), c1a, c2a, c1b, c2b, P.k0, P.k1, nz);
-                    const int4 tb = g.tab[n];
-                    const float v = __int_as_float(tb.w);
-                    // eval_sigma<false, MODEL> for both paths
-                    float Sa, Sb;
-                    f32x2 y;
-                    if (kOnS) {
-                        Sa = lo2(x);
-                        Sb = hi2(x);
-                        y = pk2(lg2_approx(fmaxf(Sa, 1e-30f)), lg2_approx(fmaxf(Sb, 1e-30f)));
-                    } else {
-                        y = x;
-                        Sa = ex2_approx(lo2(y));
-                        Sb = ex2_approx(hi2(y));
-                    }
-                    int ia, ib;
-                    if (P.log_uniform) {
-                        const f32x2 ci = fma2(y, csc, csh);
-                        ia = min(max(__float2int_rd(lo2(ci)), 0), P.I - 2);
-                        ib = min(max(__float2int_rd(hi2(ci)), 0), P.I - 2);
-                    } else {
-                        ia = spot_cell(P, g, lo2(y), Sa);
-                        ib = spot_cell(P, g, hi2(y), Sb);
-                    }
-                    const float2 aba = g.ab[ia], abb = g.ab[ib];
-                    // the spot weight is linear in S, or in y = log2 S under the ln-S weight
-                    const float ua = __saturatef(fmaf(kLnW ? lo2(y) : Sa, aba.x, aba.y));
-                    const float ub = __saturatef(fmaf(kLnW ? hi2(y) : Sb, abb.x, abb.y));
-                    const float2 loa = g.sig2[tb.x + ia], hia = g.sig2[tb.y + ia];
-                    const float2 lob = g.sig2[tb.x + ib], hib = g.sig2[tb.y + ib];
-                    const f32x2 top = pk2(fmaf(ua, loa.y, loa.x), fmaf(ub, lob.y, lob.x));
-                    const f32x2 bot = pk2(fmaf(ua, hia.y, hia.x), fmaf(ub, hib.y, hib.x));
-                    const f32x2 sig = fma2(pk2(v, v), sub2(bot, top), top);
-                    if (kOnS) {
-                        // step_state: S (1 + r dt + sigma sqrt(dt) Z), sqrt(dt) Z = (-sqrt(dt))(-Z)
-                        x = fma2(x, fma2(sig, mul2(nsqdt, nz[q & 3]), rdt), x);
-                    } else {
-                        // euler_step: y + fma(sigma, sqdt2 Z, fma(-hdt sigma, sigma, rdt))
-                        const f32x2 t3 = fma2(mul2(nhdt, sig), sig, rdt);
-                        x = add2(x, fma2(sig, mul2(nsq, nz[q & 3]), t3));
-                    }
+        time_blocks<f32x2, FAST, 2>(
+            P.N,
+            [&](int blk) {
+                if (STORE && (blk * 4) % KCK == 0) {
+                    cka[(size_t)(blk * 4 / KCK) * cks] = lo2(x);
+                    ckb[(size_t)(blk * 4 / KCK) * cks] = hi2(x);
                 }
-            }
-        }
+            },
+            [&](uint32_t blk, f32x2 (&z)[4]) { normals4x2_neg(blk, c1a, c2a, c1b, c2b, P.rk, z); },
+            [&](int n, f32x2 nz) {
+                const int4 tb = g.tab[n];
+                // eval_sigma<false, MODEL> for both paths
+                float Sa, Sb;
+                f32x2 y;
+                if (kOnS) {
+                    Sa = lo2(x);
+                    Sb = hi2(x);
+                    y = pk2(lg2_approx(fmaxf(Sa, 1e-30f)), lg2_approx(fmaxf(Sb, 1e-30f)));
+                } else {
+                    y = x;
+                    Sa = ex2_approx(lo2(y));
+                    Sb = ex2_approx(hi2(y));
+                }
+                int ia, ib;
+                if (FAST) {
+                    const f32x2 ci = add2_rd(fma2(y, csc, csh), fsh);
+                    ia = clamp_floor(P, lo2(ci));
+                    ib = clamp_floor(P, hi2(ci));
+                } else {
+                    ia = spot_cell(P, g, lo2(y), Sa);
+                    ib = spot_cell(P, g, hi2(y), Sb);
+                }
+                const float2 aba = g.ab[ia], abb = g.ab[ib];
+                // the spot weight is linear in S, or in y = log2 S under the ln-S weight
+                const float ua = __saturatef(fmaf(kLnW ? lo2(y) : Sa, aba.x, aba.y));
+                const float ub = __saturatef(fmaf(kLnW ? hi2(y) : Sb, abb.x, abb.y));
+                const float2 loa = g.sig2[tb.x + ia], hia = g.sig2[tb.x + ia + (P.I - 1)];
+                const float2 lob = g.sig2[tb.x + ib], hib = g.sig2[tb.x + ib + (P.I - 1)];
+                const f32x2 top = pk2(fmaf(ua, loa.y, loa.x), fmaf(ub, lob.y, lob.x));
+                const f32x2 bot = pk2(fmaf(ua, hia.y, hia.x), fmaf(ub, hib.y, hib.x));
+                const f32x2 sig = fma2(pk2(__int_as_float(tb.z), __int_as_float(tb.w)), sub2(bot, top), top);
+                if (kOnS) {
+                    // step_state: S (1 + r dt + sigma sqrt(dt) Z), sqrt(dt) Z = (-sqrt(dt))(-Z)
+                    x = fma2(x, fma2(sig, mul2(nsqdt, nz), rdt), x);
+                } else {
+                    // euler_step: y + fma(sigma, sqdt2 Z, fma(-hdt sigma, sigma, rdt))
+                    const f32x2 t3 = fma2(mul2(nhdt, sig), sig, rdt);
+                    x = add2(x, fma2(sig, mul2(nsq, nz), t3));
+                }
+            });
         ya_out = lo2(x);
         yb_out = hi2(x);
-        return;
-    }
-    float ya = P.x0, yb = P.x0;
-    float za[4], zb[4];
-    for (int m = 0; m < nseg; ++m) {
-        if (STORE) {
-            cka[(size_t)m * cks] = ya;
-            ckb[(size_t)m * cks] = yb;
-        }
+    } else {
+        struct Z2 { float a, b; };
+        float ya = P.x0, yb = P.x0;
+        time_blocks<Z2, FAST, 2>(
+            P.N,
+            [&](int blk) {
+                if (STORE && (blk * 4) % KCK == 0) {
+                    cka[(size_t)(blk * 4 / KCK) * cks] = ya;
+                    ckb[(size_t)(blk * 4 / KCK) * cks] = yb;
+                }
+            },
+            [&](uint32_t blk, Z2 (&z)[4]) {
+                float za[4], zb[4];
+                normals4(blk, c1a, c2a, P.rk, za);
+                normals4(blk, c1b, c2b, P.rk, zb);
 #pragma unroll
-        for (int q = 0; q < KCK; ++q) {
-            const int n = m * KCK + q;
-            if (n < P.N) {
-                if ((q & 3) == 0) {
-                    normals4((uint32_t)(n >> 2), c1a, c2a, P.k0, P.k1, za);
-                    normals4((uint32_t)(n >> 2), c1b, c2b, P.k0, P.k1, zb);
-                }
+                for (int q = 0; q < 4; ++q) z[q] = Z2{za[q], zb[q]};
+            },
+            [&](int n, Z2 z) {
                 const int4 tb = g.tab[n];
-                const StepEval ea = eval_sigma<false, MODEL>(P, g, ya, tb);
-                const StepEval eb = eval_sigma<false, MODEL>(P, g, yb, tb);
-                if (DBG) {
-                    log_cell_decision(P, g, ea, rel_a, n);
-                    if (log_b) log_cell_decision(P, g, eb, rel_b, n);
-                }
-                ya = step_state<MODEL>(P, ya, ea.sigma, za[q & 3]);
-                yb = step_state<MODEL>(P, yb, eb.sigma, zb[q & 3]);
-            }
-        }
+                const StepEval ea = eval_sigma<false, MODEL, FAST>(P, g, ya, tb);
+                const StepEval eb = eval_sigma<false, MODEL, FAST>(P, g, yb, tb);
+                ya = step_state<MODEL>(P, ya, ea.sigma, z.a);
+                yb = step_state<MODEL>(P, yb, eb.sigma, z.b);
+            });
+        ya_out = ya;
+        yb_out = yb;
     }
-    ya_out = ya;
-    yb_out = yb;
+}
+
+template <int KCK, bool STORE, int MODEL = 0, bool PACK = false>
+__device__ __forceinline__ void forward_path2(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
+                                              uint32_t c1b, uint32_t c2b, float* cka, float* ckb, size_t cks,
+                                              float& ya_out, float& yb_out)
+{
+    if (P.log_uniform == 2)
+        forward_path2_f<KCK, STORE, MODEL, PACK, true>(P, g, c1a, c2a, c1b, c2b, cka, ckb, cks, ya_out, yb_out);
+    else
+        forward_path2_f<KCK, STORE, MODEL, PACK, false>(P, g, c1a, c2a, c1b, c2b, cka, ckb, cks, ya_out, yb_out);
 }
 
 // Philox counter words of path `rel` of the call: c1 = path bits 0..31,
@@ -592,33 +659,40 @@ __device__ __forceinline__ void path_counter(const McParams& P, long long rel, u
 // With NEG (no extra sums) the recompute takes its normals from
 // normals4_neg and uses sqdt Z = (-sqdt)(-Z) and sqdt2 Z = (-sqdt2)(-Z),
 // which are exact, so every value is the same bit for bit.
-template <int KCK, int MODEL = 0, bool EXTRA = false, bool NEG = false>
-__device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                              const float* ck, size_t cks, float xbar, float* l1,
-                                              float* rho_acc = nullptr, float* t_acc = nullptr)
+template <int KCK, int MODEL, bool EXTRA, bool NEG, bool FAST>
+__device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
+                                                const float* ck, size_t cks, float xbar, float* l1, float* rho_acc,
+                                                float* t_acc)
 {
+    constexpr bool kNeg = NEG && !EXTRA;
     const int nseg = (P.N + KCK - 1) / KCK;
     int cur = -1;
     float A = 0.0f, AU = 0.0f, Bs = 0.0f, BU = 0.0f;
-    float z[4];
-    float x_next = ck[(size_t)(nseg - 1) * cks];
-    for (int m = nseg - 1; m >= 0; --m) {
-        float x = x_next;
-        if (m > 0) x_next = ck[(size_t)(m - 1) * cks];    // in flight during this segment
+    auto flush = [&]() {
+        float* p0 = l1 + cur;
+        float* p1 = p0 + P.I;
+        atomicAdd(p0, A - AU);
+        atomicAdd(p0 + 1, AU);
+        atomicAdd(p1, Bs - BU);
+        atomicAdd(p1 + 1, BU);
+    };
+    auto gen = [&](int blk, float (&z)[4]) {
+        if (kNeg) normals4_neg((uint32_t)blk, c1, c2, P.rk, z);
+        else normals4((uint32_t)blk, c1, c2, P.rk, z);
+    };
+    // one segment of up to KCK steps; ALL: every step of it is below N
+    auto segment = [&](int m, float x, const float (&zf)[4], bool all) {
         float hq[KCK], gq[KCK], uq[KCK];
         float aq[EXTRA ? KCK : 1], tq[EXTRA ? KCK : 1];
         int iq[KCK];
+        float z[4] = { zf[0], zf[1], zf[2], zf[3] };
 #pragma unroll
         for (int q = 0; q < KCK; ++q) {
             const int n = m * KCK + q;
-            if (n < P.N) {
-                constexpr bool kNeg = NEG && !EXTRA;
-                if ((q & 3) == 0) {
-                    if (kNeg) normals4_neg((uint32_t)(n >> 2), c1, c2, P.k0, P.k1, z);
-                    else normals4((uint32_t)(n >> 2), c1, c2, P.k0, P.k1, z);
-                }
+            if (all || n < P.N) {
+                if (q > 0 && (q & 3) == 0) gen(n >> 2, z);
                 const int4 tb = g.tab[n];
-                const StepEval ev = eval_sigma<true, MODEL>(P, g, x, tb);
+                const StepEval ev = eval_sigma<true, MODEL, FAST>(P, g, x, tb);
                 if (kNeg) {                    // z holds -Z: adjoint_factors with sqrt(dt) Z = (-sqrt(dt))(-Z)
                     if (MODEL & kModelEulerS) {
                         const float w = -P.sqdt * z[q & 3];
@@ -642,9 +716,9 @@ __device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid&
 #pragma unroll
         for (int q = KCK - 1; q >= 0; --q) {
             const int n = m * KCK + q;
-            if (n < P.N) {
+            if (all || n < P.N) {
                 const int4 tb = g.tab[n];
-                const int key = tb.z + iq[q];
+                const int key = tb.y + iq[q];
                 const float v = __int_as_float(tb.w);
                 const float sbar = xbar * hq[q];
                 if (EXTRA) {                             // xbar is still xbar_{n+1}
@@ -653,14 +727,7 @@ __device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid&
                 }
                 xbar = fmaf(xbar, gq[q], xbar);
                 if (key != cur) {
-                    if (cur >= 0) {
-                        float* p0 = l1 + cur;
-                        float* p1 = p0 + P.I;
-                        atomicAdd(p0, A - AU);
-                        atomicAdd(p0 + 1, AU);
-                        atomicAdd(p1, Bs - BU);
-                        atomicAdd(p1 + 1, BU);
-                    }
+                    if (cur >= 0) flush();
                     A = AU = Bs = BU = 0.0f;
                     cur = key;
                 }
@@ -672,16 +739,34 @@ __device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid&
                 BU = fmaf(b, uq[q], BU);
             }
         }
+    };
+    float x = ck[(size_t)(nseg - 1) * cks];
+    float z[4];
+    gen((nseg - 1) * (KCK / 4), z);
+    for (int m = nseg - 1; m >= 0; --m) {
+        // the next segment's checkpoint and first normals, in flight during this one
+        const int mp = max(m - 1, 0);
+        const float xn = ck[(size_t)mp * cks];
+        float zn[4];
+        gen(mp * (KCK / 4), zn);
+        if (FAST && (m + 1) * KCK <= P.N) segment(m, x, z, true);
+        else segment(m, x, z, false);
+        x = xn;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z[q] = zn[q];
     }
-    if (cur >= 0) {
-        float* p0 = l1 + cur;
-        float* p1 = p0 + P.I;
-        atomicAdd(p0, A - AU);
-        atomicAdd(p0 + 1, AU);
-        atomicAdd(p1, Bs - BU);
-        atomicAdd(p1 + 1, BU);
-    }
+    if (cur >= 0) flush();
     return xbar;
+}
+
+template <int KCK, int MODEL = 0, bool EXTRA = false, bool NEG = false>
+__device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
+                                              const float* ck, size_t cks, float xbar, float* l1,
+                                              float* rho_acc = nullptr, float* t_acc = nullptr)
+{
+    if (P.log_uniform == 2)
+        return reverse_path_f<KCK, MODEL, EXTRA, NEG, true>(P, g, c1, c2, ck, cks, xbar, l1, rho_acc, t_acc);
+    return reverse_path_f<KCK, MODEL, EXTRA, NEG, false>(P, g, c1, c2, ck, cks, xbar, l1, rho_acc, t_acc);
 }
 
 // Tangent-ratio form of the pathwise adjoint (Sec. III: the adjoint
@@ -693,33 +778,34 @@ __device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid&
 // D_N; `tiny` is set when some |1 + g_n| < 2^-20, where dividing by D loses
 // what the reverse sweep keeps. The path's arithmetic is that of
 // forward_path (same sigma, same Euler step), so y_N is the same.
+template <int MODEL, bool FAST>
+__device__ __forceinline__ float tangent_forward_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
+                                                   float& D, bool& tiny)
+{
+    float y = P.x0;
+    float d = 1.0f, fmin = 1.0f;
+    time_blocks<float, FAST, 1>(
+        P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
+        [&](int n, float z) {
+            const StepEval e = eval_sigma<true, MODEL, FAST>(P, g, y, g.tab[n]);
+            float h, gn;
+            adjoint_factors<MODEL>(P, e, z, h, gn);
+            const float f = tangent_factor<MODEL>(P, e, z, h);   // 1 + g_n
+            fmin = fminf(fmin, fabsf(f));
+            d *= f;
+            y = step_state<MODEL>(P, y, e.sigma, z);
+        });
+    D = d;
+    tiny = fmin < 0x1p-20f;
+    return y;
+}
+
 template <int MODEL = 0>
 __device__ __forceinline__ float tangent_forward(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                                  float& D, bool& tiny)
 {
-    float y = P.x0;
-    float d = 1.0f, fmin = 1.0f;
-    float z[4];
-    for (int n0 = 0; n0 < P.N; n0 += 4) {
-        normals4((uint32_t)(n0 >> 2), c1, c2, P.k0, P.k1, z);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int n = n0 + q;
-            if (n < P.N) {
-                const int4 tb = g.tab[n];
-                const StepEval e = eval_sigma<true, MODEL>(P, g, y, tb);
-                float h, gn;
-                adjoint_factors<MODEL>(P, e, z[q], h, gn);
-                const float f = tangent_factor<MODEL>(P, e, z[q], h);   // 1 + g_n
-                fmin = fminf(fmin, fabsf(f));
-                d *= f;
-                y = step_state<MODEL>(P, y, e.sigma, z[q]);
-            }
-        }
-    }
-    D = d;
-    tiny = fmin < 0x1p-20f;
-    return y;
+    if (P.log_uniform == 2) return tangent_forward_f<MODEL, true>(P, g, c1, c2, D, tiny);
+    return tangent_forward_f<MODEL, false>(P, g, c1, c2, D, tiny);
 }
 
 // Pass 1 for two paths at once (main reading), their binary32 arithmetic in
@@ -728,60 +814,56 @@ __device__ __forceinline__ float tangent_forward(const McParams& P, const SmemGr
 // spot factor, h = sqdt Z - sigma dt = (-sqdt)(-Z) + (-dt) sigma, 1 + g_n and
 // the product D run in pairs; the inside-grid test and the running minimum of
 // |1 + g_n| stay per path.
-__device__ __forceinline__ void tangent_forward2(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
-                                                 uint32_t c1b, uint32_t c2b, float& ya_out, float& yb_out,
-                                                 float& Da, float& Db, bool& tiny_a, bool& tiny_b)
+template <bool FAST>
+__device__ __forceinline__ void tangent_forward2_f(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
+                                                   uint32_t c1b, uint32_t c2b, float& ya_out, float& yb_out,
+                                                   float& Da, float& Db, bool& tiny_a, bool& tiny_b)
 {
     const f32x2 csc = pk2(P.cell_scale, P.cell_scale), csh = pk2(P.cell_shift, P.cell_shift);
     const f32x2 nsq2 = pk2(-P.sqdt2, -P.sqdt2), nhdt = pk2(-P.hdt, -P.hdt), rdt = pk2(P.rdt, P.rdt);
     const f32x2 nsqdt = pk2(-P.sqdt, -P.sqdt), ndt = pk2(-P.dt, -P.dt), one = pk2(1.0f, 1.0f);
+    const f32x2 fsh = pk2(kFloorShift, kFloorShift);
     f32x2 y = pk2(P.x0, P.x0), d = one;
     float fmin_a = 1.0f, fmin_b = 1.0f;
-    f32x2 nz[4];
-    for (int n0 = 0; n0 < P.N; n0 += 4) {
-        normals4x2_neg((uint32_t)(n0 >> 2), c1a, c2a, c1b, c2b, P.k0, P.k1, nz);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int n = n0 + q;
-            if (n < P.N) {
-                const int4 tb = g.tab[n];
-                const float v = __int_as_float(tb.w);
-                const f32x2 vv = pk2(v, v);
-                // eval_sigma<true, 0> for both paths
-                const float Sa = ex2_approx(lo2(y)), Sb = ex2_approx(hi2(y));
-                int ia, ib;
-                if (P.log_uniform) {
-                    const f32x2 ci = fma2(y, csc, csh);
-                    ia = min(max(__float2int_rd(lo2(ci)), 0), P.I - 2);
-                    ib = min(max(__float2int_rd(hi2(ci)), 0), P.I - 2);
-                } else {
-                    ia = spot_cell(P, g, lo2(y), Sa);
-                    ib = spot_cell(P, g, hi2(y), Sb);
-                }
-                const float2 aba = g.ab[ia], abb = g.ab[ib];
-                const float ua = __saturatef(fmaf(Sa, aba.x, aba.y));
-                const float ub = __saturatef(fmaf(Sb, abb.x, abb.y));
-                const float2 loa = g.sig2[tb.x + ia], hia = g.sig2[tb.y + ia];
-                const float2 lob = g.sig2[tb.x + ib], hib = g.sig2[tb.y + ib];
-                const f32x2 top = pk2(fmaf(ua, loa.y, loa.x), fmaf(ub, lob.y, lob.x));
-                const f32x2 bot = pk2(fmaf(ua, hia.y, hia.x), fmaf(ub, hib.y, hib.x));
-                const f32x2 sig = fma2(vv, sub2(bot, top), top);
-                const f32x2 ly = pk2(loa.y, lob.y);
-                const f32x2 sl = mul2(pk2(Sa, Sb), mul2(fma2(vv, sub2(pk2(hia.y, hib.y), ly), ly), pk2(aba.x, abb.x)));
-                const f32x2 slope = pk2((Sa >= P.s_lo) && (Sa <= P.s_hi) ? lo2(sl) : 0.0f,
-                                        (Sb >= P.s_lo) && (Sb <= P.s_hi) ? hi2(sl) : 0.0f);
-                // adjoint_factors<0> and tangent_factor<0>
-                const f32x2 h = fma2(nsqdt, nz[q], mul2(ndt, sig));
-                const f32x2 f = fma2(h, slope, one);
-                fmin_a = fminf(fmin_a, fabsf(lo2(f)));
-                fmin_b = fminf(fmin_b, fabsf(hi2(f)));
-                d = mul2(d, f);
-                // euler_step
-                const f32x2 t3 = fma2(mul2(nhdt, sig), sig, rdt);
-                y = add2(y, fma2(sig, mul2(nsq2, nz[q]), t3));
+    time_blocks<f32x2, FAST, 1>(
+        P.N, [](int) {},
+        [&](uint32_t blk, f32x2 (&z)[4]) { normals4x2_neg(blk, c1a, c2a, c1b, c2b, P.rk, z); },
+        [&](int n, f32x2 nz) {
+            const int4 tb = g.tab[n];
+            const f32x2 vv = pk2(__int_as_float(tb.z), __int_as_float(tb.w));
+            // eval_sigma<true, 0> for both paths
+            const float Sa = ex2_approx(lo2(y)), Sb = ex2_approx(hi2(y));
+            int ia, ib;
+            if (FAST) {
+                const f32x2 ci = add2_rd(fma2(y, csc, csh), fsh);
+                ia = clamp_floor(P, lo2(ci));
+                ib = clamp_floor(P, hi2(ci));
+            } else {
+                ia = spot_cell(P, g, lo2(y), Sa);
+                ib = spot_cell(P, g, hi2(y), Sb);
             }
-        }
-    }
+            const float2 aba = g.ab[ia], abb = g.ab[ib];
+            const float ua = __saturatef(fmaf(Sa, aba.x, aba.y));
+            const float ub = __saturatef(fmaf(Sb, abb.x, abb.y));
+            const float2 loa = g.sig2[tb.x + ia], hia = g.sig2[tb.x + ia + (P.I - 1)];
+            const float2 lob = g.sig2[tb.x + ib], hib = g.sig2[tb.x + ib + (P.I - 1)];
+            const f32x2 top = pk2(fmaf(ua, loa.y, loa.x), fmaf(ub, lob.y, lob.x));
+            const f32x2 bot = pk2(fmaf(ua, hia.y, hia.x), fmaf(ub, hib.y, hib.x));
+            const f32x2 sig = fma2(vv, sub2(bot, top), top);
+            const f32x2 ly = pk2(loa.y, lob.y);
+            const f32x2 sl = mul2(pk2(Sa, Sb), mul2(fma2(vv, sub2(pk2(hia.y, hib.y), ly), ly), pk2(aba.x, abb.x)));
+            const f32x2 slope = pk2((Sa >= P.s_lo) && (Sa <= P.s_hi) ? lo2(sl) : 0.0f,
+                                    (Sb >= P.s_lo) && (Sb <= P.s_hi) ? hi2(sl) : 0.0f);
+            // adjoint_factors<0> and tangent_factor<0>
+            const f32x2 h = fma2(nsqdt, nz, mul2(ndt, sig));
+            const f32x2 f = fma2(h, slope, one);
+            fmin_a = fminf(fmin_a, fabsf(lo2(f)));
+            fmin_b = fminf(fmin_b, fabsf(hi2(f)));
+            d = mul2(d, f);
+            // euler_step
+            const f32x2 t3 = fma2(mul2(nhdt, sig), sig, rdt);
+            y = add2(y, fma2(sig, mul2(nsq2, nz), t3));
+        });
     ya_out = lo2(y);
     yb_out = hi2(y);
     Da = lo2(d);
@@ -790,61 +872,67 @@ __device__ __forceinline__ void tangent_forward2(const McParams& P, const SmemGr
     tiny_b = fmin_b < 0x1p-20f;
 }
 
+__device__ __forceinline__ void tangent_forward2(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
+                                                 uint32_t c1b, uint32_t c2b, float& ya_out, float& yb_out,
+                                                 float& Da, float& Db, bool& tiny_a, bool& tiny_b)
+{
+    if (P.log_uniform == 2)
+        tangent_forward2_f<true>(P, g, c1a, c2a, c1b, c2b, ya_out, yb_out, Da, Db, tiny_a, tiny_b);
+    else
+        tangent_forward2_f<false>(P, g, c1a, c2a, c1b, c2b, ya_out, yb_out, Da, Db, tiny_a, tiny_b);
+}
+
 // Pass 2: regenerates one path (same counters, same arithmetic) and spreads
 // sigma_bar_n = c h_n / D_{n+1}, c = xbar_N D_N, over the corner buckets of
 // its cell with the bilinear weights, through the same run-length register
 // sums and binary32 reductions into `l1` as reverse_path, in time order.
-template <int MODEL = 0>
-__device__ __forceinline__ void tangent_scatter(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                                float c, float* l1)
+template <int MODEL, bool FAST>
+__device__ __forceinline__ void tangent_scatter_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
+                                                  float c, float* l1)
 {
     float y = P.x0, d = 1.0f;
     int cur = -1;
     float A = 0.0f, AU = 0.0f, Bs = 0.0f, BU = 0.0f;
-    float z[4];
-    for (int n0 = 0; n0 < P.N; n0 += 4) {
-        normals4((uint32_t)(n0 >> 2), c1, c2, P.k0, P.k1, z);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int n = n0 + q;
-            if (n < P.N) {
-                const int4 tb = g.tab[n];
-                const StepEval e = eval_sigma<true, MODEL>(P, g, y, tb);
-                float h, gn;
-                adjoint_factors<MODEL>(P, e, z[q], h, gn);
-                d *= tangent_factor<MODEL>(P, e, z[q], h);          // D_{n+1}
-                const float sbar = __fdividef(c * h, d);
-                const int key = tb.z + e.i;
-                if (key != cur) {
-                    if (cur >= 0) {
-                        float* p0 = l1 + cur;
-                        float* p1 = p0 + P.I;
-                        atomicAdd(p0, A - AU);
-                        atomicAdd(p0 + 1, AU);
-                        atomicAdd(p1, Bs - BU);
-                        atomicAdd(p1 + 1, BU);
-                    }
-                    A = AU = Bs = BU = 0.0f;
-                    cur = key;
-                }
-                const float b = sbar * __int_as_float(tb.w);
-                const float a = sbar - b;
-                A += a;
-                AU = fmaf(a, e.u, AU);
-                Bs += b;
-                BU = fmaf(b, e.u, BU);
-                y = step_state<MODEL>(P, y, e.sigma, z[q]);
-            }
-        }
-    }
-    if (cur >= 0) {
+    auto flush = [&]() {
         float* p0 = l1 + cur;
         float* p1 = p0 + P.I;
         atomicAdd(p0, A - AU);
         atomicAdd(p0 + 1, AU);
         atomicAdd(p1, Bs - BU);
         atomicAdd(p1 + 1, BU);
-    }
+    };
+    time_blocks<float, FAST, 1>(
+        P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
+        [&](int n, float z) {
+            const int4 tb = g.tab[n];
+            const StepEval e = eval_sigma<true, MODEL, FAST>(P, g, y, tb);
+            float h, gn;
+            adjoint_factors<MODEL>(P, e, z, h, gn);
+            d *= tangent_factor<MODEL>(P, e, z, h);          // D_{n+1}
+            const float sbar = __fdividef(c * h, d);
+            const int key = tb.y + e.i;
+            if (key != cur) {
+                if (cur >= 0) flush();
+                A = AU = Bs = BU = 0.0f;
+                cur = key;
+            }
+            const float b = sbar * __int_as_float(tb.w);
+            const float a = sbar - b;
+            A += a;
+            AU = fmaf(a, e.u, AU);
+            Bs += b;
+            BU = fmaf(b, e.u, BU);
+            y = step_state<MODEL>(P, y, e.sigma, z);
+        });
+    if (cur >= 0) flush();
+}
+
+template <int MODEL = 0>
+__device__ __forceinline__ void tangent_scatter(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
+                                                float c, float* l1)
+{
+    if (P.log_uniform == 2) tangent_scatter_f<MODEL, true>(P, g, c1, c2, c, l1);
+    else tangent_scatter_f<MODEL, false>(P, g, c1, c2, c, l1);
 }
 
 // Second-order buckets d^2 price / (d S0 d sigma_ij), pass 2 of one live
@@ -859,64 +947,59 @@ __device__ __forceinline__ void tangent_scatter(const McParams& P, const SmemGri
 // nodes. Run-length sums in registers while the cell is unchanged (the
 // weight terms as in reverse_path, the slope terms E0 = sum (1 - v) d,
 // E1 = sum v d), then binary32 reductions into `l1`.
-__device__ __forceinline__ void vanna_scatter(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                              float delta, float* l1)
+template <bool FAST>
+__device__ __forceinline__ void vanna_scatter_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
+                                                float delta, float* l1)
 {
     float y = P.x0;
     int cur = -1;
     float A = 0.0f, AU = 0.0f, Bs = 0.0f, BU = 0.0f, E0 = 0.0f, E1 = 0.0f;
-    float z[4];
-    for (int n0 = 0; n0 < P.N; n0 += 4) {
-        normals4((uint32_t)(n0 >> 2), c1, c2, P.k0, P.k1, z);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int n = n0 + q;
-            if (n < P.N) {
-                const int4 tb = g.tab[n];
-                const StepEval e = eval_sigma<true, 0>(P, g, y, tb);
-                const float zq = z[q];
-                const float h = fmaf(P.sqdt, zq, -e.sigma * P.dt);
-                const float f = fmaf(h, e.sslope, 1.0f);                      // 1 + g_n
-                const float a = __fdividef(fmaf(zq, zq, -1.0f), e.sigma) -
-                                P.sqdt * zq * (1.0f + __fdividef(e.sslope, e.sigma * f));
-                const bool inside = (e.S >= P.s_lo) && (e.S <= P.s_hi);
-                const float sdu = inside ? e.S * g.ab[e.i].x : 0.0f;          // S d u / d S
-                const float c = delta * a;
-                const float d = delta * __fdividef(h, f) * sdu;
-                const int key = tb.z + e.i;
-                if (key != cur) {
-                    if (cur >= 0) {
-                        float* p0 = l1 + cur;
-                        float* p1 = p0 + P.I;
-                        atomicAdd(p0, A - AU - E0);
-                        atomicAdd(p0 + 1, AU + E0);
-                        atomicAdd(p1, Bs - BU - E1);
-                        atomicAdd(p1 + 1, BU + E1);
-                    }
-                    A = AU = Bs = BU = E0 = E1 = 0.0f;
-                    cur = key;
-                }
-                const float v = __int_as_float(tb.w);
-                const float cb = c * v, ca = c - cb;
-                const float db = d * v;
-                A += ca;
-                AU = fmaf(ca, e.u, AU);
-                Bs += cb;
-                BU = fmaf(cb, e.u, BU);
-                E0 += d - db;
-                E1 += db;
-                y = step_state<0>(P, y, e.sigma, zq);
-            }
-        }
-    }
-    if (cur >= 0) {
+    auto flush = [&]() {
         float* p0 = l1 + cur;
         float* p1 = p0 + P.I;
         atomicAdd(p0, A - AU - E0);
         atomicAdd(p0 + 1, AU + E0);
         atomicAdd(p1, Bs - BU - E1);
         atomicAdd(p1 + 1, BU + E1);
-    }
+    };
+    time_blocks<float, FAST, 1>(
+        P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
+        [&](int n, float zq) {
+            const int4 tb = g.tab[n];
+            const StepEval e = eval_sigma<true, 0, FAST>(P, g, y, tb);
+            const float h = fmaf(P.sqdt, zq, -e.sigma * P.dt);
+            const float f = fmaf(h, e.sslope, 1.0f);                      // 1 + g_n
+            const float a = __fdividef(fmaf(zq, zq, -1.0f), e.sigma) -
+                            P.sqdt * zq * (1.0f + __fdividef(e.sslope, e.sigma * f));
+            const bool inside = (e.S >= P.s_lo) && (e.S <= P.s_hi);
+            const float sdu = inside ? e.S * g.ab[e.i].x : 0.0f;          // S d u / d S
+            const float c = delta * a;
+            const float d = delta * __fdividef(h, f) * sdu;
+            const int key = tb.y + e.i;
+            if (key != cur) {
+                if (cur >= 0) flush();
+                A = AU = Bs = BU = E0 = E1 = 0.0f;
+                cur = key;
+            }
+            const float v = __int_as_float(tb.w);
+            const float cb = c * v, ca = c - cb;
+            const float db = d * v;
+            A += ca;
+            AU = fmaf(ca, e.u, AU);
+            Bs += cb;
+            BU = fmaf(cb, e.u, BU);
+            E0 += d - db;
+            E1 += db;
+            y = step_state<0>(P, y, e.sigma, zq);
+        });
+    if (cur >= 0) flush();
+}
+
+__device__ __forceinline__ void vanna_scatter(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
+                                              float delta, float* l1)
+{
+    if (P.log_uniform == 2) vanna_scatter_f<true>(P, g, c1, c2, delta, l1);
+    else vanna_scatter_f<false>(P, g, c1, c2, delta, l1);
 }
 
 }  // namespace lv

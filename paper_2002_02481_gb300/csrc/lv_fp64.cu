@@ -33,7 +33,7 @@ __device__ __forceinline__ void normals4_f64(uint32_t blk, uint32_t c1, uint32_t
                                              double z[4])
 {
     uint32_t w[4] = { blk, c1, c2, 0u };
-    philox4x32_10(w[0], w[1], w[2], w[3], k0, k1);
+    philox4x32_10(w[0], w[1], w[2], w[3], philox_keys(k0, k1));
 #pragma unroll
     for (int pair = 0; pair < 2; ++pair) {
         const double ua = ((double)(w[2 * pair] >> 9) + 0.5) * 0x1p-23;

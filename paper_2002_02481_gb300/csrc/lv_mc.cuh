@@ -200,13 +200,19 @@ __device__ __forceinline__ void drain_buckets(float* l1, int nIJ, double* wrow)
     }
 }
 
+// Launch bound: the straight-line time loops (time_blocks, reverse_path) want
+// registers more than warps. Four blocks per SM at 124-128 registers against
+// five at 96 and six at 80, same code: 0.615, 0.643 and 0.684 ms at 2^20 paths on
+// the 30 x 60 grid with 156 steps, 2.06, 2.20 and 2.30 ms at 2^22 (the loops with
+// a bound check in every step, six blocks: 0.660 and 2.23 ms).
+//
 // PPL: paths per lane of a forward tile. With PPL = 2 a warp claims two
 // consecutive 32-path tiles and runs them interleaved (forward_path2: two
 // independent dependency chains per lane, the per-step time data loaded once);
 // each path's arithmetic is that of PPL = 1, the ring groups and the FIFO
 // hold twice as many entries, and the reverse batches are unchanged.
 template <int KCK, int ACC, bool DBG, bool GS, int MODEL, bool EXTRA = false, int PPL = 1>
-__global__ void __launch_bounds__(128, 5) adjoint_kernel(const __grid_constant__ McParams P)
+__global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int kSlots = kTile * PPL;      // checkpoint slots per ring group
@@ -299,8 +305,8 @@ __global__ void __launch_bounds__(128, 5) adjoint_kernel(const __grid_constant__
                 float ya, yb;
                 // packed pairs on the log-Euler readings; Euler on S keeps scalar pairs in
                 // this kernel (packed, it needs 82 registers: 5 blocks per SM instead of 6)
-                forward_path2<KCK, true, false, MODEL, (MODEL & kModelEulerS) == 0>(
-                    P, g, c1a, c2a, c1b, c2b, ckw + slot_a, ckw + slot_b, cks, rel_a, rel_b, false, ya, yb);
+                forward_path2<KCK, true, MODEL, (MODEL & kModelEulerS) == 0>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a,
+                                                                             ckw + slot_b, cks, ya, yb);
                 float V;
                 payoff<MODEL>(P, ya, V, xa);
                 acc_add<ACC>(acc[0], V);
@@ -401,7 +407,7 @@ __global__ void __launch_bounds__(128, 5) adjoint_kernel(const __grid_constant__
 // 32 queued paths (and at the end) the warp runs pass 2 (tangent_scatter)
 // on them as a full-warp batch. Buckets go through the same levels 0-3.
 template <int ACC, bool GS, int MODEL, int PPL = 1>
-__global__ void __launch_bounds__(128, 6) tangent_kernel(const __grid_constant__ McParams P)
+__global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int B = blockDim.x, W = B >> 5;
@@ -543,7 +549,7 @@ __global__ void __launch_bounds__(128, 6) tangent_kernel(const __grid_constant__
 // binary64 level 2. Rows: price sums as usual, buckets d^2 price / (d S0 d
 // sigma_ij) summed over paths.
 template <bool GS, int PPL = 1>
-__global__ void __launch_bounds__(128, 6) vanna_kernel(const __grid_constant__ McParams P)
+__global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int B = blockDim.x;
@@ -659,8 +665,15 @@ __global__ void __launch_bounds__(128, 6) vanna_kernel(const __grid_constant__ M
     block_scalars(acc_value<0>(acc[0]), acc_value<0>(acc[B]), acc_value<0>(acc[2 * B]), s_red, row);
 }
 
+// The forward pass alone. Bound by the FMA pipe (its 64-bit integer products
+// hold it for four cycles each) and the issue slots. With the straight-line
+// time loop unrolled over two blocks of steps, the index without a conversion
+// and the round keys in the parameter bank it runs 35 thread instructions per
+// path-step (43 before): 0.229 ms at 2^20 paths on the 30 x 60 grid with 156
+// steps, from 0.265 ms. 66 registers under a bound of three 256-thread blocks;
+// held to 64 by a bound of four it spilled.
 template <int ACC, bool GS, int MODEL>
-__global__ void __launch_bounds__(256, 4) price_kernel(const __grid_constant__ McParams P)
+__global__ void __launch_bounds__(256, 3) price_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const SmemLayout L = smem_layout(P.I, P.Je, P.N, blockDim.x, false, GS);
@@ -679,8 +692,7 @@ __global__ void __launch_bounds__(256, 4) price_kernel(const __grid_constant__ M
             path_counter(P, rel_a, c1a, c2a);
             path_counter(P, rel_b, c1b, c2b);
             float ya, yb;
-            forward_path2<4, false, false, MODEL, true>(P, g, c1a, c2a, c1b, c2b, nullptr, nullptr, 0, rel_a, rel_b,
-                                                        false, ya, yb);
+            forward_path2<4, false, MODEL, true>(P, g, c1a, c2a, c1b, c2b, nullptr, nullptr, 0, ya, yb);
             float V, xb;
             payoff<MODEL>(P, ya, V, xb);
             acc_add<ACC>(acc[0], V);
