@@ -147,6 +147,47 @@ void pack_sigma(lv_surface_s* h, const double* sigma, float2* dst)
     }
 }
 
+// Cell table of a grid that is not log-uniform: equal bins in y = log2 S over
+// [y_0, y_{I-1}], narrow enough that a bin widened by a tenth on either side
+// holds at most two nodes (a width of 1.5 times the smallest gap: 1.8 gaps
+// against the two that three nodes span). Entry b: the largest cell whose node
+// is at or below the widened bin, and the next two nodes. The tenth covers the
+// binary32 rounding of y, of the bin index and of S = 2^y (about 5e-7 of y
+// together) while a bin is at least 4e-5 wide. Grids that need more than
+// kMaxBins bins, or narrower ones, keep the binary search.
+constexpr int kMaxBins = 512;
+constexpr double kMinBinWidth = 4e-5;
+
+std::vector<float4> spot_bins(const std::vector<double>& spot, float* scale, float* shift)
+{
+    const int I = (int)spot.size();
+    std::vector<double> y(I);
+    for (int i = 0; i < I; ++i) y[i] = std::log2(spot[i]);
+    double gap = y[I - 1] - y[0];
+    for (int i = 1; i < I; ++i) gap = std::fmin(gap, y[i] - y[i - 1]);
+    const double range = y[I - 1] - y[0];
+    const double want = std::ceil(range / (1.5 * gap));
+    const double ymax = std::fmax(4.0, std::fmax(std::fabs(y[0]), std::fabs(y[I - 1])));
+    if (!(want >= 1.0) || want > kMaxBins || range / want < kMinBinWidth * ymax) return {};
+    const int n = (int)want;
+    const double w = range / n;
+    std::vector<float4> bins(n);
+    int base = 0;
+    for (int b = 0; b < n; ++b) {
+        const double lo = y[0] + b * w - 0.1 * w;
+        while (base + 1 <= I - 2 && y[base + 1] <= lo) ++base;
+        float4 t;
+        std::memcpy(&t.x, &base, sizeof(float));
+        t.y = base + 1 <= I - 2 ? (float)spot[base + 1] : INFINITY;
+        t.z = base + 2 <= I - 2 ? (float)spot[base + 2] : INFINITY;
+        t.w = 0.0f;
+        bins[b] = t;
+    }
+    *scale = (float)(1.0 / w);
+    *shift = (float)(-y[0] / w);
+    return bins;
+}
+
 void free_surface(lv_surface_s* h)
 {
     if (!h) return;
@@ -155,6 +196,7 @@ void free_surface(lv_surface_s* h)
     cudaFree(h->d_ab);
     cudaFree(h->d_abl);
     cudaFree(h->d_tau);
+    cudaFree(h->d_bins);
     cudaFree(h->d_spot64);
     cudaFree(h->d_sig64);
     cudaFreeHost(h->h_sig64_stage);
@@ -204,7 +246,7 @@ constexpr size_t kGridSmemLimit = 44 * 1024;
 // sweep, binary64 level 2, k = 4 or 8).
 // Blocks per SM of one kernel instantiation and launch shape, per device:
 // the runtime's occupancy query costs microseconds, so each answer is kept.
-using OccKey = std::tuple<int, int, int, bool, int, bool, bool, int, int, bool, size_t, int>;
+using OccKey = std::tuple<int, int, int, bool, int, bool, bool, int, int, int, bool, size_t, int>;
 std::mutex g_occ_mu;
 std::map<OccKey, int> g_occ;
 
@@ -257,17 +299,22 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
                        ((vanna || h->adj_method == LV_ADJ_TANGENT) ? model == 0 : (*k == 4 || *k == 8));
     if (!pairs) ppl = 1;
     if (ppl_out) *ppl_out = ppl;
-    const bool gs = lv::mc_smem_bytes(h->I, h->Je, n_steps, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
+    const bool gs = lv::mc_smem_bytes(h->I, h->Je, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
     if (grid_smem) *grid_smem = gs;
-    const size_t smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, *block, greeks, gs, extra, ppl);
+    const size_t smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, h->n_bins, *block, greeks, gs, extra, ppl);
     if (smem > 200 * 1024)
         return fail(LV_EINVAL, "time table does not fit in shared memory (" + std::to_string(smem) + " bytes)");
     int occ = 0;
     const int acc = dbg || extra || vanna ? 0 : h->acc_mode;
     const int method = vanna ? lv::kMethodVanna : (dbg || extra ? LV_ADJ_REVERSE : h->adj_method);
-    const OccKey key{h->device, *block, *k, greeks, acc, dbg, gs, method, model, extra, smem, ppl};
+    // the cell mode of any call whose cell index is bounded (base_params)
+    const int cell = dbg || *k > lv::kModelMaxK ? lv::kCellSearch
+                     : h->log_uniform           ? lv::kCellUniform
+                     : h->n_bins > 0            ? lv::kCellBins
+                                                : lv::kCellSearch;
+    const OccKey key{h->device, *block, *k, greeks, acc, dbg, gs, method, model, cell, extra, smem, ppl};
     if (!occ_lookup(key, &occ)) {
-        LV_CUDA(lv::mc_occupancy(*block, *k, greeks, acc, dbg, gs, method, model, extra, smem, &occ, ppl));
+        LV_CUDA(lv::mc_occupancy(*block, *k, greeks, acc, dbg, gs, method, model, cell, extra, smem, &occ, ppl));
         occ_store(key, occ);
     }
     if (occ < 1) return fail(LV_EINVAL, "launch shape does not fit on an SM");
@@ -281,11 +328,27 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     lv_status st = choose_launch(h, n_steps, greeks, &p->block, &p->k, &p->bps, dbg, &p->grid_smem, extra, vanna,
                                  &p->ppl, n_paths);
     if (st != LV_OK) return st;
-    p->smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, p->block, greeks, p->grid_smem, extra, p->ppl);
+    p->smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, h->n_bins, p->block, greeks, p->grid_smem, extra, p->ppl);
     const int warps = p->block / 32;
     const int64_t tiles = (n_paths + lv::paths_per_tile(greeks) - 1) / lv::paths_per_tile(greeks);   // claimed by warps
     p->n_tiles = (int)tiles;
     const int64_t want_blocks = (tiles + warps - 1) / warps;
+    // The forward-only kernel's tiles all take the same time, so a last round with
+    // few tiles costs a whole one: of the upper half of the resident block counts
+    // the one with the least rounds x warps. 2^20 paths on 152 SMs are 2.99 rounds
+    // at nine blocks, 3.37 at eight and 3.85 at seven: 245, 257 and 257 us a call.
+    if (!greeks && !h->cfg_bps) {
+        int64_t best = 0;
+        for (int b = p->bps; 2 * b >= p->bps && b >= 1; --b) {
+            const int64_t warps_all = (int64_t)b * h->num_sms * warps;
+            const int64_t cost = (tiles + warps_all - 1) / warps_all * b;
+            if (best == 0 || cost < best) {
+                best = cost;
+                p->bps = b;
+            }
+            if (warps_all <= tiles / 64) break;          // many rounds: the last one does not matter
+        }
+    }
     const int64_t slots = (int64_t)p->bps * h->num_sms;
     p->grid = (int)(want_blocks < slots ? want_blocks : slots);
     if (p->grid < 1) p->grid = 1;
@@ -353,7 +416,8 @@ struct McCall {
     bool vanna = false;      // buckets are d^2 price / (d S0 d sigma_ij) instead of the vegas
 };
 
-lv::McParams base_params(const lv_surface_s* h, const McCall& c)
+// k: the launch's checkpoint interval (0: a call that searches for its cells).
+lv::McParams base_params(const lv_surface_s* h, const McCall& c, int k)
 {
     lv::McParams P{};
     P.sig2 = h->d_sig;
@@ -395,9 +459,10 @@ lv::McParams base_params(const lv_surface_s* h, const McCall& c)
     P.n_paths = c.n_paths;
     P.acc_mode = h->acc_mode;
     P.method = LV_ADJ_REVERSE;
-    if (P.log_uniform && lv::index_bounded(on_s, c.n_steps, P.x0, P.rdt, P.hdt, P.sqdt2, h->sig_max, P.cell_scale,
-                                           P.cell_shift))
-        P.log_uniform = 2;
+    P.bins = h->d_bins;
+    // checkpoints every 16 or 32 steps and the diagnostics kernel search
+    if (k > 0 && k <= lv::kModelMaxK && !c.dbg_xN)
+        lv::choose_cell_mode(P, h->sig_max, h->n_bins, h->bin_scale, h->bin_shift);
     return P;
 }
 
@@ -419,7 +484,7 @@ lv_status run_mc(lv_surface_s* h, const McCall& c)
     st = ensure_scratch(h, p.total);
     if (st != LV_OK) return st;
     char* base = static_cast<char*>(h->d_scratch);
-    lv::McParams P = base_params(h, c);
+    lv::McParams P = base_params(h, c, p.k);
     P.n_tiles = p.n_tiles;
     P.ppl = p.ppl;
     P.tile_counter = reinterpret_cast<unsigned int*>(base + p.off_counter);
@@ -579,6 +644,19 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
             abl[i] = make_float2((float)(1.0 / wl), (float)(-y0 / wl));
         } else {
             ab[i] = abl[i] = make_float2(0.0f, 0.0f);
+        }
+    }
+    std::vector<float4> bins;
+    if (!h->log_uniform) bins = spot_bins(h->spot, &h->bin_scale, &h->bin_shift);
+    h->n_bins = (int)bins.size();
+    if (h->n_bins > 0) {
+        if (cudaMalloc(&h->d_bins, sizeof(float4) * bins.size()) != cudaSuccess) {
+            cudaGetLastError();
+            return bail(LV_ENOMEM, "device or pinned allocation failed");
+        }
+        if (cudaMemcpy(h->d_bins, bins.data(), sizeof(float4) * bins.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+            e = cudaGetLastError();
+            return bail(LV_ECUDA, std::string("upload of the grid failed: ") + cudaGetErrorString(e));
         }
     }
     pack_sigma(h, sigma, h->h_sig_stage);
@@ -986,7 +1064,7 @@ lv_status lv_bump_greeks(lv_surface_t h, double S0, double r, double K, double T
     char* base = static_cast<char*>(h->d_scratch);
     McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, false, false, h->d_res};
     lv::BumpParams B{};
-    B.mc = base_params(h, c);
+    B.mc = base_params(h, c, 0);
     B.mc.n_tiles = (int)tiles;
     B.mc.tile_counter = reinterpret_cast<unsigned int*>(base);
     const double eps_S = 1e-4 * S0;
@@ -1262,7 +1340,7 @@ lv_status lv_debug_time_table(lv_surface_t h, double T, int32_t n_steps, int32_t
     DeviceGuard g(h->device);
     if (!g.ok) return fail(LV_ECUDA, "cannot select the handle's device");
     McCall c{1.0, 0.0, 1.0, T, n_steps, 0, 1, 1, 0u, true, false, h->d_res};
-    const lv::McParams P = base_params(h, c);
+    const lv::McParams P = base_params(h, c, 0);
     const size_t off_v = round_up(sizeof(int) * (size_t)n_steps, 256);
     char* d = nullptr;
     if (cudaMalloc(&d, off_v + sizeof(float) * (size_t)n_steps) != cudaSuccess) {
@@ -1402,7 +1480,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
                                std::to_string(kStaticScratchBytes));
 
     McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, true, false, d_out};
-    lv::McParams P = base_params(h, c);
+    lv::McParams P = base_params(h, c, k);
     P.n_tiles = (int)tiles;
     P.ppl = ppl;
     P.tile_counter = reinterpret_cast<unsigned int*>(base);
@@ -1421,7 +1499,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
     // the array keeps the previous call's contents: the tile counter and the
     // flag must start at zero (every other section is written before it is read)
     LV_CUDA(cudaMemsetAsync(P.tile_counter, 0, 2 * sizeof(unsigned int), h->stream));
-    const size_t smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, block, true, grid_smem, false, ppl);
+    const size_t smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, h->n_bins, block, true, grid_smem, false, ppl);
     LV_CUDA(lv::launch_mc(P, grid, block, k, true, smem, h->stream));
     lv::FinalizeParams F{};
     F.partials = P.partials;

@@ -27,10 +27,11 @@ constexpr int kBMaxWarps = 8;
 __host__ __device__ inline size_t b16(size_t b) { return (b + 15) & ~size_t(15); }
 
 struct BookSmem {
-    size_t params, tab, sig, node, ab, qslot, qrel, qxb, acc, red, ctl, total;
+    size_t params, tab, sig, node, ab, bins, qslot, qrel, qxb, acc, red, ctl, total;
 };
 
-__host__ __device__ inline BookSmem book_layout(int maxI, int maxJe, int maxN, int block, int ppl = 1)
+__host__ __device__ inline BookSmem book_layout(int maxI, int maxJe, int maxN, int max_bins, int block,
+                                                  int ppl = 1)
 {
     const int W = block / 32;
     BookSmem L;
@@ -40,6 +41,7 @@ __host__ __device__ inline BookSmem book_layout(int maxI, int maxJe, int maxN, i
     L.sig = o;    o += b16(sizeof(float2) * (size_t)maxJe * (maxI - 1));
     L.node = o;   o += b16(sizeof(float) * (size_t)maxI);
     L.ab = o;     o += b16(sizeof(float2) * (size_t)maxI);
+    L.bins = o;   o += sizeof(float4) * (size_t)max_bins;
     L.qslot = o;  o += b16(sizeof(int) * (size_t)W * kBQueue * ppl);
     L.qrel = o;   o += b16(sizeof(int) * (size_t)W * kBQueue * ppl);
     L.qxb = o;    o += b16(sizeof(float) * (size_t)W * kBQueue * ppl);
@@ -91,9 +93,8 @@ __device__ void build_params(const BookParams& B, int inst, McParams* out)
     P.dt_d = dt;
     P.N = o.N;
     P.rk = philox_keys((uint32_t)(run.seed & 0xffffffffu), (uint32_t)(run.seed >> 32));
-    if (P.log_uniform && index_bounded(false, o.N, P.x0, P.rdt, P.hdt, P.sqdt2, s.sig_max, P.cell_scale,
-                                       P.cell_shift))
-        P.log_uniform = 2;
+    P.bins = B.bins + s.off_bins;
+    choose_cell_mode(P, s.sig_max, s.n_bins, s.bin_scale, s.bin_shift);
     P.stream_id = (uint32_t)o.stream_id;
     P.path_begin = 0;
     P.n_paths = o.n_paths;
@@ -109,7 +110,7 @@ __device__ void build_params(const BookParams& B, int inst, McParams* out)
 // PPL: paths per lane of a forward tile, as in the single-option kernel: a
 // warp claims PPL consecutive 32-path tiles of its item and runs them
 // interleaved; the ring groups and the FIFO grow with it.
-template <int KCK, int PPL>
+template <int KCK, int PPL, int CELL>
 __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ BookParams B)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -117,7 +118,7 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
     constexpr int kQcap = kBQueue * PPL;
     const int Bk = blockDim.x, W = Bk >> 5;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const BookSmem L = book_layout(B.max_I, B.max_Je, B.max_N, Bk, PPL);
+    const BookSmem L = book_layout(B.max_I, B.max_Je, B.max_N, B.max_bins, Bk, PPL);
     McParams* s_par = reinterpret_cast<McParams*>(smem + L.params);
     int4* s_tab = reinterpret_cast<int4*>(smem + L.tab);
     float2* s_sig = reinterpret_cast<float2*>(smem + L.sig);
@@ -131,7 +132,8 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
     float* l1 = B.l1 + (size_t)blockIdx.x * B.max_IJe;
     const size_t cks = (size_t)gridDim.x * W * kBRing * kSlots;
     float* const ckw = B.ckpt + (size_t)(blockIdx.x * W + warp) * kBRing * kSlots;
-    const SmemGrid g{ s_tab, s_sig, s_node, s_ab };
+    float4* s_bins = reinterpret_cast<float4*>(smem + L.bins);
+    const SmemGrid g{ s_tab, s_sig, s_node, s_ab, s_bins };
 
     for (int e = tid; e < B.max_IJe; e += Bk) l1[e] = 0.0f;
     if (tid == 0) s_ctl[2] = -1;
@@ -151,6 +153,7 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
             for (int e = tid; e < Q.Je * (Q.I - 1); e += Bk) s_sig[e] = Q.sig2[e];
             for (int e = tid; e < Q.I; e += Bk) s_node[e] = Q.node[e];
             for (int e = tid; e < Q.I - 1; e += Bk) s_ab[e] = Q.ab[e];
+            for (int e = tid; e < Q.n_bins; e += Bk) s_bins[e] = Q.bins[e];
             for (int n = tid; n < Q.N; n += Bk) s_tab[n] = step_time(Q, n);
             if (tid == 0) s_ctl[2] = it.inst;
         }
@@ -177,7 +180,7 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
                     const long long rel = q_rel[e];
                     uint32_t c1, c2;
                     path_counter(P, rel, c1, c2);
-                    const float xbar = reverse_path<KCK>(P, g, c1, c2, ckw + q_slot[e], cks, q_xb[e], l1);
+                    const float xbar = reverse_path<CELL, KCK>(P, g, c1, c2, ckw + q_slot[e], cks, q_xb[e], l1);
                     acc[2 * Bk] += (double)xbar;
                 }
                 q_head = (q_head + nb) & (kQcap - 1);
@@ -198,7 +201,7 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
                     path_counter(P, rel_a, c1a, c2a);
                     path_counter(P, rel_b, c1b, c2b);
                     float ya, yb;
-                    forward_path2<KCK, true>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a, ckw + slot_b, cks, ya, yb);
+                    forward_path2<CELL, KCK, true>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a, ckw + slot_b, cks, ya, yb);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         if (h == 1 && !act_b) break;
@@ -235,7 +238,7 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
             if (active) {
                 uint32_t c1, c2;
                 path_counter(P, rel, c1, c2);
-                const float x = forward_path<KCK, true, false>(P, g, c1, c2, ckw + slot, cks, rel);
+                const float x = forward_path<CELL, KCK, true, false>(P, g, c1, c2, ckw + slot, cks, rel);
                 const float SN = exp2f(x);
                 const float itm = P.phi * (SN - P.K);
                 const float V = itm > 0.0f ? P.disc * itm : 0.0f;
@@ -355,60 +358,57 @@ __global__ void book_risk_finalize_kernel(const BookInst* __restrict__ insts, co
     }
 }
 
-template <int KCK, int PPL>
-cudaError_t book_launch_k(const BookParams& b, int grid, int block, size_t smem, cudaStream_t s)
-{
-    book_kernel<KCK, PPL><<<grid, block, smem, s>>>(b);
-    return cudaGetLastError();
-}
-
-// The book kernel of (k, paths per lane): k in {4, 8}, ppl in {1, 2}.
-template <typename F>
-cudaError_t with_book_kernel(int k, int ppl, F&& f)
+// The book kernel of (k, paths per lane): k in {4, 8}, ppl in {1, 2}; the one
+// with the bins' loops only for books that have a surface with bins.
+template <int CELL, typename F>
+cudaError_t with_book_kernel_c(int k, int ppl, F&& f)
 {
     switch (k * 4 + ppl) {
-    case 17: return f(book_kernel<4, 1>);
-    case 18: return f(book_kernel<4, 2>);
-    case 33: return f(book_kernel<8, 1>);
-    case 34: return f(book_kernel<8, 2>);
+    case 17: return f(book_kernel<4, 1, CELL>);
+    case 18: return f(book_kernel<4, 2, CELL>);
+    case 33: return f(book_kernel<8, 1, CELL>);
+    case 34: return f(book_kernel<8, 2, CELL>);
     default: return cudaErrorInvalidValue;
     }
 }
 
+template <typename F>
+cudaError_t with_book_kernel(int k, int ppl, bool bins, F&& f)
+{
+    return bins ? with_book_kernel_c<kCellAny>(k, ppl, f) : with_book_kernel_c<kCellNoBins>(k, ppl, f);
+}
+
 }  // namespace
 
-size_t book_smem_bytes(int maxI, int maxJe, int maxN, int block, int ppl)
+size_t book_smem_bytes(int maxI, int maxJe, int maxN, int max_bins, int block, int ppl)
 {
-    return book_layout(maxI, maxJe, maxN, block, ppl).total;
+    return book_layout(maxI, maxJe, maxN, max_bins, block, ppl).total;
 }
 
 int book_ring_slots_per_warp() { return kBRing * 32; }
 
-cudaError_t book_prepare(int k, int ppl)
+cudaError_t book_prepare(int k, int ppl, bool bins)
 {
-    return with_book_kernel(k, ppl, [](auto kernel) {
+    return with_book_kernel(k, ppl, bins, [](auto kernel) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     });
 }
 
-cudaError_t book_occupancy(int block, int k, int ppl, size_t smem, int* bps)
+cudaError_t book_occupancy(int block, int k, int ppl, bool bins, size_t smem, int* bps)
 {
-    cudaError_t e = book_prepare(k, ppl);
+    cudaError_t e = book_prepare(k, ppl, bins);
     if (e != cudaSuccess) return e;
-    return with_book_kernel(k, ppl, [&](auto kernel) {
+    return with_book_kernel(k, ppl, bins, [&](auto kernel) {
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, kernel, block, smem);
     });
 }
 
 cudaError_t launch_book(const BookParams& b, int grid, int block, int k, int ppl, size_t smem, cudaStream_t s)
 {
-    switch (k * 4 + ppl) {
-    case 17: return book_launch_k<4, 1>(b, grid, block, smem, s);
-    case 18: return book_launch_k<4, 2>(b, grid, block, smem, s);
-    case 33: return book_launch_k<8, 1>(b, grid, block, smem, s);
-    case 34: return book_launch_k<8, 2>(b, grid, block, smem, s);
-    default: return cudaErrorInvalidValue;
-    }
+    return with_book_kernel(k, ppl, b.max_bins > 0, [&](auto kernel) {
+        kernel<<<grid, block, smem, s>>>(b);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_book_risk_finalize(const BookParams& b, int n_surf, int n_inst, int max_IJ, double* out,

@@ -34,7 +34,7 @@ struct lv_book_s {
     std::vector<lv::BookSurf> surfs;
     std::vector<int64_t> offsets;           // [n + 1]
     std::vector<int64_t> risk_offsets;      // [n_surfaces + 1]
-    int max_I = 0, max_J = 0, max_Je = 0, max_N = 0, max_IJe = 0, max_IJ = 0;
+    int max_I = 0, max_J = 0, max_Je = 0, max_N = 0, max_IJe = 0, max_IJ = 0, max_bins = 0;
     int64_t total_paths = 0;
     // device tables and grids
     lv::BookSurf* d_surfs = nullptr;
@@ -45,6 +45,7 @@ struct lv_book_s {
     float* d_node = nullptr;
     float2* d_ab = nullptr;
     double* d_tau = nullptr;
+    float4* d_bins = nullptr;
     lv::BookRun* d_run = nullptr;
     lv::BookRun* h_run = nullptr;           // pinned; the graph copies from it
     double* d_sums = nullptr;
@@ -103,6 +104,7 @@ void free_book(lv_book_s* b)
     cudaFree(b->d_node);
     cudaFree(b->d_ab);
     cudaFree(b->d_tau);
+    cudaFree(b->d_bins);
     cudaFree(b->d_run);
     cudaFree(b->d_sums);
     cudaFree(b->d_out);
@@ -142,10 +144,10 @@ lv_status configure(lv_book_s* b, int block, int k, int item_tiles, int ppl)
 {
     drop_graph(b);
     LV_BCUDA(cudaStreamSynchronize(b->stream));
-    const size_t smem = lv::book_smem_bytes(b->max_I, b->max_Je, b->max_N, block, ppl);
+    const size_t smem = lv::book_smem_bytes(b->max_I, b->max_Je, b->max_N, b->max_bins, block, ppl);
     if (smem > 200 * 1024) return set_error(LV_EINVAL, "book grids too large for shared memory");
     int bps = 0;
-    LV_BCUDA(lv::book_occupancy(block, k, ppl, smem, &bps));
+    LV_BCUDA(lv::book_occupancy(block, k, ppl, b->max_bins > 0, smem, &bps));
     if (bps < 1) return set_error(LV_EINVAL, "book launch shape does not fit on an SM");
     std::vector<lv::BookItem> items = make_items(b->insts, item_tiles);
     cudaFree(b->d_items);
@@ -198,6 +200,7 @@ lv::BookParams params(const lv_book_s* b)
     P.node = b->d_node;
     P.ab = b->d_ab;
     P.tau = b->d_tau;
+    P.bins = b->d_bins;
     P.run = b->d_run;
     P.item_counter = b->d_counter;
     P.sums = b->d_sums;
@@ -208,6 +211,7 @@ lv::BookParams params(const lv_book_s* b)
     P.max_Je = b->max_Je;
     P.max_N = b->max_N;
     P.max_IJe = b->max_IJe;
+    P.max_bins = b->max_bins;
     return P;
 }
 
@@ -296,7 +300,7 @@ lv_status run_captured(lv_book_s* b, double S0, double r, uint64_t seed, bool ri
     double* d_res = risk ? b->d_rout : b->d_out;
     double* h_res = risk ? b->h_rout : b->h_out;
     if (!exec) {
-        LV_BCUDA(lv::book_prepare(b->k, b->ppl));
+        LV_BCUDA(lv::book_prepare(b->k, b->ppl, b->max_bins > 0));
         cudaGraph_t graph = nullptr;
         LV_BCUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
         lv_status cst = LV_OK;
@@ -366,7 +370,7 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
         return bail(set_error(LV_ECUDA, "cannot read the SM count"));
 
     // grids: concatenate every surface's device arrays
-    long long n_sig = 0, n_node = 0, n_ab = 0, n_tau = 0;
+    long long n_sig = 0, n_node = 0, n_ab = 0, n_tau = 0, n_bins = 0;
     for (int s = 0; s < n_surfaces; ++s) {
         const lv_surface_s* h = surfaces[s];
         lv::BookSurf bs{};
@@ -379,6 +383,10 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
         bs.s_lo = h->s_lo;
         bs.s_hi = h->s_hi;
         bs.sig_max = h->sig_max;
+        bs.n_bins = h->n_bins;
+        bs.bin_scale = h->bin_scale;
+        bs.bin_shift = h->bin_shift;
+        bs.off_bins = n_bins;
         bs.off_sig2 = n_sig;
         bs.off_node = n_node;
         bs.off_ab = n_ab;
@@ -388,9 +396,11 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
         n_node += h->I;
         n_ab += h->I;
         n_tau += h->J;
+        n_bins += h->n_bins;
         b->surfs.push_back(bs);
         b->max_I = std::max(b->max_I, h->I);
         b->max_J = std::max(b->max_J, h->J);
+        b->max_bins = std::max(b->max_bins, h->n_bins);
         b->max_Je = std::max(b->max_Je, h->Je);
         b->max_IJe = std::max(b->max_IJe, h->Je * h->I);
         b->max_IJ = std::max(b->max_IJ, h->I * h->J);
@@ -425,6 +435,7 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
         cudaMalloc(&b->d_node, sizeof(float) * n_node) != cudaSuccess ||
         cudaMalloc(&b->d_ab, sizeof(float2) * n_ab) != cudaSuccess ||
         cudaMalloc(&b->d_tau, sizeof(double) * n_tau) != cudaSuccess ||
+        cudaMalloc(&b->d_bins, sizeof(float4) * (n_bins > 0 ? n_bins : 1)) != cudaSuccess ||
         cudaMalloc(&b->d_run, sizeof(lv::BookRun)) != cudaSuccess ||
         cudaMalloc(&b->d_sums, sizeof(double) * n_out) != cudaSuccess ||
         cudaMalloc(&b->d_out, sizeof(double) * n_out) != cudaSuccess ||
@@ -444,6 +455,8 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
             cudaMemcpy(b->d_node + bs.off_node, h->d_node, sizeof(float) * h->I, cudaMemcpyDeviceToDevice) !=
                 cudaSuccess ||
             cudaMemcpy(b->d_ab + bs.off_ab, h->d_ab, sizeof(float2) * h->I, cudaMemcpyDeviceToDevice) != cudaSuccess ||
+            (h->n_bins > 0 && cudaMemcpy(b->d_bins + bs.off_bins, h->d_bins, sizeof(float4) * h->n_bins,
+                                         cudaMemcpyDeviceToDevice) != cudaSuccess) ||
             cudaMemcpy(b->d_tau + bs.off_tau, h->d_tau, sizeof(double) * h->J, cudaMemcpyDeviceToDevice) !=
                 cudaSuccess)
             return bail(set_error(LV_ECUDA, "copying a surface into the book failed"));

@@ -264,31 +264,47 @@ struct SmemGrid {
     const float2* sig2;    // [Je][I-1]: (sigma_{i,j}, sigma_{i+1,j} - sigma_{i,j})
     const float* node;     // [I]
     const float2* ab;      // [I - 1]
+    const float4* bins;    // [n_bins] spot_bins (kCellBins)
     const float* tdt;      // [N] step_tdt (kernels that compute d price / d T)
 };
 
-// floor(c) clamped to [0, I-2] for |c| < 2^22 (the launcher's bound on every
-// path of the call, McParams::log_uniform == 2): adding 1.5 * 2^23 rounded
+// floor(c) clamped to [0, hi] for |c| < 2^22 (the launcher's bound on every
+// path of the call, McParams::cell_mode kCellUniform and kCellBins): adding 1.5 * 2^23 rounded
 // down leaves floor(c) in the low bits, and one integer instruction takes the
 // offset off and clamps both sides. A float-to-integer conversion would hold
 // the transcendental unit for 8 cycles a warp, as long as a sine.
 constexpr float kFloorShift = 12582912.0f;          // 1.5 * 2^23 = 0x4B400000
 constexpr int kFloorBits = 0x4B400000;
 
-__device__ __forceinline__ int clamp_floor(const McParams& P, float shifted)
+__device__ __forceinline__ int clamp_floor(float shifted, int hi)
 {
-    return __viaddmin_s32_relu(__float_as_int(shifted), -kFloorBits, P.I - 2);
+    return __viaddmin_s32_relu(__float_as_int(shifted), -kFloorBits, hi);
 }
 
-// Spot cell: the largest i <= I-2 with s_i <= S. On log-uniform grids the
-// index comes from y = log2 S directly (off by one only when S is within
-// binary32 rounding of a node, where the clamped weight gives the same
-// value); on other grids a binary search over the nodes. FAST: the call has
-// log_uniform == 2 (same index, no branch inside the step).
-template <bool FAST = false>
+// Cell of S in bin b: the bin's first cell and the two nodes after it (infinite
+// past the last cell).
+__device__ __forceinline__ int bin_cell(const SmemGrid& g, int b, float S)
+{
+    const float4 t = g.bins[b];
+    return __float_as_int(t.x) + (t.y <= S ? 1 : 0) + (t.z <= S ? 1 : 0);
+}
+
+// Spot cell: the largest i <= I-2 with s_i <= S, found as the call's cell mode
+// says (CELL, or kCellSearch for any mode):
+//  - kCellUniform: on log-uniform grids the index comes from y = log2 S
+//    directly (off by one only when S is within binary32 rounding of a node,
+//    where the clamped weight gives the same value);
+//  - kCellBins: on other grids from a table of equal bins in y, at most two
+//    nodes in each: the bin's first cell plus two comparisons with S;
+//  - kCellSearch: the same index from a conversion, or a binary search over the
+//    nodes.
+template <int CELL = kCellSearch>
 __device__ __forceinline__ int spot_cell(const McParams& P, const SmemGrid& g, float y, float S)
 {
-    if (FAST) return clamp_floor(P, __fadd_rd(fmaf(y, P.cell_scale, P.cell_shift), kFloorShift));
+    if (CELL == kCellUniform)
+        return clamp_floor(__fadd_rd(fmaf(y, P.cell_scale, P.cell_shift), kFloorShift), P.I - 2);
+    if (CELL == kCellBins)
+        return bin_cell(g, clamp_floor(__fadd_rd(fmaf(y, P.cell_scale, P.cell_shift), kFloorShift), P.n_bins - 1), S);
     if (P.log_uniform) {
         const int i = __float2int_rd(fmaf(y, P.cell_scale, P.cell_shift));
         return min(max(i, 0), P.I - 2);
@@ -324,7 +340,7 @@ struct StepEval {
 // slope only when WANT_SLOPE. With the ln-S weight the cell coefficients ab
 // are (1 / (y_{i+1} - y_i), -y_i / (y_{i+1} - y_i)) in y = log2 s, so that
 // d u / d ln S = ab.x log2(e); otherwise they are in S.
-template <bool WANT_SLOPE, int MODEL = 0, bool FAST = false>
+template <bool WANT_SLOPE, int MODEL = 0, int CELL = kCellSearch>
 __device__ __forceinline__ StepEval eval_sigma(const McParams& P, const SmemGrid& g, float x,
                                                const int4& tb)
 {
@@ -337,7 +353,7 @@ __device__ __forceinline__ StepEval eval_sigma(const McParams& P, const SmemGrid
         e.S = ex2_approx(x);
         y = x;
     }
-    e.i = spot_cell<FAST>(P, g, y, e.S);
+    e.i = spot_cell<CELL>(P, g, y, e.S);
     const float2 ab = g.ab[e.i];
     e.u = __saturatef(fmaf((MODEL & kModelLogWeight) ? y : e.S, ab.x, ab.y));
     const float2 lo = g.sig2[tb.x + e.i];      // time row j:     sigma_{i,j},   its spot step
@@ -455,14 +471,39 @@ __device__ __forceinline__ void log_cell_decision(const McParams& P, const SmemG
     }
 }
 
+// Calls f with the cell mode as a compile-time constant: CELL itself, or with
+// kCellAny the one in P, chosen once per path (kCellAny: any of the three,
+// kCellNoBins: no surface has bins). The single-option kernels are compiled per
+// mode: with all three loops in one kernel the adjoint took 0.633 ms instead
+// of 0.609 at 2^20 paths on a log-spaced grid.
+template <int C>
+struct CellMode {
+    static constexpr int value = C;
+};
+
+template <int CELL, typename F>
+__device__ __forceinline__ auto cell_dispatch(const McParams& P, F&& f)
+{
+    if constexpr (CELL != kCellAny && CELL != kCellNoBins) {
+        return f(CellMode<CELL>{});
+    } else {
+        if (P.cell_mode == kCellUniform) return f(CellMode<kCellUniform>{});
+        if constexpr (CELL == kCellAny) {
+            if (P.cell_mode == kCellBins) return f(CellMode<kCellBins>{});
+        }
+        return f(CellMode<kCellSearch>{});
+    }
+}
+
 // The time loop of a forward pass: blocks of four steps on four normals,
 // every block but the last without a bound check. The next block's normals
 // are computed in the same straight-line code as the current block's steps:
 // the Philox products (FMA pipe) and the Box-Muller functions (transcendental
 // unit) then fill the latencies of the steps' loads instead of forming phases
 // of their own in which every warp waits for the same pipe (forward only, 2^20
-// paths: 0.265 -> 0.238 ms; with the body unrolled over two blocks 0.226 ms; the
-// slope-carrying loops spill when unrolled and take one block). PIPE false: the
+// paths: 0.265 -> 0.229 ms). UNROLL blocks to a body: two for the adjoint's pairs,
+// one where two only cost registers (forward only) or spill (the slope-carrying
+// loops: second-order buckets 0.731 ms with two, 0.675 with one). PIPE false: the
 // plain loop, for grids whose cell search branches inside the step anyway.
 // `first(blk)` runs before a block's steps, `gen(blk, z)` makes its normals,
 // `step(n, z)` is one step.
@@ -499,28 +540,29 @@ __device__ __forceinline__ void time_blocks(int N, First&& first, Gen&& gen, Ste
 }
 
 // Forward pass of one path from x0; checkpoints every KCK steps when STORE.
-template <int KCK, bool STORE, bool DBG, int MODEL, bool FAST>
+template <int KCK, bool STORE, bool DBG, int MODEL, int CELL>
 __device__ __forceinline__ float forward_path_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                                 float* ck, size_t cks, long long rel)
 {
     float x = P.x0;
-    time_blocks<float, FAST, 2>(
+    time_blocks<float, CELL != kCellSearch, 2>(
         P.N, [&](int blk) { if (STORE && (blk * 4) % KCK == 0) ck[(size_t)(blk * 4 / KCK) * cks] = x; },
         [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
         [&](int n, float z) {
-            const StepEval e = eval_sigma<false, MODEL, FAST>(P, g, x, g.tab[n]);
+            const StepEval e = eval_sigma<false, MODEL, CELL>(P, g, x, g.tab[n]);
             if (DBG) log_cell_decision(P, g, e, rel, n);
             x = step_state<MODEL>(P, x, e.sigma, z);
         });
     return x;
 }
 
-template <int KCK, bool STORE, bool DBG, int MODEL = 0>
+template <int CELL, int KCK, bool STORE, bool DBG, int MODEL = 0>
 __device__ __forceinline__ float forward_path(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                               float* ck, size_t cks, long long rel)
 {
-    if (!DBG && P.log_uniform == 2) return forward_path_f<KCK, STORE, DBG, MODEL, true>(P, g, c1, c2, ck, cks, rel);
-    return forward_path_f<KCK, STORE, DBG, MODEL, false>(P, g, c1, c2, ck, cks, rel);
+    if constexpr (DBG) return forward_path_f<KCK, STORE, DBG, MODEL, kCellSearch>(P, g, c1, c2, ck, cks, rel);
+    return cell_dispatch<CELL>(
+        P, [&](auto c) { return forward_path_f<KCK, STORE, false, MODEL, decltype(c)::value>(P, g, c1, c2, ck, cks, rel); });
 }
 
 // Forward passes of two paths, interleaved so the scheduler has two
@@ -532,7 +574,7 @@ __device__ __forceinline__ float forward_path(const McParams& P, const SmemGrid&
 // step (on y = log2 S or on S); the loads and the transcendental unit stay per
 // path. The step uses sqdt2 Z = (-sqdt2)(-Z) (sqdt Z on S), exact, so the
 // negated normals need no sign flip.
-template <int KCK, bool STORE, int MODEL, bool PACK, bool FAST>
+template <int KCK, bool STORE, int MODEL, bool PACK, int CELL>
 __device__ __forceinline__ void forward_path2_f(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
                                                 uint32_t c1b, uint32_t c2b, float* cka, float* ckb, size_t cks,
                                                 float& ya_out, float& yb_out)
@@ -544,7 +586,7 @@ __device__ __forceinline__ void forward_path2_f(const McParams& P, const SmemGri
         const f32x2 nsq = pk2(-P.sqdt2, -P.sqdt2), nhdt = pk2(-P.hdt, -P.hdt), rdt = pk2(P.rdt, P.rdt);
         const f32x2 nsqdt = pk2(-P.sqdt, -P.sqdt), fsh = pk2(kFloorShift, kFloorShift);
         f32x2 x = pk2(P.x0, P.x0);
-        time_blocks<f32x2, FAST, 2>(
+        time_blocks<f32x2, CELL != kCellSearch, STORE ? 2 : 1>(
             P.N,
             [&](int blk) {
                 if (STORE && (blk * 4) % KCK == 0) {
@@ -568,13 +610,13 @@ __device__ __forceinline__ void forward_path2_f(const McParams& P, const SmemGri
                     Sb = ex2_approx(hi2(y));
                 }
                 int ia, ib;
-                if (FAST) {
+                if (CELL == kCellUniform) {
                     const f32x2 ci = add2_rd(fma2(y, csc, csh), fsh);
-                    ia = clamp_floor(P, lo2(ci));
-                    ib = clamp_floor(P, hi2(ci));
+                    ia = clamp_floor(lo2(ci), P.I - 2);
+                    ib = clamp_floor(hi2(ci), P.I - 2);
                 } else {
-                    ia = spot_cell(P, g, lo2(y), Sa);
-                    ib = spot_cell(P, g, hi2(y), Sb);
+                    ia = spot_cell<CELL>(P, g, lo2(y), Sa);
+                    ib = spot_cell<CELL>(P, g, hi2(y), Sb);
                 }
                 const float2 aba = g.ab[ia], abb = g.ab[ib];
                 // the spot weight is linear in S, or in y = log2 S under the ln-S weight
@@ -599,7 +641,7 @@ __device__ __forceinline__ void forward_path2_f(const McParams& P, const SmemGri
     } else {
         struct Z2 { float a, b; };
         float ya = P.x0, yb = P.x0;
-        time_blocks<Z2, FAST, 2>(
+        time_blocks<Z2, CELL != kCellSearch, 2>(
             P.N,
             [&](int blk) {
                 if (STORE && (blk * 4) % KCK == 0) {
@@ -616,8 +658,8 @@ __device__ __forceinline__ void forward_path2_f(const McParams& P, const SmemGri
             },
             [&](int n, Z2 z) {
                 const int4 tb = g.tab[n];
-                const StepEval ea = eval_sigma<false, MODEL, FAST>(P, g, ya, tb);
-                const StepEval eb = eval_sigma<false, MODEL, FAST>(P, g, yb, tb);
+                const StepEval ea = eval_sigma<false, MODEL, CELL>(P, g, ya, tb);
+                const StepEval eb = eval_sigma<false, MODEL, CELL>(P, g, yb, tb);
                 ya = step_state<MODEL>(P, ya, ea.sigma, z.a);
                 yb = step_state<MODEL>(P, yb, eb.sigma, z.b);
             });
@@ -626,15 +668,15 @@ __device__ __forceinline__ void forward_path2_f(const McParams& P, const SmemGri
     }
 }
 
-template <int KCK, bool STORE, int MODEL = 0, bool PACK = false>
+template <int CELL, int KCK, bool STORE, int MODEL = 0, bool PACK = false>
 __device__ __forceinline__ void forward_path2(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
                                               uint32_t c1b, uint32_t c2b, float* cka, float* ckb, size_t cks,
                                               float& ya_out, float& yb_out)
 {
-    if (P.log_uniform == 2)
-        forward_path2_f<KCK, STORE, MODEL, PACK, true>(P, g, c1a, c2a, c1b, c2b, cka, ckb, cks, ya_out, yb_out);
-    else
-        forward_path2_f<KCK, STORE, MODEL, PACK, false>(P, g, c1a, c2a, c1b, c2b, cka, ckb, cks, ya_out, yb_out);
+    cell_dispatch<CELL>(P, [&](auto c) {
+        forward_path2_f<KCK, STORE, MODEL, PACK, decltype(c)::value>(P, g, c1a, c2a, c1b, c2b, cka, ckb, cks, ya_out,
+                                                                     yb_out);
+    });
 }
 
 // Philox counter words of path `rel` of the call: c1 = path bits 0..31,
@@ -659,7 +701,7 @@ __device__ __forceinline__ void path_counter(const McParams& P, long long rel, u
 // With NEG (no extra sums) the recompute takes its normals from
 // normals4_neg and uses sqdt Z = (-sqdt)(-Z) and sqdt2 Z = (-sqdt2)(-Z),
 // which are exact, so every value is the same bit for bit.
-template <int KCK, int MODEL, bool EXTRA, bool NEG, bool FAST>
+template <int KCK, int MODEL, bool EXTRA, bool NEG, int CELL>
 __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                                 const float* ck, size_t cks, float xbar, float* l1, float* rho_acc,
                                                 float* t_acc)
@@ -692,7 +734,7 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
             if (all || n < P.N) {
                 if (q > 0 && (q & 3) == 0) gen(n >> 2, z);
                 const int4 tb = g.tab[n];
-                const StepEval ev = eval_sigma<true, MODEL, FAST>(P, g, x, tb);
+                const StepEval ev = eval_sigma<true, MODEL, CELL>(P, g, x, tb);
                 if (kNeg) {                    // z holds -Z: adjoint_factors with sqrt(dt) Z = (-sqrt(dt))(-Z)
                     if (MODEL & kModelEulerS) {
                         const float w = -P.sqdt * z[q & 3];
@@ -749,7 +791,7 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
         const float xn = ck[(size_t)mp * cks];
         float zn[4];
         gen(mp * (KCK / 4), zn);
-        if (FAST && (m + 1) * KCK <= P.N) segment(m, x, z, true);
+        if (CELL != kCellSearch && (m + 1) * KCK <= P.N) segment(m, x, z, true);
         else segment(m, x, z, false);
         x = xn;
 #pragma unroll
@@ -759,14 +801,15 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
     return xbar;
 }
 
-template <int KCK, int MODEL = 0, bool EXTRA = false, bool NEG = false>
+template <int CELL, int KCK, int MODEL = 0, bool EXTRA = false, bool NEG = false>
 __device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                               const float* ck, size_t cks, float xbar, float* l1,
                                               float* rho_acc = nullptr, float* t_acc = nullptr)
 {
-    if (P.log_uniform == 2)
-        return reverse_path_f<KCK, MODEL, EXTRA, NEG, true>(P, g, c1, c2, ck, cks, xbar, l1, rho_acc, t_acc);
-    return reverse_path_f<KCK, MODEL, EXTRA, NEG, false>(P, g, c1, c2, ck, cks, xbar, l1, rho_acc, t_acc);
+    return cell_dispatch<CELL>(P, [&](auto c) {
+        return reverse_path_f<KCK, MODEL, EXTRA, NEG, decltype(c)::value>(P, g, c1, c2, ck, cks, xbar, l1, rho_acc,
+                                                                          t_acc);
+    });
 }
 
 // Tangent-ratio form of the pathwise adjoint (Sec. III: the adjoint
@@ -778,16 +821,16 @@ __device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid&
 // D_N; `tiny` is set when some |1 + g_n| < 2^-20, where dividing by D loses
 // what the reverse sweep keeps. The path's arithmetic is that of
 // forward_path (same sigma, same Euler step), so y_N is the same.
-template <int MODEL, bool FAST>
+template <int MODEL, int CELL>
 __device__ __forceinline__ float tangent_forward_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                                    float& D, bool& tiny)
 {
     float y = P.x0;
     float d = 1.0f, fmin = 1.0f;
-    time_blocks<float, FAST, 1>(
+    time_blocks<float, CELL != kCellSearch, 1>(
         P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
         [&](int n, float z) {
-            const StepEval e = eval_sigma<true, MODEL, FAST>(P, g, y, g.tab[n]);
+            const StepEval e = eval_sigma<true, MODEL, CELL>(P, g, y, g.tab[n]);
             float h, gn;
             adjoint_factors<MODEL>(P, e, z, h, gn);
             const float f = tangent_factor<MODEL>(P, e, z, h);   // 1 + g_n
@@ -800,12 +843,12 @@ __device__ __forceinline__ float tangent_forward_f(const McParams& P, const Smem
     return y;
 }
 
-template <int MODEL = 0>
+template <int CELL, int MODEL = 0>
 __device__ __forceinline__ float tangent_forward(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                                  float& D, bool& tiny)
 {
-    if (P.log_uniform == 2) return tangent_forward_f<MODEL, true>(P, g, c1, c2, D, tiny);
-    return tangent_forward_f<MODEL, false>(P, g, c1, c2, D, tiny);
+    return cell_dispatch<CELL>(P,
+                         [&](auto c) { return tangent_forward_f<MODEL, decltype(c)::value>(P, g, c1, c2, D, tiny); });
 }
 
 // Pass 1 for two paths at once (main reading), their binary32 arithmetic in
@@ -814,7 +857,7 @@ __device__ __forceinline__ float tangent_forward(const McParams& P, const SmemGr
 // spot factor, h = sqdt Z - sigma dt = (-sqdt)(-Z) + (-dt) sigma, 1 + g_n and
 // the product D run in pairs; the inside-grid test and the running minimum of
 // |1 + g_n| stay per path.
-template <bool FAST>
+template <int CELL>
 __device__ __forceinline__ void tangent_forward2_f(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
                                                    uint32_t c1b, uint32_t c2b, float& ya_out, float& yb_out,
                                                    float& Da, float& Db, bool& tiny_a, bool& tiny_b)
@@ -825,7 +868,7 @@ __device__ __forceinline__ void tangent_forward2_f(const McParams& P, const Smem
     const f32x2 fsh = pk2(kFloorShift, kFloorShift);
     f32x2 y = pk2(P.x0, P.x0), d = one;
     float fmin_a = 1.0f, fmin_b = 1.0f;
-    time_blocks<f32x2, FAST, 1>(
+    time_blocks<f32x2, CELL != kCellSearch, 1>(
         P.N, [](int) {},
         [&](uint32_t blk, f32x2 (&z)[4]) { normals4x2_neg(blk, c1a, c2a, c1b, c2b, P.rk, z); },
         [&](int n, f32x2 nz) {
@@ -834,13 +877,13 @@ __device__ __forceinline__ void tangent_forward2_f(const McParams& P, const Smem
             // eval_sigma<true, 0> for both paths
             const float Sa = ex2_approx(lo2(y)), Sb = ex2_approx(hi2(y));
             int ia, ib;
-            if (FAST) {
+            if (CELL == kCellUniform) {
                 const f32x2 ci = add2_rd(fma2(y, csc, csh), fsh);
-                ia = clamp_floor(P, lo2(ci));
-                ib = clamp_floor(P, hi2(ci));
+                ia = clamp_floor(lo2(ci), P.I - 2);
+                ib = clamp_floor(hi2(ci), P.I - 2);
             } else {
-                ia = spot_cell(P, g, lo2(y), Sa);
-                ib = spot_cell(P, g, hi2(y), Sb);
+                ia = spot_cell<CELL>(P, g, lo2(y), Sa);
+                ib = spot_cell<CELL>(P, g, hi2(y), Sb);
             }
             const float2 aba = g.ab[ia], abb = g.ab[ib];
             const float ua = __saturatef(fmaf(Sa, aba.x, aba.y));
@@ -872,21 +915,21 @@ __device__ __forceinline__ void tangent_forward2_f(const McParams& P, const Smem
     tiny_b = fmin_b < 0x1p-20f;
 }
 
+template <int CELL>
 __device__ __forceinline__ void tangent_forward2(const McParams& P, const SmemGrid& g, uint32_t c1a, uint32_t c2a,
                                                  uint32_t c1b, uint32_t c2b, float& ya_out, float& yb_out,
                                                  float& Da, float& Db, bool& tiny_a, bool& tiny_b)
 {
-    if (P.log_uniform == 2)
-        tangent_forward2_f<true>(P, g, c1a, c2a, c1b, c2b, ya_out, yb_out, Da, Db, tiny_a, tiny_b);
-    else
-        tangent_forward2_f<false>(P, g, c1a, c2a, c1b, c2b, ya_out, yb_out, Da, Db, tiny_a, tiny_b);
+    cell_dispatch<CELL>(P, [&](auto c) {
+        tangent_forward2_f<decltype(c)::value>(P, g, c1a, c2a, c1b, c2b, ya_out, yb_out, Da, Db, tiny_a, tiny_b);
+    });
 }
 
 // Pass 2: regenerates one path (same counters, same arithmetic) and spreads
 // sigma_bar_n = c h_n / D_{n+1}, c = xbar_N D_N, over the corner buckets of
 // its cell with the bilinear weights, through the same run-length register
 // sums and binary32 reductions into `l1` as reverse_path, in time order.
-template <int MODEL, bool FAST>
+template <int MODEL, int CELL>
 __device__ __forceinline__ void tangent_scatter_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                                   float c, float* l1)
 {
@@ -901,11 +944,11 @@ __device__ __forceinline__ void tangent_scatter_f(const McParams& P, const SmemG
         atomicAdd(p1, Bs - BU);
         atomicAdd(p1 + 1, BU);
     };
-    time_blocks<float, FAST, 1>(
+    time_blocks<float, CELL != kCellSearch, 1>(
         P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
         [&](int n, float z) {
             const int4 tb = g.tab[n];
-            const StepEval e = eval_sigma<true, MODEL, FAST>(P, g, y, tb);
+            const StepEval e = eval_sigma<true, MODEL, CELL>(P, g, y, tb);
             float h, gn;
             adjoint_factors<MODEL>(P, e, z, h, gn);
             d *= tangent_factor<MODEL>(P, e, z, h);          // D_{n+1}
@@ -927,12 +970,11 @@ __device__ __forceinline__ void tangent_scatter_f(const McParams& P, const SmemG
     if (cur >= 0) flush();
 }
 
-template <int MODEL = 0>
+template <int CELL, int MODEL = 0>
 __device__ __forceinline__ void tangent_scatter(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                                 float c, float* l1)
 {
-    if (P.log_uniform == 2) tangent_scatter_f<MODEL, true>(P, g, c1, c2, c, l1);
-    else tangent_scatter_f<MODEL, false>(P, g, c1, c2, c, l1);
+    cell_dispatch<CELL>(P, [&](auto m) { tangent_scatter_f<MODEL, decltype(m)::value>(P, g, c1, c2, c, l1); });
 }
 
 // Second-order buckets d^2 price / (d S0 d sigma_ij), pass 2 of one live
@@ -947,7 +989,7 @@ __device__ __forceinline__ void tangent_scatter(const McParams& P, const SmemGri
 // nodes. Run-length sums in registers while the cell is unchanged (the
 // weight terms as in reverse_path, the slope terms E0 = sum (1 - v) d,
 // E1 = sum v d), then binary32 reductions into `l1`.
-template <bool FAST>
+template <int CELL>
 __device__ __forceinline__ void vanna_scatter_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                                 float delta, float* l1)
 {
@@ -962,11 +1004,11 @@ __device__ __forceinline__ void vanna_scatter_f(const McParams& P, const SmemGri
         atomicAdd(p1, Bs - BU - E1);
         atomicAdd(p1 + 1, BU + E1);
     };
-    time_blocks<float, FAST, 1>(
+    time_blocks<float, CELL != kCellSearch, 1>(
         P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
         [&](int n, float zq) {
             const int4 tb = g.tab[n];
-            const StepEval e = eval_sigma<true, 0, FAST>(P, g, y, tb);
+            const StepEval e = eval_sigma<true, 0, CELL>(P, g, y, tb);
             const float h = fmaf(P.sqdt, zq, -e.sigma * P.dt);
             const float f = fmaf(h, e.sslope, 1.0f);                      // 1 + g_n
             const float a = __fdividef(fmaf(zq, zq, -1.0f), e.sigma) -
@@ -995,11 +1037,11 @@ __device__ __forceinline__ void vanna_scatter_f(const McParams& P, const SmemGri
     if (cur >= 0) flush();
 }
 
+template <int CELL>
 __device__ __forceinline__ void vanna_scatter(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
                                               float delta, float* l1)
 {
-    if (P.log_uniform == 2) vanna_scatter_f<true>(P, g, c1, c2, delta, l1);
-    else vanna_scatter_f<false>(P, g, c1, c2, delta, l1);
+    cell_dispatch<CELL>(P, [&](auto c) { vanna_scatter_f<decltype(c)::value>(P, g, c1, c2, delta, l1); });
 }
 
 }  // namespace lv

@@ -1,5 +1,5 @@
 // lv_internal.h -- interface between the host runtime (lv_api.cu) and the
-// device kernels (lv_kernels.cu). Not part of the public ABI.
+// device kernels (lv_mc.cuh). Not part of the public ABI.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -34,6 +34,11 @@ __host__ __device__ inline PhiloxKeys philox_keys(uint32_t k0, uint32_t k1)
     return K;
 }
 
+// How the loops find the spot cell (lv_device.cuh spot_cell). The two without a
+// search need every index of the call bounded (index_bounded).
+constexpr int kCellSearch = 0, kCellUniform = 1, kCellBins = 2;
+constexpr int kCellAny = 3, kCellNoBins = 4;       // chosen on the device (the book)
+
 // Whether |cell_scale y + cell_shift| stays below 2^22 on every path of a call,
 // y = log2 S. On ln S the path moves by at most |rdt| + hdt sigma^2 +
 // sqdt2 sigma |Z| a step, and |Z| <= sqrt(-2 ln 2^-24) < 5.8 (23-bit
@@ -57,8 +62,10 @@ struct McParams {
     const float2* ab;      // [I - 1] (1 / (s_{i+1} - s_i), -s_i / (s_{i+1} - s_i))
     const double* tau;     // [J] time nodes
     int I, J, Je;
-    int log_uniform;       // spot nodes equally spaced in ln S (1), and the cell index of every
-                           // path of the call is below 2^22 (2, index_bounded)
+    int log_uniform;       // spot nodes equally spaced in ln S
+    int cell_mode;         // kCellSearch, kCellUniform or kCellBins
+    const float4* bins;    // [n_bins] (kCellBins)
+    int n_bins;
     float cell_scale;      // ln 2 / d(ln s): cell index from y = log2 S
     float cell_shift;      // -ln(s_0) / d(ln s)
     float s_lo, s_hi;      // s_0, s_{I-1}
@@ -115,6 +122,26 @@ struct McParams {
     float dbg_band;                     // relative distance to a node that is logged
 };
 
+// Sets cell_mode, and for kCellBins the bins' scale, shift and count in place
+// of the cells'; every other field is set. sig_max is the grid's largest sigma.
+__host__ __device__ inline void choose_cell_mode(McParams& P, double sig_max, int n_bins, float bin_scale,
+                                                 float bin_shift)
+{
+    const bool on_s = (P.model & 2) != 0;
+    P.cell_mode = kCellSearch;
+    P.n_bins = 0;
+    if (P.log_uniform) {
+        if (index_bounded(on_s, P.N, P.x0, P.rdt, P.hdt, P.sqdt2, sig_max, P.cell_scale, P.cell_shift))
+            P.cell_mode = kCellUniform;
+    } else if (n_bins > 0 &&
+               index_bounded(on_s, P.N, P.x0, P.rdt, P.hdt, P.sqdt2, sig_max, bin_scale, bin_shift)) {
+        P.cell_mode = kCellBins;
+        P.n_bins = n_bins;
+        P.cell_scale = bin_scale;
+        P.cell_shift = bin_shift;
+    }
+}
+
 // McParams::method of the second-order bucket kernel (besides LV_ADJ_REVERSE
 // and LV_ADJ_TANGENT of lv.h).
 constexpr int kMethodVanna = 2;
@@ -158,7 +185,7 @@ cudaError_t launch_bump_finalize(const double* partials, int G, int row_words, d
                                  long long n_paths, double eps, double eps_S, double* out,
                                  unsigned int* tile_counter, cudaStream_t s);
 
-size_t mc_smem_bytes(int I, int Je, int N, int block, bool greeks, bool grid_smem, bool extra = false,
+size_t mc_smem_bytes(int I, int Je, int N, int n_bins, int block, bool greeks, bool grid_smem, bool extra = false,
                      int ppl = 1);
 
 // Binary64 paths (lv_fp64.cu): the full-FP64 reference adjoint and the
@@ -201,20 +228,24 @@ cudaError_t launch_mc(const McParams& p, int grid, int block, int k, bool greeks
                       cudaStream_t s);
 cudaError_t launch_finalize(const FinalizeParams& f, cudaStream_t s);
 cudaError_t mc_occupancy(int block, int k, bool greeks, int acc, bool dbg, bool grid_smem, int method, int model,
-                         bool extra, size_t smem, int* blocks_per_sm, int ppl = 1);
+                         int cell, bool extra, size_t smem, int* blocks_per_sm, int ppl = 1);
 
-// The kernels of the other models (lv_model1.cu .. lv_model3.cu, one
-// translation unit each so that they compile in parallel); they exist for
-// checkpoint intervals k = 4 and 8, at one or two paths per lane.
-#define LV_DECLARE_MODEL(N)                                                                                \
-    cudaError_t launch_mc_model##N(const McParams& p, int grid, int block, int k, bool greeks, size_t smem, \
-                                   cudaStream_t s);                                                        \
-    cudaError_t mc_occupancy_model##N(int block, int k, bool greeks, int acc, bool dbg, bool grid_smem,    \
-                                      int method, bool extra, size_t smem, int* blocks_per_sm, int ppl);
+// One translation unit per model and cell mode (lv_m<model>c<cell>.cu, so that
+// they compile in parallel). Models 1 to 3 exist for checkpoint intervals k = 4
+// and 8, model 0 also for 16 and 32 (kCellSearch only), at one or two paths per
+// lane; the logging kernels are kCellSearch.
+#define LV_DECLARE_KERNELS(M, C)                                                                             \
+    cudaError_t launch_mc_m##M##c##C(const McParams& p, int grid, int block, int k, bool greeks, size_t smem, \
+                                     cudaStream_t s);                                                        \
+    cudaError_t mc_occupancy_m##M##c##C(int block, int k, bool greeks, int acc, bool dbg, bool grid_smem,    \
+                                        int method, bool extra, size_t smem, int* blocks_per_sm, int ppl);
+#define LV_DECLARE_MODEL(M) LV_DECLARE_KERNELS(M, 0) LV_DECLARE_KERNELS(M, 1) LV_DECLARE_KERNELS(M, 2)
+LV_DECLARE_MODEL(0)
 LV_DECLARE_MODEL(1)
 LV_DECLARE_MODEL(2)
 LV_DECLARE_MODEL(3)
 #undef LV_DECLARE_MODEL
+#undef LV_DECLARE_KERNELS
 constexpr int kModelMaxK = 8;
 int ring_slots_per_warp();
 int paths_per_tile(bool greeks);   // paths a warp claims at a time (adjoint / price kernel)
@@ -228,6 +259,9 @@ struct BookSurf {
     int I, J, Je, log_uniform;
     float cell_scale, cell_shift, s_lo, s_hi;
     double sig_max;                                  // largest sigma of the grid (index_bounded)
+    int n_bins;
+    float bin_scale, bin_shift;
+    long long off_bins;
     long long off_sig2, off_node, off_ab, off_tau;   // offsets into the book's grid arrays
     long long risk_off;                              // first double of this surface's aggregated risk
 };
@@ -259,6 +293,7 @@ struct BookParams {
     const float* node;
     const float2* ab;
     const double* tau;
+    const float4* bins;
     const BookRun* run;
     unsigned int* item_counter;
     double* sums;          // per option [3 + I J] binary64 sums (zeroed before a run)
@@ -266,15 +301,15 @@ struct BookParams {
                            // weights w / n_paths (zeroed before a run); null: per-option vegas
     float* l1;             // [gridDim.x][max_IJe] binary32 buckets per block
     float* ckpt;           // [ceil(max_N / k)][gridDim.x * warps * ring slots]
-    int max_I, max_Je, max_N, max_IJe;
+    int max_I, max_Je, max_N, max_IJe, max_bins;
 };
 
 // ppl: paths per lane of the forward tiles (1 or 2); the FIFO and the
 // checkpoint ring (book_ring_slots_per_warp() * ppl per warp) grow with it.
-size_t book_smem_bytes(int maxI, int maxJe, int maxN, int block, int ppl);
+size_t book_smem_bytes(int maxI, int maxJe, int maxN, int max_bins, int block, int ppl);
 int book_ring_slots_per_warp();
-cudaError_t book_prepare(int k, int ppl);
-cudaError_t book_occupancy(int block, int k, int ppl, size_t smem, int* blocks_per_sm);
+cudaError_t book_prepare(int k, int ppl, bool bins);
+cudaError_t book_occupancy(int block, int k, int ppl, bool bins, size_t smem, int* blocks_per_sm);
 cudaError_t launch_book(const BookParams& b, int grid, int block, int k, int ppl, size_t smem, cudaStream_t s);
 cudaError_t launch_book_finalize(const BookParams& b, int n_inst, int max_IJ, double* out, cudaStream_t s);
 cudaError_t launch_book_risk_finalize(const BookParams& b, int n_surf, int n_inst, int max_IJ, double* out,
@@ -318,6 +353,9 @@ struct lv_surface_s {
     float2* h_sig_stage = nullptr;   // pinned staging for sigma uploads
     int log_uniform = 0;
     double sig_max = 0.0;            // largest sigma of the grid (index_bounded)
+    float4* d_bins = nullptr;        // [n_bins] cell table of a grid not log-uniform (lv_api.cu spot_bins)
+    int n_bins = 0;
+    float bin_scale = 0.0f, bin_shift = 0.0f;
     float cell_scale = 0.0f, cell_shift = 0.0f, s_lo = 0.0f, s_hi = 0.0f;
     int phi = 1;
     cudaStream_t stream = nullptr;

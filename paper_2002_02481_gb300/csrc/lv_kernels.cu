@@ -1,6 +1,6 @@
-// lv_kernels.cu -- the main model's Monte Carlo kernels (instantiated from
-// lv_mc.cuh), the launchers that route every model to its translation unit,
-// and the fixed-order binary64 finalize (level 3 of the bucket sums).
+// lv_kernels.cu -- the launchers that route every model and cell mode to its
+// translation unit, and the fixed-order binary64 finalize (level 3 of the
+// bucket sums).
 #include "lv_mc.cuh"
 
 namespace lv {
@@ -102,37 +102,44 @@ __global__ void __launch_bounds__(32) finalize_kernel(const double* __restrict__
 
 }  // namespace
 
-size_t mc_smem_bytes(int I, int Je, int N, int block, bool greeks, bool grid_smem, bool extra, int ppl)
+size_t mc_smem_bytes(int I, int Je, int N, int n_bins, int block, bool greeks, bool grid_smem, bool extra, int ppl)
 {
-    return smem_layout(I, Je, N, block, greeks, grid_smem, extra, ppl).total;
+    return smem_layout(I, Je, N, n_bins, block, greeks, grid_smem, extra, ppl).total;
 }
 
 int ring_slots_per_warp() { return kRing * kTile; }
 int paths_per_tile(bool greeks) { return greeks ? kTile : kPriceTile; }
 
+#define LV_ROUTE(CALL, ...)                            \
+    switch (model * 3 + cell) {                        \
+    case 0: return CALL##_m0c0(__VA_ARGS__);           \
+    case 1: return CALL##_m0c1(__VA_ARGS__);           \
+    case 2: return CALL##_m0c2(__VA_ARGS__);           \
+    case 3: return CALL##_m1c0(__VA_ARGS__);           \
+    case 4: return CALL##_m1c1(__VA_ARGS__);           \
+    case 5: return CALL##_m1c2(__VA_ARGS__);           \
+    case 6: return CALL##_m2c0(__VA_ARGS__);           \
+    case 7: return CALL##_m2c1(__VA_ARGS__);           \
+    case 8: return CALL##_m2c2(__VA_ARGS__);           \
+    case 9: return CALL##_m3c0(__VA_ARGS__);           \
+    case 10: return CALL##_m3c1(__VA_ARGS__);          \
+    case 11: return CALL##_m3c2(__VA_ARGS__);          \
+    default: return cudaErrorInvalidValue;             \
+    }
+
 cudaError_t launch_mc(const McParams& p, int grid, int block, int k, bool greeks, size_t smem,
                       cudaStream_t s)
 {
-    switch (p.model) {
-    case 0: return launch_model_impl<0>(p, grid, block, k, greeks, smem, s);
-    case 1: return launch_mc_model1(p, grid, block, k, greeks, smem, s);
-    case 2: return launch_mc_model2(p, grid, block, k, greeks, smem, s);
-    case 3: return launch_mc_model3(p, grid, block, k, greeks, smem, s);
-    default: return cudaErrorInvalidValue;
-    }
+    const int model = p.model, cell = p.cell_mode;
+    LV_ROUTE(launch_mc, p, grid, block, k, greeks, smem, s)
 }
 
 cudaError_t mc_occupancy(int block, int k, bool greeks, int acc, bool dbg, bool grid_smem, int method, int model,
-                         bool extra, size_t smem, int* bps, int ppl)
+                         int cell, bool extra, size_t smem, int* bps, int ppl)
 {
-    switch (model) {
-    case 0: return occupancy_model_impl<0>(block, k, greeks, acc, dbg, grid_smem, method, extra, smem, bps, ppl);
-    case 1: return mc_occupancy_model1(block, k, greeks, acc, dbg, grid_smem, method, extra, smem, bps, ppl);
-    case 2: return mc_occupancy_model2(block, k, greeks, acc, dbg, grid_smem, method, extra, smem, bps, ppl);
-    case 3: return mc_occupancy_model3(block, k, greeks, acc, dbg, grid_smem, method, extra, smem, bps, ppl);
-    default: return cudaErrorInvalidValue;
-    }
+    LV_ROUTE(mc_occupancy, block, k, greeks, acc, dbg, grid_smem, method, extra, smem, bps, ppl)
 }
+#undef LV_ROUTE
 
 cudaError_t launch_finalize(const FinalizeParams& f, cudaStream_t s)
 {

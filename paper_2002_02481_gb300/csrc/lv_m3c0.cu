@@ -1,0 +1,5 @@
+// Monte Carlo kernels of model 3 (the Euler scheme on S with the weight linear in ln S), cell mode 0
+// (the cell found by a conversion or a binary search).
+#include "lv_mc.cuh"
+
+LV_DEFINE_KERNELS(3, 0)

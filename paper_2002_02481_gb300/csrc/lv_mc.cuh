@@ -2,7 +2,7 @@
 // 2002.02481, Sec. III, IV-A..IV-D), templated on the model (the reading of
 // the scheme and of the interpolation, see lv_device.cuh). Every translation
 // unit that includes this header instantiates its own kernels with internal
-// linkage: lv_kernels.cu the main model, lv_model1..3.cu the others.
+// linkage: lv_m<model>c<cell>.cu one model and one way to find the spot cell.
 //
 // Adjoint kernel: persistent, warp-centric, no block-wide barrier in its
 // main loop. Every warp repeatedly either
@@ -58,7 +58,7 @@ constexpr int kRing = 4;       // checkpoint slot groups of kTile per warp
 
 constexpr int kQueue = 64;     // per-warp FIFO capacity per path a lane runs in a forward tile
                                // (entries; < 32 + kTile * ppl never overflows kQueue * ppl)
-constexpr int kMaxWarps = 8;   // blockDim.x <= 256 (the adjoint kernel runs at most 128)
+constexpr int kMaxWarps = 8;   // blockDim.x <= 256 (every kernel here runs at most 128)
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
@@ -71,14 +71,14 @@ struct AccSlot {
 };
 
 struct SmemLayout {
-    size_t tab, sig, node, ab, tdt, qslot, qrel, qxb, acc, red, total;
+    size_t tab, sig, node, ab, bins, tdt, qslot, qrel, qxb, acc, red, total;
 };
 
 // extra: the adjoint kernel that also sums d V / d r and d V / d T (the time
 // slope table and two more accumulators per thread); ppl: paths per lane of
 // the adjoint's forward tiles (the FIFO grows with it).
-__host__ __device__ inline SmemLayout smem_layout(int I, int Je, int N, int block, bool greeks, bool grid_smem,
-                                                  bool extra = false, int ppl = 1)
+__host__ __device__ inline SmemLayout smem_layout(int I, int Je, int N, int n_bins, int block, bool greeks,
+                                                  bool grid_smem, bool extra = false, int ppl = 1)
 {
     const int W = block / 32;
     SmemLayout L;
@@ -87,6 +87,7 @@ __host__ __device__ inline SmemLayout smem_layout(int I, int Je, int N, int bloc
     L.sig = o;   if (grid_smem) o += align16(sizeof(float2) * (size_t)Je * (I - 1));
     L.node = o;  o += align16(sizeof(float) * (size_t)I);
     L.ab = o;    o += align16(sizeof(float2) * (size_t)I);
+    L.bins = o;  o += sizeof(float4) * (size_t)n_bins;
     L.tdt = o;   if (extra) o += align16(sizeof(float) * (size_t)N);
     // the adjoint kernel slices these three per warp from L.qslot: they stay
     // contiguous because each size is a multiple of 16 bytes (kQueue is)
@@ -135,6 +136,8 @@ __device__ __forceinline__ void stage_grid(const McParams& P, unsigned char* sme
         for (int e = tid; e < P.Je * (P.I - 1); e += B) s_sig[e] = P.sig2[e];
     for (int e = tid; e < P.I; e += B) s_node[e] = P.node[e];
     for (int e = tid; e < P.I - 1; e += B) s_ab[e] = P.ab[e];
+    float4* s_bins = reinterpret_cast<float4*>(smem + L.bins);
+    for (int e = tid; e < P.n_bins; e += B) s_bins[e] = P.bins[e];
     for (int n = tid; n < P.N; n += B) s_tab[n] = step_time(P, n);
     if (EXTRA) {
         float* s_tdt = reinterpret_cast<float*>(smem + L.tdt);
@@ -211,7 +214,7 @@ __device__ __forceinline__ void drain_buckets(float* l1, int nIJ, double* wrow)
 // independent dependency chains per lane, the per-step time data loaded once);
 // each path's arithmetic is that of PPL = 1, the ring groups and the FIFO
 // hold twice as many entries, and the reverse batches are unchanged.
-template <int KCK, int ACC, bool DBG, bool GS, int MODEL, bool EXTRA = false, int PPL = 1>
+template <int KCK, int ACC, bool DBG, bool GS, int MODEL, bool EXTRA, int PPL, int CELL>
 __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -219,7 +222,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
     constexpr int kQcap = kQueue * PPL;      // FIFO entries per warp
     const int B = blockDim.x, W = B >> 5;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const SmemLayout L = smem_layout(P.I, P.Je, P.N, B, true, GS, EXTRA, PPL);
+    const SmemLayout L = smem_layout(P.I, P.Je, P.N, P.n_bins, B, true, GS, EXTRA, PPL);
     stage_grid<GS, EXTRA>(P, smem, L);
     float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);    // this block's level-1 buckets
     // the three FIFO arrays of all warps are contiguous from L.qslot (each
@@ -248,7 +251,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
                       reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
-                      reinterpret_cast<const float*>(smem + L.tdt) };
+                      reinterpret_cast<const float4*>(smem + L.bins), reinterpret_cast<const float*>(smem + L.tdt) };
     const size_t cks = (size_t)gridDim.x * W * kRing * kSlots;  // checkpoint stride
     float* const ckw = P.ckpt + (size_t)wid * kRing * kSlots;    // this warp's slots
 
@@ -274,7 +277,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
                 uint32_t c1, c2;
                 path_counter(P, rel, c1, c2);
                 float ra = 0.0f, ta = 0.0f;
-                xbar = reverse_path<KCK, MODEL, EXTRA, PPL == 2 && (MODEL & kModelEulerS) == 0>(
+                xbar = reverse_path<CELL, KCK, MODEL, EXTRA, PPL == 2 && (MODEL & kModelEulerS) == 0>(
                     P, g, c1, c2, ckw + slot, cks, xbar, l1, &ra, &ta);
                 acc_add<ACC>(acc[2 * B], xbar);
                 if (EXTRA) {
@@ -305,7 +308,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
                 float ya, yb;
                 // packed pairs on the log-Euler readings; Euler on S keeps scalar pairs in
                 // this kernel (packed, it needs 82 registers: 5 blocks per SM instead of 6)
-                forward_path2<KCK, true, MODEL, (MODEL & kModelEulerS) == 0>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a,
+                forward_path2<CELL, KCK, true, MODEL, (MODEL & kModelEulerS) == 0>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a,
                                                                              ckw + slot_b, cks, ya, yb);
                 float V;
                 payoff<MODEL>(P, ya, V, xa);
@@ -344,7 +347,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
         if (active) {
             uint32_t c1, c2;
             path_counter(P, rel, c1, c2);
-            const float x = forward_path<KCK, true, DBG, MODEL>(P, g, c1, c2, ckw + slot, cks, rel);
+            const float x = forward_path<CELL, KCK, true, DBG, MODEL>(P, g, c1, c2, ckw + slot, cks, rel);
             float V;
             payoff<MODEL>(P, x, V, xbarN);
             acc_add<ACC>(acc[0], V);
@@ -406,14 +409,14 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
 // the paths with xbar_N != 0 join the warp's queue with c = xbar_N D_N. At
 // 32 queued paths (and at the end) the warp runs pass 2 (tangent_scatter)
 // on them as a full-warp batch. Buckets go through the same levels 0-3.
-template <int ACC, bool GS, int MODEL, int PPL = 1>
+template <int ACC, bool GS, int MODEL, int PPL, int CELL>
 __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int B = blockDim.x, W = B >> 5;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kQcap = kQueue * PPL;
-    const SmemLayout L = smem_layout(P.I, P.Je, P.N, B, true, GS, false, PPL);
+    const SmemLayout L = smem_layout(P.I, P.Je, P.N, P.n_bins, B, true, GS, false, PPL);
     stage_grid<GS>(P, smem, L);
     float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);
     int* q_rel = reinterpret_cast<int*>(smem + L.qrel) + warp * kQcap;
@@ -434,7 +437,8 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
     __syncthreads();
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
-                      reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab) };
+                      reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
+                      reinterpret_cast<const float4*>(smem + L.bins) };
     AccSlot* acc = reinterpret_cast<AccSlot*>(smem + L.acc) + tid;   // [3][block]: V, V^2, xbar_0
     acc[0] = acc[B] = acc[2 * B] = AccSlot{0.0, 0.0f, 0.0f};
     int q_head = 0, q_count = 0, batches = 0;
@@ -447,7 +451,7 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
                 const int e = (q_head + lane) & (kQcap - 1);
                 uint32_t c1, c2;
                 path_counter(P, q_rel[e], c1, c2);
-                tangent_scatter<MODEL>(P, g, c1, c2, q_c[e], l1);
+                tangent_scatter<CELL, MODEL>(P, g, c1, c2, q_c[e], l1);
             }
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
@@ -466,7 +470,7 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
                 path_counter(P, rel_b, c1b, c2b);
                 float ya, yb, Da, Db, V;
                 bool ta, tb;
-                tangent_forward2(P, g, c1a, c2a, c1b, c2b, ya, yb, Da, Db, ta, tb);
+                tangent_forward2<CELL>(P, g, c1a, c2a, c1b, c2b, ya, yb, Da, Db, ta, tb);
                 payoff<0>(P, ya, V, xa);
                 ca = xa * Da;
                 acc_add<ACC>(acc[0], V);
@@ -505,7 +509,7 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
             path_counter(P, rel, c1, c2);
             float D;
             bool tiny;
-            const float y = tangent_forward<MODEL>(P, g, c1, c2, D, tiny);
+            const float y = tangent_forward<CELL, MODEL>(P, g, c1, c2, D, tiny);
             float V;
             payoff<MODEL>(P, y, V, xbarN);
             c = xbarN * D;
@@ -548,14 +552,14 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
 // live paths are queued and scattered in full-warp batches. Main reading,
 // binary64 level 2. Rows: price sums as usual, buckets d^2 price / (d S0 d
 // sigma_ij) summed over paths.
-template <bool GS, int PPL = 1>
+template <bool GS, int PPL, int CELL>
 __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int B = blockDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kQcap = kQueue * PPL;
-    const SmemLayout L = smem_layout(P.I, P.Je, P.N, B, true, GS, false, PPL);
+    const SmemLayout L = smem_layout(P.I, P.Je, P.N, P.n_bins, B, true, GS, false, PPL);
     stage_grid<GS>(P, smem, L);
     float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);
     int* q_rel = reinterpret_cast<int*>(smem + L.qrel) + warp * kQcap;
@@ -569,7 +573,8 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
     __syncthreads();
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
-                      reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab) };
+                      reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
+                      reinterpret_cast<const float4*>(smem + L.bins) };
     AccSlot* acc = reinterpret_cast<AccSlot*>(smem + L.acc) + tid;   // [3][block]: V, V^2, xbar_0
     acc[0] = acc[B] = acc[2 * B] = AccSlot{0.0, 0.0f, 0.0f};
     int q_head = 0, q_count = 0, batches = 0;
@@ -582,7 +587,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
                 const int e = (q_head + lane) & (kQcap - 1);
                 uint32_t c1, c2;
                 path_counter(P, q_rel[e], c1, c2);
-                vanna_scatter(P, g, c1, c2, q_c[e] * P.inv_S0, l1);
+                vanna_scatter<CELL>(P, g, c1, c2, q_c[e] * P.inv_S0, l1);
             }
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
@@ -601,7 +606,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
                 path_counter(P, rel_b, c1b, c2b);
                 float ya, yb, Da, Db, V;
                 bool ta, tb;
-                tangent_forward2(P, g, c1a, c2a, c1b, c2b, ya, yb, Da, Db, ta, tb);
+                tangent_forward2<CELL>(P, g, c1a, c2a, c1b, c2b, ya, yb, Da, Db, ta, tb);
                 payoff<0>(P, ya, V, xa);
                 ca = xa * Da;
                 acc_add<0>(acc[0], V);
@@ -640,7 +645,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
             path_counter(P, rel, c1, c2);
             float D;
             bool tiny;
-            const float y = tangent_forward<0>(P, g, c1, c2, D, tiny);
+            const float y = tangent_forward<CELL, 0>(P, g, c1, c2, D, tiny);
             float V;
             payoff<0>(P, y, V, xbarN);
             c = xbarN * D;
@@ -667,21 +672,23 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
 
 // The forward pass alone. Bound by the FMA pipe (its 64-bit integer products
 // hold it for four cycles each) and the issue slots. With the straight-line
-// time loop unrolled over two blocks of steps, the index without a conversion
-// and the round keys in the parameter bank it runs 35 thread instructions per
-// path-step (43 before): 0.229 ms at 2^20 paths on the 30 x 60 grid with 156
-// steps, from 0.265 ms. 66 registers under a bound of three 256-thread blocks;
-// held to 64 by a bound of four it spilled.
-template <int ACC, bool GS, int MODEL>
-__global__ void __launch_bounds__(256, 3) price_kernel(const __grid_constant__ McParams P)
+// time loop, the index without a conversion and the round keys in the parameter
+// bank it runs 35 thread instructions per path-step (43 before): 0.229 ms at
+// 2^20 paths on the 30 x 60 grid with 156 steps, from 0.265 ms. Every tile takes
+// the same time, so the registers are held to nine blocks (2^20 paths: 245 us a
+// call against 257 with eight) and the launcher picks the blocks per SM that leave the last
+// round of tiles fullest (make_plan).
+template <int ACC, bool GS, int MODEL, int CELL>
+__global__ void __launch_bounds__(128, 9) price_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const SmemLayout L = smem_layout(P.I, P.Je, P.N, blockDim.x, false, GS);
+    const SmemLayout L = smem_layout(P.I, P.Je, P.N, P.n_bins, blockDim.x, false, GS);
     stage_grid<GS>(P, smem, L);
     __syncthreads();
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
-                      reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab) };
+                      reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
+                      reinterpret_cast<const float4*>(smem + L.bins) };
     const int lane = threadIdx.x & 31;
     AccSlot* acc = reinterpret_cast<AccSlot*>(smem + L.acc) + threadIdx.x;
     acc[0] = acc[blockDim.x] = AccSlot{0.0, 0.0f, 0.0f};
@@ -692,7 +699,7 @@ __global__ void __launch_bounds__(256, 3) price_kernel(const __grid_constant__ M
             path_counter(P, rel_a, c1a, c2a);
             path_counter(P, rel_b, c1b, c2b);
             float ya, yb;
-            forward_path2<4, false, MODEL, true>(P, g, c1a, c2a, c1b, c2b, nullptr, nullptr, 0, ya, yb);
+            forward_path2<CELL, 4, false, MODEL, true>(P, g, c1a, c2a, c1b, c2b, nullptr, nullptr, 0, ya, yb);
             float V, xb;
             payoff<MODEL>(P, ya, V, xb);
             acc_add<ACC>(acc[0], V);
@@ -737,8 +744,9 @@ cudaError_t occupancy(K kernel, int block, size_t smem, int* bps)
 }
 
 // Calls f(kernel, flag) with the instantiation for (greeks, k, acc, dbg, gs)
-// of model MODEL: k in {4, 8, 16, 32} for model 0, {4, 8} for the others.
-template <int MODEL, bool GS, typename F>
+// of model MODEL and cell mode CELL: k in {4, 8}, and for model 0 with the search
+// also 16 and 32.
+template <int MODEL, bool GS, int CELL, typename F>
 cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bool extra, F&& f, int ppl = 1)
 {
     if (ppl == 2) {        // two paths per lane: the reverse sweep (k = 4 or 8) of every reading,
@@ -747,17 +755,17 @@ cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bo
         if constexpr (MODEL == 0) {
             static bool cv2 = false, ct2[2] = {};
             if (method == kMethodVanna)
-                return acc == 0 ? f(vanna_kernel<GS, 2>, cv2) : cudaErrorInvalidValue;
+                return acc == 0 ? f(vanna_kernel<GS, 2, CELL>, cv2) : cudaErrorInvalidValue;
             if (method == LV_ADJ_TANGENT)
-                return acc ? f(tangent_kernel<1, GS, 0, 2>, ct2[1]) : f(tangent_kernel<0, GS, 0, 2>, ct2[0]);
+                return acc ? f(tangent_kernel<1, GS, 0, 2, CELL>, ct2[1]) : f(tangent_kernel<0, GS, 0, 2, CELL>, ct2[0]);
         }
         if (method != LV_ADJ_REVERSE) return cudaErrorInvalidValue;
         static bool cp[4] = {};
         switch (k * 2 + acc) {
-        case 8: return f(adjoint_kernel<4, 0, false, GS, MODEL, false, 2>, cp[0]);
-        case 9: return f(adjoint_kernel<4, 1, false, GS, MODEL, false, 2>, cp[1]);
-        case 16: return f(adjoint_kernel<8, 0, false, GS, MODEL, false, 2>, cp[2]);
-        case 17: return f(adjoint_kernel<8, 1, false, GS, MODEL, false, 2>, cp[3]);
+        case 8: return f(adjoint_kernel<4, 0, false, GS, MODEL, false, 2, CELL>, cp[0]);
+        case 9: return f(adjoint_kernel<4, 1, false, GS, MODEL, false, 2, CELL>, cp[1]);
+        case 16: return f(adjoint_kernel<8, 0, false, GS, MODEL, false, 2, CELL>, cp[2]);
+        case 17: return f(adjoint_kernel<8, 1, false, GS, MODEL, false, 2, CELL>, cp[3]);
         default: break;
         }
         return cudaErrorInvalidValue;
@@ -767,51 +775,54 @@ cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bo
         if constexpr (MODEL == 0) {
             static bool cv = false;
             if (!greeks || dbg || extra || acc != 0) return cudaErrorInvalidValue;
-            return f(vanna_kernel<GS>, cv);
+            return f(vanna_kernel<GS, 1, CELL>, cv);
         }
         return cudaErrorInvalidValue;
     }
     if (extra) {           // d V / d r and d V / d T: reverse sweep, binary64 level 2, k = 4 or 8
         static bool ce[2] = {};
         if (!greeks || dbg || method != LV_ADJ_REVERSE || acc != 0) return cudaErrorInvalidValue;
-        if (k == 4) return f(adjoint_kernel<4, 0, false, GS, MODEL, true>, ce[0]);
-        if (k == 8) return f(adjoint_kernel<8, 0, false, GS, MODEL, true>, ce[1]);
+        if (k == 4) return f(adjoint_kernel<4, 0, false, GS, MODEL, true, 1, CELL>, ce[0]);
+        if (k == 8) return f(adjoint_kernel<8, 0, false, GS, MODEL, true, 1, CELL>, ce[1]);
         return cudaErrorInvalidValue;
     }
     if (!greeks) {
         static bool c0 = false, c1 = false;
-        return acc ? f(price_kernel<1, GS, MODEL>, c1) : f(price_kernel<0, GS, MODEL>, c0);
+        return acc ? f(price_kernel<1, GS, MODEL, CELL>, c1) : f(price_kernel<0, GS, MODEL, CELL>, c0);
     }
     if (method == LV_ADJ_TANGENT && !dbg) {
         static bool t0 = false, t1 = false;
-        return acc ? f(tangent_kernel<1, GS, MODEL>, t1) : f(tangent_kernel<0, GS, MODEL>, t0);
+        return acc ? f(tangent_kernel<1, GS, MODEL, 1, CELL>, t1) : f(tangent_kernel<0, GS, MODEL, 1, CELL>, t0);
     }
     if (dbg) {
-        static bool cd = false;
-        if (k != 4) return cudaErrorInvalidValue;       // scratch must be planned with k = 4
-        return f(adjoint_kernel<4, 0, true, GS, MODEL>, cd);
+        if constexpr (CELL == kCellSearch) {
+            static bool cd = false;
+            if (k != 4) return cudaErrorInvalidValue;       // scratch must be planned with k = 4
+            return f(adjoint_kernel<4, 0, true, GS, MODEL, false, 1, CELL>, cd);
+        }
+        return cudaErrorInvalidValue;
     }
     static bool c[8] = {};
     switch (k * 2 + acc) {
-    case 8: return f(adjoint_kernel<4, 0, false, GS, MODEL>, c[0]);
-    case 9: return f(adjoint_kernel<4, 1, false, GS, MODEL>, c[1]);
-    case 16: return f(adjoint_kernel<8, 0, false, GS, MODEL>, c[2]);
-    case 17: return f(adjoint_kernel<8, 1, false, GS, MODEL>, c[3]);
+    case 8: return f(adjoint_kernel<4, 0, false, GS, MODEL, false, 1, CELL>, c[0]);
+    case 9: return f(adjoint_kernel<4, 1, false, GS, MODEL, false, 1, CELL>, c[1]);
+    case 16: return f(adjoint_kernel<8, 0, false, GS, MODEL, false, 1, CELL>, c[2]);
+    case 17: return f(adjoint_kernel<8, 1, false, GS, MODEL, false, 1, CELL>, c[3]);
     default: break;
     }
-    if constexpr (MODEL == 0) {
+    if constexpr (MODEL == 0 && CELL == kCellSearch) {
         switch (k * 2 + acc) {
-        case 32: return f(adjoint_kernel<16, 0, false, GS, 0>, c[4]);
-        case 33: return f(adjoint_kernel<16, 1, false, GS, 0>, c[5]);
-        case 64: return f(adjoint_kernel<32, 0, false, GS, 0>, c[6]);
-        case 65: return f(adjoint_kernel<32, 1, false, GS, 0>, c[7]);
+        case 32: return f(adjoint_kernel<16, 0, false, GS, 0, false, 1, CELL>, c[4]);
+        case 33: return f(adjoint_kernel<16, 1, false, GS, 0, false, 1, CELL>, c[5]);
+        case 64: return f(adjoint_kernel<32, 0, false, GS, 0, false, 1, CELL>, c[6]);
+        case 65: return f(adjoint_kernel<32, 1, false, GS, 0, false, 1, CELL>, c[7]);
         default: break;
         }
     }
     return cudaErrorInvalidValue;
 }
 
-template <int MODEL>
+template <int MODEL, int CELL>
 cudaError_t launch_model_impl(const McParams& p, int grid, int block, int k, bool greeks, size_t smem,
                               cudaStream_t s)
 {
@@ -820,19 +831,35 @@ cudaError_t launch_model_impl(const McParams& p, int grid, int block, int k, boo
     };
     const bool dbg = p.dbg_xN != nullptr;
     const int ppl = p.ppl > 1 ? p.ppl : 1;
-    return p.grid_smem ? with_kernel_gs<MODEL, true>(greeks, k, p.acc_mode, dbg, p.method, p.extra != 0, run, ppl)
-                       : with_kernel_gs<MODEL, false>(greeks, k, p.acc_mode, dbg, p.method, p.extra != 0, run, ppl);
+    return p.grid_smem
+               ? with_kernel_gs<MODEL, true, CELL>(greeks, k, p.acc_mode, dbg, p.method, p.extra != 0, run, ppl)
+               : with_kernel_gs<MODEL, false, CELL>(greeks, k, p.acc_mode, dbg, p.method, p.extra != 0, run, ppl);
 }
 
-template <int MODEL>
+template <int MODEL, int CELL>
 cudaError_t occupancy_model_impl(int block, int k, bool greeks, int acc, bool dbg, bool gs, int method, bool extra,
                                  size_t smem, int* bps, int ppl = 1)
 {
     auto occ = [&](auto kernel, bool&) { return occupancy(kernel, block, smem, bps); };
-    return gs ? with_kernel_gs<MODEL, true>(greeks, k, acc, dbg, method, extra, occ, ppl)
-              : with_kernel_gs<MODEL, false>(greeks, k, acc, dbg, method, extra, occ, ppl);
+    return gs ? with_kernel_gs<MODEL, true, CELL>(greeks, k, acc, dbg, method, extra, occ, ppl)
+              : with_kernel_gs<MODEL, false, CELL>(greeks, k, acc, dbg, method, extra, occ, ppl);
 }
 
 }  // namespace
 
 }  // namespace lv
+
+// Defines the launcher and the occupancy query of one model and cell mode.
+#define LV_DEFINE_KERNELS(M, C)                                                                                  \
+    namespace lv {                                                                                               \
+    cudaError_t launch_mc_m##M##c##C(const McParams& p, int grid, int block, int k, bool greeks, size_t smem,     \
+                                     cudaStream_t s)                                                             \
+    {                                                                                                            \
+        return launch_model_impl<M, C>(p, grid, block, k, greeks, smem, s);                                      \
+    }                                                                                                            \
+    cudaError_t mc_occupancy_m##M##c##C(int block, int k, bool greeks, int acc, bool dbg, bool grid_smem,        \
+                                        int method, bool extra, size_t smem, int* bps, int ppl)                  \
+    {                                                                                                            \
+        return occupancy_model_impl<M, C>(block, k, greeks, acc, dbg, grid_smem, method, extra, smem, bps, ppl); \
+    }                                                                                                            \
+    }

@@ -2,8 +2,9 @@
 (needs a GB300).
 
 A call whose cell index is bounded below 2^22 on every path takes the index
-from an addition rounded down, inside loops without a bound check; any other
-call on a log-spaced grid takes it from a float-to-integer conversion, inside
+from an addition rounded down (the cell itself on a log-spaced grid, a bin of
+at most two nodes on another one), inside loops without a bound check; any other
+call takes it from a float-to-integer conversion or a binary search, inside
 loops that check every step. A grid value that no path can reach (the last time
 row, at a maturity inside the time cell before it) moves a call from one to the
 other without touching any path: both must then give every path the same
@@ -53,13 +54,32 @@ def _run(surf, opt, lib, reading, call):
     return r
 
 
-@pytest.mark.parametrize("n_steps", [1, 3, 4, 5, 8, 9, 41])
+def _grids():
+    """20 x 10 grid, log-spaced; the same values on irregular nodes (bins); on
+    nodes with gaps between 1 and 400 of the smallest (up to 512 bins); on two
+    spot nodes 0.2 % off a log-spaced grid's, S0 itself a node. The last time
+    cell is [8/9, 1] in all of them."""
+    surf, _ = W.config_small()
+    rng = np.random.Generator(np.random.PCG64(11))
+    gaps = rng.uniform(0.4, 1.6, size=19)
+    uneven = 50.0 * 4.0 ** (np.concatenate([[0.0], np.cumsum(gaps)]) / gaps.sum())
+    tight = np.concatenate([np.linspace(98.0, 102.0, 15), [50.0, 70.0, 130.0, 160.0, 200.0]])
+    off = surf.spot.copy()
+    off[[7, 12]] *= 1.002
+    off[9] = 100.0
+    return [("log-spaced", surf.spot), ("irregular", uneven), ("tight around S0", np.sort(tight)),
+            ("S0 a node", off)]
+
+
+@pytest.mark.parametrize("grid", _grids(), ids=[g[0] for g in _grids()])
+@pytest.mark.parametrize("n_steps", [1, 3, 5, 8, 41])
 @pytest.mark.parametrize("call", CALLS)
 @pytest.mark.parametrize("reading", READINGS, ids=[r[2] for r in READINGS])
-def test_both_loops_give_the_same_paths(reading, call, n_steps, lib):
+def test_both_loops_give_the_same_paths(reading, call, n_steps, grid, lib):
     if reading[2] != "main reading" and (call.startswith("vanna") or call == "tangent pairs"):
         pytest.skip("main reading only")
-    surf, opt = W.config_small()                       # last time cell: [8/9, 1]
+    surf, opt = W.config_small()
+    surf = W.Surface(grid[1], surf.time, surf.sigma)
     opt = W.Option(**{**opt.__dict__, "T": 0.85, "r": 0.01, "n_steps": n_steps, "n_paths": 97})
     far = W.Surface(surf.spot, surf.time, surf.sigma.copy())
     far.sigma[-1, -1] = 1.0e7                          # unreachable: t_n < 0.85 < 8/9
