@@ -222,8 +222,8 @@ struct Plan {
     int block = 128, k = 4, bps = 1, grid = 1, ppl = 1;
     bool grid_smem = true;
     size_t smem = 0;
-    int n_tiles = 0, n_ck = 0, row_words = 0, n_chunks = 0;
-    size_t off_counter = 0, off_part = 0, off_chunks = 0, off_wrows = 0, off_l1 = 0, off_ckpt = 0, total = 0;
+    int n_tiles = 0, n_ck = 0, row_words = 0;
+    size_t off_part = 0, off_wrows = 0, off_l1 = 0, off_ckpt = 0, total = 0;
 };
 
 size_t round_up(size_t b, size_t a) { return (b + a - 1) / a * a; }
@@ -273,6 +273,22 @@ void occ_store(const OccKey& key, int occ)
 constexpr int64_t kPairMinPathsPerSm = 4 * 64 * 24;
 
 // n_paths < 0: a call large enough for two paths per lane.
+// The head of the handle's scratch, at the same place in every launch's layout:
+// the tile counter, the flag and the block counter, then the call's binary64 sums.
+// Zero between launches: cleared when allocated, left at zero by every launch.
+constexpr size_t kOffSums = 256;
+size_t scratch_header(const lv_surface_s* h)
+{
+    return round_up(kOffSums + sizeof(double) * (5 + (size_t)h->Je * h->I), 256);
+}
+
+void bind_header(lv::McParams& P, char* base)
+{
+    P.tile_counter = reinterpret_cast<unsigned int*>(base);
+    P.done = P.tile_counter + 2;          // word 1 is the flag
+    P.sums = reinterpret_cast<double*>(base + kOffSums);
+}
+
 lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* block, int* k, int* bps,
                         bool dbg = false, bool* grid_smem = nullptr, bool extra = false, bool vanna = false,
                         int* ppl_out = nullptr, int64_t n_paths = -1)
@@ -299,9 +315,9 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
                        ((vanna || h->adj_method == LV_ADJ_TANGENT) ? model == 0 : (*k == 4 || *k == 8));
     if (!pairs) ppl = 1;
     if (ppl_out) *ppl_out = ppl;
-    const bool gs = lv::mc_smem_bytes(h->I, h->Je, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
+    const bool gs = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
     if (grid_smem) *grid_smem = gs;
-    const size_t smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, h->n_bins, *block, greeks, gs, extra, ppl);
+    const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, gs, extra, ppl);
     if (smem > 200 * 1024)
         return fail(LV_EINVAL, "time table does not fit in shared memory (" + std::to_string(smem) + " bytes)");
     int occ = 0;
@@ -328,7 +344,7 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     lv_status st = choose_launch(h, n_steps, greeks, &p->block, &p->k, &p->bps, dbg, &p->grid_smem, extra, vanna,
                                  &p->ppl, n_paths);
     if (st != LV_OK) return st;
-    p->smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, h->n_bins, p->block, greeks, p->grid_smem, extra, p->ppl);
+    p->smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, p->block, greeks, p->grid_smem, extra, p->ppl);
     const int warps = p->block / 32;
     const int64_t tiles = (n_paths + lv::paths_per_tile(greeks) - 1) / lv::paths_per_tile(greeks);   // claimed by warps
     p->n_tiles = (int)tiles;
@@ -358,12 +374,9 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     const size_t nIJ = (size_t)h->Je * h->I;
     // price-only rows hold the scalars; extra rows end with the sums of d V / d r and d V / d T
     p->row_words = greeks ? 3 + (int)nIJ + (extra ? 2 : 0) : 3;
-    p->n_chunks = lv::finalize_chunks(p->grid);
     const size_t total_warps = (size_t)p->grid * warps;
-    size_t o = 0;
-    p->off_counter = o; o += 256;
+    size_t o = scratch_header(h);
     p->off_part = o;    o = round_up(o + sizeof(double) * (size_t)p->grid * p->row_words, 256);
-    p->off_chunks = o;  o = round_up(o + sizeof(double) * (size_t)p->n_chunks * p->row_words, 256);
     p->off_wrows = o;                   // per-warp rows: Kahan mode only
     if (greeks && !extra && !vanna && h->acc_mode == LV_ACC_KAHAN)
         o = round_up(o + sizeof(double) * total_warps * nIJ, 256);
@@ -390,8 +403,7 @@ lv_status ensure_scratch(lv_surface_s* h, size_t bytes)
         return fail(LV_ENOMEM, "cannot allocate " + std::to_string(want) + " bytes of scratch");
     }
     h->scratch_bytes = want;
-    // the tile counter starts at zero; every finalize resets it
-    LV_CUDA(cudaMemsetAsync(h->d_scratch, 0, 256, h->stream));
+    LV_CUDA(cudaMemsetAsync(h->d_scratch, 0, scratch_header(h), h->stream));
     return LV_OK;
 }
 
@@ -457,6 +469,11 @@ lv::McParams base_params(const lv_surface_s* h, const McCall& c, int k)
     P.stream_id = c.stream_id;
     P.path_begin = c.path_begin;
     P.n_paths = c.n_paths;
+    P.out = c.d_out;
+    P.want_sums = c.want_sums ? 1 : 0;
+    P.inv_paths = 1.0 / (double)c.n_paths;
+    P.var_scale = c.n_paths > 1 ? (double)c.n_paths / ((double)c.n_paths - 1.0) : 0.0;
+    P.inv_delta = 1.0 / ((double)c.n_paths * c.S0);
     P.acc_mode = h->acc_mode;
     P.method = LV_ADJ_REVERSE;
     P.bins = h->d_bins;
@@ -487,7 +504,7 @@ lv_status run_mc(lv_surface_s* h, const McCall& c)
     lv::McParams P = base_params(h, c, p.k);
     P.n_tiles = p.n_tiles;
     P.ppl = p.ppl;
-    P.tile_counter = reinterpret_cast<unsigned int*>(base + p.off_counter);
+    bind_header(P, base);
     P.partials = reinterpret_cast<double*>(base + p.off_part);
     P.row_words = p.row_words;
     P.warp_rows = reinterpret_cast<double*>(base + p.off_wrows);
@@ -519,21 +536,6 @@ lv_status run_mc(lv_surface_s* h, const McCall& c)
     if (h->ev_start) LV_CUDA(cudaEventRecord(h->ev_start, h->stream));
     LV_CUDA(lv::launch_mc(P, p.grid, p.block, p.k, c.greeks, p.smem, h->stream));
     if (h->ev_end) LV_CUDA(cudaEventRecord(h->ev_end, h->stream));
-    lv::FinalizeParams F{};
-    F.partials = P.partials;
-    F.G = p.grid;
-    F.row_words = p.row_words;
-    F.I = h->I;
-    F.J = h->J;
-    F.n_paths = c.n_paths;
-    F.S0 = c.S0;
-    F.want_sums = c.want_sums ? 1 : 0;
-    F.chunks = reinterpret_cast<double*>(base + p.off_chunks);
-    F.out = c.d_out;
-    F.tile_counter = P.tile_counter;
-    F.flag = P.flag;
-    F.extra = c.extra ? 1 : 0;
-    LV_CUDA(lv::launch_finalize(F, h->stream));
     return LV_OK;
 }
 
@@ -549,9 +551,18 @@ lv_status sigma64_current(lv_surface_s* h)
     return LV_OK;
 }
 
-lv_status fetch_result(lv_surface_s* h, bool extra = false)
+// Waits for a call that wrote its results to h_res (pinned host memory, written
+// by the kernel's last block: no copy follows it).
+lv_status wait_result(lv_surface_s* h)
 {
-    const size_t n = 3 + (size_t)h->I * h->J + (extra ? 2 : 0);
+    LV_CUDA(cudaStreamSynchronize(h->stream));
+    return LV_OK;
+}
+
+// Copies the bump baselines' results from d_res to h_res and waits.
+lv_status fetch_result(lv_surface_s* h)
+{
+    const size_t n = 3 + (size_t)h->I * h->J;
     LV_CUDA(cudaMemcpyAsync(h->h_res, h->d_res, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
     LV_CUDA(cudaStreamSynchronize(h->stream));
     return LV_OK;
@@ -828,10 +839,10 @@ lv_status lv_price(lv_surface_t h, double S0, double r, double K, double T, int3
     if (!h || !out_price) return fail(LV_EINVAL, "NULL argument");
     DeviceGuard g(h->device);
     if (!g.ok) return fail(LV_ECUDA, "cannot select the handle's device");
-    McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, false, false, h->d_res};
+    McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, false, false, h->h_res};
     lv_status st = run_mc(h, c);
     if (st != LV_OK) return st;
-    st = fetch_result(h);
+    st = wait_result(h);
     if (st != LV_OK) return st;
     *out_price = h->h_res[LV_OUT_PRICE];
     if (out_stderr) *out_stderr = h->h_res[LV_OUT_STDERR];
@@ -855,10 +866,10 @@ lv_status lv_price_greeks(lv_surface_t h, double S0, double r, double K, double 
     if (!h || !out_price || !out_delta || !out_vega) return fail(LV_EINVAL, "NULL argument");
     DeviceGuard g(h->device);
     if (!g.ok) return fail(LV_ECUDA, "cannot select the handle's device");
-    McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, true, false, h->d_res};
+    McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, true, false, h->h_res};
     lv_status st = run_mc(h, c);
     if (st != LV_OK) return st;
-    st = fetch_result(h);
+    st = wait_result(h);
     if (st != LV_OK) return st;
     if (std::isnan(h->h_res[LV_OUT_PRICE]))    // outputs left untouched, like every failure
         return fail(LV_ENUMERIC, "a factor 1 + g_n vanished on a live path: use LV_ADJ_REVERSE for this grid");
@@ -875,11 +886,11 @@ lv_status lv_price_greeks_ext(lv_surface_t h, double S0, double r, double K, dou
     if (!h || !out_price || !out_delta || !out_vega || !out_rho || !out_dVdT) return fail(LV_EINVAL, "NULL argument");
     DeviceGuard g(h->device);
     if (!g.ok) return fail(LV_ECUDA, "cannot select the handle's device");
-    McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, true, false, h->d_res};
+    McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, true, false, h->h_res};
     c.extra = true;
     lv_status st = run_mc(h, c);
     if (st != LV_OK) return st;
-    st = fetch_result(h, true);
+    st = wait_result(h);
     if (st != LV_OK) return st;
     const size_t IJ = (size_t)h->I * h->J;
     *out_price = h->h_res[LV_OUT_PRICE];
@@ -919,11 +930,11 @@ lv_status lv_price_greeks_vanna(lv_surface_t h, double S0, double r, double K, d
     if (!h || !out_price || !out_delta || !out_vanna) return fail(LV_EINVAL, "NULL argument");
     DeviceGuard g(h->device);
     if (!g.ok) return fail(LV_ECUDA, "cannot select the handle's device");
-    McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, true, false, h->d_res};
+    McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, true, false, h->h_res};
     c.vanna = true;
     lv_status st = run_mc(h, c);
     if (st != LV_OK) return st;
-    st = fetch_result(h);
+    st = wait_result(h);
     if (st != LV_OK) return st;
     if (std::isnan(h->h_res[LV_OUT_PRICE]))    // outputs left untouched, like every failure
         return fail(LV_ENUMERIC, "a factor 1 + g_n vanished on a live path");
@@ -1054,7 +1065,7 @@ lv_status lv_bump_greeks(lv_surface_t h, double S0, double r, double K, double T
     const int64_t slots = (int64_t)bps * h->num_sms;
     const int grid = (int)(items < slots ? items : slots);
     const int nch = lv::bump_chunks(grid);
-    size_t o = 256;
+    size_t o = scratch_header(h);
     const size_t off_part = o;
     o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
     const size_t off_chunks = o;
@@ -1116,7 +1127,7 @@ lv_status lv_price_greeks_fp64_device(lv_surface_t h, double S0, double r, doubl
     const int64_t slots = (int64_t)bps * h->num_sms;
     const int grid = (int)(want < slots ? want : slots);
     const int row_words = 3 + h->Je * h->I;
-    size_t o = 256;                                   // [0, 256): tile counter (unused), flag
+    size_t o = scratch_header(h);
     const size_t off_part = o;
     o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
     const size_t off_chunks = o;
@@ -1192,7 +1203,7 @@ lv_status lv_bump_greeks_fp64(lv_surface_t h, double S0, double r, double K, dou
     const int64_t slots = (int64_t)bps * h->num_sms;
     const int grid = (int)(items < slots ? items : slots);
     const int nch = lv::bump_chunks(grid);
-    size_t o = 256;
+    size_t o = scratch_header(h);
     const size_t off_part = o;
     o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
     const size_t off_chunks = o;
@@ -1401,15 +1412,14 @@ lv_status static_scratch(int device, char** out)
 // Scratch layout of one adjoint launch with `grid` blocks (same sections as
 // the allocating path); returns the bytes needed.
 size_t static_plan_bytes(const lv_surface_s* h, int grid, int block, int k, int ppl, int n_steps, size_t* off_part,
-                         size_t* off_chunks, size_t* off_wrows, size_t* off_l1, size_t* off_ckpt)
+                         size_t* off_wrows, size_t* off_l1, size_t* off_ckpt)
 {
     const size_t nIJ = (size_t)h->Je * h->I;
     const size_t row_words = 3 + nIJ;
     const size_t warps = (size_t)grid * (block / 32);
     const size_t n_ck = h->adj_method == LV_ADJ_TANGENT ? 0 : (size_t)((n_steps + k - 1) / k);
-    size_t o = 256;                                               // [0, 256): tile counter, flag
+    size_t o = scratch_header(h);
     *off_part = o;   o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
-    *off_chunks = o; o = round_up(o + sizeof(double) * (size_t)lv::finalize_chunks(grid) * row_words, 256);
     *off_wrows = o;                                               // per-warp rows: Kahan mode only
     if (h->acc_mode == LV_ACC_KAHAN) o = round_up(o + sizeof(double) * warps * nIJ, 256);
     *off_l1 = o;     o = round_up(o + sizeof(float) * (size_t)grid * nIJ, 256);
@@ -1440,13 +1450,13 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
     const int warps = block / 32;
     const int64_t tiles = (n_paths + lv::paths_per_tile(true) - 1) / lv::paths_per_tile(true);
     const int64_t want_blocks = (tiles + warps - 1) / warps;
-    size_t off_part = 0, off_chunks = 0, off_wrows = 0, off_l1 = 0, off_ckpt = 0;
+    size_t off_part = 0, off_wrows = 0, off_l1 = 0, off_ckpt = 0;
     // two paths per lane double each block's checkpoint ring: unless the caller
     // asked for them, run one path per lane when the full-width grid would not
     // fit in the static array at two (one fits about twice as many blocks)
     if (ppl == 2 && h->cfg_ppl == 0) {
         const int64_t full = want_blocks < (int64_t)bps * h->num_sms ? want_blocks : (int64_t)bps * h->num_sms;
-        if (static_plan_bytes(h, (int)full, block, k, 2, n_steps, &off_part, &off_chunks, &off_wrows, &off_l1,
+        if (static_plan_bytes(h, (int)full, block, k, 2, n_steps, &off_part, &off_wrows, &off_l1,
                               &off_ckpt) > kStaticScratchBytes) {
             h->cfg_ppl = 1;
             st = choose_launch(h, n_steps, true, &block, &k, &bps, false, &grid_smem, false, false, &ppl, n_paths);
@@ -1458,12 +1468,12 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
     int grid = (int)(want_blocks < slots ? want_blocks : slots);
     // the most blocks (at most the full-width grid) whose scratch fits in the static array;
     // the plan's size grows with the grid, so bisect
-    if (static_plan_bytes(h, grid, block, k, ppl, n_steps, &off_part, &off_chunks, &off_wrows, &off_l1, &off_ckpt) >
+    if (static_plan_bytes(h, grid, block, k, ppl, n_steps, &off_part, &off_wrows, &off_l1, &off_ckpt) >
         kStaticScratchBytes) {
         int lo = 1, hi = grid - 1;
         while (lo < hi) {
             const int mid = lo + (hi - lo + 1) / 2;
-            if (static_plan_bytes(h, mid, block, k, ppl, n_steps, &off_part, &off_chunks, &off_wrows, &off_l1,
+            if (static_plan_bytes(h, mid, block, k, ppl, n_steps, &off_part, &off_wrows, &off_l1,
                                   &off_ckpt) <= kStaticScratchBytes)
                 lo = mid;
             else
@@ -1471,7 +1481,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
         }
         grid = lo;
     }
-    const size_t need = static_plan_bytes(h, grid, block, k, ppl, n_steps, &off_part, &off_chunks, &off_wrows,
+    const size_t need = static_plan_bytes(h, grid, block, k, ppl, n_steps, &off_part, &off_wrows,
                                           &off_l1, &off_ckpt);
     if (need > kStaticScratchBytes)
         return fail(LV_EINVAL, "grid of " + std::to_string(h->I) + " x " + std::to_string(h->J) + " nodes with " +
@@ -1483,7 +1493,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
     lv::McParams P = base_params(h, c, k);
     P.n_tiles = (int)tiles;
     P.ppl = ppl;
-    P.tile_counter = reinterpret_cast<unsigned int*>(base);
+    bind_header(P, base);
     P.partials = reinterpret_cast<double*>(base + off_part);
     P.row_words = 3 + h->Je * h->I;
     P.warp_rows = reinterpret_cast<double*>(base + off_wrows);
@@ -1496,24 +1506,11 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
         P.method = LV_ADJ_TANGENT;
         P.flag = P.tile_counter + 1;
     }
-    // the array keeps the previous call's contents: the tile counter and the
-    // flag must start at zero (every other section is written before it is read)
-    LV_CUDA(cudaMemsetAsync(P.tile_counter, 0, 2 * sizeof(unsigned int), h->stream));
-    const size_t smem = lv::mc_smem_bytes(h->I, h->Je, n_steps, h->n_bins, block, true, grid_smem, false, ppl);
+    // the array keeps the previous call's contents (another handle's, perhaps): the
+    // counters, the flag and the sums must start at zero (every other section is
+    // written before it is read)
+    LV_CUDA(cudaMemsetAsync(base, 0, scratch_header(h), h->stream));
+    const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, block, true, grid_smem, false, ppl);
     LV_CUDA(lv::launch_mc(P, grid, block, k, true, smem, h->stream));
-    lv::FinalizeParams F{};
-    F.partials = P.partials;
-    F.G = grid;
-    F.row_words = P.row_words;
-    F.I = h->I;
-    F.J = h->J;
-    F.n_paths = n_paths;
-    F.S0 = S0;
-    F.want_sums = 0;
-    F.chunks = reinterpret_cast<double*>(base + off_chunks);
-    F.out = d_out;
-    F.tile_counter = P.tile_counter;
-    F.flag = P.flag;
-    LV_CUDA(lv::launch_finalize(F, h->stream));
     return LV_OK;
 }

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
             for (int e = tid; e < Q.I; e += Bk) s_node[e] = Q.node[e];
             for (int e = tid; e < Q.I - 1; e += Bk) s_ab[e] = Q.ab[e];
             for (int e = tid; e < Q.n_bins; e += Bk) s_bins[e] = Q.bins[e];
-            for (int n = tid; n < Q.N; n += Bk) s_tab[n] = step_time(Q, n);
+            for (int n = tid; n < Q.N; n += Bk) s_tab[n] = step_time(Q, Q.tau, n);
             if (tid == 0) s_ctl[2] = it.inst;
         }
         if (tid == 0) s_ctl[1] = it.first_tile;

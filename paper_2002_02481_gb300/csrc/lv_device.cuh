@@ -222,7 +222,7 @@ __device__ __forceinline__ void normals4_neg(uint32_t blk, uint32_t c1, uint32_t
 // [0, 1], decided in binary64. Returned as (j (I-1), j I, bits of v twice):
 // the row of the sigma pairs for j (row j + 1 is I - 1 pairs further on), the
 // bucket row, and v as the pair the packed arithmetic takes.
-__device__ __forceinline__ int4 step_time(const McParams& P, int n)
+__device__ __forceinline__ int4 step_time(const McParams& P, const double* tau, int n)
 {
     const double t = (double)n * P.dt_d;
     int j = 0;
@@ -231,11 +231,11 @@ __device__ __forceinline__ int4 step_time(const McParams& P, int n)
         int lo = 0, hi = P.J - 2;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (P.tau[mid] <= t) lo = mid;
+            if (tau[mid] <= t) lo = mid;
             else hi = mid - 1;
         }
         j = lo;
-        v = (t - P.tau[j]) / (P.tau[j + 1] - P.tau[j]);
+        v = (t - tau[j]) / (tau[j + 1] - tau[j]);
         v = fmin(fmax(v, 0.0), 1.0);
     }
     const int vb = __float_as_int((float)v);
@@ -245,17 +245,17 @@ __device__ __forceinline__ int4 step_time(const McParams& P, int n)
 // Time slope factor of step n for d price / d T: (n / N) / (tau_{j+1} - tau_j)
 // with the cell of step_time while t_n lies in [tau_0, tau_{J-1}) (the grid is
 // flat in t outside, and with one time node), else 0; decided in binary64.
-__device__ __forceinline__ float step_tdt(const McParams& P, int n)
+__device__ __forceinline__ float step_tdt(const McParams& P, const double* tau, int n)
 {
     const double t = (double)n * P.dt_d;
-    if (P.J < 2 || t < P.tau[0] || t >= P.tau[P.J - 1]) return 0.0f;
+    if (P.J < 2 || t < tau[0] || t >= tau[P.J - 1]) return 0.0f;
     int lo = 0, hi = P.J - 2;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (P.tau[mid] <= t) lo = mid;
+        if (tau[mid] <= t) lo = mid;
         else hi = mid - 1;
     }
-    return (float)(((double)n / (double)P.N) / (P.tau[lo + 1] - P.tau[lo]));
+    return (float)(((double)n / (double)P.N) / (tau[lo + 1] - tau[lo]));
 }
 
 // Shared-memory view of the grid for one block.
@@ -679,6 +679,14 @@ __device__ __forceinline__ void forward_path2(const McParams& P, const SmemGrid&
     });
 }
 
+// A binary32 reduction in L2 without a return value. Written out because in a
+// kernel that also has a memory fence the compiler turns atomicAdd into the
+// returning form, whose replies took the adjoint from 0.601 to 0.756 ms.
+__device__ __forceinline__ void red_add(float* p, float v)
+{
+    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(v) : "memory");
+}
+
 // Philox counter words of path `rel` of the call: c1 = path bits 0..31,
 // c2 = path bits 32..47 | stream_id << 16 (the path index is path_begin + rel).
 __device__ __forceinline__ void path_counter(const McParams& P, long long rel, uint32_t& c1, uint32_t& c2)
@@ -713,10 +721,10 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
     auto flush = [&]() {
         float* p0 = l1 + cur;
         float* p1 = p0 + P.I;
-        atomicAdd(p0, A - AU);
-        atomicAdd(p0 + 1, AU);
-        atomicAdd(p1, Bs - BU);
-        atomicAdd(p1 + 1, BU);
+        red_add(p0, A - AU);
+        red_add(p0 + 1, AU);
+        red_add(p1, Bs - BU);
+        red_add(p1 + 1, BU);
     };
     auto gen = [&](int blk, float (&z)[4]) {
         if (kNeg) normals4_neg((uint32_t)blk, c1, c2, P.rk, z);
@@ -782,18 +790,19 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
             }
         }
     };
-    float x = ck[(size_t)(nseg - 1) * cks];
+    // checkpoints are read two segments ahead: one segment ahead the compiler may
+    // place the load behind the recompute, which leaves its latency exposed
+    float x = ck[(size_t)(nseg - 1) * cks], xn = ck[(size_t)max(nseg - 2, 0) * cks];
     float z[4];
     gen((nseg - 1) * (KCK / 4), z);
     for (int m = nseg - 1; m >= 0; --m) {
-        // the next segment's checkpoint and first normals, in flight during this one
-        const int mp = max(m - 1, 0);
-        const float xn = ck[(size_t)mp * cks];
-        float zn[4];
-        gen(mp * (KCK / 4), zn);
+        const float xf = ck[(size_t)max(m - 2, 0) * cks];
+        float zn[4];                              // the next segment's first normals, beside this one
+        gen(max(m - 1, 0) * (KCK / 4), zn);
         if (CELL != kCellSearch && (m + 1) * KCK <= P.N) segment(m, x, z, true);
         else segment(m, x, z, false);
         x = xn;
+        xn = xf;
 #pragma unroll
         for (int q = 0; q < 4; ++q) z[q] = zn[q];
     }
@@ -939,10 +948,10 @@ __device__ __forceinline__ void tangent_scatter_f(const McParams& P, const SmemG
     auto flush = [&]() {
         float* p0 = l1 + cur;
         float* p1 = p0 + P.I;
-        atomicAdd(p0, A - AU);
-        atomicAdd(p0 + 1, AU);
-        atomicAdd(p1, Bs - BU);
-        atomicAdd(p1 + 1, BU);
+        red_add(p0, A - AU);
+        red_add(p0 + 1, AU);
+        red_add(p1, Bs - BU);
+        red_add(p1 + 1, BU);
     };
     time_blocks<float, CELL != kCellSearch, 1>(
         P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
@@ -999,10 +1008,10 @@ __device__ __forceinline__ void vanna_scatter_f(const McParams& P, const SmemGri
     auto flush = [&]() {
         float* p0 = l1 + cur;
         float* p1 = p0 + P.I;
-        atomicAdd(p0, A - AU - E0);
-        atomicAdd(p0 + 1, AU + E0);
-        atomicAdd(p1, Bs - BU - E1);
-        atomicAdd(p1 + 1, BU + E1);
+        red_add(p0, A - AU - E0);
+        red_add(p0 + 1, AU + E0);
+        red_add(p1, Bs - BU - E1);
+        red_add(p1 + 1, BU + E1);
     };
     time_blocks<float, CELL != kCellSearch, 1>(
         P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },

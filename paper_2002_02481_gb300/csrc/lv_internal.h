@@ -98,7 +98,10 @@ struct McParams {
     // work decomposition and scratch
     int n_tiles;           // ceil(n_paths / paths_per_tile()): tiles claimed by warps
     int ppl;               // adjoint: paths per lane of a forward tile (1 or 2; a warp claims ppl tiles)
-    unsigned int* tile_counter;   // zero before the launch, reset by the finalize
+    unsigned int* tile_counter;   // zero before the launch, reset by its last block, as are the next two
+    unsigned int* done;    // blocks that have added their sums
+    double* sums;          // [5 + Je * I] binary64 sums of the call: V, V^2, x_bar_0, buckets
+                           // (time-major), then d V / d r and d V / d T
     double* partials;      // [gridDim.x][row_words] per-block binary64 rows
     int row_words;         // 3 + Je * I (adjoint) or 3 (price only)
     double* warp_rows;     // [gridDim.x * warps][Je * I] per-warp level-2 rows
@@ -110,6 +113,13 @@ struct McParams {
     int acc_mode;          // 0 binary64, 1 Kahan binary32
     int method;            // LV_ADJ_REVERSE or LV_ADJ_TANGENT
     unsigned int* flag;    // tangent-ratio adjoint: count of live paths with a vanishing 1 + g_n
+
+    // results, written by the launch's last block
+    double* out;           // device memory or pinned host memory
+    int want_sums;         // 1: raw sums, 0: price / delta / stderr / vega
+    double inv_paths;      // 1 / n_paths
+    double var_scale;      // n_paths / (n_paths - 1) (0 for one path)
+    double inv_delta;      // 1 / (n_paths S0)
 
     // per-path outputs and near-node decision log (debug entry point only;
     // dbg_xN != null selects the logging instantiation)
@@ -185,7 +195,7 @@ cudaError_t launch_bump_finalize(const double* partials, int G, int row_words, d
                                  long long n_paths, double eps, double eps_S, double* out,
                                  unsigned int* tile_counter, cudaStream_t s);
 
-size_t mc_smem_bytes(int I, int Je, int N, int n_bins, int block, bool greeks, bool grid_smem, bool extra = false,
+size_t mc_smem_bytes(int I, int J, int N, int n_bins, int block, bool greeks, bool grid_smem, bool extra = false,
                      int ppl = 1);
 
 // Binary64 paths (lv_fp64.cu): the full-FP64 reference adjoint and the

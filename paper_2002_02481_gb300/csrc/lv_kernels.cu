@@ -102,9 +102,9 @@ __global__ void __launch_bounds__(32) finalize_kernel(const double* __restrict__
 
 }  // namespace
 
-size_t mc_smem_bytes(int I, int Je, int N, int n_bins, int block, bool greeks, bool grid_smem, bool extra, int ppl)
+size_t mc_smem_bytes(int I, int J, int N, int n_bins, int block, bool greeks, bool grid_smem, bool extra, int ppl)
 {
-    return smem_layout(I, Je, N, n_bins, block, greeks, grid_smem, extra, ppl).total;
+    return smem_layout(I, J, N, n_bins, block, greeks, grid_smem, extra, ppl).total;
 }
 
 int ring_slots_per_warp() { return kRing * kTile; }

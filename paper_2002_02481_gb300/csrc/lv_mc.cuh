@@ -34,9 +34,9 @@
 // L2 without a retry loop) into a per-block bucket array in global memory
 // (level 1); every few batches a warp drains that array (atomicExch) into
 // level 2: the block's binary64 row through binary64 reductions, or in Kahan
-// mode a compensated binary32 row the warp owns; at the end each block folds
-// what is left into its binary64 row, and a separate fixed-order binary64
-// reduction over blocks gives the outputs (level 3).
+// mode a compensated binary32 row the warp owns; at the end each block adds
+// what it holds to the call's binary64 sums, and the last block to arrive writes
+// the outputs (level 3).
 //
 // The DBG instantiation additionally writes per-path results and logs
 // every forward step whose spot lies within a relative band of its cell's
@@ -62,6 +62,8 @@ constexpr int kMaxWarps = 8;   // blockDim.x <= 256 (every kernel here runs at m
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
+constexpr int kStagedTau = 256;   // time nodes staged in shared memory for the time table's search
+
 // Level-2 accumulator of one value: binary64 or Kahan-compensated binary32.
 // The slots live in shared memory (one per thread and value), which keeps
 // them out of the registers the reverse sweep needs.
@@ -71,16 +73,16 @@ struct AccSlot {
 };
 
 struct SmemLayout {
-    size_t tab, sig, node, ab, bins, tdt, qslot, qrel, qxb, acc, red, total;
+    size_t tab, sig, node, ab, bins, tau, tdt, qslot, qrel, qxb, acc, red, total;
 };
 
 // extra: the adjoint kernel that also sums d V / d r and d V / d T (the time
 // slope table and two more accumulators per thread); ppl: paths per lane of
 // the adjoint's forward tiles (the FIFO grows with it).
-__host__ __device__ inline SmemLayout smem_layout(int I, int Je, int N, int n_bins, int block, bool greeks,
+__host__ __device__ inline SmemLayout smem_layout(int I, int J, int N, int n_bins, int block, bool greeks,
                                                   bool grid_smem, bool extra = false, int ppl = 1)
 {
-    const int W = block / 32;
+    const int W = block / 32, Je = J > 1 ? J : 2;
     SmemLayout L;
     size_t o = 0;
     L.tab = o;   o += align16(sizeof(int4) * (size_t)N);
@@ -88,6 +90,7 @@ __host__ __device__ inline SmemLayout smem_layout(int I, int Je, int N, int n_bi
     L.node = o;  o += align16(sizeof(float) * (size_t)I);
     L.ab = o;    o += align16(sizeof(float2) * (size_t)I);
     L.bins = o;  o += sizeof(float4) * (size_t)n_bins;
+    L.tau = o;   if (J <= kStagedTau) o += align16(sizeof(double) * (size_t)J);
     L.tdt = o;   if (extra) o += align16(sizeof(float) * (size_t)N);
     // the adjoint kernel slices these three per warp from L.qslot: they stay
     // contiguous because each size is a multiple of 16 bytes (kQueue is)
@@ -138,39 +141,125 @@ __device__ __forceinline__ void stage_grid(const McParams& P, unsigned char* sme
     for (int e = tid; e < P.I - 1; e += B) s_ab[e] = P.ab[e];
     float4* s_bins = reinterpret_cast<float4*>(smem + L.bins);
     for (int e = tid; e < P.n_bins; e += B) s_bins[e] = P.bins[e];
-    for (int n = tid; n < P.N; n += B) s_tab[n] = step_time(P, n);
+    // the time table's binary searches read the nodes from shared memory: from
+    // global memory each was a chain of up to eight dependent loads (1.5 us of a
+    // small call's launch)
+    const double* tau = P.tau;
+    if (P.J <= kStagedTau) {
+        double* s_tau = reinterpret_cast<double*>(smem + L.tau);
+        for (int e = tid; e < P.J; e += B) s_tau[e] = P.tau[e];
+        __syncthreads();
+        tau = s_tau;
+    }
+    for (int n = tid; n < P.N; n += B) s_tab[n] = step_time(P, tau, n);
     if (EXTRA) {
         float* s_tdt = reinterpret_cast<float*>(smem + L.tdt);
-        for (int n = tid; n < P.N; n += B) s_tdt[n] = step_tdt(P, n);
+        for (int n = tid; n < P.N; n += B) s_tdt[n] = step_tdt(P, tau, n);
     }
 }
 
-// Block sum of three per-thread binary64 values into row[0..2] (fixed order).
-__device__ __forceinline__ void block_scalars(double a, double b, double c, double* s_red, double* row, int n = 3)
+// Adds the block's sum of NV per-thread binary64 values (over the block in a
+// fixed order) to sums[0 .. NV-1].
+template <int NV>
+__device__ __forceinline__ void add_scalars(const double (&v)[NV], double* s_red, double* sums)
 {
+    static_assert(NV <= 3, "s_red holds three values a warp");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-        c += __shfl_down_sync(0xffffffffu, c, o);
-    }
-    if (lane == 0) {
-        s_red[3 * warp + 0] = a;
-        s_red[3 * warp + 1] = b;
-        s_red[3 * warp + 2] = c;
+    for (int k = 0; k < NV; ++k) {
+        double a = v[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+        if (lane == 0) s_red[NV * warp + k] = a;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double sa = 0.0, sb = 0.0, sc = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            sa += s_red[3 * w + 0];
-            sb += s_red[3 * w + 1];
-            sc += s_red[3 * w + 2];
+    if (threadIdx.x < NV) {
+        double s = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += s_red[NV * w + threadIdx.x];
+        atomicAdd(&sums[threadIdx.x], s);
+    }
+}
+
+// Adds what the block's buckets hold (its binary64 row, or in Kahan mode its
+// warps' rows, and the binary32 buckets not drained yet) to the call's sums.
+template <int ACC>
+__device__ __forceinline__ void fold_buckets(const McParams& P, const float* l1, const double* row)
+{
+    const int nIJ = P.Je * P.I, B = blockDim.x, W = B >> 5;
+    const double* rows0 = P.warp_rows + (size_t)blockIdx.x * W * nIJ;
+    for (int e = threadIdx.x; e < nIJ; e += B) {
+        double s = (double)__ldcg(l1 + e);       // reductions are resolved in L2
+        if (ACC == 1) {
+            for (int w = 0; w < W; ++w) {
+                const float2 k = reinterpret_cast<const float2*>(rows0 + (size_t)w * nIJ)[e];
+                s += (double)k.x - (double)k.y;
+            }
+        } else {
+            s += __ldcg(row + 3 + e);
         }
-        row[0] = sa;
-        row[1] = sb;
-        if (n > 2) row[2] = sc;
+        if (s != 0.0) atomicAdd(&P.sums[3 + e], s);
+    }
+}
+
+// End of a launch (level 3). Every block has added its sums to P.sums; the last
+// one to arrive turns them into the call's outputs and leaves the sums and the
+// counters at zero for the next launch. It replaces two launches that summed the
+// blocks' rows: where the blocks end at different times their additions hide
+// behind the blocks still running, and only the last block's pass over the outputs
+// is left. 30 x 60 grid, 156 steps, 2^20 paths: 601 -> 584 us a call, forward only
+// 245 -> 234; 20 x 10 grid, 52 steps, 2^14 paths: 31.1 -> 26.7 us. The divisions by the path count are products with its inverse: a binary64 division
+// takes 551 cycles here. A nonzero flag (a vanishing 1 + g_n on a live path of the
+// tangent-ratio forms) makes every output NaN. Outputs in the ABI layout (vega
+// spot-major); EXTRA: d price / d r and d price / d T after the vegas.
+template <bool GREEKS, bool EXTRA = false>
+__device__ __forceinline__ void finish_call(const McParams& P)
+{
+    __shared__ int s_last;
+    __threadfence();                      // this thread's additions before the block's arrival
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(P.done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();                      // every block's additions before the reads below
+    const int B = blockDim.x, tid = threadIdx.x;
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    const bool bad = P.flag && __ldcg(P.flag) != 0u;
+    const int nIJ = P.Je * P.I;
+    if (tid == 0) {
+        const double s0 = __ldcg(P.sums), s1 = __ldcg(P.sums + 1), s2 = __ldcg(P.sums + 2);
+        if (P.want_sums) {
+            P.out[0] = bad ? nan : s0;
+            P.out[1] = bad ? nan : s1;
+            P.out[2] = bad ? nan : s2;
+        } else {
+            const double mean = s0 * P.inv_paths;
+            const double var = (s1 * P.inv_paths - mean * mean) * P.var_scale;
+            P.out[LV_OUT_PRICE_DEV] = bad ? nan : mean;
+            P.out[LV_OUT_STDERR_DEV] = bad ? nan : (var > 0.0 || var != var) ? sqrt(var * P.inv_paths) : 0.0;
+            P.out[LV_OUT_DELTA_DEV] = bad ? nan : s2 * P.inv_delta;
+        }
+        P.sums[0] = P.sums[1] = P.sums[2] = 0.0;
+        *P.tile_counter = 0u;
+        *P.done = 0u;
+    }
+    const double scale = P.want_sums ? 1.0 : P.inv_paths;
+    if (GREEKS) {
+        double* s = P.sums + 3;           // time-major buckets j I + i
+        for (int e = tid; e < nIJ; e += B) {
+            const double v = __ldcg(s + e);
+            s[e] = 0.0;
+            const int j = e / P.I, i = e - j * P.I;
+            if (j < P.J) P.out[3 + i * P.J + j] = bad ? nan : v * scale;   // not the padding row of one time node
+        }
+    }
+    if (EXTRA && tid < 2) {
+        double* s = P.sums + 3 + nIJ + tid;
+        P.out[3 + P.I * P.J + tid] = __ldcg(s) * scale;
+        *s = 0.0;
+    }
+    if (P.flag) {
+        __syncthreads();                  // every thread has read it
+        if (tid == 0) *P.flag = 0u;
     }
 }
 
@@ -182,23 +271,36 @@ __device__ __forceinline__ int claim_tile(unsigned int* counter, unsigned n = 1u
     return __shfl_sync(0xffffffffu, t, 0);
 }
 
+// Moves the block's binary32 buckets into its level-2 row (binary64) or the
+// warp's (Kahan). A bucket that reads zero is left for a later drain. Eight
+// buckets of a lane are in flight at a time: one by one, each waited for a
+// load and an exchange in L2.
 template <int ACC>
 __device__ __forceinline__ void drain_buckets(float* l1, int nIJ, double* wrow)
 {
+    constexpr int kFly = 8;
     const int lane = threadIdx.x & 31;
-    for (int e = lane; e < nIJ; e += 32) {
-        if (l1[e] == 0.0f) continue;            // a skipped bucket is drained later
-        const float v = atomicExch(&l1[e], 0.0f);
-        if (ACC == 1) {
-            float2* k = reinterpret_cast<float2*>(wrow) + e;
-            float2 p = *k;
-            const float y = v - p.y;
-            const float t = p.x + y;
-            p.y = (t - p.x) - y;
-            p.x = t;
-            *k = p;
-        } else {
-            atomicAdd(&wrow[e], (double)v);       // the block's row, shared by its warps
+    for (int e0 = lane; e0 < nIJ; e0 += 32 * kFly) {
+        float v[kFly];
+#pragma unroll
+        for (int q = 0; q < kFly; ++q) v[q] = e0 + 32 * q < nIJ ? __ldcg(l1 + e0 + 32 * q) : 0.0f;
+#pragma unroll
+        for (int q = 0; q < kFly; ++q)
+            if (v[q] != 0.0f) v[q] = atomicExch(l1 + e0 + 32 * q, 0.0f);
+#pragma unroll
+        for (int q = 0; q < kFly; ++q) {
+            if (v[q] == 0.0f) continue;
+            if (ACC == 1) {
+                float2* k = reinterpret_cast<float2*>(wrow) + e0 + 32 * q;
+                float2 p = *k;
+                const float y = v[q] - p.y;
+                const float t = p.x + y;
+                p.y = (t - p.x) - y;
+                p.x = t;
+                *k = p;
+            } else {
+                atomicAdd(wrow + e0 + 32 * q, (double)v[q]);      // the block's row, shared by its warps
+            }
         }
     }
 }
@@ -222,7 +324,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
     constexpr int kQcap = kQueue * PPL;      // FIFO entries per warp
     const int B = blockDim.x, W = B >> 5;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const SmemLayout L = smem_layout(P.I, P.Je, P.N, P.n_bins, B, true, GS, EXTRA, PPL);
+    const SmemLayout L = smem_layout(P.I, P.J, P.N, P.n_bins, B, true, GS, EXTRA, PPL);
     stage_grid<GS, EXTRA>(P, smem, L);
     float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);    // this block's level-1 buckets
     // the three FIFO arrays of all warps are contiguous from L.qslot (each
@@ -376,31 +478,15 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
         tile = claim_tile(P.tile_counter, PPL);
     }
 
-    // fold: remaining level-1 buckets (and, in Kahan mode, every warp row of
-    // this block) into the block's binary64 row (after the barrier nothing adds)
-    __syncthreads();
-    // the kernel that also sums d V / d r and d V / d T recomputes its row here
-    // instead of keeping the pointer live through the loop (80 registers, 6
-    // blocks per SM, instead of 87 and 5)
-    double* const row_f = EXTRA ? P.partials + (size_t)blockIdx.x * P.row_words : row;
-    const double* rows0 = P.warp_rows + (size_t)blockIdx.x * W * nIJ;
-    for (int e = tid; e < nIJ; e += B) {
-        if (ACC == 1) {
-            double s = (double)l1[e];
-            for (int w = 0; w < W; ++w) {
-                const float2 k = reinterpret_cast<const float2*>(rows0 + (size_t)w * nIJ)[e];
-                s += (double)k.x - (double)k.y;
-            }
-            row_f[3 + e] = s;
-        } else {
-            row_f[3 + e] += (double)l1[e];
-        }
-    }
-    block_scalars(acc_value<ACC>(acc[0]), acc_value<ACC>(acc[B]), acc_value<ACC>(acc[2 * B]), s_red, row_f);
+    __syncthreads();                           // after it nothing adds to this block's buckets
+    const double* row_f = P.partials + (size_t)blockIdx.x * P.row_words;     // recomputed, not live through the loop
+    fold_buckets<ACC>(P, l1, row_f);
+    add_scalars({acc_value<ACC>(acc[0]), acc_value<ACC>(acc[B]), acc_value<ACC>(acc[2 * B])}, s_red, P.sums);
     if (EXTRA) {
         __syncthreads();                       // s_red is reused
-        block_scalars(acc_value<ACC>(acc[3 * B]), acc_value<ACC>(acc[4 * B]), 0.0, s_red, row_f + 3 + nIJ, 2);
+        add_scalars({acc_value<ACC>(acc[3 * B]), acc_value<ACC>(acc[4 * B])}, s_red, P.sums + 3 + nIJ);
     }
+    finish_call<true, EXTRA>(P);
 }
 
 // Tangent-ratio adjoint (LV_ADJ_TANGENT): persistent and warp-centric like
@@ -416,7 +502,7 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
     const int B = blockDim.x, W = B >> 5;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kQcap = kQueue * PPL;
-    const SmemLayout L = smem_layout(P.I, P.Je, P.N, P.n_bins, B, true, GS, false, PPL);
+    const SmemLayout L = smem_layout(P.I, P.J, P.N, P.n_bins, B, true, GS, false, PPL);
     stage_grid<GS>(P, smem, L);
     float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);
     int* q_rel = reinterpret_cast<int*>(smem + L.qrel) + warp * kQcap;
@@ -530,20 +616,9 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
         tile = claim_tile(P.tile_counter, PPL);
     }
     __syncthreads();
-    const double* rows0 = P.warp_rows + (size_t)blockIdx.x * W * nIJ;
-    for (int e = tid; e < nIJ; e += B) {
-        if (ACC == 1) {
-            double s = (double)l1[e];
-            for (int w = 0; w < W; ++w) {
-                const float2 k = reinterpret_cast<const float2*>(rows0 + (size_t)w * nIJ)[e];
-                s += (double)k.x - (double)k.y;
-            }
-            row[3 + e] = s;
-        } else {
-            row[3 + e] += (double)l1[e];
-        }
-    }
-    block_scalars(acc_value<ACC>(acc[0]), acc_value<ACC>(acc[B]), acc_value<ACC>(acc[2 * B]), s_red, row);
+    fold_buckets<ACC>(P, l1, row);
+    add_scalars({acc_value<ACC>(acc[0]), acc_value<ACC>(acc[B]), acc_value<ACC>(acc[2 * B])}, s_red, P.sums);
+    finish_call<true>(P);
 }
 
 // Second-order buckets (lv_price_greeks_vanna): the tangent-ratio kernel's
@@ -559,7 +634,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
     const int B = blockDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kQcap = kQueue * PPL;
-    const SmemLayout L = smem_layout(P.I, P.Je, P.N, P.n_bins, B, true, GS, false, PPL);
+    const SmemLayout L = smem_layout(P.I, P.J, P.N, P.n_bins, B, true, GS, false, PPL);
     stage_grid<GS>(P, smem, L);
     float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);
     int* q_rel = reinterpret_cast<int*>(smem + L.qrel) + warp * kQcap;
@@ -666,8 +741,9 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
         tile = claim_tile(P.tile_counter, PPL);
     }
     __syncthreads();
-    for (int e = tid; e < nIJ; e += B) row[3 + e] += (double)l1[e];
-    block_scalars(acc_value<0>(acc[0]), acc_value<0>(acc[B]), acc_value<0>(acc[2 * B]), s_red, row);
+    fold_buckets<0>(P, l1, row);
+    add_scalars({acc_value<0>(acc[0]), acc_value<0>(acc[B]), acc_value<0>(acc[2 * B])}, s_red, P.sums);
+    finish_call<true>(P);
 }
 
 // The forward pass alone. Bound by the FMA pipe (its 64-bit integer products
@@ -682,7 +758,7 @@ template <int ACC, bool GS, int MODEL, int CELL>
 __global__ void __launch_bounds__(128, 9) price_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const SmemLayout L = smem_layout(P.I, P.Je, P.N, P.n_bins, blockDim.x, false, GS);
+    const SmemLayout L = smem_layout(P.I, P.J, P.N, P.n_bins, blockDim.x, false, GS);
     stage_grid<GS>(P, smem, L);
     __syncthreads();
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
@@ -712,8 +788,8 @@ __global__ void __launch_bounds__(128, 9) price_kernel(const __grid_constant__ M
         }
     }
     double* s_red = reinterpret_cast<double*>(smem + L.red);
-    block_scalars(acc_value<ACC>(acc[0]), acc_value<ACC>(acc[blockDim.x]), 0.0, s_red,
-                  P.partials + (size_t)blockIdx.x * P.row_words);
+    add_scalars({acc_value<ACC>(acc[0]), acc_value<ACC>(acc[blockDim.x])}, s_red, P.sums);
+    finish_call<false>(P);
 }
 
 template <typename K>
