@@ -266,11 +266,12 @@ void occ_store(const OccKey& key, int occ)
 }
 
 // A call of at least this many paths per SM runs two paths per lane unless
-// told otherwise: every warp of the adjoint kernel (at most 24 resident per
-// SM) then gets at least four pairs of 32-path tiles. Smaller calls run one
-// path per lane; measured on a GB300 (k = 4), two paths per lane took 1.03-1.07x
-// the time at 2^18 and 2^19 paths and 0.96-0.99x from 2^20 on.
-constexpr int64_t kPairMinPathsPerSm = 4 * 64 * 24;
+// told otherwise: one and a half pairs of 32-path tiles for each of the 16 warps
+// of the adjoint kernel resident on an SM. Measured on a GB300 (30 x 60 grid, 156
+// steps, k = 4; one and two paths per lane): 2^18 paths 182 and 181 us, 500,000 297
+// and 290, 2^20 578 and 567, 2^22 1,980 and 1,880; below, a pair leaves warps idle
+// (2^17 121 and 134).
+constexpr int64_t kPairMinPathsPerSm = 3 * 32 * 16;
 
 // n_paths < 0: a call large enough for two paths per lane.
 // The head of the handle's scratch, at the same place in every launch's layout:
@@ -380,7 +381,8 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     p->off_wrows = o;                   // per-warp rows: Kahan mode only
     if (greeks && !extra && !vanna && h->acc_mode == LV_ACC_KAHAN)
         o = round_up(o + sizeof(double) * total_warps * nIJ, 256);
-    p->off_l1 = o;      if (greeks) o = round_up(o + sizeof(float) * (size_t)p->grid * nIJ, 256);
+    p->off_l1 = o;
+    if (greeks) o = round_up(o + sizeof(float4) * (size_t)p->grid * (h->Je - 1) * (h->I - 1), 256);
     p->off_ckpt = o;
     o = round_up(o + sizeof(float) * (size_t)p->n_ck * total_warps * lv::ring_slots_per_warp() * p->ppl, 256);
     p->total = o;
@@ -508,7 +510,7 @@ lv_status run_mc(lv_surface_s* h, const McCall& c)
     P.partials = reinterpret_cast<double*>(base + p.off_part);
     P.row_words = p.row_words;
     P.warp_rows = reinterpret_cast<double*>(base + p.off_wrows);
-    P.l1 = reinterpret_cast<float*>(base + p.off_l1);
+    P.l1 = reinterpret_cast<float4*>(base + p.off_l1);
     P.ckpt = reinterpret_cast<float*>(base + p.off_ckpt);
     P.n_ck = p.n_ck;
     P.flush_every = 8;
@@ -633,7 +635,7 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
         cudaMalloc(&h->d_node, sizeof(float) * n_spot) != cudaSuccess ||
         cudaMalloc(&h->d_ab, sizeof(float2) * n_spot) != cudaSuccess ||
         cudaMalloc(&h->d_abl, sizeof(float2) * n_spot) != cudaSuccess ||
-        cudaMalloc(&h->d_tau, sizeof(double) * n_time) != cudaSuccess ||
+        cudaMalloc(&h->d_tau, 2 * sizeof(double) * n_time) != cudaSuccess ||
         cudaMalloc(&h->d_spot64, sizeof(double) * n_spot) != cudaSuccess ||
         cudaMalloc(&h->d_sig64, sizeof(double) * (size_t)n_spot * n_time) != cudaSuccess ||
         cudaMallocHost(&h->h_sig64_stage, sizeof(double) * (size_t)n_spot * n_time) != cudaSuccess ||
@@ -642,6 +644,13 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
         cudaMallocHost(&h->h_res, sizeof(double) * nres) != cudaSuccess) {
         cudaGetLastError();
         return bail(LV_ENOMEM, "device or pinned allocation failed");
+    }
+    // time nodes and inverse gaps (0 where the inverse is not a normal number)
+    std::vector<double> tau(2 * (size_t)n_time, 0.0);
+    for (int j = 0; j < n_time; ++j) {
+        tau[j] = time_nodes[j];
+        const double inv = j + 1 < n_time ? 1.0 / (time_nodes[j + 1] - time_nodes[j]) : 0.0;
+        tau[n_time + j] = std::isnormal(inv) && inv < 1e290 ? inv : 0.0;
     }
     std::vector<float> node(n_spot);
     std::vector<float2> ab(n_spot), abl(n_spot);
@@ -675,7 +684,7 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
         cudaMemcpy(h->d_node, node.data(), sizeof(float) * n_spot, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_ab, ab.data(), sizeof(float2) * n_spot, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_abl, abl.data(), sizeof(float2) * n_spot, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(h->d_tau, time_nodes, sizeof(double) * n_time, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(h->d_tau, tau.data(), 2 * sizeof(double) * n_time, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_spot64, spot_nodes, sizeof(double) * n_spot, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_sig64, sigma, sizeof(double) * (size_t)n_spot * n_time, cudaMemcpyHostToDevice) !=
             cudaSuccess) {
@@ -1422,7 +1431,7 @@ size_t static_plan_bytes(const lv_surface_s* h, int grid, int block, int k, int 
     *off_part = o;   o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
     *off_wrows = o;                                               // per-warp rows: Kahan mode only
     if (h->acc_mode == LV_ACC_KAHAN) o = round_up(o + sizeof(double) * warps * nIJ, 256);
-    *off_l1 = o;     o = round_up(o + sizeof(float) * (size_t)grid * nIJ, 256);
+    *off_l1 = o;     o = round_up(o + sizeof(float4) * (size_t)grid * (h->Je - 1) * (h->I - 1), 256);
     *off_ckpt = o;   o = round_up(o + sizeof(float) * n_ck * warps * lv::ring_slots_per_warp() * ppl, 256);
     return o;
 }
@@ -1497,7 +1506,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
     P.partials = reinterpret_cast<double*>(base + off_part);
     P.row_words = 3 + h->Je * h->I;
     P.warp_rows = reinterpret_cast<double*>(base + off_wrows);
-    P.l1 = reinterpret_cast<float*>(base + off_l1);
+    P.l1 = reinterpret_cast<float4*>(base + off_l1);
     P.ckpt = reinterpret_cast<float*>(base + off_ckpt);
     P.n_ck = h->adj_method == LV_ADJ_TANGENT ? 0 : (n_steps + k - 1) / k;
     P.flush_every = 8;

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
             for (int e = tid; e < Q.I; e += Bk) s_node[e] = Q.node[e];
             for (int e = tid; e < Q.I - 1; e += Bk) s_ab[e] = Q.ab[e];
             for (int e = tid; e < Q.n_bins; e += Bk) s_bins[e] = Q.bins[e];
-            for (int n = tid; n < Q.N; n += Bk) s_tab[n] = step_time(Q, Q.tau, n);
+            for (int n = tid; n < Q.N; n += Bk) s_tab[n] = step_time(Q, Q.tau, Q.tau + Q.J, n);
             if (tid == 0) s_ctl[2] = it.inst;
         }
         if (tid == 0) s_ctl[1] = it.first_tile;
@@ -285,13 +285,21 @@ __global__ void __launch_bounds__(128, 4) book_kernel(const __grid_constant__ Bo
         const BookInst& inst = B.insts[it.inst];
         double* vsum = B.risk ? B.risk + B.surfs[inst.surf].risk_off + 3 : sums + 3;
         const double vscale = B.risk ? inst.scale : 1.0;
+        // eight buckets of a thread in flight: one by one each waited for L2
         const int nIJ = P.Je * P.I;
-        for (int e = tid; e < nIJ; e += Bk) {
-            const float v = l1[e];
-            if (v != 0.0f) {
-                const int j = e / P.I, i = e - j * P.I;
-                if (j < P.J) atomicAdd(&vsum[i * P.J + j], (double)v * vscale);   // spot-major sums
-                l1[e] = 0.0f;
+        constexpr int kFly = 8;
+        for (int e0 = tid; e0 < nIJ; e0 += kFly * Bk) {
+            float v[kFly];
+#pragma unroll
+            for (int q = 0; q < kFly; ++q) v[q] = e0 + q * Bk < nIJ ? __ldcg(l1 + e0 + q * Bk) : 0.0f;
+#pragma unroll
+            for (int q = 0; q < kFly; ++q) {
+                const int e = e0 + q * Bk;
+                if (v[q] != 0.0f) {
+                    const int j = e / P.I, i = e - j * P.I;
+                    if (j < P.J) atomicAdd(&vsum[i * P.J + j], (double)v[q] * vscale);   // spot-major sums
+                    l1[e] = 0.0f;
+                }
             }
         }
         __syncthreads();

@@ -395,7 +395,7 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
         n_sig += (long long)h->Je * (h->I - 1);
         n_node += h->I;
         n_ab += h->I;
-        n_tau += h->J;
+        n_tau += 2 * h->J;              // nodes and inverse gaps
         n_bins += h->n_bins;
         b->surfs.push_back(bs);
         b->max_I = std::max(b->max_I, h->I);
@@ -457,7 +457,7 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
             cudaMemcpy(b->d_ab + bs.off_ab, h->d_ab, sizeof(float2) * h->I, cudaMemcpyDeviceToDevice) != cudaSuccess ||
             (h->n_bins > 0 && cudaMemcpy(b->d_bins + bs.off_bins, h->d_bins, sizeof(float4) * h->n_bins,
                                          cudaMemcpyDeviceToDevice) != cudaSuccess) ||
-            cudaMemcpy(b->d_tau + bs.off_tau, h->d_tau, sizeof(double) * h->J, cudaMemcpyDeviceToDevice) !=
+            cudaMemcpy(b->d_tau + bs.off_tau, h->d_tau, 2 * sizeof(double) * h->J, cudaMemcpyDeviceToDevice) !=
                 cudaSuccess)
             return bail(set_error(LV_ECUDA, "copying a surface into the book failed"));
     }

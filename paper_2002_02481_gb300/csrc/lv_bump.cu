@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(256) bump_kernel(const __grid_constant__ BumpP
     for (int e = tid; e < P.Je * (P.I - 1); e += B) s_sig[e] = P.sig2[e];
     for (int e = tid; e < P.I; e += B) s_node[e] = P.node[e];
     for (int e = tid; e < P.I - 1; e += B) s_ab[e] = P.ab[e];
-    for (int n = tid; n < P.N; n += B) s_tab[n] = step_time(P, P.tau, n);
+    for (int n = tid; n < P.N; n += B) s_tab[n] = step_time(P, P.tau, P.tau + P.J, n);
     for (int e = tid; e < Q.row_words; e += B) s_acc[e] = 0.0;
     if (tid == 0) s_tile[0] = (int)atomicAdd(P.tile_counter, 1u);
     __syncthreads();

@@ -32,7 +32,7 @@ __global__ void time_table_kernel(const McParams P, int* __restrict__ out_j, flo
 {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= P.N) return;
-    const int4 tb = step_time(P, P.tau, n);
+    const int4 tb = step_time(P, P.tau, P.tau + P.J, n);
     out_j[n] = tb.y / P.I;                    // tb.y is the bucket row j I
     out_v[n] = __int_as_float(tb.w);
 }

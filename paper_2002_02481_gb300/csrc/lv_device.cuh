@@ -222,23 +222,32 @@ __device__ __forceinline__ void normals4_neg(uint32_t blk, uint32_t c1, uint32_t
 // [0, 1], decided in binary64. Returned as (j (I-1), j I, bits of v twice):
 // the row of the sigma pairs for j (row j + 1 is I - 1 pairs further on), the
 // bucket row, and v as the pair the packed arithmetic takes.
-__device__ __forceinline__ int4 step_time(const McParams& P, const double* tau, int n)
+// Every block makes the whole table, and binary64 operations run at 1.7 per SM
+// and cycle here, so it takes few of them: times are at least 0, so their bits
+// compare like them as integers; the quotient is a product with the correctly
+// rounded inverse gap rtau_j and one residual step, which rounds like the
+// division (Markstein, 1990); rtau_j = 0 marks a gap whose inverse is not normal.
+__device__ __forceinline__ int4 step_time(const McParams& P, const double* tau, const double* rtau, int n)
 {
     const double t = (double)n * P.dt_d;
     int j = 0;
-    double v = 0.0;
+    float v = 0.0f;
     if (P.J > 1) {
+        const long long tb = __double_as_longlong(t);
         int lo = 0, hi = P.J - 2;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (tau[mid] <= t) lo = mid;
+            if (__double_as_longlong(tau[mid]) <= tb) lo = mid;
             else hi = mid - 1;
         }
         j = lo;
-        v = (t - tau[j]) / (tau[j + 1] - tau[j]);
-        v = fmin(fmax(v, 0.0), 1.0);
+        const double a = t - tau[j], b = tau[j + 1] - tau[j], r = rtau[j];
+        double q = a * r;
+        q = fma(fma(-q, b, a), r, q);
+        if (r == 0.0) q = a / b;
+        v = fminf(fmaxf((float)q, 0.0f), 1.0f);
     }
-    const int vb = __float_as_int((float)v);
+    const int vb = __float_as_int(v);
     return make_int4(j * (P.I - 1), j * P.I, vb, vb);
 }
 
@@ -679,12 +688,31 @@ __device__ __forceinline__ void forward_path2(const McParams& P, const SmemGrid&
     });
 }
 
-// A binary32 reduction in L2 without a return value. Written out because in a
-// kernel that also has a memory fence the compiler turns atomicAdd into the
-// returning form, whose replies took the adjoint from 0.601 to 0.756 ms.
-__device__ __forceinline__ void red_add(float* p, float v)
+// Level 1: adds a cell's four corner sums to its bucket, one 16-byte reduction
+// resolved in L2. Lanes in random cells of one grid retire 0.80-0.85 of these per
+// SM and cycle, against 0.24-0.29 flushes as four scalar reductions of per-node
+// buckets, which is about what the adjoint needs (0.22): the scalar form held it
+// back. Written out also because in a kernel that has a memory fence the compiler
+// turns atomicAdd into the returning form, whose replies took the adjoint from
+// 0.601 to 0.756 ms.
+__device__ __forceinline__ void red_add4(float4* p, float a, float b, float c, float d)
 {
-    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(v) : "memory");
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(a),
+                 "f"(b), "f"(c), "f"(d));
+}
+
+// The same sums to the four nodes' buckets (node (i, j) at j I + i), in the book:
+// its blocks keep up to 8,192 paths of an option in binary32 buckets without a
+// drain, so their rounding is part of its results (2e-7 of a coarse grid's vegas
+// from run to run), and per-cell buckets moved them by up to 7e-7.
+__device__ __forceinline__ void red_nodes(float* p0, int I, float a, float b, float c, float d)
+{
+    float* q[2] = { p0, p0 + I };
+    const float v[4] = { a, b, c, d };
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(q[k >> 1] + (k & 1))),
+                     "f"(v[k]));
 }
 
 // Philox counter words of path `rel` of the call: c1 = path bits 0..31,
@@ -704,27 +732,24 @@ __device__ __forceinline__ void path_counter(const McParams& P, long long rel, u
 // walk them back: sigma_bar_n = xbar_{n+1} h_n, xbar_n = xbar_{n+1} (1 + g_n),
 // and spread sigma_bar_n over the corner buckets (i, j), (i+1, j), (i, j+1),
 // (i+1, j+1) with the bilinear weights. Corner sums are kept in registers
-// while the cell is unchanged and then added to the block's binary32 buckets
-// `l1` (time-major, row j * I) with red.global.add.f32. Returns d V / d x_0.
+// while the cell is unchanged and then added to the cell's binary32 bucket in
+// `l1` (row j (I - 1), as the sigma pairs) with red_add4. Returns d V / d x_0.
 // With NEG (no extra sums) the recompute takes its normals from
 // normals4_neg and uses sqdt Z = (-sqdt)(-Z) and sqdt2 Z = (-sqdt2)(-Z),
 // which are exact, so every value is the same bit for bit.
-template <int KCK, int MODEL, bool EXTRA, bool NEG, int CELL>
+template <int KCK, int MODEL, bool EXTRA, bool NEG, int CELL, typename BUCKET>
 __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                                const float* ck, size_t cks, float xbar, float* l1, float* rho_acc,
+                                                const float* ck, size_t cks, float xbar, BUCKET* l1, float* rho_acc,
                                                 float* t_acc)
 {
     constexpr bool kNeg = NEG && !EXTRA;
     const int nseg = (P.N + KCK - 1) / KCK;
     int cur = -1;
     float A = 0.0f, AU = 0.0f, Bs = 0.0f, BU = 0.0f;
+    constexpr bool kNodes = sizeof(BUCKET) == sizeof(float);    // a bucket per node, not per cell
     auto flush = [&]() {
-        float* p0 = l1 + cur;
-        float* p1 = p0 + P.I;
-        red_add(p0, A - AU);
-        red_add(p0 + 1, AU);
-        red_add(p1, Bs - BU);
-        red_add(p1 + 1, BU);
+        if constexpr (kNodes) red_nodes(l1 + cur, P.I, A - AU, AU, Bs - BU, BU);
+        else red_add4(l1 + cur, A - AU, AU, Bs - BU, BU);
     };
     auto gen = [&](int blk, float (&z)[4]) {
         if (kNeg) normals4_neg((uint32_t)blk, c1, c2, P.rk, z);
@@ -763,30 +788,36 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
                 else x = step_state<MODEL>(P, x, ev.sigma, z[q & 3]);
             }
         }
+        // back through the segment: first everything that needs no decision (hq, gq
+        // become the time-weighted shares a, b of sigma_bar), then the run-length sums
 #pragma unroll
         for (int q = KCK - 1; q >= 0; --q) {
             const int n = m * KCK + q;
             if (all || n < P.N) {
                 const int4 tb = g.tab[n];
-                const int key = tb.y + iq[q];
-                const float v = __int_as_float(tb.w);
+                iq[q] += kNodes ? tb.y : tb.x;           // the cell's bucket, or its lower node's
                 const float sbar = xbar * hq[q];
                 if (EXTRA) {                             // xbar is still xbar_{n+1}
                     *rho_acc = fmaf(xbar, aq[EXTRA ? q : 0], *rho_acc);
                     *t_acc = fmaf(xbar, tq[EXTRA ? q : 0], *t_acc);
                 }
                 xbar = fmaf(xbar, gq[q], xbar);
-                if (key != cur) {
+                gq[q] = sbar * __int_as_float(tb.w);
+                hq[q] = sbar - gq[q];
+            }
+        }
+#pragma unroll
+        for (int q = KCK - 1; q >= 0; --q) {
+            if (all || m * KCK + q < P.N) {
+                if (iq[q] != cur) {
                     if (cur >= 0) flush();
                     A = AU = Bs = BU = 0.0f;
-                    cur = key;
+                    cur = iq[q];
                 }
-                const float b = sbar * v;
-                const float a = sbar - b;
-                A += a;
-                AU = fmaf(a, uq[q], AU);
-                Bs += b;
-                BU = fmaf(b, uq[q], BU);
+                A += hq[q];
+                AU = fmaf(hq[q], uq[q], AU);
+                Bs += gq[q];
+                BU = fmaf(gq[q], uq[q], BU);
             }
         }
     };
@@ -810,9 +841,9 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
     return xbar;
 }
 
-template <int CELL, int KCK, int MODEL = 0, bool EXTRA = false, bool NEG = false>
+template <int CELL, int KCK, int MODEL = 0, bool EXTRA = false, bool NEG = false, typename BUCKET>
 __device__ __forceinline__ float reverse_path(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                              const float* ck, size_t cks, float xbar, float* l1,
+                                              const float* ck, size_t cks, float xbar, BUCKET* l1,
                                               float* rho_acc = nullptr, float* t_acc = nullptr)
 {
     return cell_dispatch<CELL>(P, [&](auto c) {
@@ -940,19 +971,12 @@ __device__ __forceinline__ void tangent_forward2(const McParams& P, const SmemGr
 // sums and binary32 reductions into `l1` as reverse_path, in time order.
 template <int MODEL, int CELL>
 __device__ __forceinline__ void tangent_scatter_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                                  float c, float* l1)
+                                                  float c, float4* l1)
 {
     float y = P.x0, d = 1.0f;
     int cur = -1;
     float A = 0.0f, AU = 0.0f, Bs = 0.0f, BU = 0.0f;
-    auto flush = [&]() {
-        float* p0 = l1 + cur;
-        float* p1 = p0 + P.I;
-        red_add(p0, A - AU);
-        red_add(p0 + 1, AU);
-        red_add(p1, Bs - BU);
-        red_add(p1 + 1, BU);
-    };
+    auto flush = [&]() { red_add4(l1 + cur, A - AU, AU, Bs - BU, BU); };
     time_blocks<float, CELL != kCellSearch, 1>(
         P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
         [&](int n, float z) {
@@ -962,7 +986,7 @@ __device__ __forceinline__ void tangent_scatter_f(const McParams& P, const SmemG
             adjoint_factors<MODEL>(P, e, z, h, gn);
             d *= tangent_factor<MODEL>(P, e, z, h);          // D_{n+1}
             const float sbar = __fdividef(c * h, d);
-            const int key = tb.y + e.i;
+            const int key = tb.x + e.i;
             if (key != cur) {
                 if (cur >= 0) flush();
                 A = AU = Bs = BU = 0.0f;
@@ -981,7 +1005,7 @@ __device__ __forceinline__ void tangent_scatter_f(const McParams& P, const SmemG
 
 template <int CELL, int MODEL = 0>
 __device__ __forceinline__ void tangent_scatter(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                                float c, float* l1)
+                                                float c, float4* l1)
 {
     cell_dispatch<CELL>(P, [&](auto m) { tangent_scatter_f<MODEL, decltype(m)::value>(P, g, c1, c2, c, l1); });
 }
@@ -1000,19 +1024,12 @@ __device__ __forceinline__ void tangent_scatter(const McParams& P, const SmemGri
 // E1 = sum v d), then binary32 reductions into `l1`.
 template <int CELL>
 __device__ __forceinline__ void vanna_scatter_f(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                                float delta, float* l1)
+                                                float delta, float4* l1)
 {
     float y = P.x0;
     int cur = -1;
     float A = 0.0f, AU = 0.0f, Bs = 0.0f, BU = 0.0f, E0 = 0.0f, E1 = 0.0f;
-    auto flush = [&]() {
-        float* p0 = l1 + cur;
-        float* p1 = p0 + P.I;
-        red_add(p0, A - AU - E0);
-        red_add(p0 + 1, AU + E0);
-        red_add(p1, Bs - BU - E1);
-        red_add(p1 + 1, BU + E1);
-    };
+    auto flush = [&]() { red_add4(l1 + cur, A - AU - E0, AU + E0, Bs - BU - E1, BU + E1); };
     time_blocks<float, CELL != kCellSearch, 1>(
         P.N, [](int) {}, [&](uint32_t blk, float (&z)[4]) { normals4(blk, c1, c2, P.rk, z); },
         [&](int n, float zq) {
@@ -1026,7 +1043,7 @@ __device__ __forceinline__ void vanna_scatter_f(const McParams& P, const SmemGri
             const float sdu = inside ? e.S * g.ab[e.i].x : 0.0f;          // S d u / d S
             const float c = delta * a;
             const float d = delta * __fdividef(h, f) * sdu;
-            const int key = tb.y + e.i;
+            const int key = tb.x + e.i;
             if (key != cur) {
                 if (cur >= 0) flush();
                 A = AU = Bs = BU = E0 = E1 = 0.0f;
@@ -1048,7 +1065,7 @@ __device__ __forceinline__ void vanna_scatter_f(const McParams& P, const SmemGri
 
 template <int CELL>
 __device__ __forceinline__ void vanna_scatter(const McParams& P, const SmemGrid& g, uint32_t c1, uint32_t c2,
-                                              float delta, float* l1)
+                                              float delta, float4* l1)
 {
     cell_dispatch<CELL>(P, [&](auto c) { vanna_scatter_f<decltype(c)::value>(P, g, c1, c2, delta, l1); });
 }

@@ -60,7 +60,7 @@ struct McParams {
                            // Je = max(J, 2), row 1 repeats row 0 when J == 1
     const float* node;     // [I] spot nodes s_i
     const float2* ab;      // [I - 1] (1 / (s_{i+1} - s_i), -s_i / (s_{i+1} - s_i))
-    const double* tau;     // [J] time nodes
+    const double* tau;     // [J] time nodes, then [J] inverse gaps 1 / (tau_{j+1} - tau_j) (step_time)
     int I, J, Je;
     int log_uniform;       // spot nodes equally spaced in ln S
     int cell_mode;         // kCellSearch, kCellUniform or kCellBins
@@ -105,7 +105,8 @@ struct McParams {
     double* partials;      // [gridDim.x][row_words] per-block binary64 rows
     int row_words;         // 3 + Je * I (adjoint) or 3 (price only)
     double* warp_rows;     // [gridDim.x * warps][Je * I] per-warp level-2 rows
-    float* l1;             // [gridDim.x][Je * I] per-block level-1 binary32 buckets
+    float4* l1;            // [gridDim.x][(Je - 1) (I - 1)] per-block level-1 buckets: the corner sums of a cell
+                           // (nodes (i, j), (i+1, j), (i, j+1), (i+1, j+1))
     float* ckpt;           // [n_ck][gridDim.x * warps * ring_slots_per_warp() * ppl] checkpoints of x
     int n_ck;
     int flush_every;       // reverse batches between level-1 -> level-2 drains
@@ -309,7 +310,7 @@ struct BookParams {
     double* sums;          // per option [3 + I J] binary64 sums (zeroed before a run)
     double* risk;          // aggregated runs: per surface [3 + I J], the vega part summed with
                            // weights w / n_paths (zeroed before a run); null: per-option vegas
-    float* l1;             // [gridDim.x][max_IJe] binary32 buckets per block
+    float* l1;             // [gridDim.x][max_IJe] binary32 node buckets per block
     float* ckpt;           // [ceil(max_N / k)][gridDim.x * warps * ring slots]
     int max_I, max_Je, max_N, max_IJe, max_bins;
 };

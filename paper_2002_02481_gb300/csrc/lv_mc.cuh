@@ -30,9 +30,9 @@
 // batches stay at 32 paths.
 //
 // Bucket accumulation: run-length sums in registers while the cell is
-// unchanged (level 0); binary32 reductions (red.global.add.f32, resolved in
-// L2 without a retry loop) into a per-block bucket array in global memory
-// (level 1); every few batches a warp drains that array (atomicExch) into
+// unchanged (level 0); binary32 reductions (one 16-byte red per cell, resolved in
+// L2 without a retry loop) into a per-block array of the cells' corner sums in
+// global memory (level 1); every few batches a warp drains that array into
 // level 2: the block's binary64 row through binary64 reductions, or in Kahan
 // mode a compensated binary32 row the warp owns; at the end each block adds
 // what it holds to the call's binary64 sums, and the last block to arrive writes
@@ -58,11 +58,10 @@ constexpr int kRing = 4;       // checkpoint slot groups of kTile per warp
 
 constexpr int kQueue = 64;     // per-warp FIFO capacity per path a lane runs in a forward tile
                                // (entries; < 32 + kTile * ppl never overflows kQueue * ppl)
-constexpr int kMaxWarps = 8;   // blockDim.x <= 256 (every kernel here runs at most 128)
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
-constexpr int kStagedTau = 256;   // time nodes staged in shared memory for the time table's search
+constexpr int kStagedTau = 256;   // time nodes (and inverse gaps) staged in shared memory for the time table
 
 // Level-2 accumulator of one value: binary64 or Kahan-compensated binary32.
 // The slots live in shared memory (one per thread and value), which keeps
@@ -73,7 +72,7 @@ struct AccSlot {
 };
 
 struct SmemLayout {
-    size_t tab, sig, node, ab, bins, tau, tdt, qslot, qrel, qxb, acc, red, total;
+    size_t tab, sig, node, ab, bins, tau, tdt, qslot, qrel, qxb, acc, flag, total;
 };
 
 // extra: the adjoint kernel that also sums d V / d r and d V / d T (the time
@@ -90,7 +89,7 @@ __host__ __device__ inline SmemLayout smem_layout(int I, int J, int N, int n_bin
     L.node = o;  o += align16(sizeof(float) * (size_t)I);
     L.ab = o;    o += align16(sizeof(float2) * (size_t)I);
     L.bins = o;  o += sizeof(float4) * (size_t)n_bins;
-    L.tau = o;   if (J <= kStagedTau) o += align16(sizeof(double) * (size_t)J);
+    L.tau = o;   if (J <= kStagedTau) o += align16(2 * sizeof(double) * (size_t)J);
     L.tdt = o;   if (extra) o += align16(sizeof(float) * (size_t)N);
     // the adjoint kernel slices these three per warp from L.qslot: they stay
     // contiguous because each size is a multiple of 16 bytes (kQueue is)
@@ -99,7 +98,7 @@ __host__ __device__ inline SmemLayout smem_layout(int I, int J, int N, int n_bin
     L.qrel = o;  if (greeks) o += align16(sizeof(int) * (size_t)W * kQueue * ppl);
     L.qxb = o;   if (greeks) o += align16(sizeof(float) * (size_t)W * kQueue * ppl);
     L.acc = o;   o += align16(sizeof(AccSlot) * (extra ? 5 : 3) * (size_t)block);
-    L.red = o;   o += align16(sizeof(double) * 3 * kMaxWarps);
+    L.flag = o;  o += 16;
     L.total = o;
     return L;
 }
@@ -124,80 +123,139 @@ __device__ __forceinline__ double acc_value(const AccSlot& a)
     return ACC == 1 ? (double)a.s - (double)a.c : a.d;
 }
 
+// Asynchronous copy of n elements of SIZE bytes (4, 8 or 16) to shared memory.
+template <int SIZE>
+__device__ __forceinline__ void copy_async(void* dst, const void* src, int n)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    for (int e = threadIdx.x; e < n; e += blockDim.x)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d + SIZE * e),
+                     "l"(__cvta_generic_to_global(static_cast<const char*>(src) + (size_t)SIZE * e)), "n"(SIZE)
+                     : "memory");
+}
+
 // Stages the time table, the spot nodes, the cell coefficients and (when GS)
 // the sigma pairs in shared memory; large grids are read from global memory
-// through L1 instead, which leaves room for more resident blocks.
-template <bool GS, bool EXTRA = false>
-__device__ __forceinline__ void stage_grid(const McParams& P, unsigned char* smem, const SmemLayout& L)
+// through L1 instead, which leaves room for more resident blocks. `clear` runs
+// while the copies are in flight: every element is on its way before the first
+// is waited for, and the time table's searches read the time nodes from
+// shared memory (loads of one thread in turn and searches in global memory took
+// 5.4 us at the start of every launch on the 30 x 60 grid with 156 steps).
+template <bool GS, bool EXTRA = false, typename F>
+__device__ __forceinline__ void stage_grid(const McParams& P, unsigned char* smem, const SmemLayout& L, F&& clear)
 {
     const int B = blockDim.x, tid = threadIdx.x;
     int4* s_tab = reinterpret_cast<int4*>(smem + L.tab);
-    float2* s_sig = reinterpret_cast<float2*>(smem + L.sig);
-    float* s_node = reinterpret_cast<float*>(smem + L.node);
-    float2* s_ab = reinterpret_cast<float2*>(smem + L.ab);
-    if (GS)
-        for (int e = tid; e < P.Je * (P.I - 1); e += B) s_sig[e] = P.sig2[e];
-    for (int e = tid; e < P.I; e += B) s_node[e] = P.node[e];
-    for (int e = tid; e < P.I - 1; e += B) s_ab[e] = P.ab[e];
-    float4* s_bins = reinterpret_cast<float4*>(smem + L.bins);
-    for (int e = tid; e < P.n_bins; e += B) s_bins[e] = P.bins[e];
-    // the time table's binary searches read the nodes from shared memory: from
-    // global memory each was a chain of up to eight dependent loads (1.5 us of a
-    // small call's launch)
     const double* tau = P.tau;
+    const double* rtau = P.tau + P.J;
     if (P.J <= kStagedTau) {
-        double* s_tau = reinterpret_cast<double*>(smem + L.tau);
-        for (int e = tid; e < P.J; e += B) s_tau[e] = P.tau[e];
-        __syncthreads();
-        tau = s_tau;
+        copy_async<8>(smem + L.tau, P.tau, 2 * P.J);
+        tau = reinterpret_cast<const double*>(smem + L.tau);
+        rtau = tau + P.J;
     }
-    for (int n = tid; n < P.N; n += B) s_tab[n] = step_time(P, tau, n);
+    if (GS) copy_async<8>(smem + L.sig, P.sig2, P.Je * (P.I - 1));
+    copy_async<4>(smem + L.node, P.node, P.I);
+    copy_async<8>(smem + L.ab, P.ab, P.I - 1);
+    copy_async<16>(smem + L.bins, P.bins, P.n_bins);
+    clear();
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    for (int n = tid; n < P.N; n += B) s_tab[n] = step_time(P, tau, rtau, n);
     if (EXTRA) {
         float* s_tdt = reinterpret_cast<float*>(smem + L.tdt);
         for (int n = tid; n < P.N; n += B) s_tdt[n] = step_tdt(P, tau, n);
     }
+    __syncthreads();
 }
 
-// Adds the block's sum of NV per-thread binary64 values (over the block in a
-// fixed order) to sums[0 .. NV-1].
-template <int NV>
-__device__ __forceinline__ void add_scalars(const double (&v)[NV], double* s_red, double* sums)
+// Cells with a level-1 bucket: (Je - 1) rows of I - 1.
+__host__ __device__ inline int n_cells(const McParams& P) { return (P.Je - 1) * (P.I - 1); }
+
+// The level-2 row of the warp: binary64 mode drains into the block's own row
+// with binary64 reductions; Kahan pairs cannot be updated atomically, so each
+// warp owns one.
+template <int ACC>
+__device__ __forceinline__ double* level2_row(const McParams& P)
 {
-    static_assert(NV <= 3, "s_red holds three values a warp");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double a = v[k];
+    if (ACC == 1)
+        return P.warp_rows + (size_t)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (P.Je * P.I);
+    return P.partials + (size_t)blockIdx.x * P.row_words + 3;
+}
+
+// Zeroes the block's level-1 buckets and level-2 rows, and the flag that some
+// warp drained.
+template <int ACC>
+__device__ __forceinline__ void clear_buckets(const McParams& P, int* drained)
+{
+    const int nIJ = P.Je * P.I, B = blockDim.x, W = B >> 5, tid = threadIdx.x;
+    const int nc = n_cells(P);
+    float4* l1 = P.l1 + (size_t)blockIdx.x * nc;
+    for (int e = tid; e < nc; e += B) l1[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (ACC == 1) {
+        double* rows = P.warp_rows + (size_t)blockIdx.x * W * nIJ;
+        for (int e = tid; e < W * nIJ; e += B) rows[e] = 0.0;     // zero as a float2 pair too
+    } else {
+        double* row = P.partials + (size_t)blockIdx.x * P.row_words + 3;
+        for (int e = tid; e < nIJ; e += B) row[e] = 0.0;
+    }
+    if (tid == 0) *drained = 0;
+}
+
+// Adds the block's sums of the first `n` accumulators (slot k of thread t at
+// acc0[k B + t]) to sums[0 .. n-1], one warp per accumulator, after a barrier.
+template <int ACC>
+__device__ __forceinline__ void add_scalars(const AccSlot* acc0, int n, double* sums)
+{
+    const int B = blockDim.x, W = B >> 5, lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < n; k += W) {
+        double a = acc_value<ACC>(acc0[k * B + lane]);
+        for (int w = 1; w < W; ++w) a += acc_value<ACC>(acc0[k * B + 32 * w + lane]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        if (lane == 0) s_red[NV * warp + k] = a;
-    }
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += s_red[NV * w + threadIdx.x];
-        atomicAdd(&sums[threadIdx.x], s);
+        if (lane == 0) atomicAdd(&sums[k], a);
     }
 }
 
-// Adds what the block's buckets hold (its binary64 row, or in Kahan mode its
-// warps' rows, and the binary32 buckets not drained yet) to the call's sums.
+// Adds what the block's buckets hold to the call's sums: per node the corners of
+// the up to four cells around it that were not drained yet and, if some warp
+// drained, the block's binary64 row (in Kahan mode its warps' rows). Four nodes
+// of a thread are in flight at a time. The four corners are added in binary32
+// (binary64 adds run at 1.7 per SM and cycle): each is a sum of a quarter of the
+// contributions that a node's own bucket would hold.
 template <int ACC>
-__device__ __forceinline__ void fold_buckets(const McParams& P, const float* l1, const double* row)
+__device__ __forceinline__ void fold_buckets(const McParams& P, const float4* l1, const double* row, bool drained)
 {
-    const int nIJ = P.Je * P.I, B = blockDim.x, W = B >> 5;
+    constexpr int kFly = 4;
+    const int I = P.I, nIJ = P.Je * I, B = blockDim.x, W = B >> 5;
+    const float* c = reinterpret_cast<const float*>(l1);         // reductions are resolved in L2: __ldcg
     const double* rows0 = P.warp_rows + (size_t)blockIdx.x * W * nIJ;
-    for (int e = threadIdx.x; e < nIJ; e += B) {
-        double s = (double)__ldcg(l1 + e);       // reductions are resolved in L2
-        if (ACC == 1) {
-            for (int w = 0; w < W; ++w) {
-                const float2 k = reinterpret_cast<const float2*>(rows0 + (size_t)w * nIJ)[e];
-                s += (double)k.x - (double)k.y;
-            }
-        } else {
-            s += __ldcg(row + 3 + e);
+    for (int e0 = threadIdx.x; e0 < nIJ; e0 += kFly * B) {
+        float f[kFly][4];
+        double d[kFly];
+#pragma unroll
+        for (int q = 0; q < kFly; ++q) {
+            const int e = e0 + q * B, j = e / I, i = e - j * I;
+            const int cell = 4 * (j * (I - 1) + i);              // the cell whose lower corner is node e
+            const bool in = e < nIJ, up = j < P.Je - 1, rt = i < I - 1;
+            f[q][0] = in && up && rt ? __ldcg(c + cell) : 0.0f;
+            f[q][1] = in && up && i > 0 ? __ldcg(c + cell - 4 + 1) : 0.0f;
+            f[q][2] = in && j > 0 && rt ? __ldcg(c + cell - 4 * (I - 1) + 2) : 0.0f;
+            f[q][3] = in && j > 0 && i > 0 ? __ldcg(c + cell - 4 * (I - 1) - 4 + 3) : 0.0f;
+            d[q] = ACC != 1 && drained && in ? __ldcg(row + 3 + e) : 0.0;
         }
-        if (s != 0.0) atomicAdd(&P.sums[3 + e], s);
+#pragma unroll
+        for (int q = 0; q < kFly; ++q) {
+            const int e = e0 + q * B;
+            double s = (double)((f[q][0] + f[q][1]) + (f[q][2] + f[q][3]));
+            if (ACC != 1 && drained) s += d[q];
+            if (ACC == 1 && drained && e < nIJ) {
+                for (int w = 0; w < W; ++w) {
+                    const float2 k = reinterpret_cast<const float2*>(rows0 + (size_t)w * nIJ)[e];
+                    s += (double)k.x - (double)k.y;
+                }
+            }
+            if (s != 0.0) atomicAdd(&P.sums[3 + e], s);
+        }
     }
 }
 
@@ -245,11 +303,19 @@ __device__ __forceinline__ void finish_call(const McParams& P)
     const double scale = P.want_sums ? 1.0 : P.inv_paths;
     if (GREEKS) {
         double* s = P.sums + 3;           // time-major buckets j I + i
-        for (int e = tid; e < nIJ; e += B) {
-            const double v = __ldcg(s + e);
-            s[e] = 0.0;
-            const int j = e / P.I, i = e - j * P.I;
-            if (j < P.J) P.out[3 + i * P.J + j] = bad ? nan : v * scale;   // not the padding row of one time node
+        constexpr int kFly = 8;           // buckets of a thread in flight
+        for (int e0 = tid; e0 < nIJ; e0 += kFly * B) {
+            double v[kFly];
+#pragma unroll
+            for (int q = 0; q < kFly; ++q) v[q] = e0 + q * B < nIJ ? __ldcg(s + e0 + q * B) : 0.0;
+#pragma unroll
+            for (int q = 0; q < kFly; ++q) {
+                const int e = e0 + q * B;
+                if (e >= nIJ) break;
+                s[e] = 0.0;
+                const int j = e / P.I, i = e - j * P.I;
+                if (j < P.J) P.out[3 + i * P.J + j] = bad ? nan : v[q] * scale;   // not the padding row of one time node
+            }
         }
     }
     if (EXTRA && tid < 2) {
@@ -263,44 +329,88 @@ __device__ __forceinline__ void finish_call(const McParams& P)
     }
 }
 
-// Claims n consecutive tiles for the warp; returns the first.
-__device__ __forceinline__ int claim_tile(unsigned int* counter, unsigned n = 1u)
+// Claims the warp's next n consecutive tiles; returns the first. Every warp of
+// the grid starts on the tiles of its own index without a claim, so the counter
+// gives those after them, and a call with no more than that many claims nothing.
+__device__ __forceinline__ int claim_tile(const McParams& P, int n = 1)
 {
+    const int first = (int)(gridDim.x * (blockDim.x >> 5)) * n;
+    if (P.n_tiles <= first) return P.n_tiles;
     int t = 0;
-    if ((threadIdx.x & 31) == 0) t = (int)atomicAdd(counter, n);
+    if ((threadIdx.x & 31) == 0) t = first + (int)atomicAdd(P.tile_counter, (unsigned)n);
     return __shfl_sync(0xffffffffu, t, 0);
 }
 
-// Moves the block's binary32 buckets into its level-2 row (binary64) or the
-// warp's (Kahan). A bucket that reads zero is left for a later drain. Eight
-// buckets of a lane are in flight at a time: one by one, each waited for a
-// load and an exchange in L2.
-template <int ACC>
-__device__ __forceinline__ void drain_buckets(float* l1, int nIJ, double* wrow)
+__device__ __forceinline__ int first_tile(int n = 1)
 {
-    constexpr int kFly = 8;
-    const int lane = threadIdx.x & 31;
-    for (int e0 = lane; e0 < nIJ; e0 += 32 * kFly) {
-        float v[kFly];
-#pragma unroll
-        for (int q = 0; q < kFly; ++q) v[q] = e0 + 32 * q < nIJ ? __ldcg(l1 + e0 + 32 * q) : 0.0f;
-#pragma unroll
-        for (int q = 0; q < kFly; ++q)
-            if (v[q] != 0.0f) v[q] = atomicExch(l1 + e0 + 32 * q, 0.0f);
+    return (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * n;
+}
+
+// Takes a bucket's four sums, leaving zeros.
+__device__ __forceinline__ float4 take4(float4* p)
+{
+    unsigned long long a, b;
+    asm volatile("{\n\t.reg .b128 d, z;\n\tmov.b128 z, {%3, %3};\n\t"
+                 "atom.relaxed.gpu.global.exch.b128 d, [%2], z;\n\tmov.b128 {%0, %1}, d;\n\t}"
+                 : "=l"(a), "=l"(b)
+                 : "l"(__cvta_generic_to_global(p)), "l"(0ull)
+                 : "memory");
+    return make_float4(__uint_as_float((unsigned)a), __uint_as_float((unsigned)(a >> 32)), __uint_as_float((unsigned)b),
+                       __uint_as_float((unsigned)(b >> 32)));
+}
+
+// Adds v to entry e of a level-2 row (binary64, shared by the block's warps; or
+// the warp's Kahan pairs).
+template <int ACC>
+__device__ __forceinline__ void level2_add(double* wrow, int e, float v)
+{
+    if (v == 0.0f) return;
+    if (ACC == 1) {
+        float2* k = reinterpret_cast<float2*>(wrow) + e;
+        float2 p = *k;
+        const float y = v - p.y;
+        const float t = p.x + y;
+        p.y = (t - p.x) - y;
+        p.x = t;
+        *k = p;
+    } else {
+        atomicAdd(wrow + e, (double)v);
+    }
+}
+
+// Moves the block's binary32 buckets into its level-2 row (binary64) or the
+// warp's (Kahan). A lane takes one cell of a row of cells and hands its right
+// corners to the next lane, which adds them to its own left ones: two additions
+// per cell to the nodes below and above. 31 cells a warp at a time (the last lane
+// only receives). A bucket that reads zero is left for a later drain; two rows
+// of cells are in flight at a time.
+template <int ACC>
+__device__ __forceinline__ void drain_buckets(const McParams& P, float4* l1, double* wrow, int* drained)
+{
+    constexpr int kFly = 2;
+    const int lane = threadIdx.x & 31, C = P.I - 1, chunks = (C + 30) / 31, n = chunks * (P.Je - 1);
+    if (lane == 0) *drained = 1;
+    for (int t0 = 0; t0 < n; t0 += kFly) {
+        float4 v[kFly];
 #pragma unroll
         for (int q = 0; q < kFly; ++q) {
-            if (v[q] == 0.0f) continue;
-            if (ACC == 1) {
-                float2* k = reinterpret_cast<float2*>(wrow) + e0 + 32 * q;
-                float2 p = *k;
-                const float y = v[q] - p.y;
-                const float t = p.x + y;
-                p.y = (t - p.x) - y;
-                p.x = t;
-                *k = p;
-            } else {
-                atomicAdd(wrow + e0 + 32 * q, (double)v[q]);      // the block's row, shared by its warps
+            const int t = t0 + q, j = t / chunks, i = 31 * (t - j * chunks) + lane;
+            v[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (t < n && lane < 31 && i < C) {
+                float4* p = l1 + j * C + i;
+                v[q] = __ldcg(p);
+                if (v[q].x != 0.0f || v[q].y != 0.0f || v[q].z != 0.0f || v[q].w != 0.0f) v[q] = take4(p);
             }
+        }
+#pragma unroll
+        for (int q = 0; q < kFly; ++q) {
+            const int t = t0 + q, j = t / chunks, i = 31 * (t - j * chunks) + lane;
+            const float y = __shfl_up_sync(0xffffffffu, v[q].y, 1), w = __shfl_up_sync(0xffffffffu, v[q].w, 1);
+            if (t < n && i <= C) {
+                level2_add<ACC>(wrow, j * P.I + i, v[q].x + (lane > 0 ? y : 0.0f));
+                level2_add<ACC>(wrow, (j + 1) * P.I + i, v[q].z + (lane > 0 ? w : 0.0f));
+            }
+            if (ACC == 1) __syncwarp();      // another lane may update the same pair next
         }
     }
 }
@@ -309,7 +419,9 @@ __device__ __forceinline__ void drain_buckets(float* l1, int nIJ, double* wrow)
 // registers more than warps. Four blocks per SM at 124-128 registers against
 // five at 96 and six at 80, same code: 0.615, 0.643 and 0.684 ms at 2^20 paths on
 // the 30 x 60 grid with 156 steps, 2.06, 2.20 and 2.30 ms at 2^22 (the loops with
-// a bound check in every step, six blocks: 0.660 and 2.23 ms).
+// a bound check in every step, six blocks: 0.660 and 2.23 ms). One path per lane
+// needs 110 registers; held to five blocks it gains 1-4 % from 2^20 paths on, where
+// two paths per lane are faster still, and loses 4-5 % below.
 //
 // PPL: paths per lane of a forward tile. With PPL = 2 a warp claims two
 // consecutive 32-path tiles and runs them interleaved (forward_path2: two
@@ -325,31 +437,22 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
     const int B = blockDim.x, W = B >> 5;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const SmemLayout L = smem_layout(P.I, P.J, P.N, P.n_bins, B, true, GS, EXTRA, PPL);
-    stage_grid<GS, EXTRA>(P, smem, L);
-    float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);    // this block's level-1 buckets
+    int* const drained = reinterpret_cast<int*>(smem + L.flag);
+    AccSlot* const acc0 = reinterpret_cast<AccSlot*>(smem + L.acc);
+    AccSlot* acc = acc0 + tid;               // [3][block]: V, V^2, xbar_0; then d V / d r, d V / d T
+    stage_grid<GS, EXTRA>(P, smem, L, [&]() {
+        clear_buckets<ACC>(P, drained);
+        for (int k = 0; k < (EXTRA ? 5 : 3); ++k) acc[k * B] = AccSlot{0.0, 0.0f, 0.0f};
+    });
+    float4* l1 = P.l1 + (size_t)blockIdx.x * n_cells(P);    // this block\'s level-1 buckets
     // the three FIFO arrays of all warps are contiguous from L.qslot (each
     // W * kQcap words): one base per warp, the others at fixed offsets, which
     // keeps two registers free for the packed forward pass
     int* const q_slot = reinterpret_cast<int*>(smem + L.qslot) + warp * 3 * kQcap;
     int* const q_rel = q_slot + kQcap;
     float* const q_xb = reinterpret_cast<float*>(q_slot + 2 * kQcap);
-    double* s_red = reinterpret_cast<double*>(smem + L.red);
     const int nIJ = P.Je * P.I;
-    for (int e = tid; e < nIJ; e += B) l1[e] = 0.0f;
     const int wid = blockIdx.x * W + warp;                    // global warp id
-    // level 2: binary64 mode drains into the block's own row with binary64
-    // reductions; Kahan pairs cannot be updated atomically, so each warp owns one
-    double* const row = P.partials + (size_t)blockIdx.x * P.row_words;
-    double* wrow;
-    if (ACC == 1) {
-        wrow = P.warp_rows + (size_t)wid * nIJ;
-        for (int e = lane; e < nIJ; e += 32) wrow[e] = 0.0;   // zero as a float2 pair too
-    } else {
-        wrow = row + 3;
-        for (int e = tid; e < nIJ; e += B) wrow[e] = 0.0;
-    }
-    __syncthreads();
-
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
                       reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
@@ -357,12 +460,9 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
     const size_t cks = (size_t)gridDim.x * W * kRing * kSlots;  // checkpoint stride
     float* const ckw = P.ckpt + (size_t)wid * kRing * kSlots;    // this warp's slots
 
-    AccSlot* acc = reinterpret_cast<AccSlot*>(smem + L.acc) + tid;   // [3][block]: V, V^2, xbar_0
-    acc[0] = acc[B] = acc[2 * B] = AccSlot{0.0, 0.0f, 0.0f};
-    if (EXTRA) acc[3 * B] = acc[4 * B] = AccSlot{0.0, 0.0f, 0.0f};    // d V / d r, d V / d T
     int q_head = 0, q_count = 0, batches = 0;
     unsigned fwd_count = 0;
-    int tile = claim_tile(P.tile_counter, PPL);
+    int tile = first_tile(PPL);
 
     while (true) {
         const int g_next = (int)(fwd_count % kRing);
@@ -392,8 +492,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
             q_count -= nb;
             __syncwarp();
             if (++batches % P.flush_every == 0)      // the level-2 row, recomputed (one register less)
-                drain_buckets<ACC>(l1, nIJ, ACC == 1 ? P.warp_rows + (size_t)wid * nIJ
-                                                     : P.partials + (size_t)blockIdx.x * P.row_words + 3);
+                drain_buckets<ACC>(P, l1, level2_row<ACC>(P), drained);
             continue;
         }
         if (!more) break;
@@ -437,7 +536,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
             }
             ++fwd_count;
             __syncwarp();
-            tile = claim_tile(P.tile_counter, PPL);
+            tile = claim_tile(P, PPL);
             continue;
         }
 
@@ -475,17 +574,13 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
         q_count += __popc(bal);
         ++fwd_count;
         __syncwarp();
-        tile = claim_tile(P.tile_counter, PPL);
+        tile = claim_tile(P, PPL);
     }
 
     __syncthreads();                           // after it nothing adds to this block's buckets
-    const double* row_f = P.partials + (size_t)blockIdx.x * P.row_words;     // recomputed, not live through the loop
-    fold_buckets<ACC>(P, l1, row_f);
-    add_scalars({acc_value<ACC>(acc[0]), acc_value<ACC>(acc[B]), acc_value<ACC>(acc[2 * B])}, s_red, P.sums);
-    if (EXTRA) {
-        __syncthreads();                       // s_red is reused
-        add_scalars({acc_value<ACC>(acc[3 * B]), acc_value<ACC>(acc[4 * B])}, s_red, P.sums + 3 + nIJ);
-    }
+    fold_buckets<ACC>(P, l1, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    add_scalars<ACC>(acc0, 3, P.sums);
+    if (EXTRA) add_scalars<ACC>(acc0 + 3 * B, 2, P.sums + 3 + nIJ);
     finish_call<true, EXTRA>(P);
 }
 
@@ -499,36 +594,26 @@ template <int ACC, bool GS, int MODEL, int PPL, int CELL>
 __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int B = blockDim.x, W = B >> 5;
+    const int B = blockDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kQcap = kQueue * PPL;
     const SmemLayout L = smem_layout(P.I, P.J, P.N, P.n_bins, B, true, GS, false, PPL);
-    stage_grid<GS>(P, smem, L);
-    float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);
+    int* const drained = reinterpret_cast<int*>(smem + L.flag);
+    AccSlot* const acc0 = reinterpret_cast<AccSlot*>(smem + L.acc);
+    AccSlot* acc = acc0 + tid;               // [3][block]: V, V^2, xbar_0
+    stage_grid<GS>(P, smem, L, [&]() {
+        clear_buckets<ACC>(P, drained);
+        for (int k = 0; k < 3; ++k) acc[k * B] = AccSlot{0.0, 0.0f, 0.0f};
+    });
+    float4* l1 = P.l1 + (size_t)blockIdx.x * n_cells(P);    // this block\'s level-1 buckets
     int* q_rel = reinterpret_cast<int*>(smem + L.qrel) + warp * kQcap;
     float* q_c = reinterpret_cast<float*>(smem + L.qxb) + warp * kQcap;
-    double* s_red = reinterpret_cast<double*>(smem + L.red);
-    const int nIJ = P.Je * P.I;
-    for (int e = tid; e < nIJ; e += B) l1[e] = 0.0f;
-    const int wid = blockIdx.x * W + warp;
-    double* const row = P.partials + (size_t)blockIdx.x * P.row_words;
-    double* wrow;
-    if (ACC == 1) {
-        wrow = P.warp_rows + (size_t)wid * nIJ;
-        for (int e = lane; e < nIJ; e += 32) wrow[e] = 0.0;
-    } else {
-        wrow = row + 3;
-        for (int e = tid; e < nIJ; e += B) wrow[e] = 0.0;
-    }
-    __syncthreads();
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
                       reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
                       reinterpret_cast<const float4*>(smem + L.bins) };
-    AccSlot* acc = reinterpret_cast<AccSlot*>(smem + L.acc) + tid;   // [3][block]: V, V^2, xbar_0
-    acc[0] = acc[B] = acc[2 * B] = AccSlot{0.0, 0.0f, 0.0f};
     int q_head = 0, q_count = 0, batches = 0;
-    int tile = claim_tile(P.tile_counter, PPL);
+    int tile = first_tile(PPL);
     while (true) {
         const bool more = tile < P.n_tiles;
         if (q_count >= 32 || (!more && q_count > 0)) {
@@ -542,7 +627,7 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
             __syncwarp();
-            if (++batches % P.flush_every == 0) drain_buckets<ACC>(l1, nIJ, wrow);
+            if (++batches % P.flush_every == 0) drain_buckets<ACC>(P, l1, level2_row<ACC>(P), drained);
             continue;
         }
         if (!more) break;
@@ -585,7 +670,7 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
                 q_count += __popc(bal);
             }
             __syncwarp();
-            tile = claim_tile(P.tile_counter, PPL);
+            tile = claim_tile(P, PPL);
             continue;
         }
         const long long rel = (long long)tile * kTile + lane;
@@ -613,11 +698,11 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
         }
         q_count += __popc(bal);
         __syncwarp();
-        tile = claim_tile(P.tile_counter, PPL);
+        tile = claim_tile(P, PPL);
     }
     __syncthreads();
-    fold_buckets<ACC>(P, l1, row);
-    add_scalars({acc_value<ACC>(acc[0]), acc_value<ACC>(acc[B]), acc_value<ACC>(acc[2 * B])}, s_red, P.sums);
+    fold_buckets<ACC>(P, l1, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    add_scalars<ACC>(acc0, 3, P.sums);
     finish_call<true>(P);
 }
 
@@ -635,25 +720,22 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kQcap = kQueue * PPL;
     const SmemLayout L = smem_layout(P.I, P.J, P.N, P.n_bins, B, true, GS, false, PPL);
-    stage_grid<GS>(P, smem, L);
-    float* l1 = P.l1 + (size_t)blockIdx.x * (P.Je * P.I);
+    int* const drained = reinterpret_cast<int*>(smem + L.flag);
+    AccSlot* const acc0 = reinterpret_cast<AccSlot*>(smem + L.acc);
+    AccSlot* acc = acc0 + tid;               // [3][block]: V, V^2, xbar_0
+    stage_grid<GS>(P, smem, L, [&]() {
+        clear_buckets<0>(P, drained);
+        for (int k = 0; k < 3; ++k) acc[k * B] = AccSlot{0.0, 0.0f, 0.0f};
+    });
+    float4* l1 = P.l1 + (size_t)blockIdx.x * n_cells(P);    // this block\'s level-1 buckets
     int* q_rel = reinterpret_cast<int*>(smem + L.qrel) + warp * kQcap;
     float* q_c = reinterpret_cast<float*>(smem + L.qxb) + warp * kQcap;
-    double* s_red = reinterpret_cast<double*>(smem + L.red);
-    const int nIJ = P.Je * P.I;
-    for (int e = tid; e < nIJ; e += B) l1[e] = 0.0f;
-    double* const row = P.partials + (size_t)blockIdx.x * P.row_words;
-    double* const wrow = row + 3;
-    for (int e = tid; e < nIJ; e += B) wrow[e] = 0.0;
-    __syncthreads();
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
                       reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
                       reinterpret_cast<const float4*>(smem + L.bins) };
-    AccSlot* acc = reinterpret_cast<AccSlot*>(smem + L.acc) + tid;   // [3][block]: V, V^2, xbar_0
-    acc[0] = acc[B] = acc[2 * B] = AccSlot{0.0, 0.0f, 0.0f};
     int q_head = 0, q_count = 0, batches = 0;
-    int tile = claim_tile(P.tile_counter, PPL);
+    int tile = first_tile(PPL);
     while (true) {
         const bool more = tile < P.n_tiles;
         if (q_count >= 32 || (!more && q_count > 0)) {
@@ -667,7 +749,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
             __syncwarp();
-            if (++batches % P.flush_every == 0) drain_buckets<0>(l1, nIJ, wrow);
+            if (++batches % P.flush_every == 0) drain_buckets<0>(P, l1, level2_row<0>(P), drained);
             continue;
         }
         if (!more) break;
@@ -710,7 +792,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
                 q_count += __popc(bal);
             }
             __syncwarp();
-            tile = claim_tile(P.tile_counter, PPL);
+            tile = claim_tile(P, PPL);
             continue;
         }
         const long long rel = (long long)tile * kTile + lane;
@@ -738,11 +820,11 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
         }
         q_count += __popc(bal);
         __syncwarp();
-        tile = claim_tile(P.tile_counter, PPL);
+        tile = claim_tile(P, PPL);
     }
     __syncthreads();
-    fold_buckets<0>(P, l1, row);
-    add_scalars({acc_value<0>(acc[0]), acc_value<0>(acc[B]), acc_value<0>(acc[2 * B])}, s_red, P.sums);
+    fold_buckets<0>(P, l1, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    add_scalars<0>(acc0, 3, P.sums);
     finish_call<true>(P);
 }
 
@@ -759,16 +841,15 @@ __global__ void __launch_bounds__(128, 9) price_kernel(const __grid_constant__ M
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const SmemLayout L = smem_layout(P.I, P.J, P.N, P.n_bins, blockDim.x, false, GS);
-    stage_grid<GS>(P, smem, L);
-    __syncthreads();
+    AccSlot* const acc0 = reinterpret_cast<AccSlot*>(smem + L.acc);
+    AccSlot* acc = acc0 + threadIdx.x;
+    stage_grid<GS>(P, smem, L, [&]() { acc[0] = acc[blockDim.x] = AccSlot{0.0, 0.0f, 0.0f}; });
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
                       reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
                       reinterpret_cast<const float4*>(smem + L.bins) };
     const int lane = threadIdx.x & 31;
-    AccSlot* acc = reinterpret_cast<AccSlot*>(smem + L.acc) + threadIdx.x;
-    acc[0] = acc[blockDim.x] = AccSlot{0.0, 0.0f, 0.0f};
-    for (int tile = claim_tile(P.tile_counter); tile < P.n_tiles; tile = claim_tile(P.tile_counter)) {
+    for (int tile = first_tile(); tile < P.n_tiles; tile = claim_tile(P)) {
         const long long rel_a = (long long)tile * kPriceTile + lane, rel_b = rel_a + 32;
         if (rel_a < P.n_paths) {
             uint32_t c1a, c2a, c1b, c2b;
@@ -787,8 +868,8 @@ __global__ void __launch_bounds__(128, 9) price_kernel(const __grid_constant__ M
             }
         }
     }
-    double* s_red = reinterpret_cast<double*>(smem + L.red);
-    add_scalars({acc_value<ACC>(acc[0]), acc_value<ACC>(acc[blockDim.x])}, s_red, P.sums);
+    __syncthreads();
+    add_scalars<ACC>(acc0, 2, P.sums);
     finish_call<false>(P);
 }
 
