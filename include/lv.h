@@ -157,16 +157,18 @@ lv_status lv_set_scheme(lv_surface_t h, int32_t scheme);
 
 /* Launch shape: threads per block (32..128, multiple of 32), checkpoint
  * interval k of the reverse sweep (4, 8, 16 or 32 steps) and resident
- * blocks per SM; 0 keeps the tuned or default value. Results do not depend
- * on it beyond reduction-order rounding. */
+ * blocks per SM; 0 keeps the tuned or default value. With 128 threads, k = 4
+ * and no blocks_per_sm, a reverse sweep of at least 512 paths per SM runs the
+ * SM's four blocks as one of 512 threads that share the staged grid. Results do
+ * not depend on it beyond reduction-order rounding. */
 lv_status lv_set_launch(lv_surface_t h, int32_t block, int32_t k, int32_t blocks_per_sm);
 
 /* Paths per lane of the adjoint's forward tiles: 1, or 2 (each lane runs two
  * paths interleaved: two independent dependency chains per thread, the
  * per-step grid data loaded once for both, and on the main reading their
  * binary32 arithmetic in packed pairs where that keeps the occupancy); 0 keeps
- * the tuned value, or the default: 2 for calls of at least 6,144 paths per SM
- * (933,888 on 152 SMs), where every warp still gets four pairs of tiles, else 1.
+ * the tuned value, or the default: 2 for calls of at least 1,536 paths per SM
+ * (233,472 on 152 SMs), one and a half pairs of tiles per resident warp, else 1.
  * Two paths per lane exist for the reverse sweep with checkpoints every 4
  * or 8 steps (every reading of the scheme), the main reading's tangent-ratio
  * adjoint and its second-order buckets; elsewhere the call runs one. The results do not

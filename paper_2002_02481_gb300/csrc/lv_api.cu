@@ -220,7 +220,7 @@ lv_status check_option(double S0, double r, double K, double T, int32_t n_steps)
 
 struct Plan {
     int block = 128, k = 4, bps = 1, grid = 1, ppl = 1;
-    bool grid_smem = true;
+    bool grid_smem = true, wide = false;
     size_t smem = 0;
     int n_tiles = 0, n_ck = 0, row_words = 0;
     size_t off_part = 0, off_wrows = 0, off_l1 = 0, off_ckpt = 0, total = 0;
@@ -273,7 +273,10 @@ void occ_store(const OccKey& key, int occ)
 // (2^17 121 and 134).
 constexpr int64_t kPairMinPathsPerSm = 3 * 32 * 16;
 
-// n_paths < 0: a call large enough for two paths per lane.
+// A call of at least this many paths per SM (one tile for each of its warps) runs
+// one 512-thread block per SM where it could run four of 128.
+constexpr int64_t kWideMinPathsPerSm = 32 * 16;
+
 // The head of the handle's scratch, at the same place in every launch's layout:
 // the tile counter, the flag and the block counter, then the call's binary64 sums.
 // Zero between launches: cleared when allocated, left at zero by every launch.
@@ -290,9 +293,11 @@ void bind_header(lv::McParams& P, char* base)
     P.sums = reinterpret_cast<double*>(base + kOffSums);
 }
 
+// n_paths < 0: a call large enough for two paths per lane. `wide`: whether the call
+// may run 512-thread blocks (its cells need no search), set to whether it does.
 lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* block, int* k, int* bps,
                         bool dbg = false, bool* grid_smem = nullptr, bool extra = false, bool vanna = false,
-                        int* ppl_out = nullptr, int64_t n_paths = -1)
+                        int* ppl_out = nullptr, int64_t n_paths = -1, bool* wide = nullptr)
 {
     *block = h->cfg_block ? h->cfg_block : 128;
     *k = greeks ? (h->cfg_k ? h->cfg_k : 4) : 4;
@@ -316,7 +321,22 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
                        ((vanna || h->adj_method == LV_ADJ_TANGENT) ? model == 0 : (*k == 4 || *k == 8));
     if (!pairs) ppl = 1;
     if (ppl_out) *ppl_out = ppl;
-    const bool gs = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
+    // the cell mode of any call whose cell index is bounded (base_params)
+    const int cell = dbg || *k > lv::kModelMaxK ? lv::kCellSearch
+                     : h->log_uniform           ? lv::kCellUniform
+                     : h->n_bins > 0            ? lv::kCellBins
+                                                : lv::kCellSearch;
+    bool gs = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
+    // one block of 512 threads per SM instead of four of 128, if the call has work
+    // for its warps and the grid fits once
+    if (wide && *wide && greeks && !vanna && *block == 128 && !h->cfg_bps && *k == 4 &&
+        h->adj_method == LV_ADJ_REVERSE && cell != lv::kCellSearch && n_paths >= kWideMinPathsPerSm * h->num_sms &&
+        lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, lv::kWideBlock, greeks, true, extra, ppl) <= 200 * 1024) {
+        *block = lv::kWideBlock;
+        gs = true;
+    } else if (wide) {
+        *wide = false;
+    }
     if (grid_smem) *grid_smem = gs;
     const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, gs, extra, ppl);
     if (smem > 200 * 1024)
@@ -324,11 +344,6 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     int occ = 0;
     const int acc = dbg || extra || vanna ? 0 : h->acc_mode;
     const int method = vanna ? lv::kMethodVanna : (dbg || extra ? LV_ADJ_REVERSE : h->adj_method);
-    // the cell mode of any call whose cell index is bounded (base_params)
-    const int cell = dbg || *k > lv::kModelMaxK ? lv::kCellSearch
-                     : h->log_uniform           ? lv::kCellUniform
-                     : h->n_bins > 0            ? lv::kCellBins
-                                                : lv::kCellSearch;
     const OccKey key{h->device, *block, *k, greeks, acc, dbg, gs, method, model, cell, extra, smem, ppl};
     if (!occ_lookup(key, &occ)) {
         LV_CUDA(lv::mc_occupancy(*block, *k, greeks, acc, dbg, gs, method, model, cell, extra, smem, &occ, ppl));
@@ -343,7 +358,7 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
                     bool extra = false, bool vanna = false)
 {
     lv_status st = choose_launch(h, n_steps, greeks, &p->block, &p->k, &p->bps, dbg, &p->grid_smem, extra, vanna,
-                                 &p->ppl, n_paths);
+                                 &p->ppl, n_paths, &p->wide);
     if (st != LV_OK) return st;
     p->smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, p->block, greeks, p->grid_smem, extra, p->ppl);
     const int warps = p->block / 32;
@@ -498,6 +513,7 @@ lv_status run_mc(lv_surface_s* h, const McCall& c)
     if (c.vanna && (h->interp != LV_INTERP_S || h->scheme != LV_SCHEME_LOG))
         return fail(LV_EINVAL, "second-order buckets run the main reading (LV_INTERP_S, LV_SCHEME_LOG) only");
     Plan p;
+    p.wide = base_params(h, c, 4).cell_mode != lv::kCellSearch;
     st = make_plan(h, c.n_steps, c.n_paths, c.greeks, c.dbg_xN != nullptr, &p, c.extra, c.vanna);
     if (st != LV_OK) return st;
     st = ensure_scratch(h, p.total);

@@ -258,6 +258,7 @@ LV_DECLARE_MODEL(3)
 #undef LV_DECLARE_MODEL
 #undef LV_DECLARE_KERNELS
 constexpr int kModelMaxK = 8;
+constexpr int kWideBlock = 512;    // threads of a block that has an SM to itself (adjoint_kernel WIDE)
 int ring_slots_per_warp();
 int paths_per_tile(bool greeks);   // paths a warp claims at a time (adjoint / price kernel)
 

@@ -198,7 +198,7 @@ __device__ __forceinline__ void clear_buckets(const McParams& P, int* drained)
         double* row = P.partials + (size_t)blockIdx.x * P.row_words + 3;
         for (int e = tid; e < nIJ; e += B) row[e] = 0.0;
     }
-    if (tid == 0) *drained = 0;
+    if (tid == 0) drained[0] = drained[1] = 0;      // the flag and the drains' lock
 }
 
 // Adds the block's sums of the first `n` accumulators (slot k of thread t at
@@ -359,62 +359,90 @@ __device__ __forceinline__ float4 take4(float4* p)
                        __uint_as_float((unsigned)(b >> 32)));
 }
 
-// Adds v to entry e of a level-2 row (binary64, shared by the block's warps; or
-// the warp's Kahan pairs).
-template <int ACC>
-__device__ __forceinline__ void level2_add(double* wrow, int e, float v)
+// Where a warp's count of reverse batches starts, so that the block's warps drain
+// in turn, every flush_every / W batches of the block's pace, and not all at once: a
+// bucket then holds a few hundred live paths whatever the block's size. The first
+// drain comes four batches later than that, which spares calls of two batches a
+// warp any drain (2^18 paths: 178 us, 188 with the turns from the start).
+__device__ __forceinline__ int first_drain(const McParams& P, int warp, int W)
 {
-    if (v == 0.0f) return;
-    if (ACC == 1) {
-        float2* k = reinterpret_cast<float2*>(wrow) + e;
-        float2 p = *k;
-        const float y = v - p.y;
-        const float t = p.x + y;
-        p.y = (t - p.x) - y;
-        p.x = t;
-        *k = p;
-    } else {
-        atomicAdd(wrow + e, (double)v);
-    }
+    return warp * P.flush_every / W - 4;
 }
 
 // Moves the block's binary32 buckets into its level-2 row (binary64) or the
-// warp's (Kahan). A lane takes one cell of a row of cells and hands its right
-// corners to the next lane, which adds them to its own left ones: two additions
-// per cell to the nodes below and above. 31 cells a warp at a time (the last lane
-// only receives). A bucket that reads zero is left for a later drain; two rows
-// of cells are in flight at a time.
+// warp's (Kahan). A lane takes one column of cells, hands their right corners to
+// the next lane and carries the upper corners to the next row, so that every node
+// gets one addition; 31 columns a warp at a time (the last lane only receives),
+// eight rows of them in flight. A bucket that reads zero is left for a later
+// drain. The binary64 row is updated by plain loads and stores under the block's
+// lock (flags[1]): as binary64 reductions, two a node, a drain took 28 us of its
+// warp's time when every warp drained. Returns false when another warp holds the
+// lock: the caller tries again after its next batch.
 template <int ACC>
-__device__ __forceinline__ void drain_buckets(const McParams& P, float4* l1, double* wrow, int* drained)
+__device__ __forceinline__ bool drain_buckets(const McParams& P, float4* l1, double* wrow, int* flags)
 {
-    constexpr int kFly = 2;
-    const int lane = threadIdx.x & 31, C = P.I - 1, chunks = (C + 30) / 31, n = chunks * (P.Je - 1);
-    if (lane == 0) *drained = 1;
-    for (int t0 = 0; t0 < n; t0 += kFly) {
-        float4 v[kFly];
-#pragma unroll
-        for (int q = 0; q < kFly; ++q) {
-            const int t = t0 + q, j = t / chunks, i = 31 * (t - j * chunks) + lane;
-            v[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (t < n && lane < 31 && i < C) {
-                float4* p = l1 + j * C + i;
-                v[q] = __ldcg(p);
-                if (v[q].x != 0.0f || v[q].y != 0.0f || v[q].z != 0.0f || v[q].w != 0.0f) v[q] = take4(p);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < kFly; ++q) {
-            const int t = t0 + q, j = t / chunks, i = 31 * (t - j * chunks) + lane;
-            const float y = __shfl_up_sync(0xffffffffu, v[q].y, 1), w = __shfl_up_sync(0xffffffffu, v[q].w, 1);
-            if (t < n && i <= C) {
-                level2_add<ACC>(wrow, j * P.I + i, v[q].x + (lane > 0 ? y : 0.0f));
-                level2_add<ACC>(wrow, (j + 1) * P.I + i, v[q].z + (lane > 0 ? w : 0.0f));
-            }
-            if (ACC == 1) __syncwarp();      // another lane may update the same pair next
-        }
+    constexpr int kFly = 8;
+    const int lane = threadIdx.x & 31, I = P.I, C = I - 1, rows = P.Je - 1;
+    if (ACC == 0) {
+        int got = 0;
+        if (lane == 0) got = atomicCAS(&flags[1], 0, 1) == 0;
+        if (!__shfl_sync(0xffffffffu, got, 0)) return false;
+        __threadfence_block();
     }
+    if (lane == 0) flags[0] = 1;
+    for (int i0 = 0; i0 < C; i0 += 31) {
+        const int i = i0 + lane;
+        const bool cell = lane < 31 && i < C, node = i <= C;
+        float carry = 0.0f;
+        auto put = [&](int e, double d, float f) {
+            if (f == 0.0f) return;
+            if (ACC == 1) {
+                float2* k = reinterpret_cast<float2*>(wrow) + e;
+                float2 p = *k;
+                const float y = f - p.y;
+                const float t = p.x + y;
+                p.y = (t - p.x) - y;
+                p.x = t;
+                *k = p;
+            } else {
+                __stcg(wrow + e, d + (double)f);
+            }
+        };
+        for (int j0 = 0; j0 <= rows; j0 += kFly) {          // node rows 0 .. rows
+            float4 v[kFly];
+            double d[kFly];
+#pragma unroll
+            for (int q = 0; q < kFly; ++q) {
+                v[q] = cell && j0 + q < rows ? __ldcg(l1 + (j0 + q) * C + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                d[q] = ACC == 0 && node && j0 + q <= rows ? __ldcg(wrow + (j0 + q) * I + i) : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < kFly; ++q)
+                if (v[q].x != 0.0f || v[q].y != 0.0f || v[q].z != 0.0f || v[q].w != 0.0f)
+                    v[q] = take4(l1 + (j0 + q) * C + i);
+#pragma unroll
+            for (int q = 0; q < kFly; ++q) {
+                const float y = __shfl_up_sync(0xffffffffu, v[q].y, 1), w = __shfl_up_sync(0xffffffffu, v[q].w, 1);
+                const float f = (v[q].x + (lane > 0 ? y : 0.0f)) + carry;
+                carry = v[q].z + (lane > 0 ? w : 0.0f);
+                if (node && j0 + q <= rows) put((j0 + q) * I + i, d[q], f);
+            }
+        }
+        __threadfence_block();                   // the next columns' first lane updates this one's last node
+        __syncwarp();
+    }
+    if (ACC == 0 && lane == 0) atomicExch(&flags[1], 0);
+    return true;
 }
 
+// WIDE: one block of 512 threads per SM (choose_launch): the sixteen warps share one copy of the sigma
+// pairs in shared memory instead of reading them through L1, and one array of
+// level-1 buckets (24 MB instead of 95 MB over the chip on a 100 x 100 grid). 100 x
+// 100 grid, 1,260 steps, 2^22 paths: 18.2 -> 15.3 ms. Other grids gain from the
+// quarter of the stagings, folds and buckets (30 x 60, 156 steps, 2^20 paths, with
+// the drains in turn: 558 -> 510 us), so every call with a tile for each warp of
+// the chip runs this form unless its launch shape was chosen otherwise.
+//
 // Launch bound: the straight-line time loops (time_blocks, reverse_path) want
 // registers more than warps. Four blocks per SM at 124-128 registers against
 // five at 96 and six at 80, same code: 0.615, 0.643 and 0.684 ms at 2^20 paths on
@@ -428,8 +456,8 @@ __device__ __forceinline__ void drain_buckets(const McParams& P, float4* l1, dou
 // independent dependency chains per lane, the per-step time data loaded once);
 // each path's arithmetic is that of PPL = 1, the ring groups and the FIFO
 // hold twice as many entries, and the reverse batches are unchanged.
-template <int KCK, int ACC, bool DBG, bool GS, int MODEL, bool EXTRA, int PPL, int CELL>
-__global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__ McParams P)
+template <int KCK, int ACC, bool DBG, bool GS, int MODEL, bool EXTRA, int PPL, int CELL, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int kSlots = kTile * PPL;      // checkpoint slots per ring group
@@ -460,7 +488,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
     const size_t cks = (size_t)gridDim.x * W * kRing * kSlots;  // checkpoint stride
     float* const ckw = P.ckpt + (size_t)wid * kRing * kSlots;    // this warp's slots
 
-    int q_head = 0, q_count = 0, batches = 0;
+    int q_head = 0, q_count = 0, batches = first_drain(P, warp, B >> 5);
     unsigned fwd_count = 0;
     int tile = first_tile(PPL);
 
@@ -491,8 +519,7 @@ __global__ void __launch_bounds__(128, 4) adjoint_kernel(const __grid_constant__
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
             __syncwarp();
-            if (++batches % P.flush_every == 0)      // the level-2 row, recomputed (one register less)
-                drain_buckets<ACC>(P, l1, level2_row<ACC>(P), drained);
+            if (++batches >= P.flush_every && drain_buckets<ACC>(P, l1, level2_row<ACC>(P), drained)) batches = 0;
             continue;
         }
         if (!more) break;
@@ -612,7 +639,7 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
                       reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
                       reinterpret_cast<const float4*>(smem + L.bins) };
-    int q_head = 0, q_count = 0, batches = 0;
+    int q_head = 0, q_count = 0, batches = first_drain(P, warp, B >> 5);
     int tile = first_tile(PPL);
     while (true) {
         const bool more = tile < P.n_tiles;
@@ -627,7 +654,7 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
             __syncwarp();
-            if (++batches % P.flush_every == 0) drain_buckets<ACC>(P, l1, level2_row<ACC>(P), drained);
+            if (++batches >= P.flush_every && drain_buckets<ACC>(P, l1, level2_row<ACC>(P), drained)) batches = 0;
             continue;
         }
         if (!more) break;
@@ -734,7 +761,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
                       GS ? reinterpret_cast<const float2*>(smem + L.sig) : P.sig2,
                       reinterpret_cast<const float*>(smem + L.node), reinterpret_cast<const float2*>(smem + L.ab),
                       reinterpret_cast<const float4*>(smem + L.bins) };
-    int q_head = 0, q_count = 0, batches = 0;
+    int q_head = 0, q_count = 0, batches = first_drain(P, warp, B >> 5);
     int tile = first_tile(PPL);
     while (true) {
         const bool more = tile < P.n_tiles;
@@ -749,7 +776,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
             __syncwarp();
-            if (++batches % P.flush_every == 0) drain_buckets<0>(P, l1, level2_row<0>(P), drained);
+            if (++batches >= P.flush_every && drain_buckets<0>(P, l1, level2_row<0>(P), drained)) batches = 0;
             continue;
         }
         if (!more) break;
@@ -904,8 +931,26 @@ cudaError_t occupancy(K kernel, int block, size_t smem, int* bps)
 // of model MODEL and cell mode CELL: k in {4, 8}, and for model 0 with the search
 // also 16 and 32.
 template <int MODEL, bool GS, int CELL, typename F>
-cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bool extra, F&& f, int ppl = 1)
+cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bool extra, F&& f, int ppl = 1,
+                           bool wide = false)
 {
+    if (wide) {            // 512-thread blocks: the reverse sweep with checkpoints every 4 steps
+        if constexpr (GS && CELL != kCellSearch) {
+            static bool cw[5] = {};
+            if (!greeks || dbg || method != LV_ADJ_REVERSE || k != 4) return cudaErrorInvalidValue;
+            if (extra)
+                return ppl == 1 && acc == 0 ? f(adjoint_kernel<4, 0, false, true, MODEL, true, 1, CELL, true>, cw[4])
+                                            : cudaErrorInvalidValue;
+            switch (2 * ppl + acc) {
+            case 2: return f(adjoint_kernel<4, 0, false, true, MODEL, false, 1, CELL, true>, cw[0]);
+            case 3: return f(adjoint_kernel<4, 1, false, true, MODEL, false, 1, CELL, true>, cw[1]);
+            case 4: return f(adjoint_kernel<4, 0, false, true, MODEL, false, 2, CELL, true>, cw[2]);
+            case 5: return f(adjoint_kernel<4, 1, false, true, MODEL, false, 2, CELL, true>, cw[3]);
+            default: break;
+            }
+        }
+        return cudaErrorInvalidValue;
+    }
     if (ppl == 2) {        // two paths per lane: the reverse sweep (k = 4 or 8) of every reading,
                            // the main reading's tangent-ratio adjoint and second-order buckets
         if (!greeks || dbg || extra) return cudaErrorInvalidValue;
@@ -988,9 +1033,10 @@ cudaError_t launch_model_impl(const McParams& p, int grid, int block, int k, boo
     };
     const bool dbg = p.dbg_xN != nullptr;
     const int ppl = p.ppl > 1 ? p.ppl : 1;
+    const bool wide = block == kWideBlock;
     return p.grid_smem
-               ? with_kernel_gs<MODEL, true, CELL>(greeks, k, p.acc_mode, dbg, p.method, p.extra != 0, run, ppl)
-               : with_kernel_gs<MODEL, false, CELL>(greeks, k, p.acc_mode, dbg, p.method, p.extra != 0, run, ppl);
+               ? with_kernel_gs<MODEL, true, CELL>(greeks, k, p.acc_mode, dbg, p.method, p.extra != 0, run, ppl, wide)
+               : with_kernel_gs<MODEL, false, CELL>(greeks, k, p.acc_mode, dbg, p.method, p.extra != 0, run, ppl, wide);
 }
 
 template <int MODEL, int CELL>
@@ -998,8 +1044,9 @@ cudaError_t occupancy_model_impl(int block, int k, bool greeks, int acc, bool db
                                  size_t smem, int* bps, int ppl = 1)
 {
     auto occ = [&](auto kernel, bool&) { return occupancy(kernel, block, smem, bps); };
-    return gs ? with_kernel_gs<MODEL, true, CELL>(greeks, k, acc, dbg, method, extra, occ, ppl)
-              : with_kernel_gs<MODEL, false, CELL>(greeks, k, acc, dbg, method, extra, occ, ppl);
+    const bool wide = block == kWideBlock;
+    return gs ? with_kernel_gs<MODEL, true, CELL>(greeks, k, acc, dbg, method, extra, occ, ppl, wide)
+              : with_kernel_gs<MODEL, false, CELL>(greeks, k, acc, dbg, method, extra, occ, ppl, wide);
 }
 
 }  // namespace
