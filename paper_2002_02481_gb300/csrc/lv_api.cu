@@ -424,6 +424,15 @@ lv_status ensure_scratch(lv_surface_s* h, size_t bytes)
     return LV_OK;
 }
 
+// Reverse batches of a warp between its drains of the block's buckets: eight on
+// grids of a thousand cells and more. On coarse grids every path adds to the same
+// few buckets, whose binary32 sums lose more, and a drain is short: two.
+int flush_every(const lv_surface_s* h)
+{
+    const int cells = (h->Je - 1) * (h->I - 1);
+    return cells >= 1000 ? 8 : cells >= 250 ? 4 : 2;
+}
+
 struct McCall {
     double S0, r, K, T;
     int32_t n_steps;
@@ -529,7 +538,7 @@ lv_status run_mc(lv_surface_s* h, const McCall& c)
     P.l1 = reinterpret_cast<float4*>(base + p.off_l1);
     P.ckpt = reinterpret_cast<float*>(base + p.off_ckpt);
     P.n_ck = p.n_ck;
-    P.flush_every = 8;
+    P.flush_every = flush_every(h);
     P.grid_smem = p.grid_smem ? 1 : 0;
     P.dbg_xN = c.dbg_xN;
     P.dbg_V = c.dbg_V;
@@ -1525,7 +1534,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
     P.l1 = reinterpret_cast<float4*>(base + off_l1);
     P.ckpt = reinterpret_cast<float*>(base + off_ckpt);
     P.n_ck = h->adj_method == LV_ADJ_TANGENT ? 0 : (n_steps + k - 1) / k;
-    P.flush_every = 8;
+    P.flush_every = flush_every(h);
     P.grid_smem = grid_smem ? 1 : 0;
     if (h->adj_method == LV_ADJ_TANGENT) {
         P.method = LV_ADJ_TANGENT;

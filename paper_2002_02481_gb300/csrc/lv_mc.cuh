@@ -362,11 +362,11 @@ __device__ __forceinline__ float4 take4(float4* p)
 // Where a warp's count of reverse batches starts, so that the block's warps drain
 // in turn, every flush_every / W batches of the block's pace, and not all at once: a
 // bucket then holds a few hundred live paths whatever the block's size. The first
-// drain comes four batches later than that, which spares calls of two batches a
-// warp any drain (2^18 paths: 178 us, 188 with the turns from the start).
+// drain comes half a turn later than that (four batches), which spares calls of two
+// batches a warp any drain (2^18 paths: 178 us, 188 with the turns from the start).
 __device__ __forceinline__ int first_drain(const McParams& P, int warp, int W)
 {
-    return warp * P.flush_every / W - 4;
+    return warp * P.flush_every / W - P.flush_every / 2;
 }
 
 // Moves the block's binary32 buckets into its level-2 row (binary64) or the
