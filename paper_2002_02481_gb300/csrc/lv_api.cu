@@ -1,6 +1,7 @@
 // lv_api.cu -- host runtime behind the C ABI of include/lv.h: handle
 // lifetime, argument validation, launch planning, scratch management and
 // the host-output wrappers.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -661,7 +662,7 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
         cudaMalloc(&h->d_ab, sizeof(float2) * n_spot) != cudaSuccess ||
         cudaMalloc(&h->d_abl, sizeof(float2) * n_spot) != cudaSuccess ||
         cudaMalloc(&h->d_tau, 2 * sizeof(double) * n_time) != cudaSuccess ||
-        cudaMalloc(&h->d_spot64, sizeof(double) * n_spot) != cudaSuccess ||
+        cudaMalloc(&h->d_spot64, 2 * sizeof(double) * n_spot) != cudaSuccess ||
         cudaMalloc(&h->d_sig64, sizeof(double) * (size_t)n_spot * n_time) != cudaSuccess ||
         cudaMallocHost(&h->h_sig64_stage, sizeof(double) * (size_t)n_spot * n_time) != cudaSuccess ||
         cudaMalloc(&h->d_res, sizeof(double) * nres) != cudaSuccess ||
@@ -669,6 +670,12 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
         cudaMallocHost(&h->h_res, sizeof(double) * nres) != cudaSuccess) {
         cudaGetLastError();
         return bail(LV_ENOMEM, "device or pinned allocation failed");
+    }
+    // spot nodes and inverse gaps, binary64
+    std::vector<double> spot64(2 * (size_t)n_spot, 0.0);
+    for (int i = 0; i < n_spot; ++i) {
+        spot64[i] = spot_nodes[i];
+        if (i + 1 < n_spot) spot64[n_spot + i] = 1.0 / (spot_nodes[i + 1] - spot_nodes[i]);
     }
     // time nodes and inverse gaps (0 where the inverse is not a normal number)
     std::vector<double> tau(2 * (size_t)n_time, 0.0);
@@ -710,7 +717,7 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
         cudaMemcpy(h->d_ab, ab.data(), sizeof(float2) * n_spot, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_abl, abl.data(), sizeof(float2) * n_spot, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_tau, tau.data(), 2 * sizeof(double) * n_time, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(h->d_spot64, spot_nodes, sizeof(double) * n_spot, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(h->d_spot64, spot64.data(), 2 * sizeof(double) * n_spot, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_sig64, sigma, sizeof(double) * (size_t)n_spot * n_time, cudaMemcpyHostToDevice) !=
             cudaSuccess) {
         e = cudaGetLastError();
@@ -1142,6 +1149,10 @@ lv_status lv_measure_pipe_peaks(double* out_ops_per_s)
     return LV_OK;
 }
 
+// Most scratch the binary64 adjoint's tapes take: every thread of one 512-thread
+// block per SM up to 980 steps; longer calls run fewer threads.
+static constexpr size_t kTape64 = (size_t)2 << 30;
+
 lv_status lv_price_greeks_fp64_device(lv_surface_t h, double S0, double r, double K, double T,
                                       int32_t n_steps, int64_t n_paths, uint64_t seed, double* d_out)
 {
@@ -1157,15 +1168,23 @@ lv_status lv_price_greeks_fp64_device(lv_surface_t h, double S0, double r, doubl
     int bps = 0;
     LV_CUDA(lv::f64_occupancy(false, smem, &bps));
     if (bps < 1) return fail(LV_EINVAL, "binary64 launch does not fit on an SM");
-    const int64_t want = (n_paths + 127) / 128;
-    const int64_t slots = (int64_t)bps * h->num_sms;
-    const int grid = (int)(want < slots ? want : slots);
+    // one block per SM, smaller ones for calls that would leave SMs without paths; no
+    // more threads than the tapes of kTape64 bytes hold (at least one warp's)
+    const int64_t per_sm = ((n_paths + h->num_sms - 1) / h->num_sms + 31) / 32 * 32;
+    const int block = (int)std::min<int64_t>(lv::adjoint64_block(), per_sm);
+    const int64_t want = (n_paths + block - 1) / block;
+    const size_t tape = lv::adjoint64_tape_bytes(n_steps);
+    const int64_t room = std::max<int64_t>(1, (int64_t)(kTape64 / (tape * block)));
+    const int grid = (int)std::min({want, (int64_t)h->num_sms, room});
+    const size_t threads = (size_t)grid * block;
     const int row_words = 3 + h->Je * h->I;
     size_t o = scratch_header(h);
     const size_t off_part = o;
     o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
     const size_t off_chunks = o;
     o = round_up(o + sizeof(double) * (size_t)lv::finalize_chunks(grid) * row_words, 256);
+    const size_t off_tape = o;
+    o = round_up(o + tape * threads, 256);
     st = ensure_scratch(h, o);
     if (st != LV_OK) return st;
     char* base = static_cast<char*>(h->d_scratch);
@@ -1192,8 +1211,11 @@ lv_status lv_price_greeks_fp64_device(lv_surface_t h, double S0, double r, doubl
     P.partials = reinterpret_cast<double*>(base + off_part);
     P.row_words = row_words;
     P.flag = reinterpret_cast<unsigned int*>(base) + 1;    // zero; every finalize resets it
+    P.tape_hf = reinterpret_cast<double2*>(base + off_tape);
+    P.tape_u = reinterpret_cast<double*>(P.tape_hf + threads * n_steps);
+    P.tape_k = reinterpret_cast<int*>(P.tape_u + threads * n_steps);
     if (h->ev_start) LV_CUDA(cudaEventRecord(h->ev_start, h->stream));
-    LV_CUDA(lv::launch_adjoint64(P, grid, smem, h->stream));
+    LV_CUDA(lv::launch_adjoint64(P, grid, block, smem, h->stream));
     if (h->ev_end) LV_CUDA(cudaEventRecord(h->ev_end, h->stream));
     lv::FinalizeParams F{};
     F.partials = P.partials;

@@ -202,7 +202,7 @@ size_t mc_smem_bytes(int I, int J, int N, int n_bins, int block, bool greeks, bo
 // Binary64 paths (lv_fp64.cu): the full-FP64 reference adjoint and the
 // binary64 bump baseline, main reading only.
 struct F64Params {
-    const double* spot;    // [I] spot nodes
+    const double* spot;    // [I] spot nodes, then [I] inverse gaps 1 / (s_{i+1} - s_i)
     const double* sig;     // [I * J] sigma, spot-major (as the ABI takes it)
     const double* tau;     // [J] time nodes
     int I, J, N;
@@ -213,6 +213,9 @@ struct F64Params {
     double* partials;      // [gridDim.x][row_words]: adjoint 3 + Je I (time-major), bump 2 + I J
     int row_words;
     unsigned int* flag;    // adjoint: live paths with a vanishing 1 + g_n
+    double2* tape_hf;      // adjoint, [N][threads]: (h_n, 1 + g_n)
+    double* tape_u;        // [N][threads]: spot weight
+    int* tape_k;           // [N][threads]: bucket of the cell's lower node
     int n_scen, n_groups;  // bump: 3 + 2 I J scenarios in groups of bump64_slots_per_thread()
 };
 
@@ -220,7 +223,9 @@ size_t adjoint64_smem_bytes(int N);
 size_t bump64_smem_bytes(int N, int row_words);
 int bump64_slots_per_thread();
 cudaError_t f64_occupancy(bool bump, size_t smem, int* blocks_per_sm);
-cudaError_t launch_adjoint64(const F64Params& P, int grid, size_t smem, cudaStream_t s);
+cudaError_t launch_adjoint64(const F64Params& P, int grid, int block, size_t smem, cudaStream_t s);
+int adjoint64_block();                    // most threads per block
+size_t adjoint64_tape_bytes(int N);       // per thread
 cudaError_t launch_bump64(const F64Params& P, int grid, size_t smem, cudaStream_t s);
 
 // Pipe-rate probes (lv_probe.cu): out[LV_PIPE_COUNT] operations per second.
