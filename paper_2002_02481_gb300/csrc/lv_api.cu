@@ -274,6 +274,11 @@ void occ_store(const OccKey& key, int occ)
 // (2^17 121 and 134).
 constexpr int64_t kPairMinPathsPerSm = 3 * 32 * 16;
 
+// The forward-only kernel runs two paths per lane from this many paths per SM on:
+// below, one path per lane has the shorter chain (2^14 paths on the 30 x 60 grid, 156
+// steps: 30.9 and 34.5 us a call; 2^16 42.4 and 39.7; 2^20 259 and 224).
+constexpr int64_t kPricePairMinPathsPerSm = 200;
+
 // A call of at least this many paths per SM (one tile for each of its warps) runs
 // one 512-thread block per SM where it could run four of 128.
 constexpr int64_t kWideMinPathsPerSm = 32 * 16;
@@ -321,6 +326,7 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     const bool pairs = greeks && !dbg && !extra &&
                        ((vanna || h->adj_method == LV_ADJ_TANGENT) ? model == 0 : (*k == 4 || *k == 8));
     if (!pairs) ppl = 1;
+    if (!greeks) ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= kPricePairMinPathsPerSm * h->num_sms ? 2 : 1);
     if (ppl_out) *ppl_out = ppl;
     // the cell mode of any call whose cell index is bounded (base_params)
     const int cell = dbg || *k > lv::kModelMaxK ? lv::kCellSearch
@@ -363,7 +369,7 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     if (st != LV_OK) return st;
     p->smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, p->block, greeks, p->grid_smem, extra, p->ppl);
     const int warps = p->block / 32;
-    const int64_t tiles = (n_paths + lv::paths_per_tile(greeks) - 1) / lv::paths_per_tile(greeks);   // claimed by warps
+    const int64_t tiles = (n_paths + lv::paths_per_tile(greeks, p->ppl) - 1) / lv::paths_per_tile(greeks, p->ppl);   // claimed by warps
     p->n_tiles = (int)tiles;
     const int64_t want_blocks = (tiles + warps - 1) / warps;
     // The forward-only kernel's tiles all take the same time, so a last round with
@@ -1504,7 +1510,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
     st = choose_launch(h, n_steps, true, &block, &k, &bps, false, &grid_smem, false, false, &ppl, n_paths);
     if (st != LV_OK) return st;
     const int warps = block / 32;
-    const int64_t tiles = (n_paths + lv::paths_per_tile(true) - 1) / lv::paths_per_tile(true);
+    const int64_t tiles = (n_paths + lv::paths_per_tile(true, 1) - 1) / lv::paths_per_tile(true, 1);
     const int64_t want_blocks = (tiles + warps - 1) / warps;
     size_t off_part = 0, off_wrows = 0, off_l1 = 0, off_ckpt = 0;
     // two paths per lane double each block's checkpoint ring: unless the caller

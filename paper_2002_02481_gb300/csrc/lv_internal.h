@@ -265,7 +265,7 @@ LV_DECLARE_MODEL(3)
 constexpr int kModelMaxK = 8;
 constexpr int kWideBlock = 512;    // threads of a block that has an SM to itself (adjoint_kernel WIDE)
 int ring_slots_per_warp();
-int paths_per_tile(bool greeks);   // paths a warp claims at a time (adjoint / price kernel)
+int paths_per_tile(bool greeks, int ppl);   // paths of a tile (the adjoint claims ppl tiles at a time)
 
 }  // namespace lv
 

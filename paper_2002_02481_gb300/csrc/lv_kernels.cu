@@ -108,7 +108,7 @@ size_t mc_smem_bytes(int I, int J, int N, int n_bins, int block, bool greeks, bo
 }
 
 int ring_slots_per_warp() { return kRing * kTile; }
-int paths_per_tile(bool greeks) { return greeks ? kTile : kPriceTile; }
+int paths_per_tile(bool greeks, int ppl) { return greeks ? kTile : kTile * ppl; }
 
 #define LV_ROUTE(CALL, ...)                            \
     switch (model * 3 + cell) {                        \

@@ -52,8 +52,7 @@ namespace lv {
 
 namespace {
 
-constexpr int kTile = 32;      // paths per warp tile of the adjoint kernel (one per lane)
-constexpr int kPriceTile = 64; // paths per warp tile of the price kernel (two per lane)
+constexpr int kTile = 32;      // paths per warp tile (one per lane); the forward-only kernel's hold 32 PPL
 constexpr int kRing = 4;       // checkpoint slot groups of kTile per warp
 
 constexpr int kQueue = 64;     // per-warp FIFO capacity per path a lane runs in a forward tile
@@ -863,7 +862,7 @@ __global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ M
 // the same time, so the registers are held to nine blocks (2^20 paths: 245 us a
 // call against 257 with eight) and the launcher picks the blocks per SM that leave the last
 // round of tiles fullest (make_plan).
-template <int ACC, bool GS, int MODEL, int CELL>
+template <int ACC, bool GS, int MODEL, int CELL, int PPL>
 __global__ void __launch_bounds__(128, 9) price_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -877,14 +876,20 @@ __global__ void __launch_bounds__(128, 9) price_kernel(const __grid_constant__ M
                       reinterpret_cast<const float4*>(smem + L.bins) };
     const int lane = threadIdx.x & 31;
     for (int tile = first_tile(); tile < P.n_tiles; tile = claim_tile(P)) {
-        const long long rel_a = (long long)tile * kPriceTile + lane, rel_b = rel_a + 32;
+        const long long rel_a = (long long)tile * (kTile * PPL) + lane, rel_b = rel_a + 32;
         if (rel_a < P.n_paths) {
             uint32_t c1a, c2a, c1b, c2b;
             path_counter(P, rel_a, c1a, c2a);
+            float ya, yb, V, xb;
+            if constexpr (PPL == 1) {
+                ya = forward_path<CELL, 4, false, false, MODEL>(P, g, c1a, c2a, nullptr, 0, rel_a);
+                payoff<MODEL>(P, ya, V, xb);
+                acc_add<ACC>(acc[0], V);
+                acc_add<ACC>(acc[blockDim.x], V * V);
+                continue;
+            }
             path_counter(P, rel_b, c1b, c2b);
-            float ya, yb;
             forward_path2<CELL, 4, false, MODEL, true>(P, g, c1a, c2a, c1b, c2b, nullptr, nullptr, 0, ya, yb);
-            float V, xb;
             payoff<MODEL>(P, ya, V, xb);
             acc_add<ACC>(acc[0], V);
             acc_add<ACC>(acc[blockDim.x], V * V);
@@ -951,6 +956,11 @@ cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bo
         }
         return cudaErrorInvalidValue;
     }
+    if (!greeks) {
+        static bool c0[2] = {}, c1[2] = {};
+        if (ppl == 2) return acc ? f(price_kernel<1, GS, MODEL, CELL, 2>, c1[1]) : f(price_kernel<0, GS, MODEL, CELL, 2>, c0[1]);
+        return acc ? f(price_kernel<1, GS, MODEL, CELL, 1>, c1[0]) : f(price_kernel<0, GS, MODEL, CELL, 1>, c0[0]);
+    }
     if (ppl == 2) {        // two paths per lane: the reverse sweep (k = 4 or 8) of every reading,
                            // the main reading's tangent-ratio adjoint and second-order buckets
         if (!greeks || dbg || extra) return cudaErrorInvalidValue;
@@ -987,10 +997,6 @@ cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bo
         if (k == 4) return f(adjoint_kernel<4, 0, false, GS, MODEL, true, 1, CELL>, ce[0]);
         if (k == 8) return f(adjoint_kernel<8, 0, false, GS, MODEL, true, 1, CELL>, ce[1]);
         return cudaErrorInvalidValue;
-    }
-    if (!greeks) {
-        static bool c0 = false, c1 = false;
-        return acc ? f(price_kernel<1, GS, MODEL, CELL>, c1) : f(price_kernel<0, GS, MODEL, CELL>, c0);
     }
     if (method == LV_ADJ_TANGENT && !dbg) {
         static bool t0 = false, t1 = false;
