@@ -30,8 +30,8 @@ class LVPrice(torch.autograd.Function):
     @staticmethod
     def forward(ctx, S0, sigma, surface, r, K, T, n_steps, n_paths, seed):
         s0 = float(S0.detach().cpu())
-        sig = sigma.detach().to("cpu", torch.float64).numpy()
-        surface.set_sigma(np.ascontiguousarray(sig))
+        # copied in its own type and widened on the host: no conversion kernel before the copy
+        surface.set_sigma(np.ascontiguousarray(sigma.detach().cpu().to(torch.float64).numpy()))
         price, _ = surface.price(s0, r, K, T, n_steps, n_paths, seed)
         ctx.surface = surface
         ctx.state = surface.state()
@@ -39,7 +39,7 @@ class LVPrice(torch.autograd.Function):
         ctx.shape = sigma.shape
         ctx.sigma_dtype, ctx.s0_dtype = sigma.dtype, S0.dtype
         ctx.device = sigma.device
-        return torch.tensor(price, dtype=torch.float64, device=sigma.device)
+        return torch.full((), price, dtype=torch.float64, device=sigma.device)   # a fill, not a blocking copy
 
     @staticmethod
     def backward(ctx, grad_out):
@@ -51,9 +51,9 @@ class LVPrice(torch.autograd.Function):
         surface.set_stream(torch.cuda.current_stream(dev).cuda_stream)
         surface.restore(ctx.state)               # the settings this term was priced with
         surface.price_greeks_device(s0, r, K, T, n_steps, n_paths, seed, out.data_ptr())
-        g = grad_out.to(dev, torch.float64)
-        d_s0 = (g * out[lv.LV_OUT_DELTA]).to(ctx.device, ctx.s0_dtype)
-        d_sig = (g * out[lv.LV_OUT_VEGA:]).reshape(ctx.shape).to(ctx.device, ctx.sigma_dtype)
+        v = grad_out.to(dev, torch.float64) * out
+        d_s0 = v[lv.LV_OUT_DELTA].to(ctx.device, ctx.s0_dtype)
+        d_sig = v[lv.LV_OUT_VEGA:].reshape(ctx.shape).to(ctx.device, ctx.sigma_dtype)
         return d_s0, d_sig, None, None, None, None, None, None, None
 
 

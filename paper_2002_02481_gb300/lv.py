@@ -195,8 +195,10 @@ class Surface:
                     interp=self.interp, scheme=self.scheme)
 
     def restore(self, st: dict) -> None:
-        """Passes the settings of state() back to the handle."""
-        self.set_sigma(st["sigma"])
+        """Passes the settings of state() back to the handle (sigma only when its values differ:
+        an upload waits for the handle's stream)."""
+        if not np.array_equal(self.sigma, st["sigma"]):
+            self.set_sigma(st["sigma"])
         self.set_option_type(st["phi"])
         self.set_accumulation(st["accumulation"])
         self.set_adjoint_method(st["method"])
