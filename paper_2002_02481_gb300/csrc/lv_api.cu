@@ -280,7 +280,10 @@ constexpr int64_t kPairMinPathsPerSm = 3 * 32 * 16;
 constexpr int64_t kPricePairMinPathsPerSm = 200;
 
 // A call of at least this many paths per SM (one tile for each of its warps) runs
-// one 512-thread block per SM where it could run four of 128.
+// one 512-thread block per SM where it could run four or five of 128: every kernel
+// with buckets gains. 30 x 60 grid, 156 steps, 128 and 512 threads: second-order buckets
+// 2^17 paths 143 and 139 us, 500,000 363 and 346, 2^20 638 and 618, 2^22 2,280 and
+// 2,247; tangent ratio 2^17 127 and 123 us, 2^18 206 and 191, 2^20 588 and 556.
 constexpr int64_t kWideMinPathsPerSm = 32 * 16;
 
 // The head of the handle's scratch, at the same place in every launch's layout:
@@ -327,23 +330,22 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
                        ((vanna || h->adj_method == LV_ADJ_TANGENT) ? model == 0 : (*k == 4 || *k == 8));
     if (!pairs) ppl = 1;
     if (!greeks) ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= kPricePairMinPathsPerSm * h->num_sms ? 2 : 1);
-    if (ppl_out) *ppl_out = ppl;
     // the cell mode of any call whose cell index is bounded (base_params)
     const int cell = dbg || *k > lv::kModelMaxK ? lv::kCellSearch
                      : h->log_uniform           ? lv::kCellUniform
                      : h->n_bins > 0            ? lv::kCellBins
                                                 : lv::kCellSearch;
-    bool gs = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
     // one block of 512 threads per SM instead of four of 128, if the call has work
     // for its warps and the grid fits once
-    if (wide && *wide && greeks && !vanna && *block == 128 && !h->cfg_bps && *k == 4 &&
-        h->adj_method == LV_ADJ_REVERSE && cell != lv::kCellSearch && n_paths >= kWideMinPathsPerSm * h->num_sms &&
-        lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, lv::kWideBlock, greeks, true, extra, ppl) <= 200 * 1024) {
-        *block = lv::kWideBlock;
-        gs = true;
-    } else if (wide) {
-        *wide = false;
-    }
+    const bool run_wide =
+        wide && *wide && greeks && *block == 128 && !h->cfg_bps && *k == 4 && cell != lv::kCellSearch &&
+        n_paths >= kWideMinPathsPerSm * h->num_sms &&
+        lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, lv::kWideBlock, greeks, true, extra, ppl) <= 200 * 1024;
+    if (wide) *wide = run_wide;
+    if (run_wide) *block = lv::kWideBlock;
+    const bool gs =
+        run_wide || lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
+    if (ppl_out) *ppl_out = ppl;
     if (grid_smem) *grid_smem = gs;
     const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, gs, extra, ppl);
     if (smem > 200 * 1024)

@@ -616,8 +616,8 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
 // the paths with xbar_N != 0 join the warp's queue with c = xbar_N D_N. At
 // 32 queued paths (and at the end) the warp runs pass 2 (tangent_scatter)
 // on them as a full-warp batch. Buckets go through the same levels 0-3.
-template <int ACC, bool GS, int MODEL, int PPL, int CELL>
-__global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__ McParams P)
+template <int ACC, bool GS, int MODEL, int PPL, int CELL, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) tangent_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int B = blockDim.x;
@@ -738,8 +738,8 @@ __global__ void __launch_bounds__(128, 5) tangent_kernel(const __grid_constant__
 // live paths are queued and scattered in full-warp batches. Main reading,
 // binary64 level 2. Rows: price sums as usual, buckets d^2 price / (d S0 d
 // sigma_ij) summed over paths.
-template <bool GS, int PPL, int CELL>
-__global__ void __launch_bounds__(128, 5) vanna_kernel(const __grid_constant__ McParams P)
+template <bool GS, int PPL, int CELL, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) vanna_kernel(const __grid_constant__ McParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int B = blockDim.x;
@@ -939,10 +939,21 @@ template <int MODEL, bool GS, int CELL, typename F>
 cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bool extra, F&& f, int ppl = 1,
                            bool wide = false)
 {
-    if (wide) {            // 512-thread blocks: the reverse sweep with checkpoints every 4 steps
+    if (wide) {            // 512-thread blocks: every Greeks kernel, the reverse sweep with checkpoints every 4 steps
         if constexpr (GS && CELL != kCellSearch) {
-            static bool cw[5] = {};
-            if (!greeks || dbg || method != LV_ADJ_REVERSE || k != 4) return cudaErrorInvalidValue;
+            static bool cw[12] = {};
+            if (!greeks || dbg) return cudaErrorInvalidValue;
+            if constexpr (MODEL == 0) {
+                if (method == kMethodVanna && acc == 0)
+                    return ppl == 2 ? f(vanna_kernel<true, 2, CELL, true>, cw[6]) : f(vanna_kernel<true, 1, CELL, true>, cw[7]);
+                if (method == LV_ADJ_TANGENT && ppl == 2)
+                    return acc ? f(tangent_kernel<1, true, 0, 2, CELL, true>, cw[8])
+                               : f(tangent_kernel<0, true, 0, 2, CELL, true>, cw[9]);
+            }
+            if (method == LV_ADJ_TANGENT && ppl == 1)
+                return acc ? f(tangent_kernel<1, true, MODEL, 1, CELL, true>, cw[10])
+                           : f(tangent_kernel<0, true, MODEL, 1, CELL, true>, cw[11]);
+            if (method != LV_ADJ_REVERSE || k != 4) return cudaErrorInvalidValue;
             if (extra)
                 return ppl == 1 && acc == 0 ? f(adjoint_kernel<4, 0, false, true, MODEL, true, 1, CELL, true>, cw[4])
                                             : cudaErrorInvalidValue;
