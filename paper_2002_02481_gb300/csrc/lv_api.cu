@@ -274,6 +274,11 @@ void occ_store(const OccKey& key, int occ)
 // (2^17 121 and 134).
 constexpr int64_t kPairMinPathsPerSm = 3 * 32 * 16;
 
+// The kernel that also sums d V / d r and d V / d T has fewer registers to spare for
+// the second path and pairs later: 2^18 paths 185 us at one and 195 at two, 500,000 300 and
+// 321, 2^20 557 and 545, 2^22 2,012 and 1,939 (an irregular grid, 2^20: 666 and 633).
+constexpr int64_t kExtPairMinPathsPerSm = 4 * kPairMinPathsPerSm;
+
 // The forward-only kernel runs two paths per lane from this many paths per SM on:
 // below, one path per lane has the shorter chain (2^14 paths on the 30 x 60 grid, 156
 // steps: 30.9 and 34.5 us a call; 2^16 42.4 and 39.7; 2^20 259 and 224).
@@ -310,7 +315,8 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
 {
     *block = h->cfg_block ? h->cfg_block : 128;
     *k = greeks ? (h->cfg_k ? h->cfg_k : 4) : 4;
-    int ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= kPairMinPathsPerSm * h->num_sms ? 2 : 1);
+    const int64_t pair_min = extra ? kExtPairMinPathsPerSm : kPairMinPathsPerSm;
+    int ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= pair_min * h->num_sms ? 2 : 1);
     const char* cache = std::getenv("LV_TUNE_CACHE");
     if (greeks && !dbg && !h->cfg_block && !h->cfg_k && !h->cfg_ppl && cache && *cache) {
         int v[4];
@@ -328,7 +334,9 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     // the main reading's tangent-ratio adjoint and its second-order buckets (no checkpoints)
     const bool pairs = greeks && !dbg && !extra &&
                        ((vanna || h->adj_method == LV_ADJ_TANGENT) ? model == 0 : (*k == 4 || *k == 8));
-    if (!pairs) ppl = 1;
+    // the kernel that also sums d V / d r and d V / d T pairs its paths in 512-thread blocks only
+    const bool ext_pairs = extra && !dbg && *k == 4;
+    if (!pairs && !ext_pairs) ppl = 1;
     if (!greeks) ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= kPricePairMinPathsPerSm * h->num_sms ? 2 : 1);
     // the cell mode of any call whose cell index is bounded (base_params)
     const int cell = dbg || *k > lv::kModelMaxK ? lv::kCellSearch
@@ -342,7 +350,10 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
         n_paths >= kWideMinPathsPerSm * h->num_sms &&
         lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, lv::kWideBlock, greeks, true, extra, ppl) <= 200 * 1024;
     if (wide) *wide = run_wide;
-    if (run_wide) *block = lv::kWideBlock;
+    if (run_wide)
+        *block = lv::kWideBlock;
+    else if (ext_pairs)
+        ppl = 1;
     const bool gs =
         run_wide || lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
     if (ppl_out) *ppl_out = ppl;

@@ -537,14 +537,20 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
                 // this kernel (packed, it needs 82 registers: 5 blocks per SM instead of 6)
                 forward_path2<CELL, KCK, true, MODEL, (MODEL & kModelEulerS) == 0>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a,
                                                                              ckw + slot_b, cks, ya, yb);
-                float V;
-                payoff<MODEL>(P, ya, V, xa);
-                acc_add<ACC>(acc[0], V);
-                acc_add<ACC>(acc[B], V * V);
-                if (rel_b < P.n_paths) {
-                    payoff<MODEL>(P, yb, V, xb);
+                auto add = [&](float V) {
                     acc_add<ACC>(acc[0], V);
                     acc_add<ACC>(acc[B], V * V);
+                    if (EXTRA) {                   // the discount's share: -T V and -r V
+                        acc_add<ACC>(acc[3 * B], -P.Tf * V);
+                        acc_add<ACC>(acc[4 * B], -P.r_nat * V);
+                    }
+                };
+                float V;
+                payoff<MODEL>(P, ya, V, xa);
+                add(V);
+                if (rel_b < P.n_paths) {
+                    payoff<MODEL>(P, yb, V, xb);
+                    add(V);
                 }
             }
 #pragma unroll
@@ -954,9 +960,10 @@ cudaError_t with_kernel_gs(bool greeks, int k, int acc, bool dbg, int method, bo
                 return acc ? f(tangent_kernel<1, true, MODEL, 1, CELL, true>, cw[10])
                            : f(tangent_kernel<0, true, MODEL, 1, CELL, true>, cw[11]);
             if (method != LV_ADJ_REVERSE || k != 4) return cudaErrorInvalidValue;
-            if (extra)
-                return ppl == 1 && acc == 0 ? f(adjoint_kernel<4, 0, false, true, MODEL, true, 1, CELL, true>, cw[4])
-                                            : cudaErrorInvalidValue;
+            if (extra && acc == 0)
+                return ppl == 2 ? f(adjoint_kernel<4, 0, false, true, MODEL, true, 2, CELL, true>, cw[5])
+                                : f(adjoint_kernel<4, 0, false, true, MODEL, true, 1, CELL, true>, cw[4]);
+            if (extra) return cudaErrorInvalidValue;
             switch (2 * ppl + acc) {
             case 2: return f(adjoint_kernel<4, 0, false, true, MODEL, false, 1, CELL, true>, cw[0]);
             case 3: return f(adjoint_kernel<4, 1, false, true, MODEL, false, 1, CELL, true>, cw[1]);
