@@ -573,7 +573,7 @@ lv_status run_mc(lv_surface_s* h, const McCall& c)
     }
     if (c.greeks && !c.dbg_xN && !c.extra && h->adj_method == LV_ADJ_TANGENT) {
         P.method = LV_ADJ_TANGENT;
-        P.flag = P.tile_counter + 1;      // in the zeroed counter section; the finalize resets it
+        P.flag = P.tile_counter + 1;      // in the zeroed header; the last block of the launch resets it
     }
     if (c.vanna) {                        // two forward passes, binary64 level 2, the same flag
         P.method = lv::kMethodVanna;

@@ -33,7 +33,7 @@
 // unchanged (level 0); binary32 reductions (one 16-byte red per cell, resolved in
 // L2 without a retry loop) into a per-block array of the cells' corner sums in
 // global memory (level 1); every few batches a warp drains that array into
-// level 2: the block's binary64 row through binary64 reductions, or in Kahan
+// level 2: the block's binary64 row, one warp at a time under a lock, or in Kahan
 // mode a compensated binary32 row the warp owns; at the end each block adds
 // what it holds to the call's binary64 sums, and the last block to arrive writes
 // the outputs (level 3).
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
                 uint32_t c1, c2;
                 path_counter(P, rel, c1, c2);
                 float ra = 0.0f, ta = 0.0f;
-                xbar = reverse_path<CELL, KCK, MODEL, EXTRA, PPL == 2 && (MODEL & kModelEulerS) == 0>(
+                xbar = reverse_path<CELL, KCK, MODEL, EXTRA, PPL == 2>(
                     P, g, c1, c2, ckw + slot, cks, xbar, l1, &ra, &ta);
                 acc_add<ACC>(acc[2 * B], xbar);
                 if (EXTRA) {
@@ -533,9 +533,8 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
                 path_counter(P, rel_a, c1a, c2a);
                 path_counter(P, rel_b, c1b, c2b);
                 float ya, yb;
-                // packed pairs on the log-Euler readings; Euler on S keeps scalar pairs in
-                // this kernel (packed, it needs 82 registers: 5 blocks per SM instead of 6)
-                forward_path2<CELL, KCK, true, MODEL, (MODEL & kModelEulerS) == 0>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a,
+                // packed under every reading (Euler on S: 2^20 paths 514 -> 511 us, 2^22 1,850 -> 1,832)
+                forward_path2<CELL, KCK, true, MODEL, true>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a,
                                                                              ckw + slot_b, cks, ya, yb);
                 auto add = [&](float V) {
                     acc_add<ACC>(acc[0], V);
