@@ -668,7 +668,7 @@ def run_ours(args):
                        "l2": "256 MB buffer rewritten between timed steps (outside the timed region)",
                        "parallelism": f"path-range shards x{ws}" + (", one all-reduce of 3+1800 sums per step"
                                                                      if ws > 1 else "")},
-            "clocks": clocks, "gpu_launches": (3 if ws == 1 else 4) * args.steps, "roofline": roofline,
+            "clocks": clocks, "gpu_launches": (1 if ws == 1 else 2) * args.steps, "roofline": roofline,
             "pipe_peaks_gops": {k: v / 1e9 for k, v in pipe_peaks.items()} if pipe_peaks else None,
             "cpu_baseline": cpu, "accuracy": accuracy, "e2e": e2e,
             "forward_only": {"kernel_ms": statistics.mean(fwd_ms),
