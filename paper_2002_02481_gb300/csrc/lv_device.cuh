@@ -743,6 +743,7 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
                                                 float* t_acc)
 {
     constexpr bool kNeg = NEG && !EXTRA;
+    constexpr int K = KCK > 16 ? 4 : KCK;         // steps whose factors are held in registers at a time
     const int nseg = (P.N + KCK - 1) / KCK;
     int cur = -1;
     float A = 0.0f, AU = 0.0f, Bs = 0.0f, BU = 0.0f;
@@ -755,15 +756,15 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
         if (kNeg) normals4_neg((uint32_t)blk, c1, c2, P.rk, z);
         else normals4((uint32_t)blk, c1, c2, P.rk, z);
     };
-    // one segment of up to KCK steps; ALL: every step of it is below N
+    // one segment of up to K steps; ALL: every step of it is below N
     auto segment = [&](int m, float x, const float (&zf)[4], bool all) {
-        float hq[KCK], gq[KCK], uq[KCK];
-        float aq[EXTRA ? KCK : 1], tq[EXTRA ? KCK : 1];
-        int iq[KCK];
+        float hq[K], gq[K], uq[K];
+        float aq[EXTRA ? K : 1], tq[EXTRA ? K : 1];
+        int iq[K];
         float z[4] = { zf[0], zf[1], zf[2], zf[3] };
 #pragma unroll
-        for (int q = 0; q < KCK; ++q) {
-            const int n = m * KCK + q;
+        for (int q = 0; q < K; ++q) {
+            const int n = m * K + q;
             if (all || n < P.N) {
                 if (q > 0 && (q & 3) == 0) gen(n >> 2, z);
                 const int4 tb = g.tab[n];
@@ -791,8 +792,8 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
         // back through the segment: first everything that needs no decision (hq, gq
         // become the time-weighted shares a, b of sigma_bar), then the run-length sums
 #pragma unroll
-        for (int q = KCK - 1; q >= 0; --q) {
-            const int n = m * KCK + q;
+        for (int q = K - 1; q >= 0; --q) {
+            const int n = m * K + q;
             if (all || n < P.N) {
                 const int4 tb = g.tab[n];
                 iq[q] += kNodes ? tb.y : tb.x;           // the cell's bucket, or its lower node's
@@ -807,8 +808,8 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
             }
         }
 #pragma unroll
-        for (int q = KCK - 1; q >= 0; --q) {
-            if (all || m * KCK + q < P.N) {
+        for (int q = K - 1; q >= 0; --q) {
+            if (all || m * K + q < P.N) {
                 if (iq[q] != cur) {
                     if (cur >= 0) flush();
                     A = AU = Bs = BU = 0.0f;
@@ -821,6 +822,39 @@ __device__ __forceinline__ float reverse_path_f(const McParams& P, const SmemGri
             }
         }
     };
+    if constexpr (KCK > 16) {
+        // The factors of 32 steps do not fit the registers (480 bytes of spills at 128): the
+        // segment is run forward once for the state before each of its blocks of four, then
+        // its blocks are swept as above, last to first.
+        // 30 x 60 grid, 156 steps, 2^20 paths: 1,677 -> 877 us, 2^16 219 -> 118; 100 x 100,
+        // 1,260 steps, 2^20 paths 11.7 -> 7.2 ms. At 16 steps, whose factors nearly fit, it is
+        // slower (838 and 870 us; an irregular grid 1,529 and 1,754).
+        constexpr int R = KCK / 4;
+        const int nb = (P.N + 3) >> 2;
+        float x0 = ck[(size_t)(nseg - 1) * cks];
+        for (int m = nseg - 1; m >= 0; --m) {
+            const float x0n = ck[(size_t)max(m - 1, 0) * cks];
+            float xs[R], z[4], x = x0;
+            xs[0] = x;
+            const int last = min((m + 1) * R, nb) - 1;
+            for (int b = m * R; b < last; ++b) {                 // a block with another behind it is whole
+                gen(b, z);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const StepEval ev = eval_sigma<false, MODEL, CELL>(P, g, x, g.tab[4 * b + q]);
+                    x = step_state<MODEL>(P, x, ev.sigma, z[q]);
+                }
+                xs[b + 1 - m * R] = x;
+            }
+            for (int b = last; b >= m * R; --b) {
+                gen(b, z);
+                segment(b, xs[b - m * R], z, (b + 1) * 4 <= P.N);
+            }
+            x0 = x0n;
+        }
+        if (cur >= 0) flush();
+        return xbar;
+    }
     // checkpoints are read two segments ahead: one segment ahead the compiler may
     // place the load behind the recompute, which leaves its latency exposed
     float x = ck[(size_t)(nseg - 1) * cks], xn = ck[(size_t)max(nseg - 2, 0) * cks];

@@ -1,6 +1,6 @@
 // lv_kernels.cu -- the launchers that route every model and cell mode to its
-// translation unit, and the fixed-order binary64 finalize (level 3 of the
-// bucket sums).
+// translation unit, and the fixed-order binary64 finalize of the binary64
+// run's block rows (the binary32 kernels finish in their last block).
 #include "lv_mc.cuh"
 
 namespace lv {
@@ -33,8 +33,8 @@ __device__ __forceinline__ double tree_sum32(double (&v)[32])
     return v[0];
 }
 
-// A nonzero *flag (the tangent-ratio adjoint met a vanishing 1 + g_n) makes
-// every sum, and so every output, NaN.
+// A nonzero *flag (a vanishing 1 + g_n on a live path) makes every sum, and so
+// every output, NaN.
 __global__ void __launch_bounds__(32) reduce_rows_kernel(const double* __restrict__ partials, int G, int row_words,
                                                           const unsigned int* flag, double* __restrict__ chunks)
 {
