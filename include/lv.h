@@ -158,8 +158,8 @@ lv_status lv_set_scheme(lv_surface_t h, int32_t scheme);
 /* Launch shape: threads per block (32..128, multiple of 32), checkpoint
  * interval k of the reverse sweep (4, 8, 16 or 32 steps) and resident
  * blocks per SM; 0 keeps the tuned or default value. With 128 threads, k = 4
- * and no blocks_per_sm, a reverse sweep of at least 512 paths per SM runs the
- * SM's four blocks as one of 512 threads that share the staged grid. Results do
+ * and no blocks_per_sm, a call with buckets of at least 512 paths per SM runs
+ * one block of 512 threads per SM, whose warps share the staged grid. Results do
  * not depend on it beyond reduction-order rounding. */
 lv_status lv_set_launch(lv_surface_t h, int32_t block, int32_t k, int32_t blocks_per_sm);
 
@@ -171,7 +171,9 @@ lv_status lv_set_launch(lv_surface_t h, int32_t block, int32_t k, int32_t blocks
  * (233,472 on 152 SMs), one and a half pairs of tiles per resident warp, else 1.
  * Two paths per lane exist for the reverse sweep with checkpoints every 4
  * or 8 steps (every reading of the scheme), the main reading's tangent-ratio
- * adjoint and its second-order buckets; elsewhere the call runs one. The results do not
+ * adjoint and its second-order buckets; rho and d price / d T take two from
+ * 6,144 paths per SM on, where the SM runs one 512-thread block. Elsewhere the
+ * call runs one. The results do not
  * depend on it beyond reduction-order rounding.
  * lv_get_paths_per_lane reads back the value the next call with n_steps steps
  * and n_paths >= 1 paths will use. */
