@@ -417,7 +417,7 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     if (greeks && !extra && !vanna && h->acc_mode == LV_ACC_KAHAN)
         o = round_up(o + sizeof(double) * total_warps * nIJ, 256);
     p->off_l1 = o;
-    if (greeks) o = round_up(o + sizeof(float4) * (size_t)p->grid * (h->Je - 1) * (h->I - 1), 256);
+    if (greeks) o = round_up(o + sizeof(float4) * (size_t)p->grid * lv::bucket_arrays(warps) * (h->Je - 1) * (h->I - 1), 256);
     p->off_ckpt = o;
     o = round_up(o + sizeof(float) * (size_t)p->n_ck * total_warps * lv::ring_slots_per_warp() * p->ppl, 256);
     p->total = o;
@@ -444,14 +444,15 @@ lv_status ensure_scratch(lv_surface_s* h, size_t bytes)
     return LV_OK;
 }
 
-// Reverse batches of a warp between its drains of the block's buckets: eight on
-// grids of a thousand cells and more. On coarse grids every path adds to the same
-// few buckets, whose binary32 sums lose more, and a drain is short: two.
-int flush_every(const lv_surface_s* h)
-{
-    const int cells = (h->Je - 1) * (h->I - 1);
-    return cells >= 1000 ? 8 : cells >= 250 ? 4 : 2;
-}
+// Reverse batches of a warp between its drains of the buckets it shares with three
+// others: eight, and two on coarse grids, where every path adds to the same few
+// buckets and their binary32 sums lose more. Relative 2-norm against binary64 sums of
+// the same flushes, 104 steps, drains every eight / two batches (and node buckets of
+// 128-thread blocks): second-order buckets, 5 x 2 nodes, 2^20 paths 1.2e-7 / 4.0e-8
+// (7.8e-8), 12 x 2, 2^19 8.8e-8 / 4.0e-8 (5.1e-8); from 20 x 10 nodes on eight is enough
+// (4.8e-8, 7.3e-8). Two costs 1 % on 20 x 10 nodes at 2^22 paths (1,373 -> 1,393 us) and 4 %
+// on 30 x 60 at 2^20 (411 -> 428 us). The line lies between 171 cells (20 x 10) and 361.
+int flush_every(const lv_surface_s* h) { return (h->Je - 1) * (h->I - 1) < 250 ? 2 : 8; }
 
 struct McCall {
     double S0, r, K, T;
@@ -1497,7 +1498,7 @@ size_t static_plan_bytes(const lv_surface_s* h, int grid, int block, int k, int 
     *off_part = o;   o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
     *off_wrows = o;                                               // per-warp rows: Kahan mode only
     if (h->acc_mode == LV_ACC_KAHAN) o = round_up(o + sizeof(double) * warps * nIJ, 256);
-    *off_l1 = o;     o = round_up(o + sizeof(float4) * (size_t)grid * (h->Je - 1) * (h->I - 1), 256);
+    *off_l1 = o;     o = round_up(o + sizeof(float4) * (size_t)grid * lv::bucket_arrays(block / 32) * (h->Je - 1) * (h->I - 1), 256);
     *off_ckpt = o;   o = round_up(o + sizeof(float) * n_ck * warps * lv::ring_slots_per_warp() * ppl, 256);
     return o;
 }

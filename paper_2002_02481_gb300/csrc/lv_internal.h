@@ -52,6 +52,10 @@ __host__ __device__ inline bool index_bounded(bool on_s, int n_steps, double x0,
     return fabs(cell_scale) * y + fabs(cell_shift) < 4194304.0 - 2.0;     // false for infinities and NaN
 }
 
+// Arrays of level-1 buckets of a block: one for every kBucketWarps warps (lv_mc.cuh warp_buckets).
+constexpr int kBucketWarps = 4;
+__host__ __device__ inline int bucket_arrays(int warps) { return (warps + kBucketWarps - 1) / kBucketWarps; }
+
 // Everything a Monte Carlo launch reads, passed by value as a
 // __grid_constant__ kernel parameter.
 struct McParams {
@@ -105,7 +109,7 @@ struct McParams {
     double* partials;      // [gridDim.x][row_words] per-block binary64 rows
     int row_words;         // 3 + Je * I (adjoint) or 3 (price only)
     double* warp_rows;     // [gridDim.x * warps][Je * I] per-warp level-2 rows
-    float4* l1;            // [gridDim.x][(Je - 1) (I - 1)] per-block level-1 buckets: the corner sums of a cell
+    float4* l1;            // [gridDim.x][bucket_arrays][(Je - 1) (I - 1)] level-1 buckets: the corner sums of a cell
                            // (nodes (i, j), (i+1, j), (i, j+1), (i+1, j+1))
     float* ckpt;           // [n_ck][gridDim.x * warps * ring_slots_per_warp() * ppl] checkpoints of x
     int n_ck;

@@ -31,9 +31,9 @@
 //
 // Bucket accumulation: run-length sums in registers while the cell is
 // unchanged (level 0); binary32 reductions (one 16-byte red per cell, resolved in
-// L2 without a retry loop) into a per-block array of the cells' corner sums in
-// global memory (level 1); every few batches a warp drains that array into
-// level 2: the block's binary64 row, one warp at a time under a lock, or in Kahan
+// L2 without a retry loop) into an array of the cells' corner sums in global
+// memory, one for every four warps of a block (level 1); every few batches a warp
+// drains its array into level 2: the block's binary64 row, one warp at a time under a lock, or in Kahan
 // mode a compensated binary32 row the warp owns; at the end each block adds
 // what it holds to the call's binary64 sums, and the last block to arrive writes
 // the outputs (level 3).
@@ -170,6 +170,22 @@ __device__ __forceinline__ void stage_grid(const McParams& P, unsigned char* sme
 // Cells with a level-1 bucket: (Je - 1) rows of I - 1.
 __host__ __device__ inline int n_cells(const McParams& P) { return (P.Je - 1) * (P.I - 1); }
 
+// The level-1 buckets of a warp. A block has one array for every kBucketWarps of its
+// warps, dealt out in turn, so that the warps of one array drain at different times
+// (first_drain). With one array for all sixteen warps of a 512-thread block, a
+// bucket held four times the paths in binary32 that a 128-thread block's does, and its
+// rounding grew with them (relative 2-norm against binary64 sums of the same
+// flushes, 104 steps: vegas on 5 x 2 nodes, 2^17 paths 3.9e-8, with four arrays
+// 1.2e-8, in 128-thread blocks of node buckets 1.5e-8; second-order buckets on 20 x 10
+// nodes 1.1e-7, 4.4e-8 and 7.6e-8). The four arrays' clears and folds take 3-7 us a
+// call on 30 x 60 nodes: 2^18 paths 177 -> 183 us, 2^20 509 -> 517, 2^22 1,827 -> 1,842;
+// 100 x 100 nodes, 1,260 steps, 2^22 paths 15.38 -> 15.53 ms.
+__device__ __forceinline__ float4* warp_buckets(const McParams& P, int warp, int W)
+{
+    const int G = bucket_arrays(W);
+    return P.l1 + (size_t)(blockIdx.x * G + warp % G) * n_cells(P);
+}
+
 // The level-2 row of the warp: binary64 mode drains into the block's own row
 // with binary64 reductions; Kahan pairs cannot be updated atomically, so each
 // warp owns one.
@@ -187,7 +203,7 @@ template <int ACC>
 __device__ __forceinline__ void clear_buckets(const McParams& P, int* drained)
 {
     const int nIJ = P.Je * P.I, B = blockDim.x, W = B >> 5, tid = threadIdx.x;
-    const int nc = n_cells(P);
+    const int nc = bucket_arrays(W) * n_cells(P);
     float4* l1 = P.l1 + (size_t)blockIdx.x * nc;
     for (int e = tid; e < nc; e += B) l1[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (ACC == 1) {
@@ -215,45 +231,51 @@ __device__ __forceinline__ void add_scalars(const AccSlot* acc0, int n, double* 
     }
 }
 
-// Adds what the block's buckets hold to the call's sums: per node the corners of
-// the up to four cells around it that were not drained yet and, if some warp
-// drained, the block's binary64 row (in Kahan mode its warps' rows). Four nodes
-// of a thread are in flight at a time. The four corners are added in binary32
-// (binary64 adds run at 1.7 per SM and cycle): each is a sum of a quarter of the
-// contributions that a node's own bucket would hold.
+// Adds what the block's buckets hold to the call's sums: per node and array the
+// corners of the up to four cells around it that were not drained yet and, if some
+// warp drained, the block's binary64 row (in Kahan mode its warps' rows). Four nodes
+// of a thread are in flight at a time. The four corners of one array are added in
+// binary32 (binary64 adds run at 1.7 per SM and cycle: with every corner widened
+// first, 2^14 paths on 20 x 10 nodes take 24.4 us a call instead of 23.3 and 2^18 on 30 x 60
+// 197 instead of 184, at the same rounding), each a sum of a quarter of the
+// contributions that a node's own bucket would hold; everything after in binary64.
 template <int ACC>
-__device__ __forceinline__ void fold_buckets(const McParams& P, const float4* l1, const double* row, bool drained)
+__device__ __forceinline__ void fold_buckets(const McParams& P, const double* row, bool drained)
 {
     constexpr int kFly = 4;
-    const int I = P.I, nIJ = P.Je * I, B = blockDim.x, W = B >> 5;
-    const float* c = reinterpret_cast<const float*>(l1);         // reductions are resolved in L2: __ldcg
+    const int I = P.I, nIJ = P.Je * I, B = blockDim.x, W = B >> 5, G = bucket_arrays(W), nc = n_cells(P);
+    const float* c0 = reinterpret_cast<const float*>(P.l1 + (size_t)blockIdx.x * G * nc);
     const double* rows0 = P.warp_rows + (size_t)blockIdx.x * W * nIJ;
     for (int e0 = threadIdx.x; e0 < nIJ; e0 += kFly * B) {
-        float f[kFly][4];
-        double d[kFly];
+        double s[kFly];
 #pragma unroll
-        for (int q = 0; q < kFly; ++q) {
-            const int e = e0 + q * B, j = e / I, i = e - j * I;
-            const int cell = 4 * (j * (I - 1) + i);              // the cell whose lower corner is node e
-            const bool in = e < nIJ, up = j < P.Je - 1, rt = i < I - 1;
-            f[q][0] = in && up && rt ? __ldcg(c + cell) : 0.0f;
-            f[q][1] = in && up && i > 0 ? __ldcg(c + cell - 4 + 1) : 0.0f;
-            f[q][2] = in && j > 0 && rt ? __ldcg(c + cell - 4 * (I - 1) + 2) : 0.0f;
-            f[q][3] = in && j > 0 && i > 0 ? __ldcg(c + cell - 4 * (I - 1) - 4 + 3) : 0.0f;
-            d[q] = ACC != 1 && drained && in ? __ldcg(row + 3 + e) : 0.0;
+        for (int q = 0; q < kFly; ++q) s[q] = ACC != 1 && drained && e0 + q * B < nIJ ? __ldcg(row + 3 + e0 + q * B) : 0.0;
+        for (int a = 0; a < G; ++a) {
+            const float* c = c0 + 4 * (size_t)(a * nc);                  // reductions are resolved in L2: __ldcg
+            float f[kFly][4];
+#pragma unroll
+            for (int q = 0; q < kFly; ++q) {
+                const int e = e0 + q * B, j = e / I, i = e - j * I;
+                const int cell = 4 * (j * (I - 1) + i);                  // the cell whose lower corner is node e
+                const bool in = e < nIJ, up = j < P.Je - 1, rt = i < I - 1;
+                f[q][0] = in && up && rt ? __ldcg(c + cell) : 0.0f;
+                f[q][1] = in && up && i > 0 ? __ldcg(c + cell - 4 + 1) : 0.0f;
+                f[q][2] = in && j > 0 && rt ? __ldcg(c + cell - 4 * (I - 1) + 2) : 0.0f;
+                f[q][3] = in && j > 0 && i > 0 ? __ldcg(c + cell - 4 * (I - 1) - 4 + 3) : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < kFly; ++q) s[q] += (double)((f[q][0] + f[q][1]) + (f[q][2] + f[q][3]));
         }
 #pragma unroll
         for (int q = 0; q < kFly; ++q) {
             const int e = e0 + q * B;
-            double s = (double)((f[q][0] + f[q][1]) + (f[q][2] + f[q][3]));
-            if (ACC != 1 && drained) s += d[q];
             if (ACC == 1 && drained && e < nIJ) {
                 for (int w = 0; w < W; ++w) {
                     const float2 k = reinterpret_cast<const float2*>(rows0 + (size_t)w * nIJ)[e];
-                    s += (double)k.x - (double)k.y;
+                    s[q] += (double)k.x - (double)k.y;
                 }
             }
-            if (s != 0.0) atomicAdd(&P.sums[3 + e], s);
+            if (s[q] != 0.0) atomicAdd(&P.sums[3 + e], s[q]);
         }
     }
 }
@@ -359,8 +381,8 @@ __device__ __forceinline__ float4 take4(float4* p)
 }
 
 // Where a warp's count of reverse batches starts, so that the block's warps drain
-// in turn, every flush_every / W batches of the block's pace, and not all at once: a
-// bucket then holds a few hundred live paths whatever the block's size. The first
+// in turn, every flush_every / W batches of the block's pace, and not all at once: the
+// four warps of an array then leave a few hundred live paths in a bucket. The first
 // drain comes half a turn later than that (four batches), which spares calls of two
 // batches a warp any drain (2^18 paths: 178 us, 188 with the turns from the start).
 __device__ __forceinline__ int first_drain(const McParams& P, int warp, int W)
@@ -471,7 +493,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
         clear_buckets<ACC>(P, drained);
         for (int k = 0; k < (EXTRA ? 5 : 3); ++k) acc[k * B] = AccSlot{0.0, 0.0f, 0.0f};
     });
-    float4* l1 = P.l1 + (size_t)blockIdx.x * n_cells(P);    // this block\'s level-1 buckets
+    float4* const l1 = warp_buckets(P, warp, B >> 5);
     // the three FIFO arrays of all warps are contiguous from L.qslot (each
     // W * kQcap words): one base per warp, the others at fixed offsets, which
     // keeps two registers free for the packed forward pass
@@ -609,7 +631,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
     }
 
     __syncthreads();                           // after it nothing adds to this block's buckets
-    fold_buckets<ACC>(P, l1, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    fold_buckets<ACC>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
     add_scalars<ACC>(acc0, 3, P.sums);
     if (EXTRA) add_scalars<ACC>(acc0 + 3 * B, 2, P.sums + 3 + nIJ);
     finish_call<true, EXTRA>(P);
@@ -636,7 +658,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) tangent
         clear_buckets<ACC>(P, drained);
         for (int k = 0; k < 3; ++k) acc[k * B] = AccSlot{0.0, 0.0f, 0.0f};
     });
-    float4* l1 = P.l1 + (size_t)blockIdx.x * n_cells(P);    // this block\'s level-1 buckets
+    float4* const l1 = warp_buckets(P, warp, B >> 5);
     int* q_rel = reinterpret_cast<int*>(smem + L.qrel) + warp * kQcap;
     float* q_c = reinterpret_cast<float*>(smem + L.qxb) + warp * kQcap;
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
@@ -732,7 +754,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) tangent
         tile = claim_tile(P, PPL);
     }
     __syncthreads();
-    fold_buckets<ACC>(P, l1, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    fold_buckets<ACC>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
     add_scalars<ACC>(acc0, 3, P.sums);
     finish_call<true>(P);
 }
@@ -758,7 +780,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) vanna_k
         clear_buckets<0>(P, drained);
         for (int k = 0; k < 3; ++k) acc[k * B] = AccSlot{0.0, 0.0f, 0.0f};
     });
-    float4* l1 = P.l1 + (size_t)blockIdx.x * n_cells(P);    // this block\'s level-1 buckets
+    float4* const l1 = warp_buckets(P, warp, B >> 5);
     int* q_rel = reinterpret_cast<int*>(smem + L.qrel) + warp * kQcap;
     float* q_c = reinterpret_cast<float*>(smem + L.qxb) + warp * kQcap;
     const SmemGrid g{ reinterpret_cast<const int4*>(smem + L.tab),
@@ -854,7 +876,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) vanna_k
         tile = claim_tile(P, PPL);
     }
     __syncthreads();
-    fold_buckets<0>(P, l1, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    fold_buckets<0>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
     add_scalars<0>(acc0, 3, P.sums);
     finish_call<true>(P);
 }
