@@ -152,7 +152,9 @@ void pack_sigma(lv_surface_s* h, const double* sigma, float2* dst)
 // [y_0, y_{I-1}], narrow enough that a bin widened by a tenth on either side
 // holds at most two nodes (a width of 1.5 times the smallest gap: 1.8 gaps
 // against the two that three nodes span). Entry b: the largest cell whose node
-// is at or below the widened bin, and the next two nodes. The tenth covers the
+// is at or below the widened bin, and the next two nodes of the cells after it
+// (NaN past the last cell: a spot is at or above none of them, an infinite one
+// included). The tenth covers the
 // binary32 rounding of y, of the bin index and of S = 2^y (about 5e-7 of y
 // together) while a bin is at least 4e-5 wide. Grids that need more than
 // kMaxBins bins, or narrower ones, keep the binary search.
@@ -179,8 +181,8 @@ std::vector<float4> spot_bins(const std::vector<double>& spot, float* scale, flo
         while (base + 1 <= I - 2 && y[base + 1] <= lo) ++base;
         float4 t;
         std::memcpy(&t.x, &base, sizeof(float));
-        t.y = base + 1 <= I - 2 ? (float)spot[base + 1] : INFINITY;
-        t.z = base + 2 <= I - 2 ? (float)spot[base + 2] : INFINITY;
+        t.y = base + 1 <= I - 2 ? (float)spot[base + 1] : NAN;
+        t.z = base + 2 <= I - 2 ? (float)spot[base + 2] : NAN;
         t.w = 0.0f;
         bins[b] = t;
     }

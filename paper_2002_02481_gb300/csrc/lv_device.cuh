@@ -290,8 +290,8 @@ __device__ __forceinline__ int clamp_floor(float shifted, int hi)
     return __viaddmin_s32_relu(__float_as_int(shifted), -kFloorBits, hi);
 }
 
-// Cell of S in bin b: the bin's first cell and the two nodes after it (infinite
-// past the last cell).
+// Cell of S in bin b: the bin's first cell and the two nodes after it (NaN past
+// the last cell, which no spot passes: 2^y is infinite from y = 128 on).
 __device__ __forceinline__ int bin_cell(const SmemGrid& g, int b, float S)
 {
     const float4 t = g.bins[b];
