@@ -47,10 +47,13 @@ OPT = W.Option(S0=2e38, r=0.01, K=2e36, T=0.85, n_steps=16, n_paths=4096, seed=5
 
 
 def _close(got, ref, tol):
-    assert np.isfinite(ref[0]) and ref[0] > 0.0 and abs(got[0] - ref[0]) <= 1e-11 * ref[0]
-    assert abs(got[1] - ref[1]) <= 1e-11 * abs(ref[1])
-    top = np.max(np.abs(ref[2]))
-    assert np.isfinite(top) and top > 0.0 and np.max(np.abs(got[2] - ref[2])) <= tol * top
+    """The same values; where the search's are no numbers (on 100 x 100 rough nodes adjoints
+    overflow: S d sigma / d S is above 10), the same ones are none."""
+    assert np.isfinite(ref[0]) and ref[0] > 0.0
+    np.testing.assert_allclose(got[:2], ref[:2], rtol=1e-11)
+    top = np.max(np.abs(ref[2][np.isfinite(ref[2])]))
+    assert top > 0.0
+    np.testing.assert_allclose(got[2], ref[2], rtol=0.0, atol=tol * top)
 
 
 @pytest.mark.parametrize("n_spot,n_time", [(5, 10), (20, 10), (100, 100)])
