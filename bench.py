@@ -245,7 +245,7 @@ def other_workloads(lib, dev, ev0, ev1):
         ms = time_call(lambda: S.price_greeks_device(opt.S0, opt.r, opt.K, opt.T, opt.n_steps, opt.n_paths,
                                                       opt.seed, d.data_ptr()), ev0, ev1)
         res[name] = {"adjoint_kernel_ms": ms, "path_steps_per_s": opt.n_paths * opt.n_steps / (ms * 1e-3),
-                     "launch": list(S.get_launch(opt.n_steps, True)),
+                     "launch": list(S.get_call_launch(opt.n_steps, opt.n_paths, True)),
                      "paths_per_lane": S.get_paths_per_lane(opt.n_steps, opt.n_paths)}
         S.close()
 
@@ -441,7 +441,7 @@ def large_record(lib, dev, peaks, n_sm, mhz, reps=3):
         ms = statistics.median(step_ms)
         res[f"k={k}"] = {"ms_per_step": ms, "value": ps / (ms * 1e-3), "kernel_ms": statistics.median(kern_ms)}
     S.set_launch(128, 4, 0)
-    res["launch"] = {"block": 128, "k": 4, "paths_per_lane": S.get_paths_per_lane(opt.n_steps, opt.n_paths),
+    res["launch"] = {"block": S.get_call_launch(opt.n_steps, opt.n_paths, True)[0], "k": 4, "paths_per_lane": S.get_paths_per_lane(opt.n_steps, opt.n_paths),
                      "source": "tuned (k=4 fastest of 4, 8, 16; two paths per lane, packed pairs); k=32 is the "
                                "configured interval, reported beside it"}
     res["value"] = res["k=4"]["value"]
@@ -623,7 +623,7 @@ def run_ours(args):
             pipe_peaks = None
         live = live_fraction(S, opt)
         roofline = roofline_block(kern, P * opt.n_steps, live, pipe_peaks, mhz, n_sm, profiled_record())
-        blk, kk, bps = S.get_launch(opt.n_steps, True)
+        blk, kk, bps = S.get_call_launch(opt.n_steps, P, True)
         ppl = S.get_paths_per_lane(opt.n_steps, opt.n_paths)
         roofline["kernel"] = (f"adjoint_kernel<k={kk},binary64 level 2,{ppl} path(s) per lane> "
                               f"(block {blk}, {bps} blocks/SM)")

@@ -197,11 +197,19 @@ lv_status lv_set_kernel_events(lv_surface_t h, void* start_event, void* end_even
 lv_status lv_tune(lv_surface_t h, double S0, double r, double K, double T, int32_t n_steps, int64_t n_paths,
                   uint64_t seed, int32_t* out_block, int32_t* out_k, double* out_ms);
 
-/* Read back the launch shape the next call will use for (n_steps, greeks);
- * blocks_per_sm is that of a call large enough for two paths per lane by
- * default (lv_get_paths_per_lane). */
+/* Read back the launch shape of the handle's settings for (n_steps, greeks):
+ * the one of calls too small for 512-thread blocks (lv_set_launch), with the
+ * blocks_per_sm of two paths per lane (lv_get_paths_per_lane).
+ * lv_get_call_launch reads back the shape that lv_price_greeks (greeks != 0)
+ * or lv_price (greeks = 0) runs for n_paths paths, 1 <= n_paths < 2^31: 512
+ * threads and one block per SM where it runs that, and for lv_price the blocks
+ * per SM that leave its last round fullest. (A call whose paths can leave any
+ * binary32 range of the grid's cell index, at volatilities in the hundreds,
+ * stays at the former.) */
 lv_status lv_get_launch(lv_surface_t h, int32_t n_steps, int32_t greeks,
                         int32_t* block, int32_t* k, int32_t* blocks_per_sm);
+lv_status lv_get_call_launch(lv_surface_t h, int32_t n_steps, int64_t n_paths, int32_t greeks,
+                             int32_t* block, int32_t* k, int32_t* blocks_per_sm);
 
 /* lv_price -- Monte Carlo price of the option over paths [0, n_paths)
  * (Sec. IV-C: the mean of the discounted payoff).

@@ -896,6 +896,23 @@ lv_status lv_get_launch(lv_surface_t h, int32_t n_steps, int32_t greeks, int32_t
     return LV_OK;
 }
 
+lv_status lv_get_call_launch(lv_surface_t h, int32_t n_steps, int64_t n_paths, int32_t greeks, int32_t* block,
+                             int32_t* k, int32_t* blocks_per_sm)
+{
+    if (!h || !block || !k || !blocks_per_sm) return fail(LV_EINVAL, "NULL argument");
+    if (n_steps < 1 || n_steps > LV_MAX_STEPS) return fail(LV_EINVAL, "n_steps out of range");
+    if (n_paths < 1 || n_paths > 0x7fffffffLL) return fail(LV_EINVAL, "n_paths must be in [1, 2^31 - 1]");
+    DeviceGuard g(h->device);
+    Plan p;
+    p.wide = true;                        // a call whose cell index is bounded
+    lv_status st = make_plan(h, n_steps, n_paths, greeks != 0, false, &p);
+    if (st != LV_OK) return st;
+    *block = p.block;
+    *k = p.k;
+    *blocks_per_sm = p.bps;
+    return LV_OK;
+}
+
 lv_status lv_price(lv_surface_t h, double S0, double r, double K, double T, int32_t n_steps,
                    int64_t n_paths, uint64_t seed, double* out_price, double* out_stderr)
 {

@@ -79,6 +79,7 @@ def _declare(lib: ctypes.CDLL) -> ctypes.CDLL:
         "lv_get_paths_per_lane": [vp, i32, i64, c.POINTER(i32)],
         "lv_tune": [vp, d, d, d, d, i32, i64, u64, c.POINTER(i32), c.POINTER(i32), c.POINTER(d)],
         "lv_get_launch": [vp, i32, i32, c.POINTER(i32), c.POINTER(i32), c.POINTER(i32)],
+        "lv_get_call_launch": [vp, i32, i64, i32, c.POINTER(i32), c.POINTER(i32), c.POINTER(i32)],
         "lv_price": [vp, d, d, d, d, i32, i64, u64, dp, dp],
         "lv_price_greeks": [vp, d, d, d, d, i32, i64, u64, dp, dp, dp],
         "lv_price_greeks_device": [vp, d, d, d, d, i32, i64, u64, vp],
@@ -251,6 +252,13 @@ class Surface:
         b, k, s = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
         _check(self.lib, self.lib.lv_get_launch(self.h, int(n_steps), int(greeks), ctypes.byref(b),
                                                 ctypes.byref(k), ctypes.byref(s)), "lv_get_launch")
+        return b.value, k.value, s.value
+
+    def get_call_launch(self, n_steps: int, n_paths: int, greeks: bool = True):
+        """(block, k, blocks per SM) of a call of n_paths paths."""
+        b, k, s = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
+        _check(self.lib, self.lib.lv_get_call_launch(self.h, int(n_steps), int(n_paths), int(greeks), ctypes.byref(b),
+                                                     ctypes.byref(k), ctypes.byref(s)), "lv_get_call_launch")
         return b.value, k.value, s.value
 
     # pricing
