@@ -427,7 +427,7 @@ def large_record(lib, dev, peaks, n_sm, mhz, reps=3):
                        "price+delta+10000 vegas", "metric": METRIC, "unit": "path-steps/s"}
     ps = opt.n_paths * opt.n_steps
     for k in (4, 32):
-        S.set_launch(128, k, 0)
+        S.set_launch(0, k, 0)
         S.set_kernel_events(ev[2].cuda_event, ev[3].cuda_event)
         S.price_greeks_device(opt.S0, opt.r, opt.K, opt.T, opt.n_steps, opt.n_paths, opt.seed, d.data_ptr())
         step_ms, kern_ms = [], []
@@ -440,7 +440,7 @@ def large_record(lib, dev, peaks, n_sm, mhz, reps=3):
             kern_ms.append(ev[2].elapsed_time(ev[3]))
         ms = statistics.median(step_ms)
         res[f"k={k}"] = {"ms_per_step": ms, "value": ps / (ms * 1e-3), "kernel_ms": statistics.median(kern_ms)}
-    S.set_launch(128, 4, 0)
+    S.set_launch(0, 4, 0)
     res["launch"] = {"block": S.get_call_launch(opt.n_steps, opt.n_paths, True)[0], "k": 4, "paths_per_lane": S.get_paths_per_lane(opt.n_steps, opt.n_paths),
                      "source": "tuned (k=4 fastest of 4, 8, 16; two paths per lane, packed pairs); k=32 is the "
                                "configured interval, reported beside it"}
@@ -754,7 +754,7 @@ def path_sweep():
     S = lv.Surface.from_workload(surf, lib)
     stream = torch.cuda.current_stream()
     S.set_stream(stream.cuda_stream)
-    S.set_launch(128, 4, 0)
+    S.set_launch(0, 4, 0)
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     ev0.record(stream)
     ev1.record(stream)
@@ -762,7 +762,7 @@ def path_sweep():
     S.set_kernel_events(ev0.cuda_event, ev1.cuda_event)
     d = torch.zeros(3 + S.IJ, dtype=torch.float64, device="cuda")
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
-    out = {"study": "path sweep", "workload": "30x60 grid, 156 steps", "launch": [128, 4], "points": []}
+    out = {"study": "path sweep", "workload": "30x60 grid, 156 steps", "points": []}
     for lg in range(16, 25):
         P = 1 << lg
         ts = []
@@ -773,7 +773,8 @@ def path_sweep():
             if rep:
                 ts.append(ev0.elapsed_time(ev1))
         ms = statistics.median(ts)
-        out["points"].append({"paths": P, "kernel_ms": ms, "path_steps_per_s": P * opt.n_steps / (ms * 1e-3)})
+        out["points"].append({"paths": P, "kernel_ms": ms, "path_steps_per_s": P * opt.n_steps / (ms * 1e-3),
+                              "launch": list(S.get_call_launch(opt.n_steps, P, True))})
     S.close()
     print(json.dumps(out), flush=True)
     return 0

@@ -157,10 +157,10 @@ lv_status lv_set_scheme(lv_surface_t h, int32_t scheme);
 
 /* Launch shape: threads per block (32..128, multiple of 32), checkpoint
  * interval k of the reverse sweep (4, 8, 16 or 32 steps) and resident
- * blocks per SM; 0 keeps the tuned or default value. With 128 threads, k = 4
- * and no blocks_per_sm, a call with buckets of at least 512 paths per SM runs
- * one block of 512 threads per SM, whose warps share the staged grid. Results do
- * not depend on it beyond reduction-order rounding. */
+ * blocks per SM; 0 keeps the tuned or default value. With block and
+ * blocks_per_sm 0 and k = 4, a call with buckets of at least 512 paths per SM
+ * runs one block of 512 threads per SM, whose warps share the staged grid.
+ * Results do not depend on it beyond reduction-order rounding. */
 lv_status lv_set_launch(lv_surface_t h, int32_t block, int32_t k, int32_t blocks_per_sm);
 
 /* Paths per lane of the adjoint's forward tiles: 1, or 2 (each lane runs two
@@ -187,13 +187,15 @@ lv_status lv_get_paths_per_lane(lv_surface_t h, int32_t n_steps, int64_t n_paths
 lv_status lv_set_kernel_events(lv_surface_t h, void* start_event, void* end_event);
 
 /* Autotuner for one option: times lv_price_greeks_device on this problem
- * over launch shapes (threads per block 64 / 128, checkpoint interval 4 / 8
- * / 16, and for the main reading's reverse sweep at k = 4 and 8 one or two
- * paths per lane), keeps the fastest in the handle (as lv_set_launch and
- * lv_set_paths_per_lane would) and appends it (block, k, paths per lane) to
- * the file named by LV_TUNE_CACHE when that variable is set; later handles
- * with the same grid size and step count then start from it. Runs the
- * problem about 40 times. Outputs may be NULL. */
+ * over launch shapes (threads per block 64 / 128, and the default's 512 for a
+ * call of at least 512 paths per SM, checkpoint interval 4 / 8 / 16, and at
+ * k = 4 and 8 one or two paths per lane where they exist), keeps the fastest
+ * in the handle (as lv_set_launch and lv_set_paths_per_lane would) and appends
+ * it (block, k, paths per lane, 1 if 512 threads were among them) to the file
+ * named by LV_TUNE_CACHE when that variable is set; later handles with the
+ * same grid size and step count then start from it. out_block is the block
+ * lv_set_launch takes: 0 when the default's 512 threads were fastest. Runs the
+ * problem about 50 times. Outputs may be NULL. */
 lv_status lv_tune(lv_surface_t h, double S0, double r, double K, double T, int32_t n_steps, int64_t n_paths,
                   uint64_t seed, int32_t* out_block, int32_t* out_k, double* out_ms);
 

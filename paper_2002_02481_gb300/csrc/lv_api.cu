@@ -319,14 +319,17 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     *k = greeks ? (h->cfg_k ? h->cfg_k : 4) : 4;
     const int64_t pair_min = extra ? kExtPairMinPathsPerSm : kPairMinPathsPerSm;
     int ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= pair_min * h->num_sms ? 2 : 1);
+    bool own_block = h->cfg_block != 0;              // the block was asked for, or tuned
     const char* cache = std::getenv("LV_TUNE_CACHE");
     if (greeks && !dbg && !h->cfg_block && !h->cfg_k && !h->cfg_ppl && cache && *cache) {
         int v[4];
-        if (lv::tune_cache_lookup(adjoint_tune_key(h, n_steps), v) && v[0] >= 32 && v[0] <= 128 &&
+        // block 0: the default, 512 threads where it takes them; a line that ends in 1 was timed against those
+        if (lv::tune_cache_lookup(adjoint_tune_key(h, n_steps), v) && v[0] >= 0 && v[0] <= 128 &&
             v[0] % 32 == 0 && (v[1] == 4 || v[1] == 8 || v[1] == 16 || v[1] == 32)) {
-            *block = v[0];
+            *block = v[0] ? v[0] : 128;
             *k = v[1];
             ppl = v[2] == 2 ? 2 : 1;
+            own_block = v[0] != 0 && v[3] == 1;
         }
     }
     if (dbg) *k = 4;
@@ -346,9 +349,9 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
                      : h->n_bins > 0            ? lv::kCellBins
                                                 : lv::kCellSearch;
     // one block of 512 threads per SM instead of four of 128, if the call has work
-    // for its warps and the grid fits once
+    // for its warps, the grid fits once and no block was asked for
     const bool run_wide =
-        wide && *wide && greeks && *block == 128 && !h->cfg_bps && *k == 4 && cell != lv::kCellSearch &&
+        wide && *wide && greeks && *block == 128 && !own_block && !h->cfg_bps && *k == 4 && cell != lv::kCellSearch &&
         n_paths >= kWideMinPathsPerSm * h->num_sms &&
         lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, lv::kWideBlock, greeks, true, extra, ppl) <= 200 * 1024;
     if (wide) *wide = run_wide;
@@ -1045,11 +1048,13 @@ lv_status lv_tune(lv_surface_t h, double S0, double r, double K, double T, int32
     if (n_paths < 1 || n_paths > 0x7fffffffLL) return fail(LV_EINVAL, "n_paths must be in [1, 2^31 - 1]");
     DeviceGuard g(h->device);
     if (!g.ok) return fail(LV_ECUDA, "cannot select the handle's device");
-    const int blocks[] = {64, 128};
+    // 0: the default, which runs 512-thread blocks for a call of this size (else it is 128)
+    const bool wide = n_paths >= kWideMinPathsPerSm * h->num_sms;
+    const int blocks[] = {0, 64, 128};
     const int ks[] = {4, 8, 16};
     const int keep_b = h->cfg_block, keep_k = h->cfg_k, keep_s = h->cfg_bps, keep_p = h->cfg_ppl;
-    // two paths per lane exist for the main reading's reverse sweep at k = 4 and 8
-    // the reverse sweep under every reading, the tangent-ratio adjoint under the main one
+    // two paths per lane at k = 4 and 8: the reverse sweep under every reading, the
+    // tangent-ratio adjoint under the main one
     const bool ppl2 = h->adj_method == LV_ADJ_REVERSE || (h->interp == LV_INTERP_S && h->scheme == LV_SCHEME_LOG);
     cudaEvent_t e0, e1;
     LV_CUDA(cudaEventCreate(&e0));
@@ -1059,6 +1064,7 @@ lv_status lv_tune(lv_surface_t h, double S0, double r, double K, double T, int32
     for (int blk : blocks)
         for (int k : ks)
         for (int ppl = 1; ppl <= ((ppl2 && k <= 8) ? 2 : 1); ++ppl) {
+            if (blk == 0 && (!wide || k != 4)) continue;
             h->cfg_block = blk;
             h->cfg_k = k;
             h->cfg_bps = 0;
@@ -1091,11 +1097,12 @@ lv_status lv_tune(lv_surface_t h, double S0, double r, double K, double T, int32
         h->cfg_ppl = keep_p;
         return fail(LV_EINTERNAL, "no launch shape ran");
     }
-    h->cfg_block = bb;
+    // 128 threads that were not timed against 512 leave larger calls their choice
+    h->cfg_block = bb == 128 && !wide ? 0 : bb;
     h->cfg_k = bk;
     h->cfg_bps = 0;
     h->cfg_ppl = bp;
-    const int v[4] = {bb, bk, bp, 0};
+    const int v[4] = {bb, bk, bp, wide ? 1 : 0};
     lv::tune_cache_append(adjoint_tune_key(h, n_steps), v, best);
     if (out_block) *out_block = bb;
     if (out_k) *out_k = bk;

@@ -81,3 +81,46 @@ def test_wide_blocks_on_a_fine_grid_against_the_oracle(lib):
     assert s.get_call_launch(opt.n_steps, opt.n_paths, True) == (512, 4, 1)
     s.close()
     G.full_parity(surf, opt, lib, label="100x100 grid, wide blocks")
+
+
+def test_a_block_asked_for_is_kept(lib):
+    """128 threads are 128 threads at any path count; 0 is the default's choice."""
+    s = _surface(lib, "greeks")
+    n = 2048 * _sms()
+    assert s.get_call_launch(52, n)[0] == 512
+    s.set_launch(128, 4, 0)
+    assert s.get_call_launch(52, n)[0] == 128
+    s.set_launch(0, 4, 0)
+    assert s.get_call_launch(52, n)[0] == 512
+    s.close()
+
+
+def test_tuner_times_the_default_too(lib, tmp_path, monkeypatch):
+    """What it keeps is what a later call and a later handle run, and what lv_set_launch makes of its block."""
+    monkeypatch.setenv("LV_TUNE_CACHE", str(tmp_path / "tune.txt"))
+    n = 2048 * _sms()
+    s = _surface(lib, "greeks")
+    block, k, _ = s.tune(100.0, 0.01, 100.0, 3.0, 52, n, 3)
+    assert block in (0, 64, 128)
+    shape = s.get_call_launch(52, n)
+    assert shape[0] == (block or 512) and shape[1] == k
+    for keep in (lambda t: None, lambda t: (t.set_launch(block, k, 0), t.set_paths_per_lane(s.get_paths_per_lane(52, n)))):
+        t = _surface(lib, "greeks")
+        keep(t)
+        assert t.get_call_launch(52, n) == shape
+        t.close()
+    s.close()
+
+
+@pytest.mark.parametrize("line,block", [("128 4 2 0", 512), ("128 4 2 1", 128), ("0 4 2 1", 512), ("64 4 2 0", 64)])
+def test_lines_of_a_tune_cache(line, block, lib, tmp_path, monkeypatch):
+    """A line of 128 threads that was not timed against 512 leaves a large call the default."""
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("LV_TUNE_CACHE", str(cache))
+    s = _surface(lib, "greeks")
+    s.tune(100.0, 0.01, 100.0, 3.0, 52, 4096, 3)
+    cache.write_text(cache.read_text().split()[0] + f" {line} 1.0\n")
+    t = _surface(lib, "greeks")
+    assert t.get_call_launch(52, 2048 * _sms())[0] == block
+    s.close()
+    t.close()
