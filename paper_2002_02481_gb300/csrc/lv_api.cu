@@ -395,8 +395,9 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     // the one with the least rounds x warps. 2^20 paths on 152 SMs are 2.99 rounds
     // at nine blocks, 3.37 at eight and 3.85 at seven: 245, 257 and 257 us a call.
     if (!greeks && !h->cfg_bps) {
+        const int occ = p->bps;
         int64_t best = 0;
-        for (int b = p->bps; 2 * b >= p->bps && b >= 1; --b) {
+        for (int b = occ; 2 * b >= occ; --b) {
             const int64_t warps_all = (int64_t)b * h->num_sms * warps;
             const int64_t cost = (tiles + warps_all - 1) / warps_all * b;
             if (best == 0 || cost < best) {

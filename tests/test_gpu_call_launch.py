@@ -124,3 +124,12 @@ def test_lines_of_a_tune_cache(line, block, lib, tmp_path, monkeypatch):
     assert t.get_call_launch(52, 2048 * _sms())[0] == block
     s.close()
     t.close()
+
+
+def test_forward_only_calls_keep_half_the_resident_blocks(lib):
+    """The search for the blocks per SM that leave the last round fullest stays in the upper half."""
+    s = _surface(lib, "price")
+    occ = s.get_launch(52, False)[2]
+    for tiles in [*range(1, 400, 7), *range(1216, 60000, 97), 32268, 34049, 56048]:
+        assert 2 * s.get_call_launch(52, 64 * tiles, False)[2] >= occ, tiles
+    s.close()
