@@ -35,6 +35,7 @@ struct lv_book_s {
     std::vector<int64_t> offsets;           // [n + 1]
     std::vector<int64_t> risk_offsets;      // [n_surfaces + 1]
     int max_I = 0, max_J = 0, max_Je = 0, max_N = 0, max_IJe = 0, max_IJ = 0, max_bins = 0;
+    int bins = 0;                            // bins staged per surface: max_bins, or 0 where they leave no room
     int64_t total_paths = 0;
     // device tables and grids
     lv::BookSurf* d_surfs = nullptr;
@@ -144,10 +145,16 @@ lv_status configure(lv_book_s* b, int block, int k, int item_tiles, int ppl)
 {
     drop_graph(b);
     LV_BCUDA(cudaStreamSynchronize(b->stream));
-    const size_t smem = lv::book_smem_bytes(b->max_I, b->max_Je, b->max_N, b->max_bins, block, ppl);
-    if (smem > 200 * 1024) return set_error(LV_EINVAL, "book grids too large for shared memory");
+    // grids that leave no room for the bins search for their cells
+    int bins = b->max_bins;
+    size_t smem = lv::book_smem_bytes(b->max_I, b->max_Je, b->max_N, bins, block, ppl);
+    if (smem > lv::kBookSmem && bins > 0) {
+        bins = 0;
+        smem = lv::book_smem_bytes(b->max_I, b->max_Je, b->max_N, 0, block, ppl);
+    }
+    if (smem > lv::kBookSmem) return set_error(LV_EINVAL, "book grids too large for shared memory");
     int bps = 0;
-    LV_BCUDA(lv::book_occupancy(block, k, ppl, b->max_bins > 0, smem, &bps));
+    LV_BCUDA(lv::book_occupancy(block, k, ppl, bins > 0, smem, &bps));
     if (bps < 1) return set_error(LV_EINVAL, "book launch shape does not fit on an SM");
     std::vector<lv::BookItem> items = make_items(b->insts, item_tiles);
     cudaFree(b->d_items);
@@ -184,6 +191,7 @@ lv_status configure(lv_book_s* b, int block, int k, int item_tiles, int ppl)
     b->k = k;
     b->item_tiles = item_tiles;
     b->ppl = ppl;
+    b->bins = bins;
     b->grid = grid;
     b->smem = smem;
     return LV_OK;
@@ -211,7 +219,7 @@ lv::BookParams params(const lv_book_s* b)
     P.max_Je = b->max_Je;
     P.max_N = b->max_N;
     P.max_IJe = b->max_IJe;
-    P.max_bins = b->max_bins;
+    P.max_bins = b->bins;
     return P;
 }
 
@@ -300,7 +308,7 @@ lv_status run_captured(lv_book_s* b, double S0, double r, uint64_t seed, bool ri
     double* d_res = risk ? b->d_rout : b->d_out;
     double* h_res = risk ? b->h_rout : b->h_out;
     if (!exec) {
-        LV_BCUDA(lv::book_prepare(b->k, b->ppl, b->max_bins > 0));
+        LV_BCUDA(lv::book_prepare(b->k, b->ppl, b->bins > 0));
         cudaGraph_t graph = nullptr;
         LV_BCUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
         lv_status cst = LV_OK;

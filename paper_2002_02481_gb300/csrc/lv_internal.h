@@ -327,6 +327,9 @@ struct BookParams {
 
 // ppl: paths per lane of the forward tiles (1 or 2); the FIFO and the
 // checkpoint ring (book_ring_slots_per_warp() * ppl per warp) grow with it.
+// Most shared memory of a book's block: 200 KB, and beside them the 144 bytes of the
+// option's Philox round keys and output scales, which took no room from the grids.
+constexpr size_t kBookSmem = 200 * 1024 + 144;
 size_t book_smem_bytes(int maxI, int maxJe, int maxN, int max_bins, int block, int ppl);
 int book_ring_slots_per_warp();
 cudaError_t book_prepare(int k, int ppl, bool bins);
