@@ -1216,23 +1216,28 @@ lv_status lv_price_greeks_fp64_device(lv_surface_t h, double S0, double r, doubl
     LV_CUDA(lv::f64_occupancy(false, smem, &bps));
     if (bps < 1) return fail(LV_EINVAL, "binary64 launch does not fit on an SM");
     // one block per SM, smaller ones for calls that would leave SMs without paths; no
-    // more threads than the tapes of kTape64 bytes hold (at least one warp's)
+    // more threads than the tapes of kTape64 bytes hold, and half as many again while the
+    // device has no room for those (at least one warp's)
     const int64_t per_sm = ((n_paths + h->num_sms - 1) / h->num_sms + 31) / 32 * 32;
-    const int block = (int)std::min<int64_t>(lv::adjoint64_block(), per_sm);
-    const int64_t want = (n_paths + block - 1) / block;
     const size_t tape = lv::adjoint64_tape_bytes(n_steps);
-    const int64_t room = std::max<int64_t>(1, (int64_t)(kTape64 / (tape * block)));
-    const int grid = (int)std::min({want, (int64_t)h->num_sms, room});
-    const size_t threads = (size_t)grid * block;
     const int row_words = 3 + h->Je * h->I;
-    size_t o = scratch_header(h);
-    const size_t off_part = o;
-    o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
-    const size_t off_chunks = o;
-    o = round_up(o + sizeof(double) * (size_t)lv::finalize_chunks(grid) * row_words, 256);
-    const size_t off_tape = o;
-    o = round_up(o + tape * threads, 256);
-    st = ensure_scratch(h, o);
+    int block = 0, grid = 0;
+    size_t threads = 0, off_part = 0, off_chunks = 0, off_tape = 0;
+    for (int64_t most = (int64_t)(kTape64 / tape);; most = (int64_t)threads / 2) {
+        most = std::max<int64_t>(32, most / 32 * 32);
+        block = (int)std::min({(int64_t)lv::adjoint64_block(), per_sm, most});
+        grid = (int)std::min({(n_paths + block - 1) / block, (int64_t)h->num_sms, most / block});
+        threads = (size_t)grid * block;
+        size_t o = scratch_header(h);
+        off_part = o;
+        o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
+        off_chunks = o;
+        o = round_up(o + sizeof(double) * (size_t)lv::finalize_chunks(grid) * row_words, 256);
+        off_tape = o;
+        o = round_up(o + tape * threads, 256);
+        st = ensure_scratch(h, o);
+        if (st != LV_ENOMEM || threads <= 32) break;
+    }
     if (st != LV_OK) return st;
     char* base = static_cast<char*>(h->d_scratch);
     const double dt = T / (double)n_steps;
