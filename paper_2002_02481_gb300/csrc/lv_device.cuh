@@ -242,9 +242,12 @@ __device__ __forceinline__ int4 step_time(const McParams& P, const double* tau, 
         }
         j = lo;
         const double a = t - tau[j], b = tau[j + 1] - tau[j], r = rtau[j];
-        double q = a * r;
-        q = fma(fma(-q, b, a), r, q);
-        if (r == 0.0) q = a / b;
+        double q = 1.0;                     // past the cell, where a / b may overflow (b > 0: bits again)
+        if (__double_as_longlong(a) < __double_as_longlong(b)) {
+            q = a * r;
+            q = fma(fma(-q, b, a), r, q);
+            if (r == 0.0) q = a / b;
+        }
         v = fminf(fmaxf((float)q, 0.0f), 1.0f);
     }
     const int vb = __float_as_int(v);
