@@ -697,11 +697,13 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
         cudaGetLastError();
         return bail(LV_ENOMEM, "device or pinned allocation failed");
     }
-    // spot nodes and inverse gaps, binary64
+    // spot nodes and inverse gaps (0 where the inverse overflows), binary64
     std::vector<double> spot64(2 * (size_t)n_spot, 0.0);
     for (int i = 0; i < n_spot; ++i) {
         spot64[i] = spot_nodes[i];
-        if (i + 1 < n_spot) spot64[n_spot + i] = 1.0 / (spot_nodes[i + 1] - spot_nodes[i]);
+        const double inv = i + 1 < n_spot ? 1.0 / (spot_nodes[i + 1] - spot_nodes[i]) : 0.0;
+        spot64[n_spot + i] = std::isfinite(inv) ? inv : 0.0;
+        h->gap_divide = h->gap_divide || !std::isfinite(inv);
     }
     // time nodes and inverse gaps (0 where the inverse is not a normal number)
     std::vector<double> tau(2 * (size_t)n_time, 0.0);
@@ -1262,6 +1264,7 @@ lv_status lv_price_greeks_fp64_device(lv_surface_t h, double S0, double r, doubl
     P.n_paths = n_paths;
     P.partials = reinterpret_cast<double*>(base + off_part);
     P.row_words = row_words;
+    P.divide = h->gap_divide;
     P.flag = reinterpret_cast<unsigned int*>(base) + 1;    // zero; every finalize resets it
     P.tape_hf = reinterpret_cast<double2*>(base + off_tape);
     P.tape_u = reinterpret_cast<double*>(P.tape_hf + threads * n_steps);

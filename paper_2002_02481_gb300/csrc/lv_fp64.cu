@@ -264,6 +264,9 @@ __host__ __device__ inline Smem64 smem64(int N)
 // 50 operations per path-step where two forward passes with CUDA's functions, two
 // divisions a step and a search by binary64 comparisons took 226. 30 x 60 grid, 156
 // steps, 2^16 paths: 5.08 -> 1.05 ms; 2^18 paths 26.8 -> 4.7 ms.
+// DIVIDE: some spot gap has no inverse (below 2^-1024), and its cell divides. Both in
+// one kernel took 1,097 us instead of 1,056 at 2^16 paths.
+template <bool DIVIDE>
 __global__ void __launch_bounds__(kBlock64, 1) adjoint64_kernel(const __grid_constant__ F64Params P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -284,7 +287,7 @@ __global__ void __launch_bounds__(kBlock64, 1) adjoint64_kernel(const __grid_con
     const Tab64 T{ reinterpret_cast<const double*>(smem + L.ex), reinterpret_cast<const double2*>(smem + L.lg),
                    reinterpret_cast<const double2*>(smem + L.cs), reinterpret_cast<const double*>(smem + L.eln2) };
     const PhiloxKeys K = philox_keys(P.k0, P.k1);
-    const double* gap = P.spot + P.I;                // 1 / (s_{i+1} - s_i)
+    const double* gap = P.spot + P.I;                // 1 / (s_{i+1} - s_i), 0 where that overflows
     const size_t threads = (size_t)gridDim.x * B;    // tape stride of a step
     const size_t col0 = (size_t)blockIdx.x * B;
     double2* const t_hf = P.tape_hf + col0;
@@ -316,6 +319,7 @@ __global__ void __launch_bounds__(kBlock64, 1) adjoint64_kernel(const __grid_con
                 }
                 const double inv = __ldg(gap + i);
                 double u = (S - __ldg(P.spot + i)) * inv;
+                if (DIVIDE && inv == 0.0) u = (S - __ldg(P.spot + i)) / (__ldg(P.spot + i + 1) - __ldg(P.spot + i));
                 if (__double_as_longlong(u) < 0) u = 0.0;                                   // below the grid
                 else if (__double_as_longlong(u) > 0x3ff0000000000000ll) u = 1.0;           // above it
                 const double* q = P.sig + i * J + jr.x;
@@ -332,7 +336,9 @@ __global__ void __launch_bounds__(kBlock64, 1) adjoint64_kernel(const __grid_con
                 }
                 const bool inside = sb >= s_first && sb <= s_last;
                 const double h = fma(P.sqdt, z[n & 3], -sigma * P.dt);
-                const double f = inside ? fma(h, S * (ds * inv), 1.0) : 1.0;
+                double slope = ds * inv;
+                if (DIVIDE && inv == 0.0) slope = ds / (__ldg(P.spot + i + 1) - __ldg(P.spot + i));
+                const double f = inside ? fma(h, S * slope, 1.0) : 1.0;
                 tiny = tiny || (__double2hiint(f) & 0x7fffffff) < 0x3d700000;               // |f| < 2^-40
                 const size_t at = (size_t)n * threads + tid;
                 t_hf[at] = make_double2(h, f);
@@ -502,7 +508,7 @@ int bump64_slots_per_thread() { return kM64; }
 
 cudaError_t f64_occupancy(bool bump, size_t smem, int* bps)
 {
-    const void* k = bump ? (const void*)bump64_kernel : (const void*)adjoint64_kernel;
+    const void* k = bump ? (const void*)bump64_kernel : (const void*)adjoint64_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k, bump ? 128 : kBlock64, smem);
@@ -510,9 +516,10 @@ cudaError_t f64_occupancy(bool bump, size_t smem, int* bps)
 
 cudaError_t launch_adjoint64(const F64Params& P, int grid, int block, size_t smem, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(adjoint64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    const auto kernel = P.divide ? adjoint64_kernel<true> : adjoint64_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
-    adjoint64_kernel<<<grid, block, smem, s>>>(P);
+    kernel<<<grid, block, smem, s>>>(P);
     return cudaGetLastError();
 }
 

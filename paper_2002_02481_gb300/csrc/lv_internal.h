@@ -206,7 +206,8 @@ size_t mc_smem_bytes(int I, int J, int N, int n_bins, int block, bool greeks, bo
 // Binary64 paths (lv_fp64.cu): the full-FP64 reference adjoint and the
 // binary64 bump baseline, main reading only.
 struct F64Params {
-    const double* spot;    // [I] spot nodes, then [I] inverse gaps 1 / (s_{i+1} - s_i)
+    const double* spot;    // [I] spot nodes, then [I] inverse gaps 1 / (s_{i+1} - s_i) (0 where infinite)
+    bool divide;           // adjoint: some inverse gap is 0
     const double* sig;     // [I * J] sigma, spot-major (as the ABI takes it)
     const double* tau;     // [J] time nodes
     int I, J, N;
@@ -370,7 +371,8 @@ struct lv_surface_s {
     float2* d_ab = nullptr;
     float2* d_abl = nullptr;         // [I] cell coefficients of the ln-S weight, in y = log2 S
     double* d_tau = nullptr;
-    double* d_spot64 = nullptr;      // [I] spot nodes, binary64 (the binary64 kernels)
+    double* d_spot64 = nullptr;      // [I] spot nodes, then [I] inverse gaps, binary64 (the binary64 kernels)
+    bool gap_divide = false;         // some gap has no inverse (0 in d_spot64)
     double* d_sig64 = nullptr;       // [I * J] sigma, binary64, spot-major
     double* h_sig64_stage = nullptr; // pinned staging for its uploads
     bool sig64_stale = false;        // d_sig64 behind h_sig64_stage: uploaded by the binary64 calls
