@@ -51,9 +51,10 @@ class LVPrice(torch.autograd.Function):
         surface.set_stream(torch.cuda.current_stream(dev).cuda_stream)
         surface.restore(ctx.state)               # the settings this term was priced with
         surface.price_greeks_device(s0, r, K, T, n_steps, n_paths, seed, out.data_ptr())
-        v = grad_out.to(dev, torch.float64) * out
-        d_s0 = v[lv.LV_OUT_DELTA].to(ctx.device, ctx.s0_dtype)
-        d_sig = v[lv.LV_OUT_VEGA:].reshape(ctx.shape).to(ctx.device, ctx.sigma_dtype)
+        g = grad_out.to(dev, torch.float64)
+        # two products: each gradient is a tensor of its own, not a view of one buffer
+        d_s0 = (g * out[lv.LV_OUT_DELTA]).to(ctx.device, ctx.s0_dtype)
+        d_sig = (g * out[lv.LV_OUT_VEGA:]).reshape(ctx.shape).to(ctx.device, ctx.sigma_dtype)
         return d_s0, d_sig, None, None, None, None, None, None, None
 
 
