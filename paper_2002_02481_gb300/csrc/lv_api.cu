@@ -530,9 +530,10 @@ lv::McParams base_params(const lv_surface_s* h, const McCall& c, int k)
     P.acc_mode = h->acc_mode;
     P.method = LV_ADJ_REVERSE;
     P.bins = h->d_bins;
-    // checkpoints every 16 or 32 steps and the diagnostics kernel search
-    if (k > 0 && k <= lv::kModelMaxK && !c.dbg_xN)
-        lv::choose_cell_mode(P, h->sig_max, h->n_bins, h->bin_scale, h->bin_shift);
+    // the diagnostics kernel searches; the sweeps with checkpoints every 16 or 32 steps have
+    // one loop, which reads the bins where the call has them
+    if (k > 0 && !c.dbg_xN) lv::choose_cell_mode(P, h->sig_max, h->n_bins, h->bin_scale, h->bin_shift);
+    if (k > lv::kModelMaxK) P.cell_mode = lv::kCellSearch;
     return P;
 }
 

@@ -308,8 +308,9 @@ __device__ __forceinline__ int bin_cell(const SmemGrid& g, int b, float S)
 //    where the clamped weight gives the same value);
 //  - kCellBins: on other grids from a table of equal bins in y, at most two
 //    nodes in each: the bin's first cell plus two comparisons with S;
-//  - kCellSearch: the same index from a conversion, or a binary search over the
-//    nodes.
+//  - kCellSearch: the same index from a conversion, from the bins, or from a binary
+//    search over the nodes, as the call says (the sweeps with checkpoints every 16 or 32
+//    steps, which are compiled once, and calls whose index has no bound).
 template <int CELL = kCellSearch>
 __device__ __forceinline__ int spot_cell(const McParams& P, const SmemGrid& g, float y, float S)
 {
@@ -321,6 +322,8 @@ __device__ __forceinline__ int spot_cell(const McParams& P, const SmemGrid& g, f
         const int i = __float2int_rd(fmaf(y, P.cell_scale, P.cell_shift));
         return min(max(i, 0), P.I - 2);
     }
+    if (P.n_bins > 0)
+        return bin_cell(g, clamp_floor(__fadd_rd(fmaf(y, P.cell_scale, P.cell_shift), kFloorShift), P.n_bins - 1), S);
     int lo = 0, hi = P.I - 2;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
