@@ -152,16 +152,20 @@ void pack_sigma(lv_surface_s* h, const double* sigma, float2* dst)
 // [y_0, y_{I-1}], narrow enough that a bin widened by a tenth on either side
 // holds at most two nodes (a width of 1.5 times the smallest gap: 1.8 gaps
 // against the two that three nodes span). Entry b: the largest cell whose node
-// is at or below the widened bin, and the next two nodes of the cells after it
+// is at or below the widened bin, the next two nodes of the cells after it
 // (NaN past the last cell: a spot is at or above none of them, an infinite one
-// included). The tenth covers the
+// included) and the last cell whose node is in it. The tenth covers the
 // binary32 rounding of y, of the bin index and of S = 2^y (about 5e-7 of y
 // together) while a bin is at least 4e-5 wide. Grids that need more than
-// kMaxBins bins, or narrower ones, keep the binary search.
+// kMaxBins bins, or narrower ones, have as many as they may (*two is false)
+// and search among a bin's cells: the loops that search over all cells are slower at the
+// four blocks per SM that the straight-line loops want (60 x 80 nodes, gaps from 1 to 1,600 of
+// the smallest, 156 steps: 2^20 paths 1,839 us, 1,404 at the six blocks of before, 1,274 with the
+// bins; 33 paths 175, 170 and 127).
 constexpr int kMaxBins = 512;
 constexpr double kMinBinWidth = 4e-5;
 
-std::vector<float4> spot_bins(const std::vector<double>& spot, float* scale, float* shift)
+std::vector<float4> spot_bins(const std::vector<double>& spot, float* scale, float* shift, bool* two)
 {
     const int I = (int)spot.size();
     std::vector<double> y(I);
@@ -171,19 +175,22 @@ std::vector<float4> spot_bins(const std::vector<double>& spot, float* scale, flo
     const double range = y[I - 1] - y[0];
     const double want = std::ceil(range / (1.5 * gap));
     const double ymax = std::fmax(4.0, std::fmax(std::fabs(y[0]), std::fabs(y[I - 1])));
-    if (!(want >= 1.0) || want > kMaxBins || range / want < kMinBinWidth * ymax) return {};
-    const int n = (int)want;
+    *two = want >= 1.0 && want <= kMaxBins && range / want >= kMinBinWidth * ymax;
+    const double most = std::fmin((double)kMaxBins, std::floor(range / (kMinBinWidth * ymax)));
+    if (!*two && !(most >= 2.0)) return {};
+    const int n = (int)(*two ? want : most);
     const double w = range / n;
     std::vector<float4> bins(n);
-    int base = 0;
+    int base = 0, last = 0;
     for (int b = 0; b < n; ++b) {
         const double lo = y[0] + b * w - 0.1 * w;
+        while (last + 1 <= I - 2 && (b == n - 1 || y[last + 1] <= lo + 1.2 * w)) ++last;
         while (base + 1 <= I - 2 && y[base + 1] <= lo) ++base;
         float4 t;
         std::memcpy(&t.x, &base, sizeof(float));
         t.y = base + 1 <= I - 2 ? (float)spot[base + 1] : NAN;
         t.z = base + 2 <= I - 2 ? (float)spot[base + 2] : NAN;
-        t.w = 0.0f;
+        std::memcpy(&t.w, &last, sizeof(float));
         bins[b] = t;
     }
     *scale = (float)(1.0 / w);
@@ -309,12 +316,20 @@ void bind_header(lv::McParams& P, char* base)
     P.sums = reinterpret_cast<double*>(base + kOffSums);
 }
 
+// Bins a call stages: those of the surface, or none beside a time table and nodes that
+// leave them no room (thousands of spot nodes and steps).
+int staged_bins(const lv_surface_s* h, int32_t n_steps, bool greeks, bool extra)
+{
+    return lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, 128, greeks, false, extra, 2) <= 200 * 1024 ? h->n_bins : 0;
+}
+
 // n_paths < 0: a call large enough for two paths per lane. `wide`: whether the call
 // may run 512-thread blocks (its cells need no search), set to whether it does.
 lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* block, int* k, int* bps,
                         bool dbg = false, bool* grid_smem = nullptr, bool extra = false, bool vanna = false,
                         int* ppl_out = nullptr, int64_t n_paths = -1, bool* wide = nullptr)
 {
+    const int bins = staged_bins(h, n_steps, greeks, extra);
     *block = h->cfg_block ? h->cfg_block : 128;
     *k = greeks ? (h->cfg_k ? h->cfg_k : 4) : 4;
     const int64_t pair_min = extra ? kExtPairMinPathsPerSm : kPairMinPathsPerSm;
@@ -346,24 +361,24 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     // the cell mode of any call whose cell index is bounded (base_params)
     const int cell = dbg || *k > lv::kModelMaxK ? lv::kCellSearch
                      : h->log_uniform           ? lv::kCellUniform
-                     : h->n_bins > 0            ? lv::kCellBins
+                     : bins > 0 && h->bins_two  ? lv::kCellBins
                                                 : lv::kCellSearch;
     // one block of 512 threads per SM instead of four of 128, if the call has work
     // for its warps, the grid fits once and no block was asked for
     const bool run_wide =
         wide && *wide && greeks && *block == 128 && !own_block && !h->cfg_bps && *k == 4 && cell != lv::kCellSearch &&
         n_paths >= kWideMinPathsPerSm * h->num_sms &&
-        lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, lv::kWideBlock, greeks, true, extra, ppl) <= 200 * 1024;
+        lv::mc_smem_bytes(h->I, h->J, n_steps, bins, lv::kWideBlock, greeks, true, extra, ppl) <= 200 * 1024;
     if (wide) *wide = run_wide;
     if (run_wide)
         *block = lv::kWideBlock;
     else if (ext_pairs)
         ppl = 1;
     const bool gs =
-        run_wide || lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
+        run_wide || lv::mc_smem_bytes(h->I, h->J, n_steps, bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
     if (ppl_out) *ppl_out = ppl;
     if (grid_smem) *grid_smem = gs;
-    const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, *block, greeks, gs, extra, ppl);
+    const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, bins, *block, greeks, gs, extra, ppl);
     if (smem > 200 * 1024)
         return fail(LV_EINVAL, "time table does not fit in shared memory (" + std::to_string(smem) + " bytes)");
     int occ = 0;
@@ -382,10 +397,11 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
 lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool greeks, bool dbg, Plan* p,
                     bool extra = false, bool vanna = false)
 {
+    const bool straight = p->wide;        // the call's cells need no search
     lv_status st = choose_launch(h, n_steps, greeks, &p->block, &p->k, &p->bps, dbg, &p->grid_smem, extra, vanna,
                                  &p->ppl, n_paths, &p->wide);
     if (st != LV_OK) return st;
-    p->smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, p->block, greeks, p->grid_smem, extra, p->ppl);
+    p->smem = lv::mc_smem_bytes(h->I, h->J, n_steps, staged_bins(h, n_steps, greeks, extra), p->block, greeks, p->grid_smem, extra, p->ppl);
     const int warps = p->block / 32;
     const int64_t tiles = (n_paths + lv::paths_per_tile(greeks, p->ppl) - 1) / lv::paths_per_tile(greeks, p->ppl);   // claimed by warps
     p->n_tiles = (int)tiles;
@@ -394,7 +410,7 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     // few tiles costs a whole one: of the upper half of the resident block counts
     // the one with the least rounds x warps. 2^20 paths on 152 SMs are 2.99 rounds
     // at nine blocks, 3.37 at eight and 3.85 at seven: 245, 257 and 257 us a call.
-    if (!greeks && !h->cfg_bps) {
+    if (!greeks && !h->cfg_bps && straight) {
         const int occ = p->bps;
         int64_t best = 0;
         for (int b = occ; 2 * b >= occ; --b) {
@@ -530,10 +546,12 @@ lv::McParams base_params(const lv_surface_s* h, const McCall& c, int k)
     P.acc_mode = h->acc_mode;
     P.method = LV_ADJ_REVERSE;
     P.bins = h->d_bins;
-    // the diagnostics kernel searches; the sweeps with checkpoints every 16 or 32 steps have
-    // one loop, which reads the bins where the call has them
-    if (k > 0 && !c.dbg_xN) lv::choose_cell_mode(P, h->sig_max, h->n_bins, h->bin_scale, h->bin_shift);
-    if (k > lv::kModelMaxK) P.cell_mode = lv::kCellSearch;
+    // the diagnostics kernel and the sweeps with checkpoints every 16 or 32 steps have one
+    // loop, which searches within the bins where the call has them
+    if (k > 0)
+        lv::choose_cell_mode(P, h->sig_max, staged_bins(h, c.n_steps, c.greeks, c.extra), h->bins_two, h->bin_scale,
+                             h->bin_shift);
+    if (k > lv::kModelMaxK || c.dbg_xN) P.cell_mode = lv::kCellSearch;
     return P;
 }
 
@@ -728,7 +746,7 @@ lv_status lv_surface_create(const double* spot_nodes, int32_t n_spot, const doub
         }
     }
     std::vector<float4> bins;
-    if (!h->log_uniform) bins = spot_bins(h->spot, &h->bin_scale, &h->bin_shift);
+    if (!h->log_uniform) bins = spot_bins(h->spot, &h->bin_scale, &h->bin_shift, &h->bins_two);
     h->n_bins = (int)bins.size();
     if (h->n_bins > 0) {
         if (cudaMalloc(&h->d_bins, sizeof(float4) * bins.size()) != cudaSuccess) {
@@ -911,7 +929,7 @@ lv_status lv_get_call_launch(lv_surface_t h, int32_t n_steps, int64_t n_paths, i
     if (n_paths < 1 || n_paths > 0x7fffffffLL) return fail(LV_EINVAL, "n_paths must be in [1, 2^31 - 1]");
     DeviceGuard g(h->device);
     Plan p;
-    p.wide = true;                        // a call whose cell index is bounded
+    p.wide = h->log_uniform || (h->bins_two && staged_bins(h, n_steps, greeks != 0, false) > 0);        // a call whose cell index is bounded
     lv_status st = make_plan(h, n_steps, n_paths, greeks != 0, false, &p);
     if (st != LV_OK) return st;
     *block = p.block;
@@ -1622,7 +1640,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
     // counters, the flag and the sums must start at zero (every other section is
     // written before it is read)
     LV_CUDA(cudaMemsetAsync(base, 0, scratch_header(h), h->stream));
-    const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, block, true, grid_smem, false, ppl);
+    const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, staged_bins(h, n_steps, true, false), block, true, grid_smem, false, ppl);
     LV_CUDA(lv::launch_mc(P, grid, block, k, true, smem, h->stream));
     return LV_OK;
 }

@@ -94,7 +94,7 @@ __device__ void build_params(const BookParams& B, int inst, McParams* out)
     P.N = o.N;
     P.rk = philox_keys((uint32_t)(run.seed & 0xffffffffu), (uint32_t)(run.seed >> 32));
     P.bins = B.bins + s.off_bins;
-    choose_cell_mode(P, s.sig_max, B.max_bins > 0 ? s.n_bins : 0, s.bin_scale, s.bin_shift);
+    choose_cell_mode(P, s.sig_max, B.max_bins > 0 ? s.n_bins : 0, s.bins_two != 0, s.bin_scale, s.bin_shift);
     P.stream_id = (uint32_t)o.stream_id;
     P.path_begin = 0;
     P.n_paths = o.n_paths;

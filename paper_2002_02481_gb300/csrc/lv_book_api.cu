@@ -392,6 +392,7 @@ lv_status lv_book_create(const lv_surface_t* surfaces, int32_t n_surfaces, const
         bs.s_hi = h->s_hi;
         bs.sig_max = h->sig_max;
         bs.n_bins = h->n_bins;
+        bs.bins_two = h->bins_two ? 1 : 0;
         bs.bin_scale = h->bin_scale;
         bs.bin_shift = h->bin_shift;
         bs.off_bins = n_bins;

@@ -276,7 +276,7 @@ struct SmemGrid {
     const float2* sig2;    // [Je][I-1]: (sigma_{i,j}, sigma_{i+1,j} - sigma_{i,j})
     const float* node;     // [I]
     const float2* ab;      // [I - 1]
-    const float4* bins;    // [n_bins] spot_bins (kCellBins)
+    const float4* bins;    // [n_bins] spot_bins
     const float* tdt;      // [N] step_tdt (kernels that compute d price / d T)
 };
 
@@ -308,9 +308,9 @@ __device__ __forceinline__ int bin_cell(const SmemGrid& g, int b, float S)
 //    where the clamped weight gives the same value);
 //  - kCellBins: on other grids from a table of equal bins in y, at most two
 //    nodes in each: the bin's first cell plus two comparisons with S;
-//  - kCellSearch: the same index from a conversion, from the bins, or from a binary
-//    search over the nodes, as the call says (the sweeps with checkpoints every 16 or 32
-//    steps, which are compiled once, and calls whose index has no bound).
+//  - kCellSearch: the same index from a conversion, or a binary search over the bin's
+//    cells, or over all where the call has no bins (the sweeps with checkpoints every 16 or 32
+//    steps, grids with more than two nodes in a bin, calls whose index has no bound).
 template <int CELL = kCellSearch>
 __device__ __forceinline__ int spot_cell(const McParams& P, const SmemGrid& g, float y, float S)
 {
@@ -322,9 +322,12 @@ __device__ __forceinline__ int spot_cell(const McParams& P, const SmemGrid& g, f
         const int i = __float2int_rd(fmaf(y, P.cell_scale, P.cell_shift));
         return min(max(i, 0), P.I - 2);
     }
-    if (P.n_bins > 0)
-        return bin_cell(g, clamp_floor(__fadd_rd(fmaf(y, P.cell_scale, P.cell_shift), kFloorShift), P.n_bins - 1), S);
     int lo = 0, hi = P.I - 2;
+    if (P.n_bins > 0) {
+        const float4 t = g.bins[clamp_floor(__fadd_rd(fmaf(y, P.cell_scale, P.cell_shift), kFloorShift), P.n_bins - 1)];
+        lo = __float_as_int(t.x);
+        hi = __float_as_int(t.w);
+    }
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (g.node[mid] <= S) lo = mid;

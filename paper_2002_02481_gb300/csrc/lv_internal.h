@@ -139,8 +139,8 @@ struct McParams {
 
 // Sets cell_mode, and for kCellBins the bins' scale, shift and count in place
 // of the cells'; every other field is set. sig_max is the grid's largest sigma.
-__host__ __device__ inline void choose_cell_mode(McParams& P, double sig_max, int n_bins, float bin_scale,
-                                                 float bin_shift)
+__host__ __device__ inline void choose_cell_mode(McParams& P, double sig_max, int n_bins, bool bins_two,
+                                                 float bin_scale, float bin_shift)
 {
     const bool on_s = (P.model & 2) != 0;
     P.cell_mode = kCellSearch;
@@ -150,7 +150,7 @@ __host__ __device__ inline void choose_cell_mode(McParams& P, double sig_max, in
             P.cell_mode = kCellUniform;
     } else if (n_bins > 0 &&
                index_bounded(on_s, P.N, P.x0, P.rdt, P.hdt, P.sqdt2, sig_max, bin_scale, bin_shift)) {
-        P.cell_mode = kCellBins;
+        if (bins_two) P.cell_mode = kCellBins;
         P.n_bins = n_bins;
         P.cell_scale = bin_scale;
         P.cell_shift = bin_shift;
@@ -281,7 +281,7 @@ struct BookSurf {
     int I, J, Je, log_uniform;
     float cell_scale, cell_shift, s_lo, s_hi;
     double sig_max;                                  // largest sigma of the grid (index_bounded)
-    int n_bins;
+    int n_bins, bins_two;
     float bin_scale, bin_shift;
     long long off_bins;
     long long off_sig2, off_node, off_ab, off_tau;   // offsets into the book's grid arrays
@@ -380,6 +380,7 @@ struct lv_surface_s {
     int log_uniform = 0;
     double sig_max = 0.0;            // largest sigma of the grid (index_bounded)
     float4* d_bins = nullptr;        // [n_bins] cell table of a grid not log-uniform (lv_api.cu spot_bins)
+    bool bins_two = false;           // no bin has more than two nodes
     int n_bins = 0;
     float bin_scale = 0.0f, bin_shift = 0.0f;
     float cell_scale = 0.0f, cell_shift = 0.0f, s_lo = 0.0f, s_hi = 0.0f;
