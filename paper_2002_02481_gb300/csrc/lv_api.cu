@@ -323,6 +323,13 @@ int staged_bins(const lv_surface_s* h, int32_t n_steps, bool greeks, bool extra)
     return lv::mc_smem_bytes(h->I, h->J, n_steps, h->n_bins, 128, greeks, false, extra, 2) <= 200 * 1024 ? h->n_bins : 0;
 }
 
+// The checkpoint interval a call's loops depend on: the tangent-ratio adjoint and the
+// second-order buckets keep no checkpoints, and run the same loops at every k.
+int loop_interval(const lv_surface_s* h, bool greeks, bool dbg, bool extra, bool vanna, int k)
+{
+    return vanna || (greeks && !dbg && !extra && h->adj_method == LV_ADJ_TANGENT) ? 4 : k;
+}
+
 // n_paths < 0: a call large enough for two paths per lane. `wide`: whether the call
 // may run 512-thread blocks (its cells need no search), set to whether it does.
 lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* block, int* k, int* bps,
@@ -350,6 +357,7 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     if (dbg) *k = 4;
     const int model = (h->interp == LV_INTERP_LOGS ? 1 : 0) | (h->scheme == LV_SCHEME_S ? 2 : 0);
     if ((model != 0 || extra) && *k > lv::kModelMaxK) *k = lv::kModelMaxK;
+    const int kk = loop_interval(h, greeks, dbg, extra, vanna, *k);
     // two paths per lane: the reverse sweep with checkpoints every 4 or 8 steps (every reading),
     // the main reading's tangent-ratio adjoint and its second-order buckets (no checkpoints)
     const bool pairs = greeks && !dbg && !extra &&
@@ -359,14 +367,14 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     if (!pairs && !ext_pairs) ppl = 1;
     if (!greeks) ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= kPricePairMinPathsPerSm * h->num_sms ? 2 : 1);
     // the cell mode of any call whose cell index is bounded (base_params)
-    const int cell = dbg || *k > lv::kModelMaxK ? lv::kCellSearch
+    const int cell = dbg || kk > lv::kModelMaxK ? lv::kCellSearch
                      : h->log_uniform           ? lv::kCellUniform
                      : bins > 0 && h->bins_two  ? lv::kCellBins
                                                 : lv::kCellSearch;
     // one block of 512 threads per SM instead of four of 128, if the call has work
     // for its warps, the grid fits once and no block was asked for
     const bool run_wide =
-        wide && *wide && greeks && *block == 128 && !own_block && !h->cfg_bps && *k == 4 && cell != lv::kCellSearch &&
+        wide && *wide && greeks && *block == 128 && !own_block && !h->cfg_bps && kk == 4 && cell != lv::kCellSearch &&
         n_paths >= kWideMinPathsPerSm * h->num_sms &&
         lv::mc_smem_bytes(h->I, h->J, n_steps, bins, lv::kWideBlock, greeks, true, extra, ppl) <= 200 * 1024;
     if (wide) *wide = run_wide;
@@ -574,7 +582,7 @@ lv_status run_mc(lv_surface_s* h, const McCall& c)
     st = ensure_scratch(h, p.total);
     if (st != LV_OK) return st;
     char* base = static_cast<char*>(h->d_scratch);
-    lv::McParams P = base_params(h, c, p.k);
+    lv::McParams P = base_params(h, c, loop_interval(h, c.greeks, c.dbg_xN != nullptr, c.extra, c.vanna, p.k));
     P.n_tiles = p.n_tiles;
     P.ppl = p.ppl;
     bind_header(P, base);
@@ -1620,7 +1628,7 @@ extern "C" lv_status lv_price_greeks_device_noalloc(lv_surface_t h, double S0, d
                                std::to_string(kStaticScratchBytes));
 
     McCall c{S0, r, K, T, n_steps, 0, n_paths, seed, 0u, true, false, d_out};
-    lv::McParams P = base_params(h, c, k);
+    lv::McParams P = base_params(h, c, loop_interval(h, true, false, false, false, k));
     P.n_tiles = (int)tiles;
     P.ppl = ppl;
     bind_header(P, base);

@@ -133,3 +133,17 @@ def test_forward_only_calls_keep_half_the_resident_blocks(lib):
     for tiles in [*range(1, 400, 7), *range(1216, 60000, 97), 32268, 34049, 56048]:
         assert 2 * s.get_call_launch(52, 64 * tiles, False)[2] >= occ, tiles
     s.close()
+
+
+def test_tangent_ratio_runs_the_same_at_every_interval(lib):
+    """It keeps no checkpoints: k = 16 and 32 leave it its cells and its 512-thread blocks."""
+    n = 1024 * _sms()
+    out = []
+    for k in (4, 16, 32):
+        s = _surface(lib, "tangent")
+        s.set_launch(0, k, 0)
+        assert s.get_call_launch(52, n)[0] == 512
+        out.append(s.price_greeks(100.0, 0.01, 100.0, 3.0, 52, n, 3))
+        s.close()
+    for p, d, _ in out[1:]:
+        assert abs(p - out[0][0]) <= 1e-12 * p and abs(d - out[0][1]) <= 1e-12 * abs(d)
