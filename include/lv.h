@@ -167,14 +167,14 @@ lv_status lv_set_launch(lv_surface_t h, int32_t block, int32_t k, int32_t blocks
  * paths interleaved: two independent dependency chains per thread, the
  * per-step grid data loaded once for both, and on the main reading their
  * binary32 arithmetic in packed pairs where that keeps the occupancy); 0 keeps
- * the tuned value, or the default: 2 for calls of at least 1,536 paths per SM
- * (233,472 on 152 SMs), one and a half pairs of tiles per resident warp, else 1.
+ * the tuned value, or the default: 2 for calls of at least 6,144 paths per SM
+ * (933,888 on 152 SMs), six pairs of tiles per resident warp, else 1.
  * Two paths per lane exist for the reverse sweep with checkpoints every 4
  * or 8 steps (every reading of the scheme), the main reading's tangent-ratio
- * adjoint and its second-order buckets; rho and d price / d T take two from
- * 6,144 paths per SM on, where the SM runs one 512-thread block. Elsewhere the
- * call runs one. The results do not
- * depend on it beyond reduction-order rounding.
+ * adjoint and its second-order buckets, and with rho and d price / d T where
+ * the SM runs one 512-thread block. Elsewhere the call runs one. lv_price, whose
+ * default is 2 from 200 paths per SM on, takes a 1 or 2 set here as well. The
+ * results do not depend on it beyond reduction-order rounding.
  * lv_get_paths_per_lane reads back the value the next call with n_steps steps
  * and n_paths >= 1 paths will use. */
 lv_status lv_set_paths_per_lane(lv_surface_t h, int32_t ppl);

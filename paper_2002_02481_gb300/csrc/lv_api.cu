@@ -248,9 +248,16 @@ std::string adjoint_tune_key(const lv_surface_s* h, int32_t n_steps)
            "|N2^" + std::to_string(nb);
 }
 
-// Shared memory a block may use and still leave room for the five resident
-// blocks the register budget allows; larger grids are read through L1.
-constexpr size_t kGridSmemLimit = 44 * 1024;
+// Shared memory a block may use and still leave room for the four resident
+// blocks the register budget allows; grids that need more are read through L1. 156
+// steps, read through L1 and staged: 60 x 70 log-spaced nodes 2^14 paths 74.0 and 62.1 us, 2^16 109
+// and 101, forward only on irregular nodes 48.2 and 36.1; 60 x 72, 128-thread blocks, 2^20 paths 657
+// and 588 us. Forward-only blocks, nine on an SM by their registers, gain too (60 x 80, 2^20
+// paths: 284 and 239 us; irregular 366 and 368).
+constexpr size_t kGridSmemLimit = 55 * 1024;
+// The sweep with checkpoints every 16 steps spills, and wants more of the L1 left (60 x 80 nodes,
+// 70,000 paths, read through L1 and staged: 144 and 167 us; 60 x 72, 2^18 paths 336 and 302).
+constexpr size_t kGridSmemLimitSpills = 48 * 1024;
 
 // extra: the adjoint kernel that also sums d V / d r and d V / d T (reverse
 // sweep, binary64 level 2, k = 4 or 8).
@@ -275,18 +282,15 @@ void occ_store(const OccKey& key, int occ)
     g_occ[key] = occ;
 }
 
-// A call of at least this many paths per SM runs two paths per lane unless
-// told otherwise: one and a half pairs of 32-path tiles for each of the 16 warps
-// of the adjoint kernel resident on an SM. Measured on a GB300 (30 x 60 grid, 156
-// steps, k = 4; one and two paths per lane): 2^18 paths 182 and 181 us, 500,000 297
-// and 290, 2^20 578 and 567, 2^22 1,980 and 1,880; below, a pair leaves warps idle
-// (2^17 121 and 134).
-constexpr int64_t kPairMinPathsPerSm = 3 * 32 * 16;
-
-// The kernel that also sums d V / d r and d V / d T has fewer registers to spare for
-// the second path and pairs later: 2^18 paths 185 us at one and 195 at two, 500,000 300 and
-// 321, 2^20 557 and 545, 2^22 2,012 and 1,939 (an irregular grid, 2^20: 666 and 633).
-constexpr int64_t kExtPairMinPathsPerSm = 4 * kPairMinPathsPerSm;
+// A call of at least this many paths per SM runs two paths per lane unless told
+// otherwise: six pairs of 32-path tiles for each of the sixteen warps on an SM. In
+// 512-thread blocks, 30 x 60 nodes, 156 steps, one and two paths per lane: 2^18 paths 178 and
+// 184 us, 500,000 284 and 305, 600,000 328 and 326, 800,000 420 and 431, 900,000 463 and 458, 2^20 532
+// and 519, 2^22 1,912 and 1,845; with d V / d r and d V / d T 500,000 306 and 322, 900,000 500 and 481;
+// second-order buckets 500,000 340 and 349, 900,000 560 and 542. Below six pairs a warp's last round
+// is too large a part of its work; an irregular grid pairs well from 600,000 paths on (399 and
+// 383, 500,000 346 and 361).
+constexpr int64_t kPairMinPathsPerSm = 6 * 64 * 16;
 
 // The forward-only kernel runs two paths per lane from this many paths per SM on:
 // below, one path per lane has the shorter chain (2^14 paths on the 30 x 60 grid, 156
@@ -339,8 +343,7 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     const int bins = staged_bins(h, n_steps, greeks, extra);
     *block = h->cfg_block ? h->cfg_block : 128;
     *k = greeks ? (h->cfg_k ? h->cfg_k : 4) : 4;
-    const int64_t pair_min = extra ? kExtPairMinPathsPerSm : kPairMinPathsPerSm;
-    int ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= pair_min * h->num_sms ? 2 : 1);
+    int ppl = h->cfg_ppl ? h->cfg_ppl : (n_paths < 0 || n_paths >= kPairMinPathsPerSm * h->num_sms ? 2 : 1);
     bool own_block = h->cfg_block != 0;              // the block was asked for, or tuned
     const char* cache = std::getenv("LV_TUNE_CACHE");
     if (greeks && !dbg && !h->cfg_block && !h->cfg_k && !h->cfg_ppl && cache && *cache) {
@@ -383,7 +386,8 @@ lv_status choose_launch(lv_surface_s* h, int32_t n_steps, bool greeks, int* bloc
     else if (ext_pairs)
         ppl = 1;
     const bool gs =
-        run_wide || lv::mc_smem_bytes(h->I, h->J, n_steps, bins, *block, greeks, true, extra, ppl) <= kGridSmemLimit;
+        run_wide || lv::mc_smem_bytes(h->I, h->J, n_steps, bins, *block, greeks, true, extra, ppl) <=
+                                    (kk > lv::kModelMaxK ? kGridSmemLimitSpills : kGridSmemLimit);
     if (ppl_out) *ppl_out = ppl;
     if (grid_smem) *grid_smem = gs;
     const size_t smem = lv::mc_smem_bytes(h->I, h->J, n_steps, bins, *block, greeks, gs, extra, ppl);

@@ -147,3 +147,16 @@ def test_tangent_ratio_runs_the_same_at_every_interval(lib):
         s.close()
     for p, d, _ in out[1:]:
         assert abs(p - out[0][0]) <= 1e-12 * p and abs(d - out[0][1]) <= 1e-12 * abs(d)
+
+
+def test_two_paths_per_lane_from_six_pairs_a_warp(lib):
+    s = _surface(lib, "greeks")
+    assert [s.get_paths_per_lane(52, n) for n in (6144 * _sms() - 1, 6144 * _sms())] == [1, 2]
+    s.close()
+
+
+@pytest.mark.parametrize("n_time", [80, 84, 88, 100])
+def test_grids_around_the_staging_limit(n_time, lib):
+    """60 spot nodes: 80 and 84 time rows fit beside four blocks' limit of 55 KB, 88 and 100 are read through L1."""
+    opt = W.Option(S0=100.0, r=0.01, K=100.0, T=3.0, n_steps=40, n_paths=2048, seed=6)
+    G.full_parity(W.seeded_skew_surface(4, n_spot=60, n_time=n_time), opt, lib, label=f"60 x {n_time}")
