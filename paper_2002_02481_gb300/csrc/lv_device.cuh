@@ -323,7 +323,7 @@ __device__ __forceinline__ int spot_cell(const McParams& P, const SmemGrid& g, f
         return min(max(i, 0), P.I - 2);
     }
     int lo = 0, hi = P.I - 2;
-    if (P.n_bins > 0) {
+    if (CELL != kCellNodes && P.n_bins > 0) {
         const float4 t = g.bins[clamp_floor(__fadd_rd(fmaf(y, P.cell_scale, P.cell_shift), kFloorShift), P.n_bins - 1)];
         lo = __float_as_int(t.x);
         hi = __float_as_int(t.w);
@@ -357,8 +357,9 @@ struct StepEval {
 // Bilinear sigma at (S_n, t_n), Sec. IV-D, from the path state x; the
 // slope only when WANT_SLOPE. With the ln-S weight the cell coefficients ab
 // are (1 / (y_{i+1} - y_i), -y_i / (y_{i+1} - y_i)) in y = log2 s, so that
-// d u / d ln S = ab.x log2(e); otherwise they are in S.
-template <bool WANT_SLOPE, int MODEL = 0, int CELL = kCellSearch>
+// d u / d ln S = ab.x log2(e); otherwise they are in S. ROW2: the time data's third
+// word is row j + 1 of the sigma pairs (the bump kernel).
+template <bool WANT_SLOPE, int MODEL = 0, int CELL = kCellSearch, bool ROW2 = false>
 __device__ __forceinline__ StepEval eval_sigma(const McParams& P, const SmemGrid& g, float x,
                                                const int4& tb)
 {
@@ -375,7 +376,7 @@ __device__ __forceinline__ StepEval eval_sigma(const McParams& P, const SmemGrid
     const float2 ab = g.ab[e.i];
     e.u = __saturatef(fmaf((MODEL & kModelLogWeight) ? y : e.S, ab.x, ab.y));
     const float2 lo = g.sig2[tb.x + e.i];      // time row j:     sigma_{i,j},   its spot step
-    const float2 hi = g.sig2[tb.x + e.i + (P.I - 1)];   // time row j + 1
+    const float2 hi = g.sig2[ROW2 ? tb.z + e.i : tb.x + e.i + (P.I - 1)];   // time row j + 1
     const float v = __int_as_float(tb.w);
     const float top = fmaf(e.u, lo.y, lo.x);
     const float bot = fmaf(e.u, hi.y, hi.x);

@@ -38,6 +38,7 @@ __host__ __device__ inline PhiloxKeys philox_keys(uint32_t k0, uint32_t k1)
 // search need every index of the call bounded (index_bounded).
 constexpr int kCellSearch = 0, kCellUniform = 1, kCellBins = 2;
 constexpr int kCellAny = 3, kCellNoBins = 4;       // chosen on the device (the book)
+constexpr int kCellNodes = 5;                      // the search without bins (the bump kernel, which stages none)
 
 // Whether |cell_scale y + cell_shift| stays below 2^22 on every path of a call,
 // y = log2 S. On ln S the path moves by at most |rdt| + hdt sigma^2 +
@@ -369,7 +370,7 @@ struct lv_surface_s {
     float2* d_sig = nullptr;         // [Je][I-1] pairs (sigma_{i,j}, sigma_{i+1,j} - sigma_{i,j})
     float* d_node = nullptr;
     float2* d_ab = nullptr;
-    float2* d_abl = nullptr;         // [I] cell coefficients of the ln-S weight, in y = log2 S
+    float2* d_abl = nullptr;         // [I] cell coefficients of the ln-S weight, in y = log2 S (behind the bins)
     double* d_tau = nullptr;
     double* d_spot64 = nullptr;      // [I] spot nodes, then [I] inverse gaps, binary64 (the binary64 kernels)
     bool gap_divide = false;         // some gap has no inverse (0 in d_spot64)
