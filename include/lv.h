@@ -19,9 +19,13 @@
  *    Work runs on the handle's CUDA stream (lv_set_stream; default: the
  *    legacy default stream). Entry points with host outputs synchronise that
  *    stream before returning; the *_device variants only enqueue work.
- *  - Arithmetic: paths in binary32; per-block accumulation of payoffs and
- *    vega buckets in binary64 (or Kahan-compensated binary32, see
- *    lv_set_accumulation); cross-block reduction in binary64, fixed order.
+ *  - Arithmetic: paths in binary32; payoffs accumulated per thread in
+ *    binary64 (or Kahan-compensated binary32, see lv_set_accumulation); a
+ *    path's bucket terms added in binary32 to sums shared by a few warps, which
+ *    go to binary64 (Kahan) sums of the block every few hundred paths, the four
+ *    corner sums around a node added in binary32 first; the blocks' sums added
+ *    in binary64 in the order in which the blocks arrive. The binary64 entry
+ *    points are binary64 throughout, their blocks added in a fixed order.
  *  - Random numbers: Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11) with
  *    key (seed & 0xffffffff, seed >> 32) and counter
  *    (step / 4, path & 0xffffffff, ((path >> 32) & 0xffff) | stream_id << 16, 0).

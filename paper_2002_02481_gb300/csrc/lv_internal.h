@@ -169,8 +169,6 @@ struct FinalizeParams {
     int I, J;
     long long n_paths;
     double S0;
-    int want_sums;         // 1: raw sums, 0: price / delta / stderr / vega
-    int extra;             // rows end with the sums of d V / d r and d V / d T
     double* chunks;        // [finalize_chunks(G)][row_words] stage-1 sums
     double* out;           // [3 + I * J]
     unsigned int* tile_counter;  // reset to 0

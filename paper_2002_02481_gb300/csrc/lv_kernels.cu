@@ -54,13 +54,11 @@ __global__ void __launch_bounds__(32) reduce_rows_kernel(const double* __restric
 
 // Level 3, stage 2: the chunks of one column summed in the same way (32 at a
 // time, the groups in order); outputs in the ABI layout (vega spot-major),
-// price statistics from the scalar sums. With `extra` the last two columns of
-// the rows are the sums of d V / d r and d V / d T, written after the vegas
-// (out[3 + I J], out[4 + I J]).
+// price statistics from the scalar sums.
 __global__ void __launch_bounds__(32) finalize_kernel(const double* __restrict__ chunks, int n_chunks, int row_words,
-                                                       int I, int J, long long n_paths, double S0, int want_sums,
-                                                       int extra, double* __restrict__ out,
-                                                       unsigned int* tile_counter, unsigned int* flag)
+                                                       int I, int J, long long n_paths, double S0,
+                                                       double* __restrict__ out, unsigned int* tile_counter,
+                                                       unsigned int* flag)
 {
     wait_prior_grid();
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
@@ -76,9 +74,7 @@ __global__ void __launch_bounds__(32) finalize_kernel(const double* __restrict__
     if (col >= row_words) return;
     const double P = (double)n_paths;
     if (col < 3) {
-        if (want_sums) {
-            out[col] = s;
-        } else if (col == 0) {
+        if (col == 0) {
             const double mean = s / P;
             const double var = n_paths > 1 ? (sv2 / P - mean * mean) * P / (P - 1.0) : 0.0;
             out[LV_OUT_PRICE_DEV] = mean;
@@ -90,14 +86,10 @@ __global__ void __launch_bounds__(32) finalize_kernel(const double* __restrict__
         if (col == 0 && flag) *flag = 0u;
         return;
     }
-    if (extra && col >= row_words - 2) {
-        out[3 + I * J + (col - (row_words - 2))] = want_sums ? s : s / P;
-        return;
-    }
     const int e = col - 3;             // time-major bucket j * I + i
     const int j = e / I, i = e - j * I;
     if (j >= J) return;                // padding row of a one-column grid
-    out[3 + i * J + j] = want_sums ? s : s / P;
+    out[3 + i * J + j] = s / P;
 }
 
 }  // namespace
@@ -158,7 +150,7 @@ cudaError_t launch_finalize(const FinalizeParams& f, cudaStream_t s)
     if (e != cudaSuccess) return e;
     cfg.gridDim = dim3((f.row_words + 31) / 32);
     return cudaLaunchKernelEx(&cfg, finalize_kernel, (const double*)f.chunks, n_chunks, f.row_words, f.I, f.J,
-                              f.n_paths, f.S0, f.want_sums, f.extra, f.out, f.tile_counter, f.flag);
+                              f.n_paths, f.S0, f.out, f.tile_counter, f.flag);
 }
 
 int finalize_chunks(int G) { return (G + kRowsPerChunk - 1) / kRowsPerChunk; }
