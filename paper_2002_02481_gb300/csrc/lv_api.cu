@@ -460,7 +460,7 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     if (greeks && !extra && !vanna && h->acc_mode == LV_ACC_KAHAN)
         o = round_up(o + sizeof(double) * total_warps * nIJ, 256);
     p->off_l1 = o;
-    if (greeks) o = round_up(o + sizeof(float4) * (size_t)p->grid * lv::bucket_arrays(warps) * (h->Je - 1) * (h->I - 1), 256);
+    if (greeks) o = round_up(o + sizeof(float4) * (size_t)p->grid * lv::bucket_arrays(warps) * lv::bucket_count(h->I, h->Je), 256);
     p->off_ckpt = o;
     o = round_up(o + sizeof(float) * (size_t)p->n_ck * total_warps * lv::ring_slots_per_warp() * p->ppl, 256);
     p->total = o;
@@ -1573,7 +1573,7 @@ size_t static_plan_bytes(const lv_surface_s* h, int grid, int block, int k, int 
     *off_part = o;   o = round_up(o + sizeof(double) * (size_t)grid * row_words, 256);
     *off_wrows = o;                                               // per-warp rows: Kahan mode only
     if (h->acc_mode == LV_ACC_KAHAN) o = round_up(o + sizeof(double) * warps * nIJ, 256);
-    *off_l1 = o;     o = round_up(o + sizeof(float4) * (size_t)grid * lv::bucket_arrays(block / 32) * (h->Je - 1) * (h->I - 1), 256);
+    *off_l1 = o;     o = round_up(o + sizeof(float4) * (size_t)grid * lv::bucket_arrays(block / 32) * lv::bucket_count(h->I, h->Je), 256);
     *off_ckpt = o;   o = round_up(o + sizeof(float) * n_ck * warps * lv::ring_slots_per_warp() * ppl, 256);
     return o;
 }

@@ -56,6 +56,8 @@ __host__ __device__ inline bool index_bounded(bool on_s, int n_steps, double x0,
 // Arrays of level-1 buckets of a block: one for every kBucketWarps warps (lv_mc.cuh warp_buckets).
 constexpr int kBucketWarps = 4;
 __host__ __device__ inline int bucket_arrays(int warps) { return (warps + kBucketWarps - 1) / kBucketWarps; }
+// Buckets of an array: the cells', then one a lane for the cell that the paths start in.
+__host__ __device__ inline int bucket_count(int I, int Je) { return (Je - 1) * (I - 1) + 32; }
 
 // Everything a Monte Carlo launch reads, passed by value as a
 // __grid_constant__ kernel parameter.
@@ -110,7 +112,7 @@ struct McParams {
     double* partials;      // [gridDim.x][row_words] per-block binary64 rows
     int row_words;         // 3 + Je * I (adjoint) or 3 (price only)
     double* warp_rows;     // [gridDim.x * warps][Je * I] per-warp level-2 rows
-    float4* l1;            // [gridDim.x][bucket_arrays][(Je - 1) (I - 1)] level-1 buckets: the corner sums of a cell
+    float4* l1;            // [gridDim.x][bucket_arrays][bucket_count] level-1 buckets: the corner sums of a cell
                            // (nodes (i, j), (i+1, j), (i, j+1), (i+1, j+1))
     float* ckpt;           // [n_ck][gridDim.x * warps * ring_slots_per_warp() * ppl] checkpoints of x
     int n_ck;

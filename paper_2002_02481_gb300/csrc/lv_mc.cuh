@@ -167,8 +167,14 @@ __device__ __forceinline__ void stage_grid(const McParams& P, unsigned char* sme
     __syncthreads();
 }
 
-// Cells with a level-1 bucket: (Je - 1) rows of I - 1.
-__host__ __device__ inline int n_cells(const McParams& P) { return (P.Je - 1) * (P.I - 1); }
+// The lower node (j I + i) of the cell the paths start in, for the launches whose lanes
+// have buckets of their own for it (OWN).
+template <bool OWN, int MODEL, int CELL>
+__device__ __forceinline__ int start_node(const McParams& P, const SmemGrid& g)
+{
+    if (!OWN) return 0;
+    return g.tab[0].y + start_cell<MODEL, CELL>(P, g) - g.tab[0].x;
+}
 
 // The level-1 buckets of a warp. A block has one array for every kBucketWarps of its
 // warps, dealt out in turn, so that the warps of one array drain at different times
@@ -183,7 +189,7 @@ __host__ __device__ inline int n_cells(const McParams& P) { return (P.Je - 1) * 
 __device__ __forceinline__ float4* warp_buckets(const McParams& P, int warp, int W)
 {
     const int G = bucket_arrays(W);
-    return P.l1 + (size_t)(blockIdx.x * G + warp % G) * n_cells(P);
+    return P.l1 + (size_t)(blockIdx.x * G + warp % G) * bucket_count(P.I, P.Je);
 }
 
 // The level-2 row of the warp: binary64 mode drains into the block's own row
@@ -203,7 +209,7 @@ template <int ACC>
 __device__ __forceinline__ void clear_buckets(const McParams& P, int* drained)
 {
     const int nIJ = P.Je * P.I, B = blockDim.x, W = B >> 5, tid = threadIdx.x;
-    const int nc = bucket_arrays(W) * n_cells(P);
+    const int nc = bucket_arrays(W) * bucket_count(P.I, P.Je);
     float4* l1 = P.l1 + (size_t)blockIdx.x * nc;
     for (int e = tid; e < nc; e += B) l1[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (ACC == 1) {
@@ -231,6 +237,19 @@ __device__ __forceinline__ void add_scalars(const AccSlot* acc0, int n, double* 
     }
 }
 
+// The warp's sums, in lane 0, of its lanes' corner sums.
+__device__ __forceinline__ void sum_start(const float4& v, double (&s)[4])
+{
+    s[0] = v.x;
+    s[1] = v.y;
+    s[2] = v.z;
+    s[3] = v.w;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q] += __shfl_down_sync(0xffffffffu, s[q], o);
+}
+
 // Adds what the block's buckets hold to the call's sums: per node and array the
 // corners of the up to four cells around it that were not drained yet and, if some
 // warp drained, the block's binary64 row (in Kahan mode its warps' rows). Four nodes
@@ -239,13 +258,17 @@ __device__ __forceinline__ void add_scalars(const AccSlot* acc0, int n, double* 
 // first, 2^14 paths on 20 x 10 nodes take 24.4 us a call instead of 23.3 and 2^18 on 30 x 60
 // 197 instead of 184, at the same rounding), each a sum of a quarter of the
 // contributions that a node's own bucket would hold; everything after in binary64.
-template <int ACC>
-__device__ __forceinline__ void fold_buckets(const McParams& P, const double* row, bool drained)
+template <int ACC, bool OWN>
+__device__ __forceinline__ void fold_buckets(const McParams& P, const double* row, bool drained, int start_node)
 {
     constexpr int kFly = 4;
-    const int I = P.I, nIJ = P.Je * I, B = blockDim.x, W = B >> 5, G = bucket_arrays(W), nc = n_cells(P);
+    const int I = P.I, nIJ = P.Je * I, B = blockDim.x, W = B >> 5, G = bucket_arrays(W), nc = bucket_count(I, P.Je);
     const float* c0 = reinterpret_cast<const float*>(P.l1 + (size_t)blockIdx.x * G * nc);
     const double* rows0 = P.warp_rows + (size_t)blockIdx.x * W * nIJ;
+    // the start cell, a lane's sums each: one warp an array (there are no more arrays than warps)
+    const int a0 = (int)(threadIdx.x >> 5);
+    const float4 start = OWN && a0 < G ? __ldcg(P.l1 + (size_t)(blockIdx.x * G + a0) * nc + start_bucket(P))
+                                : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (int e0 = threadIdx.x; e0 < nIJ; e0 += kFly * B) {
         double s[kFly];
 #pragma unroll
@@ -277,6 +300,12 @@ __device__ __forceinline__ void fold_buckets(const McParams& P, const double* ro
             }
             if (s[q] != 0.0) atomicAdd(&P.sums[3 + e], s[q]);
         }
+    }
+    if (OWN && a0 < G) {
+        double s[4];
+        sum_start(start, s);
+        if ((threadIdx.x & 31) == 0)
+            for (int q = 0; q < 4; ++q) atomicAdd(&P.sums[3 + start_node + (q & 1) + (q >> 1) * I], s[q]);
     }
 }
 
@@ -396,8 +425,8 @@ __device__ __forceinline__ int first_drain(const McParams& P, int warp, int W)
 // lock (flags[1]): as binary64 reductions, two a node, a drain took 28 us of its
 // warp's time when every warp drained. Returns false when another warp holds the
 // lock: the caller tries again after its next batch.
-template <int ACC>
-__device__ __forceinline__ bool drain_buckets(const McParams& P, float4* l1, double* wrow, int* flags)
+template <int ACC, bool OWN>
+__device__ __forceinline__ bool drain_buckets(const McParams& P, float4* l1, double* wrow, int* flags, int start_node)
 {
     constexpr int kFly = 8;
     const int lane = threadIdx.x & 31, I = P.I, C = I - 1, rows = P.Je - 1;
@@ -408,23 +437,37 @@ __device__ __forceinline__ bool drain_buckets(const McParams& P, float4* l1, dou
         __threadfence_block();
     }
     if (lane == 0) flags[0] = 1;
+    auto kahan = [&](int e, float f) {
+        float2* k = reinterpret_cast<float2*>(wrow) + e;
+        float2 p = *k;
+        const float y = f - p.y;
+        const float t = p.x + y;
+        p.y = (t - p.x) - y;
+        p.x = t;
+        *k = p;
+    };
+    if (OWN) {                                   // the start cell, a lane's sums each
+        double s[4];
+        sum_start(take4(l1 + start_bucket(P)), s);
+        if (lane == 0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int e = start_node + (q & 1) + (q >> 1) * I;
+                if (ACC == 1) kahan(e, (float)s[q]);
+                else __stcg(wrow + e, __ldcg(wrow + e) + s[q]);
+            }
+        }
+        __threadfence_block();
+        __syncwarp();
+    }
     for (int i0 = 0; i0 < C; i0 += 31) {
         const int i = i0 + lane;
         const bool cell = lane < 31 && i < C, node = i <= C;
         float carry = 0.0f;
         auto put = [&](int e, double d, float f) {
             if (f == 0.0f) return;
-            if (ACC == 1) {
-                float2* k = reinterpret_cast<float2*>(wrow) + e;
-                float2 p = *k;
-                const float y = f - p.y;
-                const float t = p.x + y;
-                p.y = (t - p.x) - y;
-                p.x = t;
-                *k = p;
-            } else {
-                __stcg(wrow + e, d + (double)f);
-            }
+            if (ACC == 1) kahan(e, f);
+            else __stcg(wrow + e, d + (double)f);
         };
         for (int j0 = 0; j0 <= rows; j0 += kFly) {          // node rows 0 .. rows
             float4 v[kFly];
@@ -525,7 +568,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
                 uint32_t c1, c2;
                 path_counter(P, rel, c1, c2);
                 float ra = 0.0f, ta = 0.0f;
-                xbar = reverse_path<CELL, KCK, MODEL, EXTRA, PPL == 2>(
+                xbar = reverse_path<CELL, KCK, MODEL, EXTRA, PPL == 2, WIDE>(
                     P, g, c1, c2, ckw + slot, cks, xbar, l1, &ra, &ta);
                 acc_add<ACC>(acc[2 * B], xbar);
                 if (EXTRA) {
@@ -537,7 +580,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
             __syncwarp();
-            if (++batches >= P.flush_every && drain_buckets<ACC>(P, l1, level2_row<ACC>(P), drained)) batches = 0;
+            if (++batches >= P.flush_every && drain_buckets<ACC, WIDE>(P, l1, level2_row<ACC>(P), drained, start_node<WIDE, MODEL, CELL>(P, g))) batches = 0;
             continue;
         }
         if (!more) break;
@@ -628,7 +671,8 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
     }
 
     __syncthreads();                           // after it nothing adds to this block's buckets
-    fold_buckets<ACC>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    fold_buckets<ACC, WIDE>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0,
+                            start_node<WIDE, MODEL, CELL>(P, g));
     add_scalars<ACC>(acc0, 3, P.sums);
     if (EXTRA) add_scalars<ACC>(acc0 + 3 * B, 2, P.sums + 3 + nIJ);
     finish_call<true, EXTRA>(P);
@@ -672,12 +716,12 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) tangent
                 const int e = (q_head + lane) & (kQcap - 1);
                 uint32_t c1, c2;
                 path_counter(P, q_rel[e], c1, c2);
-                tangent_scatter<CELL, MODEL>(P, g, c1, c2, q_c[e], l1);
+                tangent_scatter<CELL, MODEL, WIDE>(P, g, c1, c2, q_c[e], l1);
             }
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
             __syncwarp();
-            if (++batches >= P.flush_every && drain_buckets<ACC>(P, l1, level2_row<ACC>(P), drained)) batches = 0;
+            if (++batches >= P.flush_every && drain_buckets<ACC, WIDE>(P, l1, level2_row<ACC>(P), drained, start_node<WIDE, MODEL, CELL>(P, g))) batches = 0;
             continue;
         }
         if (!more) break;
@@ -751,7 +795,8 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) tangent
         tile = claim_tile(P, PPL);
     }
     __syncthreads();
-    fold_buckets<ACC>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    fold_buckets<ACC, WIDE>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0,
+                            start_node<WIDE, MODEL, CELL>(P, g));
     add_scalars<ACC>(acc0, 3, P.sums);
     finish_call<true>(P);
 }
@@ -794,12 +839,12 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) vanna_k
                 const int e = (q_head + lane) & (kQcap - 1);
                 uint32_t c1, c2;
                 path_counter(P, q_rel[e], c1, c2);
-                vanna_scatter<CELL>(P, g, c1, c2, q_c[e] * P.inv_S0, l1);
+                vanna_scatter<CELL, WIDE>(P, g, c1, c2, q_c[e] * P.inv_S0, l1);
             }
             q_head = (q_head + nb) & (kQcap - 1);
             q_count -= nb;
             __syncwarp();
-            if (++batches >= P.flush_every && drain_buckets<0>(P, l1, level2_row<0>(P), drained)) batches = 0;
+            if (++batches >= P.flush_every && drain_buckets<0, WIDE>(P, l1, level2_row<0>(P), drained, start_node<WIDE, 0, CELL>(P, g))) batches = 0;
             continue;
         }
         if (!more) break;
@@ -873,7 +918,8 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) vanna_k
         tile = claim_tile(P, PPL);
     }
     __syncthreads();
-    fold_buckets<0>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0);
+    fold_buckets<0, WIDE>(P, P.partials + (size_t)blockIdx.x * P.row_words, *drained != 0,
+                          start_node<WIDE, 0, CELL>(P, g));
     add_scalars<0>(acc0, 3, P.sums);
     finish_call<true>(P);
 }
