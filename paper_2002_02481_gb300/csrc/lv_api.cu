@@ -306,11 +306,13 @@ constexpr int64_t kPairMinPathsPerSm = 6 * 64 * 16;
 // steps: 30.9 and 34.5 us a call; 2^16 42.4 and 39.7; 2^20 259 and 224).
 constexpr int64_t kPricePairMinPathsPerSm = 200;
 
-// A call of at least this many paths per SM (one tile for each of its warps) runs
-// one 512-thread block per SM where it could run four or five of 128: every kernel
-// with buckets gains. 30 x 60 grid, 156 steps, 128 and 512 threads: second-order buckets
-// 2^17 paths 143 and 139 us, 500,000 363 and 346, 2^20 638 and 618, 2^22 2,280 and
-// 2,247; tangent ratio 2^17 127 and 123 us, 2^18 206 and 191, 2^20 588 and 556.
+// A call of at least this many paths per SM (one tile for each of its warps) runs one
+// 512-thread block per SM where it could run four or five of 128. 128 and 512 threads, 30 x
+// 60 grid, 156 steps: 2^17 paths 121 and 124 us, 2^18 181 and 178, 2^20 527 and 519; second-order
+// buckets 2^17 144 and 148, 2^18 226 and 220, 500,000 362 and 340; tangent ratio 2^17 128 and 133, 2^20
+// 587 and 568; 100 x 100 grid, 300 steps: 80,000 paths 333 and 240, 2^17 342 and 268. The line lies where every
+// warp has a tile: below two, small grids lose 2-3 %, but large ones gain a fifth, and from here on
+// 128-thread blocks put more paths into a bucket than one tile a warp (start_bucket).
 constexpr int64_t kWideMinPathsPerSm = 32 * 16;
 
 // The head of the handle's scratch, at the same place in every launch's layout:
@@ -430,7 +432,7 @@ lv_status make_plan(lv_surface_s* h, int32_t n_steps, int64_t n_paths, bool gree
     // The forward-only kernel's tiles all take the same time, so a last round with
     // few tiles costs a whole one: of the upper half of the resident block counts
     // the one with the least rounds x warps. 2^20 paths on 152 SMs are 2.99 rounds
-    // at nine blocks, 3.37 at eight and 3.85 at seven: 245, 257 and 257 us a call.
+    // at nine blocks, 3.37 at eight and 3.85 at seven, which take 12 us a call more.
     if (!greeks && !h->cfg_bps && straight) {
         const int occ = p->bps;
         int64_t best = 0;

@@ -513,8 +513,8 @@ __device__ __forceinline__ void log_cell_decision(const McParams& P, const SmemG
 // Calls f with the cell mode as a compile-time constant: CELL itself, or with
 // kCellAny the one in P, chosen once per path (kCellAny: any of the three,
 // kCellNoBins: no surface has bins). The single-option kernels are compiled per
-// mode: with all three loops in one kernel the adjoint took 0.633 ms instead
-// of 0.609 at 2^20 paths on a log-spaced grid.
+// mode: all three loops in one kernel made the adjoint 4 % slower at 2^20 paths on a
+// log-spaced grid.
 template <int C>
 struct CellMode {
     static constexpr int value = C;
@@ -540,9 +540,9 @@ __device__ __forceinline__ auto cell_dispatch(const McParams& P, F&& f)
 // the Philox products (FMA pipe) and the Box-Muller functions (transcendental
 // unit) then fill the latencies of the steps' loads instead of forming phases
 // of their own in which every warp waits for the same pipe (forward only, 2^20
-// paths: 0.265 -> 0.229 ms). UNROLL blocks to a body: two for the adjoint's pairs,
+// paths: a seventh of the time). UNROLL blocks to a body: two for the adjoint's pairs,
 // one where two only cost registers (forward only) or spill (the slope-carrying
-// loops: second-order buckets 0.731 ms with two, 0.675 with one). PIPE false: the
+// loops: second-order buckets 8 % slower with two). PIPE false: the
 // plain loop, for grids whose cell search branches inside the step anyway.
 // `first(blk)` runs before a block's steps, `gen(blk, z)` makes its normals,
 // `step(n, z)` is one step.
@@ -722,9 +722,9 @@ __device__ __forceinline__ void forward_path2(const McParams& P, const SmemGrid&
 // resolved in L2. Lanes in random cells of one grid retire 0.80-0.85 of these per
 // SM and cycle, against 0.24-0.29 flushes as four scalar reductions of per-node
 // buckets, which is about what the adjoint needs (0.22): the scalar form held it
-// back. Written out also because in a kernel that has a memory fence the compiler
-// turns atomicAdd into the returning form, whose replies took the adjoint from
-// 0.601 to 0.756 ms.
+// back (2^20 paths on 30 x 60 nodes: 587 us, 517 by cells; 2^18 213 and 184). Written out
+// also because in a kernel that has a memory fence the compiler turns atomicAdd into the
+// returning form, whose replies made the adjoint a quarter slower.
 __device__ __forceinline__ void red_add4(float4* p, float a, float b, float c, float d)
 {
     asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(a),

@@ -314,9 +314,10 @@ __device__ __forceinline__ void fold_buckets(const McParams& P, const double* ro
 // counters at zero for the next launch. It replaces two launches that summed the
 // blocks' rows: where the blocks end at different times their additions hide
 // behind the blocks still running, and only the last block's pass over the outputs
-// is left. 30 x 60 grid, 156 steps, 2^20 paths: 601 -> 584 us a call, forward only
-// 245 -> 234; 20 x 10 grid, 52 steps, 2^14 paths: 31.1 -> 26.7 us. The divisions by the path count are products with its inverse: a binary64 division
-// takes 551 cycles here. A nonzero flag (a vanishing 1 + g_n on a live path of the
+// is left. It took 17 us off a call of 2^20 paths on the 30 x 60 grid with 156 steps
+// (489 us now), 11 off a forward-only one (223) and 4.4 off 2^14 paths on the 20 x 10 grid
+// with 52 steps (23). The divisions by the path count are products with its inverse: a
+// binary64 division takes 551 cycles here. A nonzero flag (a vanishing 1 + g_n on a live path of the
 // tangent-ratio forms) makes every output NaN. Outputs in the ABI layout (vega
 // spot-major); EXTRA: d price / d r and d price / d T after the vegas.
 template <bool GREEKS, bool EXTRA = false>
@@ -398,8 +399,8 @@ __device__ __forceinline__ int first_tile(int n = 1)
 
 // Takes a bucket's four sums, leaving zeros. Word by word, as red_add4's reduction is
 // atomic per element: an exchange of all 16 bytes beside it would be a race of two
-// sizes, for which the memory model promises nothing. Both took 509 us at 2^20 paths (30 x 60
-// nodes, 156 steps).
+// sizes, for which the memory model promises nothing. At 2^20 paths (30 x 60 nodes, 156
+// steps) either took 509-510 us.
 __device__ __forceinline__ float4 take4(float4* p)
 {
     float* f = reinterpret_cast<float*>(p);
@@ -410,7 +411,7 @@ __device__ __forceinline__ float4 take4(float4* p)
 // in turn, every flush_every / W batches of the block's pace, and not all at once: the
 // four warps of an array then leave a few hundred live paths in a bucket. The first
 // drain comes half a turn later than that (four batches), which spares calls of two
-// batches a warp any drain (2^18 paths: 178 us, 188 with the turns from the start).
+// batches a warp any drain (2^18 paths: 177 us, 190 with the turns from the start).
 __device__ __forceinline__ int first_drain(const McParams& P, int warp, int W)
 {
     return warp * P.flush_every / W - P.flush_every / 2;
@@ -496,21 +497,22 @@ __device__ __forceinline__ bool drain_buckets(const McParams& P, float4* l1, dou
     return true;
 }
 
-// WIDE: one block of 512 threads per SM (choose_launch): the sixteen warps share one copy of the sigma
-// pairs in shared memory instead of reading them through L1, and one array of
-// level-1 buckets (24 MB instead of 95 MB over the chip on a 100 x 100 grid). 100 x
-// 100 grid, 1,260 steps, 2^22 paths: 18.2 -> 15.3 ms. Other grids gain from the
-// quarter of the stagings, folds and buckets (30 x 60, 156 steps, 2^20 paths, with
-// the drains in turn: 558 -> 510 us), so every call with a tile for each warp of
-// the chip runs this form unless its launch shape was chosen otherwise.
+// WIDE: one block of 512 threads per SM (choose_launch): the sixteen warps share one copy of
+// the sigma pairs in shared memory instead of reading them through L1 (100 x 100 grid,
+// 1,260 steps, 2^22 paths: 18.4 -> 16.1 ms; 300 steps, 2^17 paths 342 -> 268 us), and their
+// lanes have buckets of their own for the cell that the paths start in (start_bucket).
+// Grids that four blocks of 128 stage as well gain a little from the one staging and
+// the fewer blocks to fold (30 x 60, 156 steps: 2^20 paths 527 -> 519 us, tangent ratio 587 ->
+// 568; 500,000 second-order buckets 362 -> 340), so every call with a tile for each warp
+// of the chip runs this form unless its launch shape was chosen otherwise.
 //
 // Launch bound: the straight-line time loops (time_blocks, reverse_path) want
 // registers more than warps. Four blocks per SM at 124-128 registers against
-// five at 96 and six at 80, same code: 0.615, 0.643 and 0.684 ms at 2^20 paths on
-// the 30 x 60 grid with 156 steps, 2.06, 2.20 and 2.30 ms at 2^22 (the loops with
-// a bound check in every step, six blocks: 0.660 and 2.23 ms). One path per lane
-// needs 110 registers; held to five blocks it gains 1-4 % from 2^20 paths on, where
-// two paths per lane are faster still, and loses 4-5 % below.
+// five at 96 and six at 80, in 128-thread blocks before the bucket reductions of 16 bytes
+// (527 us at 2^20 paths now): 615, 643 and 684 us on the 30 x 60 grid with 156
+// steps, 2.06, 2.20 and 2.30 ms at 2^22. One path per lane needs 110 registers; held to
+// five blocks it gained 1-4 % from 2^20 paths on, where two paths per lane are
+// faster still, and lost 4-5 % below.
 //
 // PPL: paths per lane of a forward tile. With PPL = 2 a warp claims two
 // consecutive 32-path tiles and runs them interleaved (forward_path2: two
@@ -595,7 +597,7 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 4) adjoint
                 path_counter(P, rel_a, c1a, c2a);
                 path_counter(P, rel_b, c1b, c2b);
                 float ya, yb;
-                // packed under every reading (Euler on S: 2^20 paths 514 -> 511 us, 2^22 1,850 -> 1,832)
+                // packed under every reading (Euler on S, 2^22 paths: 1 % faster than scalar pairs)
                 forward_path2<CELL, KCK, true, MODEL, true>(P, g, c1a, c2a, c1b, c2b, ckw + slot_a,
                                                                              ckw + slot_b, cks, ya, yb);
                 auto add = [&](float V) {
@@ -927,11 +929,11 @@ __global__ void __launch_bounds__(WIDE ? kWideBlock : 128, WIDE ? 1 : 5) vanna_k
 // The forward pass alone. Bound by the FMA pipe (its 64-bit integer products
 // hold it for four cycles each) and the issue slots. With the straight-line
 // time loop, the index without a conversion and the round keys in the parameter
-// bank it runs 35 thread instructions per path-step (43 before): 0.229 ms at
-// 2^20 paths on the 30 x 60 grid with 156 steps, from 0.265 ms. Every tile takes
-// the same time, so the registers are held to nine blocks (2^20 paths: 245 us a
-// call against 257 with eight) and the launcher picks the blocks per SM that leave the last
-// round of tiles fullest (make_plan).
+// bank it runs 33 thread instructions per path-step, 43 with a check in every step: 223 us
+// a call of 2^20 paths on the 30 x 60 grid with 156 steps, from 291. Every tile takes
+// the same time, so the registers are held to nine blocks (12 us less than with eight
+// there) and the launcher picks the blocks per SM that leave the last round of tiles
+// fullest (make_plan).
 template <int ACC, bool GS, int MODEL, int CELL, int PPL>
 __global__ void __launch_bounds__(128, 9) price_kernel(const __grid_constant__ McParams P)
 {
