@@ -289,7 +289,7 @@ def other_workloads(lib, dev, ev0, ev1):
             single(f"precision {which} grid, 156 steps, 2^24 paths, level 2 {nm}", surf, opt, acc=acc)
     surf, opt = W.config_large()
     for k in (4, 32):
-        single(f"large 100x100, 1260 steps, 2^26 paths, k={k}", surf, opt, launch=(128, k, 0))
+        single(f"large 100x100, 1260 steps, 2^26 paths, k={k}", surf, opt, launch=(0, k, 0))
     # the book: 8 grids x 64 options, one persistent launch, graph replay
     handles = [lv.Surface.from_workload(sf, lib) for sf in W.book_surfaces()]
     items = W.book_items()
@@ -495,9 +495,8 @@ def run_ours(args):
         vals = [int(v) for v in args.launch.split(",")]
         S.set_launch(vals[0], vals[1], 0)
         S.set_paths_per_lane(vals[2] if len(vals) > 2 else 1)
-        tuned = (vals[0], vals[1], None)
     else:
-        tuned = S.tune(opt.S0, opt.r, opt.K, opt.T, opt.n_steps, P, opt.seed)
+        S.tune(opt.S0, opt.r, opt.K, opt.T, opt.n_steps, P, opt.seed)
     n_out = 3 + surf.n_spot * surf.n_time
     d_out = torch.zeros(n_out, dtype=torch.float64, device=dev)
     d_sums = torch.zeros(n_out, dtype=torch.float64, device=dev)
@@ -663,7 +662,7 @@ def run_ours(args):
             "warmup": max(3, args.warmup), "ms_per_step": ms_per_step, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": WORKLOAD, "grid": "30x60", "n_steps": opt.n_steps, "n_paths_per_gpu": P,
-                       "launch": {"block": tuned[0], "k": tuned[1], "paths_per_lane": ppl,
+                       "launch": {"block": blk, "k": kk, "paths_per_lane": ppl,
                                   "source": "--launch" if args.launch else "lv_tune"},
                        "l2": "256 MB buffer rewritten between timed steps (outside the timed region)",
                        "parallelism": f"path-range shards x{ws}" + (", one all-reduce of 3+1800 sums per step"
